@@ -101,10 +101,11 @@ typedef struct aps_graph {
 /* Work counters and phase times of the last aps_all_pairs / aps_query / batch call on
  * an index (all counts are exact; times are CUDA-event milliseconds). */
 typedef struct aps_stats {
-    int64_t visits;       /* posting-list entries Alg. 2 adds: on x's lists, y after x (self-join),
-                             |y| >= minsize when minsize is on */
+    int64_t visits;       /* entries of the join's posting lists that Alg. 2 adds: on x's lists, y
+                             after x (self-join), |y| >= minsize when minsize is on; lists that only
+                             update are left out where x has no candidate */
     int64_t candidates;   /* (x, y) pairs with a non-zero partial score */
-    int64_t verified;     /* candidates that passed upperbound and got dot(x, y') */
+    int64_t verified;     /* candidates that passed the prefix bound and got dot(x, y') */
     int64_t pairs;        /* pairs emitted */
     int64_t band;         /* pairs re-decided in float64 */
     int64_t evaluations;  /* similarity evaluations decided: sum over instances n(n-1)/2 */
@@ -113,8 +114,8 @@ typedef struct aps_stats {
     float ms_join;        /* join kernel launches only (last attempt) */
     float ms_sort;        /* output stage: count scan + gather into (i, j) order */
     float ms_total;       /* whole call */
-    int64_t entries_read; /* posting-list entries loaded by the join (visits plus the entries it
-                             reads and skips: minsize, and ids at or before x in x's first window) */
+    int64_t entries_read; /* posting-list entries on the lists the join walks (visits plus the entries
+                             it skips: minsize, ids at or before x in x's first window) */
 } aps_stats;
 
 typedef struct aps_index aps_index;
@@ -143,7 +144,7 @@ aps_status aps_build_index(const int64_t *indptr, const int32_t *idx, const floa
  * dot >= t (Alg. 1-2 with the all-pairs-2 bounds), sorted by (i, j).
  * flags: APS_NO_MINSIZE / APS_NO_REMSCORE / APS_NO_UPPERBOUND ablations and
  * APS_HOST_OUTPUT. Result buffers are allocated by the library; free with aps_pairs_free.
- * The first call on an index captures its join phase as a CUDA graph that later calls
+ * The second call on an index captures its join phase as a CUDA graph that later calls
  * replay; calls on one index must not overlap each other (aps_query may run meanwhile).
  * Errors: APS_EINVAL (NULL arguments or a batched index), APS_ENOMEM, APS_ECUDA,
  * APS_EOVERFLOW (the staging still overflowed after growing twice); *out is then empty. */
@@ -198,8 +199,9 @@ aps_status aps_index_info(const aps_index *index, int32_t *n, int32_t *m, int64_
  * device arrays i, j, score (capacity pairs each); on APS_OK *count pairs sorted by
  * (i, j) are in them. All scratch comes from one fixed 64 MiB device array inside the
  * library (held by every GPU that loads this part of the library until exit) and the
- * join uses at most 32 CTAs. Limits: the index's (vector, window) slots must fit the
- * arena with room left to stage pairs (else APS_EINVAL, before any work), and the pairs
+ * join uses at most 32 CTAs. Limits: the index's arena slots (n times the windows of 40960 / G
+ * ids that cover it, G from the tile table) must fit the arena with room left to stage pairs
+ * (else APS_EINVAL, before any work), and the pairs
  * must fit both the staging room and `capacity` (else APS_EOVERFLOW with *count = the
  * number of pairs). The current device must be the index's device, and i, j and score
  * must be device memory of that device (else APS_EINVAL). The first call on a device
@@ -262,9 +264,9 @@ aps_status aps_batch_all_pairs_csr(int32_t k, const int64_t *row_offsets, const 
                                    aps_stats *stats);
 
 /* ---- join tile shapes and the autotuner ------------------------------------------ */
-/* The join's tile shape for an instance of n vectors: G query groups per CTA (1, 2, 4 or
- * 8), each with a candidate window of 40960 / G ids in shared memory (the blocks of
- * Sec. 5.1.9 as CTA-level tiles). G is looked up by the instance's size bucket: bucket b
+/* The join's tile shape for an instance of n vectors: G = 1, 2, 4 or 8 (one warp per query
+ * vector with a candidate window in shared memory, the blocks of Sec. 5.1.9 as tiles; G = 1
+ * has the widest windows and the fewest warps). G is looked up by the instance's size bucket: bucket b
  * holds 1 + the previous bound <= n <= APS_TUNE_BOUND_b, with bounds 512, 1280, 2560,
  * 5120, 10240, 20480, 40960 and unbounded (aps_tune_bucket). The bucket bounds are the
  * work-split thresholds; the table is process-wide and read by every later index build
@@ -288,8 +290,8 @@ typedef struct aps_tune_report {
 
 /* The size bucket (0 .. APS_TUNE_BUCKETS-1) of an instance of n vectors. */
 int32_t aps_tune_bucket(int64_t n);
-/* The built-in table, the same in both columns: G = 8 up to 5120 vectors (one window),
- * 4 up to 10240, 2 above. (This and aps_get_tuning ignore a NULL out.) */
+/* The built-in table, the same in both columns: G = 8 up to 5120 vectors, 4 up to 10240, 2
+ * above. (This and aps_get_tuning ignore a NULL out.) */
 void aps_tuning_default(aps_tuning *out);
 /* The table in force for this process. */
 void aps_get_tuning(aps_tuning *out);

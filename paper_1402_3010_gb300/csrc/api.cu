@@ -212,10 +212,15 @@ aps_status aps_index_export(const aps_index *ix, int32_t *len, float *mw, int32_
     APS_TRY(export_array(split, d.split, ix->N, s));
     APS_TRY(export_array(qsplit, d.qsplit, ix->N, s));
     APS_TRY(export_array(mw_pre, d.mwpre, ix->N, s));
-    APS_TRY(export_array(list_ptr, d.lptr, ix->M + 1, s));
+    // the lists by split: the index's own, or built here where the join's are shorter
+    DBuf<int64_t> xl;
+    DBuf<int2> xp;
+    const bool own = ix->njoin == ix->nsuf;
+    if (!own && (list_ptr || post_id || post_w)) APS_TRY(export_postings(ix, xl, xp, s));
+    APS_TRY(export_array(list_ptr, own ? d.lptr : xl, ix->M + 1, s));
     if ((post_id || post_w) && ix->nsuf > 0) {
         std::vector<int2> tmp((size_t)ix->nsuf);
-        APS_CUDA(cudaMemcpyAsync(tmp.data(), d.post.p, sizeof(int2) * ix->nsuf, cudaMemcpyDeviceToHost, s));
+        APS_CUDA(cudaMemcpyAsync(tmp.data(), own ? d.post.p : xp.p, sizeof(int2) * ix->nsuf, cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
         const int32_t mask = (ix->k == 1 && ix->inst_h[0].packed) ? 0x00ffffff : 0x7fffffff;
         for (int64_t q = 0; q < ix->nsuf; q++) {

@@ -273,6 +273,12 @@ __global__ void k_canon_gather(const uint64_t *__restrict__ keys, const uint32_t
 // split may fall one component apart from a sequential one; either is a valid split (the
 // bound of the unindexed prefix stays below t up to rounding, which the float64 band of
 // the decisions covers).
+//
+// With l2, the join's own prefix and create boundary reach to the first component where the
+// norm of the leading components, summed in float32 with every operation rounded up, can
+// reach t (times 1.0025 in the square for the norm tolerance of both vectors): no row scores
+// t on such a prefix, so a match has a later component in common. On the 200k power-law set
+// this takes the visits from 1.2e10 to about 3.8e9 and the candidates from 1.6e9 to 6e8.
 __device__ __forceinline__ double warp_incl_scan_f64(double v, int lane) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -282,49 +288,79 @@ __device__ __forceinline__ double warp_incl_scan_f64(double v, int lane) {
     return v;
 }
 
+__device__ __forceinline__ float warp_incl_scan_ru(float v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v = __fadd_ru(v, y);
+    }
+    return v;
+}
+
+// The smallest 4-bit code c with c * PN4_STEP >= pn (the bound stays a bound).
+__device__ __forceinline__ int pn4_code(float pn) {
+    int c = (int)ceilf(__fdiv_ru(pn, PN4_STEP));
+    if ((double)c * (double)PN4_STEP < (double)pn) c++;
+    return min(max(c, 0), 15);
+}
+
 __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
                         const float *__restrict__ cval, const float *__restrict__ mwr,
                         const int32_t *__restrict__ vinst, const InstDesc *__restrict__ inst, int64_t N,
-                        uint32_t flags, int32_t *split, int32_t *qsplit, float *mwpre, float *pnorm, int64_t M,
-                        uint64_t *pkeys, uint32_t *pvals, unsigned long long *nsuf) {
+                        uint32_t flags, bool l2, const float *__restrict__ mw, int32_t *split, int32_t *qsplit,
+                        float *mwpre, int4 *vmeta, int4 *vcand, uint8_t *code, int64_t M, uint64_t *pkeys,
+                        uint32_t *pvals, unsigned long long *nsuf, unsigned long long *njoin) {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long nsuf_w = 0;  // this warp's indexed components (lane 0)
+    unsigned long long nsuf_w = 0, njoin_w = 0;  // this warp's indexed components (lane 0)
     for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < N; x += nwarps) {
         const InstDesc &I = inst[vinst[x]];
         const double t = (double)I.t;
+        const float t2 = __fmul_rd(I.t, I.t);
         const int64_t a = cptr[x], b = cptr[x + 1];
         const int32_t L = (int32_t)(b - a);
-        const bool need_cs = (flags & APS_QUERYABLE) != 0;  // the norm-bound split only for queryable indexes
-        int32_t qs = L, cs = L;
+        const bool need_cs = (flags & APS_QUERYABLE) != 0;  // the norm-bound split of queryable indexes
+        int32_t qs = L, cs = L, ls = L;
         double bmw = 0.0, ss = 0.0;  // sums of the components before this step
-        for (int64_t base = a; base < b && (qs == L || (need_cs && cs == L)); base += 32) {
+        float ssu = 0.f;             // the squares again, rounded up
+        for (int64_t base = a; base < b && (qs == L || (need_cs && cs == L) || (l2 && ls == L)); base += 32) {
             const int64_t p = base + lane;
-            double pr = 0.0, sq = 0.0;
+            float c = 0.f, mwc = 0.f;
             if (p < b) {
-                const double v = (double)cval[p];
-                pr = v * (double)mwr[(int64_t)I.rbase + crank[p]];
-                sq = v * v;
+                c = cval[p];
+                mwc = mwr[(int64_t)I.rbase + crank[p]];
             }
-            const double bi = bmw + warp_incl_scan_f64(pr, lane);
-            const unsigned hit = __ballot_sync(0xffffffffu, p < b && bi >= t);
-            if (qs == L && hit) qs = (int32_t)(base - a) + __ffs(hit) - 1;
-            bmw = __shfl_sync(0xffffffffu, bi, 31);
-            if (need_cs) {
-                const double si = ss + warp_incl_scan_f64(sq, lane);
+            const int32_t at = (int32_t)(base - a);
+            if (qs == L) {
+                const double bi = bmw + warp_incl_scan_f64((double)c * (double)mwc, lane);
+                const unsigned hit = __ballot_sync(0xffffffffu, p < b && bi >= t);
+                if (hit) qs = at + __ffs(hit) - 1;
+                bmw = __shfl_sync(0xffffffffu, bi, 31);
+            }
+            if (need_cs && cs == L) {
+                const double si = ss + warp_incl_scan_f64((double)c * (double)c, lane);
                 const unsigned hc = __ballot_sync(0xffffffffu, p < b && si * (1.0 + 2e-3) >= t * t);
-                if (cs == L && hc) cs = (int32_t)(base - a) + __ffs(hc) - 1;
+                if (hc) cs = at + __ffs(hc) - 1;
                 ss = __shfl_sync(0xffffffffu, si, 31);
             }
+            if (l2 && ls == L) {
+                const float si = __fadd_ru(ssu, warp_incl_scan_ru(__fmul_ru(c, c), lane));
+                const unsigned hl = __ballot_sync(0xffffffffu, p < b && __fmul_ru(si, 1.0025f) >= t2);
+                if (hl) ls = at + __ffs(hl) - 1;
+                ssu = __shfl_sync(0xffffffffu, si, 31);
+            }
         }
-        const int32_t sp = (flags & APS_NO_PARTIAL_INDEX) ? 0 : ((flags & APS_QUERYABLE) ? cs : qs);
-        // maxweight(x') and an upper bound of ||x'||_2 (float32 with every operation rounded
-        // up, so the bound can only come out above the exact norm; times 1 + 1.1e-3 for the
-        // 1e-3 norm tolerance of the vectors it will be dotted with)
+        const int32_t sp = (flags & APS_NO_PARTIAL_INDEX) ? 0 : (need_cs ? cs : qs);
+        // the join's prefix (external queries only obey the norm bound) and create boundary
+        const int32_t js = (l2 && !need_cs) ? max(sp, ls) : sp;
+        const int32_t jq = l2 ? max(qs, ls) : qs;
+        // maxweight(x') of the split and an upper bound of the join prefix's norm (float32 with
+        // every operation rounded up, so the bound can only come out above the exact norm;
+        // times 1 + 1.1e-3 for the 1e-3 norm tolerance of the vectors it will be dotted with)
         float best = 0.f, pss = 0.f;
-        for (int64_t p = a + lane; p < a + sp; p += 32) {
+        for (int64_t p = a + lane; p < a + js; p += 32) {
             const float c = cval[p];
-            best = fmaxf(best, c);
+            if (p < a + sp) best = fmaxf(best, c);
             pss = __fmaf_ru(c, c, pss);
         }
 #pragma unroll
@@ -333,21 +369,47 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
             pss = __fadd_ru(pss, __shfl_xor_sync(0xffffffffu, pss, o));
         }
         if (lane == 0) {
+            const float pn = js ? __fmul_ru(__fsqrt_ru(pss), 1.0011f) : 0.f;
+            const int32_t rlim = js < L ? crank[a + js] : 0x7fffffff;
             split[x] = sp;
             qsplit[x] = qs;
             mwpre[x] = best;
-            pnorm[x] = sp ? __fmul_ru(__fsqrt_ru(pss), 1.0011f) : 0.f;
+            vmeta[x] = make_int4((int32_t)a, L, jq, __float_as_int(mw[x]));
+            vcand[x] = make_int4((int32_t)a, js, rlim, __float_as_int(pn));
+            code[x] = (uint8_t)((rank_bucket(rlim) >> 2) << 4 | pn4_code(pn));
             nsuf_w += (unsigned long long)(L - sp);
+            njoin_w += (unsigned long long)(L - js);
         }
-        // the row's posting keys: a suffix entry its global rank, a prefix entry a sentinel
+        // the row's posting keys: an indexed entry its global rank, a prefix entry a sentinel
         // past the last rank (it sorts last); the value is the entry's index. The sort is
         // stable and entries arrive in row order, so every list comes out in increasing id.
         for (int64_t p = a + lane; p < b; p += 32) {
-            pkeys[p] = (p - a >= sp) ? (uint64_t)I.rbase + (uint64_t)crank[p] : (uint64_t)M;
+            pkeys[p] = (p - a >= js) ? (uint64_t)I.rbase + (uint64_t)crank[p] : (uint64_t)M;
             pvals[p] = (uint32_t)p;
         }
     }
     if (lane == 0 && nsuf_w) atomicAdd(nsuf, nsuf_w);
+    if (lane == 0 && njoin_w) atomicAdd(njoin, njoin_w);
+}
+
+// Posting keys by a given split (for the exported lists), one thread per component.
+__global__ void k_post_keys(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
+                            const int32_t *__restrict__ erow, const int32_t *__restrict__ vinst,
+                            const InstDesc *__restrict__ inst, const int32_t *__restrict__ split, int64_t nnz,
+                            int64_t M, uint64_t *pkeys, uint32_t *pvals) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t x = erow[p];
+        pkeys[p] = (p - cptr[x] >= split[x]) ? (uint64_t)inst[vinst[x]].rbase + (uint64_t)crank[p] : (uint64_t)M;
+        pvals[p] = (uint32_t)p;
+    }
+}
+
+// The row of every component.
+__global__ void k_rows_of(const int64_t *__restrict__ cptr, int64_t N, int32_t *erow) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < N; x += nwarps)
+        for (int64_t p = cptr[x] + lane; p < cptr[x + 1]; p += 32) erow[p] = (int32_t)x;
 }
 
 __global__ void k_post_fill(const uint32_t *__restrict__ vals, const int32_t *__restrict__ erow,
@@ -377,49 +439,36 @@ __global__ void k_lptr(const uint64_t *__restrict__ keys, int64_t nsuf, int64_t 
     }
 }
 
-// Interleaved rows and per-vector metadata read by the join.
-__global__ void k_pack(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
-                       const float *__restrict__ cval, const int32_t *__restrict__ len,
-                       const int32_t *__restrict__ split, const float *__restrict__ mwpre,
-                       const float *__restrict__ pnorm, const int32_t *__restrict__ vinst,
-                       const InstDesc *__restrict__ inst, int64_t N, int64_t nnz, int2 *crow, int4 *vmeta,
-                       int4 *vcand, uint32_t *pn4) {
+// Interleaved rows read by the join.
+__global__ void k_pack(const int32_t *__restrict__ crank, const float *__restrict__ cval, int64_t nnz, int2 *crow) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += stride)
         crow[p] = make_int2(crank[p], __float_as_int(cval[p]));
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < N; x += stride) {
-        vmeta[x] = make_int4((int32_t)cptr[x], len[x], split[x], __float_as_int(mwpre[x]));
-        vcand[x] = make_int4((int32_t)cptr[x], split[x], __float_as_int(mwpre[x]), __float_as_int(pnorm[x]));
-        // the smallest 4-bit code c with c * PN4_STEP >= ||x'||_2 (the bound stays a bound)
-        const double pn = (double)pnorm[x];
-        int c = (int)ceil(pn / (double)PN4_STEP);
-        if ((double)c * (double)PN4_STEP < pn) c++;
-        c = min(max(c, 0), 15);
-        const InstDesc &I = inst[vinst[x]];
-        const int64_t lx = x - I.vbase;
-        if (c) atomicOr(&pn4[I.pbase + (lx >> 3)], (uint32_t)c << (4 * (lx & 7)));
-    }
 }
 
-// Window offsets inside each list of a multi-window instance: w[i] = the offset in list R
-// of its first entry with local id >= i * W (lists are in increasing id; binary search).
-__global__ void k_wptr(const InstDesc *__restrict__ inst, int k, int64_t M, const int64_t *__restrict__ lptr,
-                       const int2 *__restrict__ post, int32_t *wptr) {
-    for (int64_t R = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; R < M; R += (int64_t)gridDim.x * blockDim.x) {
-        const InstDesc &I = inst[inst_of_rank(inst, k, R)];
+// Where the windows of a multi-window instance begin inside each list: w[i] = the position in
+// post of list R's first entry with local id >= i * W (lists are in increasing id; binary
+// search). One warp per list of one instance (blockIdx.y), the windows over its lanes.
+__global__ void k_wptr(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ lptr,
+                       const int2 *__restrict__ post, uint32_t *wptr) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int q = blockIdx.y; q < k; q += gridDim.y) {
+        const InstDesc &I = inst[q];
         if (I.nw <= 1) continue;
         const int32_t idmask = I.packed ? 0x00ffffff : 0x7fffffff;
-        const int64_t a = lptr[R], b = lptr[R + 1];
-        int32_t *w = wptr + I.wbase + (R - I.rbase) * (I.nw + 1);
-        int64_t lo = a;
-        for (int i = 0; i <= I.nw; i++) {
-            const int32_t bound = i * I.W;
-            int64_t hi = b;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if ((post[mid].x & idmask) < bound) lo = mid + 1; else hi = mid;
+        for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < I.m; r += nwarps) {
+            const int64_t a = lptr[I.rbase + r], b = lptr[I.rbase + r + 1];
+            uint32_t *w = wptr + I.wbase + r * (I.nw + 1);
+            for (int i = lane; i <= I.nw; i += 32) {
+                const int64_t bound = (int64_t)i * I.W;
+                int64_t lo = a, hi = b;
+                while (lo < hi) {
+                    const int64_t mid = (lo + hi) >> 1;
+                    if ((post[mid].x & idmask) < bound) lo = mid + 1; else hi = mid;
+                }
+                w[i] = (uint32_t)lo;
             }
-            w[i] = (int32_t)(lo - a);
         }
     }
 }
@@ -427,8 +476,8 @@ __global__ void k_wptr(const InstDesc *__restrict__ inst, int k, int64_t M, cons
 // Join work list: every vector with later candidates in its instance, keyed by
 // (class, decreasing estimated cost) so that the persistent join takes the most expensive
 // queries first (least-loaded-first idea of the vertical algorithm's binning). Classes 0-3
-// are the instance's tile shape (G = 1, 2, 4, 8 query groups per CTA); class 4 holds the
-// vectors with one or two components, which the join streams one warp per vector.
+// are the instance's tile shape (G = 1, 2, 4, 8); class 4 holds the vectors with one or two
+// components, which the join streams one warp per vector.
 __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
                             const int64_t *__restrict__ lptr, const int32_t *__restrict__ vinst,
                             const InstDesc *__restrict__ inst, int64_t N, uint64_t *keys, uint32_t *vals,
@@ -463,7 +512,8 @@ __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__r
             const double cost = (double)lsum * later / (double)I.n + later / 8.0 + 32.0;
             // decreasing cost inside the class, in 24 bits (the costliest saturate together)
             const uint64_t c = cost >= 16777215.0 ? 0xffffffull : (uint64_t)cost;
-            const int cls = b - a <= 2 ? 4 : I.G == 1 ? 0 : I.G == 2 ? 1 : I.G == 4 ? 2 : 3;
+            // (a merge of two long lists would be one warp's serial tail: those go by windows)
+            const int cls = b - a <= 1 || (b - a == 2 && lsum <= 8192) ? 4 : I.G == 1 ? 0 : I.G == 2 ? 1 : I.G == 4 ? 2 : 3;
             keys[x] = ((uint64_t)cls << 24) | (0xffffffull - c);
             vals[x] = (uint32_t)x;
             atomicAdd(&ccount[cls], 1ull);
@@ -499,7 +549,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     ix->stream = s;
     // ---- host-side layout of instances: ranks, windows, classes
     std::vector<InstDesc> inst = inst_in;
-    int64_t N = 0, M = 0, nqw = 0, nwptr = 0, npw = 0;
+    int64_t N = 0, M = 0, arena_slots = 0, nwptr = 0;
     int32_t maxm = 1, maxn = 1, maxnw = 1;
     // tile shape per instance: G query groups per CTA from the size-bucket table (its
     // queryable column for indexes built to answer queries)
@@ -510,14 +560,11 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         I.vbase = N;
         I.rbase = (int32_t)M;
         I.G = gtab[tune_bucket(I.n)];
-        I.W = JOIN_WMAX / I.G;
-        I.nw = I.n > 0 ? (int32_t)((I.n + I.W - 1) / I.W) : 0;
+        I.W = tile_window(I.G);
+        I.nw = I.n > 0 ? (int32_t)(((int64_t)I.n + I.W - 1) / I.W) : 0;
         I.packed = I.n < (1 << 24) ? 1 : 0;
-        I.qwbase = nqw;
         I.wbase = nwptr;
-        I.pbase = npw;
-        npw += 4 * (((int64_t)I.n + 31) / 32);  // 32 codes per 16 bytes, each instance aligned
-        nqw += (int64_t)I.n * I.nw;
+        arena_slots += (int64_t)I.n * (((int64_t)I.n * I.G + 40959) / 40960);
         if (I.nw > 1) nwptr += (int64_t)I.m * (I.nw + 1);
         N += I.n;
         M += I.m;
@@ -531,10 +578,15 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     }
     ix->N = N;
     ix->M = M;
-    ix->nqw = nqw;
+    ix->arena_slots = arena_slots;
     ix->nwptr = nwptr;
-    ix->npw = npw;
     ix->maxm = maxm;
+    ix->maxnw = maxnw;
+    // every bound on: the join may keep the norm-bounded prefixes to itself
+    ix->l2 = !(ix->flags & (APS_NO_PARTIAL_INDEX | APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
+    // A heavy vector's windows go to several warps where there are few vectors (2M slots at most)
+    // and enough windows for it: a vector's tables cost a unit about as much as a window does.
+    ix->parts = maxnw < 4 ? 1 : (int32_t)std::max<int64_t>(1, std::min<int64_t>({16, maxnw, ((int64_t)1 << 21) / std::max<int64_t>(N, 1)}));
     ix->inst_h = inst;
     IndexArrays &d = ix->d;
 
@@ -549,8 +601,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         return APS_EINVAL;
     }
     ix->nnz = nnz;
-    for (int i = 0; i < k; i++) inst[i].ebase = 0;
-
     APS_TRY(d.inst.alloc((size_t)k, s));
     APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
     APS_TRY(d.vinst.alloc((size_t)N, s));
@@ -646,7 +696,9 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         APS_LAUNCH_CHECK();
     }
     // ---- a3: partial-indexing split
-    APS_TRY(d.pnorm.alloc((size_t)std::max<int64_t>(N, 1), s));
+    APS_TRY(d.vmeta.alloc((size_t)std::max<int64_t>(N, 1), s));
+    APS_TRY(d.vcand.alloc((size_t)std::max<int64_t>(N, 1), s));
+    APS_TRY(d.code.alloc((size_t)std::max<int64_t>(N, 1), s));
     // the split also writes each row's posting keys for a4 (and counts the indexed components)
     DBuf<uint64_t> pkeys;
     DBuf<uint32_t> pvals;
@@ -654,41 +706,40 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     APS_TRY(pvals.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     unsigned long long *nsuf_d = err.p + 1;
     k_split<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N,
-                                                    ix->flags, d.split.p, d.qsplit.p, d.mwpre.p, d.pnorm.p, M,
-                                                    pkeys.p, pvals.p, nsuf_d);
+                                                    ix->flags, ix->l2, d.mw.p, d.split.p, d.qsplit.p, d.mwpre.p,
+                                                    d.vmeta.p, d.vcand.p, d.code.p, M, pkeys.p, pvals.p, nsuf_d,
+                                                    nsuf_d + 2);
     APS_LAUNCH_CHECK();
     // ---- a4: suffix inverted index
     {
         DBuf<uint64_t> &keys = pkeys;
         DBuf<uint32_t> &vals = pvals;
-        unsigned long long nsuf_h = 0;
-        APS_CUDA(cudaMemcpyAsync(&nsuf_h, nsuf_d, sizeof(nsuf_h), cudaMemcpyDeviceToHost, s));
+        unsigned long long cnt3[3] = {0, 0, 0};  // by split, (longest row), in the join's lists
+        APS_CUDA(cudaMemcpyAsync(cnt3, nsuf_d, sizeof(cnt3), cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
-        ix->nsuf = (int64_t)nsuf_h;
+        ix->nsuf = (int64_t)cnt3[0];
+        ix->njoin = (int64_t)cnt3[2];
         if (nnz > 0) APS_TRY(sort_pairs(keys.p, vals.p, nnz, bits_for((uint64_t)M), s));
-        APS_TRY(d.post.alloc((size_t)std::max<int64_t>(ix->nsuf, 1), s));
+        APS_TRY(d.post.alloc((size_t)std::max<int64_t>(ix->njoin, 1), s));
         APS_TRY(d.wptr.alloc((size_t)std::max<int64_t>(nwptr, 1), s));
-        if (nwptr) APS_CUDA(cudaMemsetAsync(d.wptr.p, 0, sizeof(int32_t) * nwptr, s));
-        if (ix->nsuf > 0) {
-            k_post_fill<<<grid_for(ix->nsuf, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p,
-                                                                  d.inst.p, ix->nsuf, d.post.p);
+        if (ix->njoin > 0) {
+            k_post_fill<<<grid_for(ix->njoin, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p,
+                                                                   d.inst.p, ix->njoin, d.post.p);
             APS_LAUNCH_CHECK();
         }
-        k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, M, d.lptr.p);
+        k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p);
         APS_LAUNCH_CHECK();
         if (nwptr) {
-            k_wptr<<<gM, T256, 0, s>>>(d.inst.p, k, M, d.lptr.p, d.post.p, d.wptr.p);
+            const dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>((maxm + 7) / 8, 65536 / k)),
+                         (unsigned)std::min(k, 65535));
+            k_wptr<<<g, T256, 0, s>>>(d.inst.p, k, d.lptr.p, d.post.p, d.wptr.p);
             APS_LAUNCH_CHECK();
         }
         APS_TRY(d.crow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
-        APS_TRY(d.vmeta.alloc((size_t)std::max<int64_t>(N, 1), s));
-        APS_TRY(d.vcand.alloc((size_t)std::max<int64_t>(N, 1), s));
-        APS_TRY(d.pn4.alloc((size_t)std::max<int64_t>(ix->npw, 4), s));
-        APS_CUDA(cudaMemsetAsync(d.pn4.p, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(ix->npw, 4), s));
-        k_pack<<<grid_for(std::max(nnz, N), T256), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.len.p, d.split.p,
-                                                                 d.mwpre.p, d.pnorm.p, d.vinst.p, d.inst.p, N, nnz,
-                                                                 d.crow.p, d.vmeta.p, d.vcand.p, d.pn4.p);
-        APS_LAUNCH_CHECK();
+        if (nnz > 0) {
+            k_pack<<<gE, T256, 0, s>>>(d.crank.p, d.cval.p, nnz, d.crow.p);
+            APS_LAUNCH_CHECK();
+        }
     }
     // ---- join work list
     {
@@ -724,6 +775,34 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     return APS_OK;
 }
 
+aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> &post, cudaStream_t s) {
+    const IndexArrays &d = ix->d;
+    DBuf<uint64_t> keys;
+    DBuf<uint32_t> vals;
+    DBuf<int32_t> erow;
+    APS_TRY(keys.alloc((size_t)std::max<int64_t>(ix->nnz, 1), s));
+    APS_TRY(vals.alloc((size_t)std::max<int64_t>(ix->nnz, 1), s));
+    APS_TRY(erow.alloc((size_t)std::max<int64_t>(ix->nnz, 1), s));
+    APS_TRY(lptr.alloc((size_t)ix->M + 1, s));
+    APS_TRY(post.alloc((size_t)std::max<int64_t>(ix->nsuf, 1), s));
+    if (ix->nnz > 0) {
+        k_rows_of<<<grid_for(ix->N * 32, T256), T256, 0, s>>>(d.cptr.p, ix->N, erow.p);
+        APS_LAUNCH_CHECK();
+        k_post_keys<<<grid_for(ix->nnz, T256), T256, 0, s>>>(d.cptr.p, d.crank.p, erow.p, d.vinst.p, d.inst.p,
+                                                             d.split.p, ix->nnz, ix->M, keys.p, vals.p);
+        APS_LAUNCH_CHECK();
+        APS_TRY(sort_pairs(keys.p, vals.p, ix->nnz, bits_for((uint64_t)ix->M), s));
+    }
+    if (ix->nsuf > 0) {
+        k_post_fill<<<grid_for(ix->nsuf, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p, d.inst.p,
+                                                              ix->nsuf, post.p);
+        APS_LAUNCH_CHECK();
+    }
+    k_lptr<<<grid_for(ix->M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, ix->M, lptr.p);
+    APS_LAUNCH_CHECK();
+    return APS_OK;
+}
+
 // ------------------------------------------------------------------ external queries
 namespace {
 
@@ -742,23 +821,39 @@ __global__ void k_q_gather(const uint64_t *__restrict__ keys, const uint32_t *__
 }
 
 // Remscore boundary of a query: the first rank-ordered component where
-// sum x[i] * maxweight_i(V) reaches t (float64, as for indexed vectors).
+// sum x[i] * maxweight_i(V) reaches t (float64, as for indexed vectors), or, with l2 and if
+// that is later, where the norm of the leading components can reach t. One warp per query.
 __global__ void k_q_split(const int64_t *__restrict__ qptr, const int2 *__restrict__ crow,
-                          const float *__restrict__ mwr, int64_t nq, float t, int32_t *qsplit, int4 *vmeta) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nq; x += (int64_t)gridDim.x * blockDim.x) {
+                          const float *__restrict__ mwr, const float *__restrict__ mw, int64_t nq, float t, bool l2,
+                          int4 *vmeta) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const float t2 = __fmul_rd(t, t);
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < nq; x += nwarps) {
         const int64_t a = qptr[x], b = qptr[x + 1];
         const int32_t L = (int32_t)(b - a);
-        int32_t qs = L;
+        int32_t qs = L, ls = l2 ? L : 0;
         double bmw = 0.0;
-        for (int64_t p = a; p < b; p++) {
-            bmw += (double)__int_as_float(crow[p].y) * (double)mwr[crow[p].x];
-            if (bmw >= (double)t) {
-                qs = (int32_t)(p - a);
-                break;
+        float ssu = 0.f;
+        for (int64_t base = a; base < b && (qs == L || ls == L); base += 32) {
+            const int64_t p = base + lane;
+            int2 e = make_int2(0, 0);
+            float mwc = 0.f;
+            if (p < b) {
+                e = crow[p];
+                mwc = mwr[e.x];
             }
+            const float c = __int_as_float(e.y);
+            const double bi = bmw + warp_incl_scan_f64((double)c * (double)mwc, lane);
+            const unsigned hit = __ballot_sync(0xffffffffu, p < b && bi >= (double)t);
+            if (qs == L && hit) qs = (int32_t)(base - a) + __ffs(hit) - 1;
+            bmw = __shfl_sync(0xffffffffu, bi, 31);
+            const float si = __fadd_ru(ssu, warp_incl_scan_ru(__fmul_ru(c, c), lane));
+            const unsigned hl = __ballot_sync(0xffffffffu, p < b && __fmul_ru(si, 1.0025f) >= t2);
+            if (ls == L && hl) ls = (int32_t)(base - a) + __ffs(hl) - 1;
+            ssu = __shfl_sync(0xffffffffu, si, 31);
         }
-        qsplit[x] = qs;
-        vmeta[x] = make_int4((int32_t)a, L, 0, 0);
+        if (lane == 0) vmeta[x] = make_int4((int32_t)a, L, max(qs, ls), __float_as_int(mw[x]));
     }
 }
 
@@ -823,10 +918,11 @@ aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32
         k_q_gather<<<grid_for(nnz, T256), T256, 0, s>>>(keys.p, vals.p, vout.p, nnz, (1ull << rb) - 1, qa.crow.p);
         APS_LAUNCH_CHECK();
     }
-    APS_TRY(qa.qsplit.alloc((size_t)std::max<int64_t>(nq, 1), s));
     APS_TRY(qa.vmeta.alloc((size_t)std::max<int64_t>(nq, 1), s));
     if (nq > 0) {
-        k_q_split<<<grid_for(nq, T256), T256, 0, s>>>(qptr, qa.crow.p, d.mwr.p, nq, t, qa.qsplit.p, qa.vmeta.p);
+        const bool l2 = !(flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
+        k_q_split<<<grid_for((int64_t)nq * 32, T256), T256, 0, s>>>(qptr, qa.crow.p, d.mwr.p, qa.mw.p, nq, t, l2,
+                                                                    qa.vmeta.p);
         APS_LAUNCH_CHECK();
     }
     return APS_OK;

@@ -9,20 +9,23 @@
 //   mwr/nnzr[M] maxweight_i(V) and non-zero count by global rank
 //   lptr[M+1]   posting-list start by global rank
 //   crow[nnz]   the same rows interleaved as {int32 rank, float32 value} (8 bytes)
-//   vmeta[N]    {int32 row offset, int32 |x|, int32 |x'|, float32 maxweight(x')} (16 bytes)
-//   pnorm[N]    an upper bound of ||x'||_2 (with the 1e-3 norm tolerance of the queries):
-//               dot(q, x') <= ||x'||_2 for any unit q
+//   The lists that the join walks keep more of a row unindexed than split does: the join's
+//   prefix x' ends at the later of split and the first component where ||x'||_2 would reach
+//   t (any y scores less than t on either kind of prefix), and the join's create boundary is
+//   the later of the remscore boundary and that component. Both only with every bound on.
+//   vmeta[N]    what the join reads of a query vector x, in one 16-byte load: {int32 row
+//               offset, int32 |x|, int32 create boundary, float32 maxweight(x)}
 //   vcand[N]    what verification reads of a candidate y, in one 16-byte load: {int32 row
-//               offset, int32 |y'|, float32 maxweight(y'), float32 ||y'||_2 bound}
-//   pn4[]       ||y'||_2 rounded up to a 4-bit code (c * 1.01/15 >= ||y'||_2), eight codes
-//               per 32-bit word, each instance from a 16-byte boundary (word pbase): the join
-//               copies a window's codes into shared memory and rejects candidates with them
+//               offset, int32 |y'|, int32 first rank after y', float32 ||y'||_2 bound}
+//   code[N]     one byte per vector: the octave of the first rank after y' in the high four
+//               bits and ||y'||_2 rounded up to c * 1.01/15 in the low four. A query vector
+//               turns the 256 codes into the least accumulated score worth verifying
 //   post[]      posting entries {int32 local vector id | min(|y|, 255) << 24, float32
 //               weight} (8 bytes), in increasing id inside each list; the size class in
 //               the top byte lets minsize skip an entry without another load (instances
 //               with n >= 2^24 store the id only and skip no entry)
-//   wptr[]      offsets of each candidate window (ids [w*W, (w+1)*W)) inside each list,
-//               only for instances with > 1 window
+//   wptr[]      position in post of each list's first entry of every candidate window (ids
+//               [w*W, (w+1)*W)), only for instances with > 1 window
 #pragma once
 
 #include <atomic>
@@ -32,42 +35,63 @@
 
 namespace aps {
 
-constexpr int JOIN_THREADS = 1024;
-constexpr int JOIN_WMAX = 40960;  // accumulator slots of a whole CTA (160 KB)
-constexpr int JOIN_RMAX = 1536;   // dense rank table for dot(x, y') lookups (6 KB)
-constexpr int JOIN_XCAP = 1280;   // x's row kept in shared memory when |x| <= XCAP / G
-// (so that every class layout of a CTA plus the join kernel's 1.5 KB of per-warp counters
-// fits the 227 KB of shared memory a CTA can have)
-// per-warp list of emitted pairs of one window: a warp scans at most W/NW slots rounded
-// up to 128 (W/NW = 1280 for every group shape)
-constexpr int JOIN_ECAP = JOIN_WMAX / (JOIN_THREADS / 32) + 128;
-constexpr int JOIN_STAGE_SLAB = 4096;  // staging slots a query group reserves at a time
-constexpr int JOIN_NCLS = 5;           // work-list classes: G = 1, 2, 4, 8 groups per CTA; vectors of <= 2 components
-// ||y'||_2 bounds in 4 bits per vector: code c stands for c * PN4_STEP (PN4_STEP = 1.01 / 15,
-// above any norm the index accepts), and PN4_UNIT = PN4_STEP in units of 2^-30, rounded up
+constexpr int JOIN_WARPS = 24;  // warps of a join CTA (one CTA per SM)
+constexpr int JOIN_THREADS = 32 * JOIN_WARPS;
+// A join tile is one warp with a window of accumulator slots of its own in shared memory. The
+// tile shape G (1, 2, 4 or 8) trades the warps that run on an SM against the window's width. The
+// join waits for memory, so the most warps that the registers allow win at every size (join ms
+// with 12 / 16 / 20 / 24 warps: 200k power-law set 27.1 / 22.0 / 20.6 / 21.0, the 512-instance
+// batch 28.4 / 21.0 / 17.1 / 14.9; 28 and 32 warps spill registers and lose 5 to 30%), and G = 2,
+// 4 and 8 are the same shape; G = 1 has windows of twice the width.
+constexpr int JOIN_LCAP = 256;  // candidate list entries of a warp
+constexpr int JOIN_SMEM = 232448 - 4096;  // of the 227 KB a CTA can have (the rest: the warps' states)
+__host__ __device__ constexpr int tile_warps(int G) { return G == 1 ? 12 : 24; }
+constexpr int JOIN_XCAP = 64;   // a query row of at most so many components is held in shared memory
+// per-warp shared memory beside the window: 64 prefix norms, 32 lists waiting, 32 lists of a run,
+// a query row, the candidate list
+constexpr int TILE_FIXED = 4 * 64 + 16 * 32 + 8 * 32 + 8 * JOIN_XCAP + 2 * JOIN_LCAP;
+// 4 bytes of accumulator and one bit of the match bitmap per slot; a multiple of 128 slots
+__host__ __device__ constexpr int tile_window(int G) {
+    return (JOIN_SMEM / tile_warps(G) - TILE_FIXED) * 8 / 33 / 128 * 128;
+}
+__host__ __device__ constexpr int tile_bytes(int G) { return TILE_FIXED + tile_window(G) * 33 / 8; }
+// per-warp list of the matches of a streamed vector before they are placed
+constexpr int JOIN_ECAP = 1408;
+constexpr int JOIN_STAGE_SLAB = 512;  // staging slots a warp reserves at a time
+constexpr int JOIN_NCLS = 5;          // work-list classes: tile shapes G = 1, 2, 4, 8; vectors of <= 2 components
+// ||y'||_2 bounds in 4 bits: code c stands for c * PN4_STEP (above any norm the index accepts)
 constexpr float PN4_STEP = 1.01f / 15.f;
-constexpr uint32_t PN4_UNIT = 72298617u;
+
+// Buckets of dimension ranks: four per octave (64 in all; the last takes every rank from
+// 114,688 on), and their octaves, used for the prefix norms of a query vector.
+__device__ __forceinline__ int rank_bucket(int r) {
+    const int e = max(31 - __clz(r), 2);
+    return r < 4 ? r : min(4 * e + ((r >> (e - 2)) & 3) - 4, 63);
+}
 
 struct InstDesc {
     int64_t vbase;   // first global vector id
-    int64_t qwbase;  // first (vector, window) slot of the per-window pair counts
     int64_t wbase;   // first wptr entry (instances with nw > 1)
-    int64_t ebase;   // first component (nnz offset)
-    int64_t pbase;   // first 32-bit word of the instance's 4-bit ||y'||_2 codes (a multiple of 4)
     int32_t n;       // vectors
     int32_t m;       // dimensions
     int32_t rbase;   // first global rank
     int32_t nw;      // candidate windows
     int32_t W;       // window width
-    int32_t G;       // query groups per CTA for this instance's class
+    int32_t G;       // tile shape of this instance's class
     float t;         // threshold
     int32_t packed;  // 1: posting ids carry the size class in their top byte
 };
 
-struct Segment {      // the run of emitted pairs of one (x, window) slot qw, stored at segs[qw]
-    int64_t src;      // offset in the staging buffer
-    int32_t cnt;      // pairs (also in the per-slot counts; destination = scan(counts)[qw])
-    int32_t i;        // local id of x
+// The first piece of the run of emitted pairs of one slot (a vector, or one part of its
+// windows), stored at segs[slot]; the slot's pairs go to scan(counts)[slot] on. A run that
+// fills its staging slab goes on at the start of another one: chain[k] = {pairs, next slab or
+// -1} describes the piece at the start of slab k.
+struct Segment {
+    int64_t src;   // offset in the staging buffer
+    int32_t cnt;   // pairs of this piece
+    int32_t i;     // local id of x
+    int32_t next;  // slab of the next piece, or -1
+    int32_t _pad;
 };
 
 struct IndexArrays {
@@ -78,20 +102,19 @@ struct IndexArrays {
     DBuf<float> cval;
     DBuf<int2> crow;
     DBuf<int4> vmeta;
-    DBuf<int4> vcand;  // {row offset, |x'|, maxweight(x'), ||x'||_2 bound} per vector
-    DBuf<uint32_t> pn4;  // 4-bit ||x'||_2 codes, eight per word, each instance 16-byte aligned
+    DBuf<int4> vcand;
+    DBuf<uint8_t> code;
     DBuf<int32_t> len, split, qsplit;
     DBuf<float> mw, mwpre;
-    DBuf<float> pnorm;  // ||x'||_2 of the unindexed prefix (rounded up, with the norm tolerance)
     DBuf<int32_t> rank_of_dim, dim_of_rank, nnz_d;
     DBuf<float> mw_d, mwr;
     DBuf<int64_t> lptr;
-    DBuf<int32_t> wptr;
+    DBuf<uint32_t> wptr;
     DBuf<int2> post;
 };
 
 // The join phase of an index as a CUDA graph: the two workspace resets and the persistent
-// join launch, captured on the index's first join; later joins update the nodes' pointers
+// join launch, captured on the index's second join; later joins update the nodes' pointers
 // and launch parameters in the instantiated graph and replay it.
 struct JoinGraph {
     cudaGraph_t graph = nullptr;
@@ -117,17 +140,20 @@ struct aps_index {
     int64_t N = 0;     // vectors
     int64_t M = 0;     // dimensions (all instances)
     int64_t nnz = 0;
-    int64_t nsuf = 0;  // indexed components
-    int64_t nqw = 0;   // (vector, window) slots
+    int64_t nsuf = 0;   // indexed components (by split)
+    int64_t njoin = 0;  // components in the join's posting lists
+    bool l2 = false;    // the join's prefixes take the norm bound too
+    int64_t arena_slots = 0;  // what the allocation-free join's documented size limit counts
     int64_t nwptr = 0;
-    int64_t npw = 0;   // words of the 4-bit ||x'||_2 codes
-    int32_t maxm = 0;
+    int32_t maxm = 0, maxnw = 0;
+    // parts that the windows of a heavy vector are cut into (its slots; 1: none)
+    int32_t parts = 1;
     float t = 0.f;     // single-instance threshold
     std::vector<aps::InstDesc> inst_h;
     aps::IndexArrays d;
     // join work list: vectors in decreasing estimated cost, grouped by class
     aps::DBuf<int32_t> items;
-    int64_t class_begin[aps::JOIN_NCLS + 1] = {};  // classes G = 1, 2, 4, 8, then vectors of <= 2 components
+    int64_t class_begin[aps::JOIN_NCLS + 1] = {};  // tile shapes G = 1, 2, 4, 8, then vectors of <= 2 components
     // output sizing from the previous join
     int64_t hint_pairs = 0;
     // pairs per query (times 16) that query batches on this index have needed at most: the
@@ -156,10 +182,7 @@ aps_status pairs_to_host(aps_pairs *p, cudaStream_t s);
 // dimension ranks and sorted by rank, with |q|, maxweight(q) and the remscore boundary.
 struct QueryArrays {
     DBuf<int2> crow;     // {rank, value} per component, rows in rank order
-    DBuf<int4> vmeta;
-    DBuf<int4> vcand;  // {row offset, |x'|, maxweight(x'), ||x'||_2 bound} per vector
-    DBuf<uint32_t> pn4;  // 4-bit ||x'||_2 codes, eight per word, each instance 16-byte aligned    // {row offset, |q|, 0, 0}
-    DBuf<int32_t> qsplit;
+    DBuf<int4> vmeta;  // {row offset, |q|, create boundary, maxweight(q)}
     DBuf<float> mw;
     int64_t nq = 0, nnz = 0;
 };
@@ -181,6 +204,9 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
 aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_t *idx,
                               const float *val, const std::vector<InstDesc> &inst_in,
                               cudaStream_t s, const aps_tuning *tune = nullptr);
+
+// The posting lists by split (the exported ones), where they are not the join's own.
+aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> &post, cudaStream_t s);
 
 // Join tile shapes (tune.cu): the size bucket of an instance, the process-wide table of
 // query groups per bucket, and the autotuner (host arrays ro, hptr, m, t; device CSR).

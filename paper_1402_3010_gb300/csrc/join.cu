@@ -1,31 +1,33 @@
 // The inverted-index join (Alg. 2, Find-Matches, with the all-pairs-2 bounds) and the
 // output stage.
 //
-// One persistent launch takes every size class in turn. A CTA of 1024 threads runs G
-// query groups (G = 1, 2, 4, 8); each group owns a dense score array A over a window of W
-// candidate ids in shared memory (the paper's all-pairs-0-array accumulator, cut into
-// windows because n floats do not fit on chip). For a query x (a whole vector of the set, taken
-// from a cost-ordered work list) and each window of candidates y > x:
-//   1. accumulate: A[y] += x[i] * y[i] over the posting lists of x's components,
-//      first over the components with remscore >= t (these may create candidates), then
-//      over the rest, which only update candidates that exist (remscore); entries with |y|
-//      below minsize are skipped using the size class stored in the entry. A holds 32-bit
-//      fixed-point sums (products rounded up to multiples of 2^-30, so a creating product
-//      is at least one unit), so its updates are native integer shared-memory atomics. A
-//      creating update that finds its slot still zero (a plain read before the add) also
-//      sets the slot's bit in a bitmap of candidates: the first update of a slot always
-//      does, so every candidate is marked, at one bitmap update per candidate rather than
-//      per entry. Lists are in id order, so a warp's 32 lanes add into 32 increasing slots;
-//   2. verify: each warp walks its share of the bitmap and takes the marked slots in slot
-//      order, one candidate per lane: A[y] + ||y'||_2 < t rejects cheaply, then the
-//      upperbound test A[y] + min(|y'|, |x|) * maxweight(x) * maxweight(y') >= t, then
-//      s = A[y] + dot(x, y') with y' the unindexed prefix of y; scores within a band of
-//      t are recomputed in float64 and decided there;
-//   3. compact: warp ballots give each emitted pair its slot; the window's run comes from
-//      a staging slab the group reserves in bulk; pairs land as (y, score) in increasing
-//      y and the run is recorded at its (x, window) slot.
-// The output stage scans the per-(x, window) counts and gathers the staged runs into
-// (i, j, score) arrays, which are then in (i, j) order without a sort.
+// One persistent launch takes every size class in turn, one CTA per SM. A join tile is one
+// warp: it holds a dense score array A over a window of W candidate ids in its own part of
+// shared memory (the paper's all-pairs-0-array accumulator, cut into windows because n floats
+// do not fit on chip), so no step of a query vector waits for another warp and the warps of an
+// SM hide one another's latency. For a query x (a whole vector of the set from a cost-ordered
+// work list, or one part of its windows where x is among the heaviest) and each window of
+// candidates y > x:
+//   1. create: A[y] += x[i] * y[i] over the posting lists of x's components from its create
+//      boundary on (remscore and norm bounds: a match has one of these in common with x). A
+//      holds 32-bit fixed-point sums (products rounded up to multiples of 2^-30, at least one
+//      unit), added with integer shared-memory atomics whose returned old value tells a slot's
+//      first update: those slots go to the warp's candidate list. Entries with |y| below minsize
+//      are skipped using the size class stored in the entry;
+//   2. update: the same over x's earlier components, which only add where A is not zero;
+//   3. filter: dot(x, y') <= ||x on the ranks before y's first indexed one|| * ||y'||
+//      (Cauchy-Schwarz). Both of y's parts are in its one-byte code, x's norms in a table made
+//      once per unit, so a candidate costs one byte of global memory;
+//   4. verify the rest, one candidate per lane: the same bound with the exact norm, then
+//      s = A[y] + dot(x, y') with y' the unindexed prefix of y; scores within a band of t are
+//      recomputed in float64 and decided there. A match leaves its score in A and a bit in the
+//      window's bitmap;
+//   5. emit: the bitmap is walked in id order and the (y, score) go to the staging slab that
+//      the warp reserves in bulk. The run of x (or of its part) is recorded at its slot.
+// A window with more candidates than the list holds is filtered from A itself, in stretches
+// of as many slots as the list has entries.
+// The output stage scans the per-slot counts and gathers the staged runs into (i, j, score)
+// arrays, which are then in (i, j) order without a sort.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -44,16 +46,20 @@ struct JoinParams {
     const InstDesc *inst;
     const int32_t *vinst;
     const int32_t *items;
+    int one;  // a single instance
     // classes, taken in order by one persistent launch: class c is the work-list range
-    // [cls_begin[c], cls_begin[c + 1]) run with cls_G[c] query groups per CTA, or, when
-    // cls_G[c] is 0, one warp per vector with one or two components
+    // [cls_begin[c], cls_begin[c + 1]) run with tile shape cls_G[c], or, when cls_G[c] is 0,
+    // one warp per vector with one or two components. The first cls_heavy[c] items are cut
+    // into `parts` parts of their windows.
     int ncls;
     int cls_G[JOIN_NCLS];
     int64_t cls_begin[JOIN_NCLS + 1];
+    int64_t cls_heavy[JOIN_NCLS];
+    int parts;
     const int2 *crow;    // rank-ordered rows {rank, value}
-    const int4 *vmeta;   // {row offset, |x|, |x'|, maxweight(x')}
-    const int4 *vcand;   // {row offset, |y'|, maxweight(y'), ||y'||_2 bound}
-    const uint32_t *pn4; // 4-bit ||y'||_2 codes, eight per word (instance I from word I.pbase)
+    const int4 *vmeta;   // {row offset, |x|, create boundary, maxweight(x)}
+    const int4 *vcand;   // {row offset, |y'|, first rank after y', ||y'||_2 bound}
+    const uint8_t *code; // per vector: octave of the first rank after y', 4-bit ||y'||_2 bound
     // dimension-block items (the vertical split with local pruning, Sec. 5.1): iblk[it] >= 0
     // makes work item it one of nblk blocks of the vector items[it]; null: none
     const int8_t *iblk;
@@ -62,62 +68,25 @@ struct JoinParams {
     uint32_t *sp_score;            // their float32 scores (bits)
     unsigned long long *sp_count;  // pairs reserved in sp_key / sp_score
     int64_t sp_cap;
-    const int32_t *qsplit;
-    const float *mw;
     const int64_t *lptr;
-    const int32_t *wptr;
+    const uint32_t *wptr;
     const int2 *post;
     uint32_t flags;
     int2 *stage;
     int64_t stage_cap;
-    unsigned long long *stage_count;  // staging slots handed out (in slabs of stage_slab)
+    unsigned long long *stage_count;  // staging slots handed out (whole slabs of stage_slab)
     int64_t stage_slab;
-    Segment *segs;                    // [slots]: the run of slot qw
-    int32_t *cntq;
+    Segment *segs;                    // [slots]: the first piece of a slot's run
+    int2 *chain;                      // [stage_cap / stage_slab + 1]: later pieces, by slab
+    int32_t *cntq;                    // [slots]: pairs
     unsigned long long *counters;  // visits, candidates, verified, pairs, band; [6] entries read
     unsigned long long *work;       // [ncls] work-list cursors
-    int2 *scratch;                  // per-warp lists of emitted pairs, JOIN_ECAP each
+    int2 *scratch;                  // per-warp lists of the streamed class, JOIN_ECAP each
     // query mode: items are external query rows matched against every indexed vector
-    int qmode;
     const int2 *qcrow;    // query rows over the index's ranks
-    const int4 *qvmeta;   // {row offset, |q|, 0, 0}
-    const int32_t *qqsplit;
-    const float *qmw;
+    const int4 *qvmeta;   // {row offset, |q|, create boundary, maxweight(q)}
     float qt;
-    int qnw;              // windows of the index: query-mode items are (query, window) pairs
 };
-
-constexpr int NWARPS = JOIN_THREADS / 32;
-
-__host__ __device__ constexpr int group_bytes(int G) {
-    return 4 * (JOIN_WMAX / G)                       // A
-           + 4 * (JOIN_WMAX / G / 8)                 // the window's 4-bit ||y'||_2 codes
-           + 8 * (JOIN_THREADS / G)                  // c_start
-           + 4 * (JOIN_THREADS / G)                  // c_cnt
-           + 4 * (JOIN_THREADS / G + 4)              // c_ch0
-           + 4 * (JOIN_THREADS / G)                  // c_xv
-           + 4 * (JOIN_RMAX / G)                     // xtab
-           + 8 * (JOIN_XCAP / G)                     // x's row
-           + 4 * (JOIN_WMAX / G / 32)                // bitmap of the window's candidates
-           + 8 * 32                                  // wsum
-           + 4 * 32                                  // wcnt
-           + 8 * 8;                                  // broadcast and the staging slab
-}
-
-// every class layout of a CTA plus the kernel's per-warp counters (static shared memory)
-// within the 227 KB a CTA can opt into on this part
-constexpr int JOIN_SMEM_LIMIT = 232448;
-static_assert(group_bytes(1) * 1 + NWARPS * 6 * 8 <= JOIN_SMEM_LIMIT, "G = 1 layout too large");
-static_assert(group_bytes(2) * 2 + NWARPS * 6 * 8 <= JOIN_SMEM_LIMIT, "G = 2 layout too large");
-static_assert(group_bytes(4) * 4 + NWARPS * 6 * 8 <= JOIN_SMEM_LIMIT, "G = 4 layout too large");
-static_assert(group_bytes(8) * 8 + NWARPS * 6 * 8 <= JOIN_SMEM_LIMIT, "G = 8 layout too large");
-
-__device__ __forceinline__ void gsync(int G, int g, int GT) {
-    if (G == 1)
-        __syncthreads();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(GT) : "memory");
-}
 
 __device__ __forceinline__ int64_t warp_incl_scan(int64_t v, int lane) {
 #pragma unroll
@@ -139,170 +108,110 @@ __device__ __forceinline__ int warp_excl_scan_int(int v, int lane, int *total) {
     return inc - v;
 }
 
-// x's value at rank r: dense table for small ranks, binary search of x's rank-ordered row
-// otherwise.
-__device__ __noinline__ float x_at_search(int r, const int2 *__restrict__ xrow, int xl) {
-    int lo = 0, hi = xl;
+// Position of the first entry at or after `lo` of a rank-ordered row whose rank is >= r.
+__device__ __forceinline__ int row_find(const int2 *row, int lo, int hi, const int r) {
+#pragma unroll 1
     while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (xrow[mid].x < r) lo = mid + 1; else hi = mid;
+        const int mid = (lo + hi) >> 1;
+        if (row[mid].x < r) lo = mid + 1; else hi = mid;
     }
-    if (lo < xl) {
-        const int2 e = xrow[lo];
+    return lo;
+}
+
+// The value at rank r of a rank-ordered row (0 when it has none).
+__device__ __forceinline__ float x_at(const int r, const int2 *xrow, const int xl) {
+    const int p = row_find(xrow, 0, xl, r);
+    if (p < xl) {
+        const int2 e = xrow[p];
         if (e.x == r) return __int_as_float(e.y);
     }
     return 0.f;
 }
 
-// x's value at rank r: dense table for small ranks, then a binary search of x's row held
-// in shared memory (xr, xs entries; xs = 0 when the row did not fit), else in global memory.
-__device__ __forceinline__ float x_at(int r, const float *xtab, int RG, const int2 *xr, int xs,
-                                      const int2 *__restrict__ xrow, int xl) {
-    if (r < RG) return xtab[r];
-    if (xs == 0) return x_at_search(r, xrow, xl);
-    int lo = 0, hi = xs;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (xr[mid].x < r) lo = mid + 1; else hi = mid;
-    }
-    return (lo < xs && xr[lo].x == r) ? __int_as_float(xr[lo].y) : 0.f;
-}
-
-// The accumulation of one warp over chunks [ch, che) of the current component batch
-// (Alg. 2's A[y] += x[i] * y[i]). Chunk ch of component cc covers entries
-// (ch - c_ch0[cc]) * 128 .. + 127 of that component's segment, and no further than its end.
-// Each product is rounded up to a multiple of 2^-30 (so a creating product is at least one
-// unit and its slot becomes non-zero); CREATE: the component may create candidates, and an
-// add that found its slot zero marks the slot in bm (the first add to a slot always finds
-// it zero, so every candidate is marked; a few concurrent first adds mark it again, which
-// is harmless); otherwise it only adds where A is already non-zero (remscore). FIRST: the
-// window holds ids at or below x's (slots below lo are skipped).
-// Asynchronous 16-byte global -> shared copy (cp.async, completes out of band) and waits.
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// A thread's work counters, 32-bit: folded (warp-reduced) into its warp's 64-bit totals in
-// shared memory after every item, so no 64-bit register pair stays live across the loops.
-struct Ctr {
-    uint32_t visits = 0, cand = 0, verified = 0, pairs = 0, band = 0, read = 0;
+// A warp's staging place and the pieces of the run that it is writing, in shared memory.
+// Reservations are whole slabs, so a piece that
+// begins a reservation is named by its slab. Nothing is left unused but the rest of the last one.
+struct Stager {
+    int64_t base;         // current reservation
+    int64_t head;         // the run's first pair
+    uint32_t used, size;  // of the reservation
+    uint32_t piece_cnt, head_cnt, cnt;
+    int32_t piece;        // slab of the current piece, -1: the run's first one
+    int32_t head_next;
+    // room handed out last: pair p goes to a + p for p < f, to b + p - f from there on
+    uint32_t f;
+    int64_t a, b;
 };
-__device__ __forceinline__ void ctr_flush(Ctr &c, unsigned long long *wtot, const int lane) {
-    uint32_t v[6] = {c.visits, c.cand, c.verified, c.pairs, c.band, c.read};
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if (lane == 0) wtot[k] += v[k];
-    }
-    c = Ctr();
+
+// Work totals of a warp: visits, candidates, verified, pairs, band, entries read.
+struct Totals {
+    unsigned long long v[6];
+};
+
+// tot[k] += the warp's sum of v. Warp-collective.
+__device__ __forceinline__ void count_add(Totals &S, const int k, const uint32_t v, const int lane) {
+    const uint32_t s = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) S.v[k] += s;
 }
 
-// One 128-entry chunk of a segment: entries off .. off + 127 of seg[0, cnt), lane l taking
-// off + l, off + l + 32, ... (see walk_chunks).
-template <bool CREATE, bool FIRST>
-__device__ __forceinline__ void walk_chunk(const int2 *__restrict__ seg, const int cnt, const int off, const float cxv,
-                                           uint32_t *A, uint32_t *bm, const uint32_t smin_tag, const int32_t idmask,
-                                           const int w0, const int lo, const int lane, uint32_t &nv) {
-    const int rem = cnt - off - lane;  // entries from this lane's first one to the segment's end
-    const int2 *pp = seg + off + lane;
-    int2 ent[4];
-#pragma unroll
-    for (int u = 0; u < 4; u++) ent[u] = u * 32 < rem ? __ldg(pp + u * 32) : make_int2(0, 0);
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-        if (u * 32 >= rem || (uint32_t)ent[u].x < smin_tag) continue;  // past the end; minsize
-        const int slot = (ent[u].x & idmask) - w0;
-        if (FIRST && slot < lo) continue;
-        nv++;  // an entry Alg. 2 visits: y after x, |y| >= minsize
-        const uint32_t q = __float2uint_ru(cxv * __int_as_float(ent[u].y));
-        const uint32_t old = A[slot];
-        if (CREATE) {
-            atomicAdd(&A[slot], q);
-            if (old == 0u) atomicOr(&bm[slot >> 5], 1u << (slot & 31));
-        } else if (old != 0u) {
-            atomicAdd(&A[slot], q);
+// Room for c more pairs of the run: S.a, S.f, S.b. One thread.
+__device__ __forceinline__ void stage_take(Stager &S, const JoinParams &P, const uint32_t c) {
+    const uint32_t f = min(c, S.size - S.used);
+    const int64_t a = S.base + S.used;
+    S.a = a;
+    S.f = f;
+    if (f == c) {
+        if (S.cnt == 0) S.head = a;
+        S.used += c;
+        S.piece_cnt += c;
+        S.cnt += c;
+        return;
+    }
+    const uint32_t slab = (uint32_t)P.stage_slab;
+    const uint32_t want = (c - f + slab - 1) / slab * slab;
+    const int64_t b = (int64_t)atomicAdd(P.stage_count, (unsigned long long)want);
+    S.b = b;
+    if (S.cnt == 0 && f == 0) {  // the run begins here
+        S.head = b;
+        S.piece_cnt = c;
+    } else {
+        if (S.cnt == 0) S.head = a;
+        const int32_t nx = (int32_t)(b / slab);
+        if (S.piece < 0) {
+            S.head_cnt = S.piece_cnt + f;
+            S.head_next = nx;
+        } else if ((int64_t)S.piece * slab < P.stage_cap) {
+            P.chain[S.piece] = make_int2((int)(S.piece_cnt + f), nx);
         }
+        S.piece = nx;
+        S.piece_cnt = c - f;
     }
+    S.base = b;
+    S.size = want;
+    S.used = c - f;
+    S.cnt += c;
 }
 
-// The accumulation of one warp over chunks [ch, che) of the current component batch
-// (Alg. 2's A[y] += x[i] * y[i]), the components' segments in shared memory. Chunk ch of
-// component cc covers entries (ch - c_ch0[cc]) * 128 .. + 127 of that component's segment,
-// and no further than its end. Each product is rounded up to a multiple of 2^-30 (so a
-// creating product is at least one unit and its slot becomes non-zero); CREATE: the
-// component may create candidates, and an add that found its slot zero marks the slot in bm
-// (the first add to a slot always finds it zero, so every candidate is marked; a few
-// concurrent first adds mark it again, which is harmless); otherwise it only adds where A
-// is already non-zero (remscore). FIRST: the window holds ids at or below x's (slots below
-// lo are skipped).
-template <bool CREATE, bool FIRST>
-__device__ __forceinline__ void walk_chunks(int ch, const int che, int cc, const int64_t *c_start,
-                                            const int32_t *c_cnt, const int32_t *c_ch0, const float *c_xv,
-                                            const int2 *__restrict__ post, uint32_t *A, uint32_t *bm,
-                                            const uint32_t smin_tag, const int32_t idmask, const int w0, const int lo,
-                                            const int lane, uint32_t &n_visits) {
-    uint32_t nv = 0;
-    const int2 *seg = post + c_start[cc];
-    int cnt = c_cnt[cc], cch0 = c_ch0[cc], cnext = c_ch0[cc + 1];
-    float cxv = c_xv[cc] * 1073741824.f;  // x's value scaled by 2^30 (exact)
-    for (; ch < che; ch++) {
-        if (ch >= cnext) {
-            cc++;
-            seg = post + c_start[cc];
-            cnt = c_cnt[cc];
-            cch0 = cnext;
-            cnext = c_ch0[cc + 1];
-            cxv = c_xv[cc] * 1073741824.f;
-        }
-        walk_chunk<CREATE, FIRST>(seg, cnt, (ch - cch0) << 7, cxv, A, bm, smin_tag, idmask, w0, lo, lane, nv);
-    }
-    n_visits += nv;
+// The run is complete: its record at `slot`. One thread.
+__device__ __forceinline__ void stage_close(Stager &S, const JoinParams &P, const int64_t slot, const int32_t id) {
+    if (S.cnt == 0) return;
+    P.cntq[slot] = (int32_t)S.cnt;
+    Segment g;
+    g.src = S.head;
+    g.cnt = (int32_t)(S.piece < 0 ? S.piece_cnt : S.head_cnt);
+    g.i = id;
+    g.next = S.piece < 0 ? -1 : S.head_next;
+    g._pad = 0;
+    P.segs[slot] = g;
+    if (S.piece >= 0 && (int64_t)S.piece * P.stage_slab < P.stage_cap)
+        P.chain[S.piece] = make_int2((int)S.piece_cnt, -1);
+    S.piece = -1;
+    S.piece_cnt = S.cnt = 0;
 }
 
-// The same with the (at most 32) components of a short x held in registers, lane c holding
-// component c: its segment start st, length cnt, first chunk ch0 and x's value xv.
-template <bool CREATE, bool FIRST>
-__device__ __forceinline__ void walk_chunks_r(int ch, const int che, int cc, const int64_t st, const int cnt_l,
-                                              const int ch0_l, const float xv_l, const int2 *__restrict__ post,
-                                              uint32_t *A, uint32_t *bm, const uint32_t smin_tag, const int32_t idmask,
-                                              const int w0, const int lo, const int lane, uint32_t &n_visits) {
-    uint32_t nv = 0;
-    const int2 *seg = post + __shfl_sync(0xffffffffu, st, cc);
-    int cnt = __shfl_sync(0xffffffffu, cnt_l, cc), cch0 = __shfl_sync(0xffffffffu, ch0_l, cc);
-    float cxv = __shfl_sync(0xffffffffu, xv_l, cc) * 1073741824.f;
-    for (; ch < che; ch++) {
-        while (ch >= cch0 + ((cnt + 127) >> 7)) {  // the next component with entries
-            cc++;
-            seg = post + __shfl_sync(0xffffffffu, st, cc);
-            cnt = __shfl_sync(0xffffffffu, cnt_l, cc);
-            cch0 = __shfl_sync(0xffffffffu, ch0_l, cc);
-            cxv = __shfl_sync(0xffffffffu, xv_l, cc) * 1073741824.f;
-        }
-        walk_chunk<CREATE, FIRST>(seg, cnt, (ch - cch0) << 7, cxv, A, bm, smin_tag, idmask, w0, lo, lane, nv);
-    }
-    n_visits += nv;
-}
-
-// dot(x, y') over the |y'| leading (unindexed) entries of y's rank-ordered row, by one
-// lane (short prefixes): two entries per step.
-__device__ __forceinline__ float dot_prefix(const int2 *__restrict__ yr, int ys, const float *xtab, int RG,
-                                           const int2 *xr, int xs, const int2 *__restrict__ xrow, int xl) {
-    float acc = 0.f;
-    int k = 0;
-    for (; k + 2 <= ys; k += 2) {
-        const int2 e0 = __ldg(yr + k), e1 = __ldg(yr + k + 1);
-        acc = fmaf(x_at(e0.x, xtab, RG, xr, xs, xrow, xl), __int_as_float(e0.y), acc);
-        acc = fmaf(x_at(e1.x, xtab, RG, xr, xs, xrow, xl), __int_as_float(e1.y), acc);
-    }
-    if (k < ys) {
-        const int2 e0 = __ldg(yr + k);
-        acc = fmaf(x_at(e0.x, xtab, RG, xr, xs, xrow, xl), __int_as_float(e0.y), acc);
-    }
-    return acc;
+__device__ __forceinline__ void stage_put(const JoinParams &P, const Stager &S, const uint32_t p, const int2 v) {
+    const int64_t at = p < S.f ? S.a + p : S.b + (p - S.f);
+    if (at < P.stage_cap) P.stage[at] = v;  // past the room: the host grows it and runs again
 }
 
 // First position in [a, b) of a posting list (ids increasing) whose id exceeds lx, or b
@@ -340,9 +249,9 @@ __device__ __forceinline__ void list_after(const JoinParams &P, const InstDesc &
     end = P.lptr[R + 1];
     int64_t a = ls, b = end;
     if (I.nw > 1) {
-        const int32_t *wp = P.wptr + I.wbase + (int64_t)r * (I.nw + 1);
-        a = ls + wp[wf];
-        b = ls + wp[wf + 1];
+        const uint32_t *wp = P.wptr + I.wbase + (int64_t)r * (I.nw + 1);
+        a = wp[wf];
+        b = wp[wf + 1];
     }
     first = first_after(P.post, a, b, lx, idmask, lane);
 }
@@ -376,37 +285,43 @@ __device__ __forceinline__ int count_below(const int v, const int key) {
 //   unless the ||y'||_2 bound already rules the pair out).
 // Each candidate is decided like the windowed path (float32 outside a band of beta around
 // t, the exact float64 sum of the products inside it). The matches, in increasing y, go to
-// the warp's scratch list and are then copied as x's run in its first window's slot, from
-// a staging slab the warp reserves in bulk; a vector with more matches than the scratch
-// list holds is streamed a second time, writing them there directly.
+// the warp's scratch list and are then copied as x's run to the staging slab that the warp
+// reserves in bulk; a vector with more matches than the scratch list holds is streamed a
+// second time, writing them there directly.
 __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long long *work, const int64_t item_begin,
                                           const int64_t item_end, const bool f_minsize, const bool f_remscore,
-                                          unsigned long long *wtot) {
+                                          Totals &tot, Stager &S) {
     const int lane = threadIdx.x & 31;
-    Ctr ct;
+    struct {
+        uint32_t visits = 0, cand = 0, verified = 0, band = 0;
+    } ct;  // folded into the warp's totals after every item
     const unsigned lt_mask = (1u << lane) - 1u;
-    const int64_t wslab = max((int64_t)32, P.stage_slab / 8);
-    int2 *const elist = P.scratch + ((size_t)blockIdx.x * NWARPS + (threadIdx.x >> 5)) * JOIN_ECAP;
-    int64_t sb = 0, su = 0, ss = 0;  // this warp's staging slab: base, used, size
+    int2 *const elist = P.scratch + ((size_t)blockIdx.x * JOIN_WARPS + (threadIdx.x >> 5)) * JOIN_ECAP;
+    // the first item is this warp's own, the next ones are asked for one item ahead (lane 0)
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * JOIN_WARPS;
+    unsigned long long nw = blockIdx.x + (unsigned long long)gridDim.x * (threadIdx.x >> 5);
     for (;;) {
-        ctr_flush(ct, wtot, lane);
-        unsigned long long iw = 0;
-        if (lane == 0) iw = atomicAdd(work, 1ull);
-        const int64_t it = (int64_t)__shfl_sync(0xffffffffu, iw, 0) + item_begin;
+        const int64_t it = (int64_t)__shfl_sync(0xffffffffu, nw, 0) + item_begin;
+        count_add(tot, 0, ct.visits, lane);
+        count_add(tot, 1, ct.cand, lane);
+        count_add(tot, 2, ct.verified, lane);
+        count_add(tot, 4, ct.band, lane);
+        ct.visits = ct.cand = ct.verified = ct.band = 0;
         if (it >= item_end) break;
+        if (lane == 0) nw = atomicAdd(work, 1ull) + nwarps;
         const int64_t x = P.items[it];
         const InstDesc I = P.inst[P.vinst[x]];
         const int32_t lx = (int32_t)(x - I.vbase);
         const int4 xm = P.vmeta[x];
         const int xl = xm.y;  // 1 or 2
-        const int qs = f_remscore ? P.qsplit[x] : 0;
+        const int qs = f_remscore ? xm.z : 0;
         if (qs >= xl) continue;  // remscore < t from the first component on: no candidate
         const int2 xe0 = P.crow[xm.x];
         const int2 xe1 = xl == 2 ? P.crow[xm.x + 1] : make_int2(0, 0);
         const float x0 = __int_as_float(xe0.y), x1 = __int_as_float(xe1.y);
         const float t = I.t;
         const float beta = fmaxf(1e-5f, (float)(xl + 2) * 1.1920929e-7f);  // (|x| + 2) * 2^-23
-        const float mwx = P.mw[x];
+        const float mwx = __int_as_float(xm.w);
         int smin = 0;  // minsize, bounded as in the windowed path
         if (f_minsize && I.packed && mwx > 0.f)
             smin = (int)ceilf(fminf(__fdiv_rd(__fsub_rd(t, beta), __fmul_ru(mwx, 1.0020001f)), 255.f));
@@ -416,12 +331,10 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
         int64_t f0, e0, f1 = 0, e1 = 0;
         list_after(P, I, xe0.x, lx, wf, idmask, lane, f0, e0);
         if (xl == 2) list_after(P, I, xe1.x, lx, wf, idmask, lane, f1, e1);
-        if (lane == 0) ct.read += (uint32_t)((e0 - f0) + (e1 - f1));
+        if (lane == 0) tot.v[5] += (unsigned long long)((e0 - f0) + (e1 - f1));
         // pass 0: count the matches, the first JOIN_ECAP into the scratch list; pass 1 (only
         // when there were more): write them all into the reserved run
         int cnt = 0;
-        int64_t dst = 0;
-        bool wr = false;
         for (int pass = 0; pass < 2; pass++) {
             int k = 0;  // matches so far
             if (xl == 1) {
@@ -453,7 +366,7 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
                         if (m) {
                             const int at = k + __popc(bal & lt_mask);
                             const int2 v2 = make_int2(e[u].x & idmask, __float_as_int(sc));
-                            if (pass == 1) P.stage[dst + at] = v2;
+                            if (pass == 1) stage_put(P, S, (uint32_t)at, v2);
                             else if (at < JOIN_ECAP) elist[at] = v2;
                         }
                         k += __popc(bal);
@@ -517,20 +430,14 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
                         float y0 = 0.f;
                         // y[r0] <= 1 + 1e-3 (the norm tolerance): most pairs stop here, unloaded
                         bool look = s1 + x0 * 1.0011f > t - beta;
-                        int4 yc = make_int4(0, 0, 0, 0);  // {row offset, |y'|, ., ||y'||_2 bound}
+                        int4 yc = make_int4(0, 0, 0, 0);  // {row offset, |y'|, rank after y', ||y'||_2 bound}
                         if (look) {
                             yc = __ldg(&P.vcand[I.vbase + idb]);
-                            look = yc.y > 0 && s1 + x0 * __int_as_float(yc.w) > t - beta;
+                            look = yc.y > 0 && xe0.x < yc.z && s1 + x0 * __int_as_float(yc.w) > t - beta;
                         }
-                        if (look) {  // r0 in y's unindexed prefix (ranks increasing)?
+                        if (look) {  // r0 in y's unindexed prefix?
                             if (pass == 0) ct.verified++;
-                            for (int q = 0; q < yc.y; q++) {
-                                const int2 ye = __ldg(&P.crow[yc.x + q]);
-                                if (ye.x >= xe0.x) {
-                                    if (ye.x == xe0.x) y0 = __int_as_float(ye.y);
-                                    break;
-                                }
-                            }
+                            y0 = x_at(xe0.x, P.crow + yc.x, yc.y);
                         }
                         sbs = fmaf(x0, y0, s1);
                         if (sbs >= t + beta) {
@@ -547,13 +454,13 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
                     if (ma) {  // (a lane may hold a match in both lists)
                         const int at = k + __popc(mm & ((1u << ra) - 1u));
                         const int2 v2 = make_int2(ida, __float_as_int(sa));
-                        if (pass == 1) P.stage[dst + at] = v2;
+                        if (pass == 1) stage_put(P, S, (uint32_t)at, v2);
                         else if (at < JOIN_ECAP) elist[at] = v2;
                     }
                     if (mb) {
                         const int at = k + __popc(mm & ((1u << rb) - 1u));
                         const int2 v2 = make_int2(idb, __float_as_int(sbs));
-                        if (pass == 1) P.stage[dst + at] = v2;
+                        if (pass == 1) stage_put(P, S, (uint32_t)at, v2);
                         else if (at < JOIN_ECAP) elist[at] = v2;
                     }
                     k += __popc(mm);
@@ -564,33 +471,16 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
             if (pass == 0) {
                 cnt = k;
                 if (cnt == 0) break;
-                if (su + cnt > ss) {  // a new slab: one global atomic per slab
-                    const int64_t want = max(wslab, (int64_t)cnt);
-                    unsigned long long bw = 0;
-                    if (lane == 0) bw = atomicAdd(P.stage_count, (unsigned long long)want);
-                    sb = (int64_t)__shfl_sync(0xffffffffu, bw, 0);
-                    su = 0;
-                    ss = want;
-                }
-                dst = sb + su;
-                su += cnt;
-                wr = dst + cnt <= P.stage_cap;
+                __syncwarp();  // (the previous run's writers have read its place)
                 if (lane == 0) {
-                    const int64_t qw = I.qwbase + (int64_t)lx * I.nw + wf;
-                    P.cntq[qw] = cnt;
-                    if (wr) {
-                        Segment S;
-                        S.src = dst;
-                        S.cnt = cnt;
-                        S.i = lx;
-                        P.segs[qw] = S;
-                    }
-                    ct.pairs += (uint32_t)cnt;
+                    stage_take(S, P, (uint32_t)cnt);
+                    stage_close(S, P, x * P.parts, lx);
+                    tot.v[3] += (unsigned long long)cnt;
                 }
-                if (!wr) break;  // no room: the host grows the staging buffer and runs again
+                __syncwarp();
                 if (cnt <= JOIN_ECAP) {  // every match is in the scratch list
-                    __syncwarp();
-                    for (int q = lane; q < cnt; q += 32) P.stage[dst + q] = elist[q];
+#pragma unroll 1
+                    for (int q = lane; q < cnt; q += 32) stage_put(P, S, (uint32_t)q, elist[q]);
                     break;
                 }
             }
@@ -598,339 +488,443 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
     }
 }
 
-// One class of windowed items (G query groups per CTA, G known at compile time so that the
-// group's shared-memory layout is constant offsets): every group takes items from the
-// class's work list until it is empty, with its own work counters (folded into wtot).
-template <bool QMODE, bool SPLIT, int G>
-__device__ __forceinline__ void join_class(const JoinParams &P, const int64_t item_begin, const int64_t item_end,
-                                        unsigned long long *const work, unsigned long long *const wtot,
-                                        const bool f_minsize, const bool f_remscore, const bool f_upper) {
+// A warp's part of shared memory.
+struct Tile {
+    uint32_t *A;     // [W] accumulated scores, fixed point, units of 2^-30
+    uint32_t *bm;    // [W / 32] the window's matches
+    float *px;       // [64] norm of x on the rank buckets 0 .. b
+    int4 *wait;      // [32] lists of a long x waiting for a walk: {first position, entries, x's value, -}
+    int2 *seg;       // [32] the lists of a run: {first position - place in the run, x's value scaled by 2^30}
+    int2 *xr;        // [JOIN_XCAP] x's row, where it fits
+    uint16_t *list;  // [JOIN_LCAP] candidate slots
+};
+
+// What a walk needs beside its lists.
+struct WinCtx {
+    uint32_t smin_tag;
+    int32_t idmask;
+    int w0, first;  // first id of the window; first id after x
+};
+
+// Predicated single instructions for the walk's steps (the compiler turns the same conditions
+// written in C++ into divergent branches, which cost more than the instruction they guard).
+__device__ __forceinline__ uint32_t shl_clamped(const uint32_t v, const uint32_t by) {  // 0 from 32 on
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(by));
+    return r;
+}
+__device__ __forceinline__ void ldg_if(const bool on, const int2 *p, int2 &v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p ld.global.nc.v2.u32 {%0, %1}, [%2];\n\t}"
+                 : "+r"(v.x), "+r"(v.y)
+                 : "l"(p), "r"((uint32_t)on));
+}
+__device__ __forceinline__ uint32_t atoms_add_if(const bool on, const uint32_t addr, const uint32_t q) {  // old, or 1
+    uint32_t old;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.u32 %0, 1;\n\t@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
+                 : "=&r"(old)
+                 : "r"(addr), "r"(q), "r"((uint32_t)on)
+                 : "memory");
+    return old;
+}
+__device__ __forceinline__ void reds_add_if(const bool on, const uint32_t addr, const uint32_t q) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.shared.add.u32 [%0], %1;\n\t}" ::"r"(addr), "r"(q),
+                 "r"((uint32_t)on)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t lds_if(const bool on, const uint32_t addr) {  // or 0
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u32 %0, 0;\n\t@p ld.shared.u32 %0, [%1];\n\t}"
+                 : "=&r"(v)
+                 : "r"(addr), "r"((uint32_t)on)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts16_if(const bool on, const uint32_t addr, const uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tcvt.u16.u32 h, %1;\n\t@p st.shared.u16 [%0], h;\n\t}" ::"r"(addr),
+                 "r"(v), "r"((uint32_t)on)
+                 : "memory");
+}
+
+// 64 consecutive entries of a run, two per lane, and x's values for them.
+struct Round {
+    int2 ent[2];
+    float xs[2];
+};
+
+// The entries of up to 32 lists (lane l: cnt entries from post[st] on, x's value xv) as one
+// run, taken 32 consecutive entries per step whichever lists they belong to, two steps per round,
+// the next round's loads in flight while a round is added, so that short lists leave no lanes
+// idle. The lists of the first ncl lanes may create candidates (their slots go to the list, n its
+// length; slots past its end are counted only); those of the others only add where A is already
+// non-zero, and are left out while there is no candidate.
+__device__ __forceinline__ void walk(const Tile &T, const int2 *__restrict__ post, const WinCtx &C, const int ncl,
+                                     const uint32_t st, const int cnt, const float xv, const int lane, int &n,
+                                     uint32_t &visits, Totals &tot) {
+    const unsigned nonempty = __ballot_sync(0xffffffffu, cnt > 0);
+    if (!nonempty) return;
+    const unsigned lt_mask = (1u << lane) - 1u, le_mask = 2u * lt_mask + 1u;
+    int total;
+    int pre = warp_excl_scan_int(cnt, lane, &total);
+    // entries before the first updating list
+    const int cend = ncl >= 32 ? total : __shfl_sync(0xffffffffu, pre, ncl);
+    __syncwarp();  // (the previous run's readers are done)
+    if (cnt > 0)   // x's value scaled by 2^30 (exact)
+        T.seg[__popc(nonempty & lt_mask)] = make_int2((int)(st - (uint32_t)pre), __float_as_int(xv * 1073741824.f));
+    else
+        pre = 0x7fffffff;  // begins in no step
+    if (lane == 0) tot.v[5] += (unsigned long long)total;
+    __syncwarp();
+    const uint32_t abase = (uint32_t)__cvta_generic_to_shared(T.A) - 4u * (uint32_t)C.w0;  // slot of id 0
+    const uint32_t lbase = (uint32_t)__cvta_generic_to_shared(T.list);
+    int kb = -1;       // the list that holds the entry before the next step to load
+    int lb = lane;     // this lane's place in that step
+    int lpre = pre;    // pre minus the step's first place
+    auto load = [&](Round &R) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            // the lists that begin in this step, a bit at their place
+            const unsigned starts = __reduce_or_sync(0xffffffffu, shl_clamped(1u, (uint32_t)lpre));
+            const int2 sg = T.seg[kb + __popc(starts & le_mask)];
+            kb += __popc(starts);
+            R.xs[u] = __int_as_float(sg.y);
+            ldg_if(lb < total, post + (uint32_t)(sg.x + lb), R.ent[u]);
+            lb += 32;
+            lpre -= 32;
+        }
+    };
+    auto add = [&](const Round &R, const int base) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int b = base + 32 * u, p = b + lane;
+            const int id = R.ent[u].x & C.idmask;
+            const bool ok = p < total && (uint32_t)R.ent[u].x >= C.smin_tag && id >= C.first;
+            const uint32_t a = abase + 4u * (uint32_t)id;
+            visits += (uint32_t)ok;  // an entry Alg. 2 visits: y after x, |y| >= minsize
+            // rounded up, and at least one unit (the smallest addend keeps a tiny product from 0)
+            const uint32_t q = __float2uint_ru(fmaf(R.xs[u], __int_as_float(R.ent[u].y), 1e-30f));
+            if (b < cend) {
+                const uint32_t old = atoms_add_if(ok && p < cend, a, q);
+                const unsigned fresh = __ballot_sync(0xffffffffu, old == 0u);
+                const int at = n + __popc(fresh & lt_mask);
+                sts16_if(old == 0u && at < JOIN_LCAP, lbase + 2u * (uint32_t)at, (uint32_t)(id - C.w0));
+                n += __popc(fresh);
+                if (b + 32 >= cend) __syncwarp();  // creations land before updates
+            }
+            if (b + 32 > cend) {
+                const uint32_t v = lds_if(ok && p >= cend, a);
+                reds_add_if(v != 0u, a, q);
+            }
+        }
+    };
+    // one copy of the code for each: a join of a few thousand vectors runs it about once per warp,
+    // and its time is then the instruction fetches
+    Round R, N;
+    N.ent[0] = N.ent[1] = make_int2(0, 0);
+#pragma unroll 1
+    for (int base = -64; base < total; base += 64) {
+        if (base >= 0 && base >= cend && n == 0) break;
+        R = N;
+        if (base + 64 < total) load(N);
+        if (base >= 0) add(R, base);
+    }
+}
+
+// One class of windowed items with tile shape G: every warp takes units (a vector, or one
+// part of a heavy vector's windows) from the class's work list until it is empty.
+template <bool QMODE, bool SPLIT>
+__device__ __forceinline__ void join_class(const JoinParams &P, const int G, const int64_t item_begin,
+                                           const int64_t item_end, const int64_t heavy, unsigned long long *const work,
+                                           const bool f_minsize, const bool f_remscore, const bool f_upper,
+                                           Stager &S, Totals &tot) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Ctr ct;
-    constexpr int GT = JOIN_THREADS / G;
-    const int g = threadIdx.x / GT, gt = threadIdx.x % GT;
-    const int lane = gt & 31, gw = gt >> 5;
-    constexpr int NW = GT >> 5;
-    constexpr int WG = JOIN_WMAX / G, RG = JOIN_RMAX / G;
-    unsigned char *base = smem + (size_t)g * group_bytes(G);
-    uint32_t *A = reinterpret_cast<uint32_t *>(base);  // fixed point, units of 2^-30
-    uint32_t *pn4s = A + WG;                                        // [WG / 8], 16-byte aligned
-    int64_t *c_start = reinterpret_cast<int64_t *>(pn4s + WG / 8);  // [GT]
-    int32_t *c_cnt = reinterpret_cast<int32_t *>(c_start + GT);    // [GT]
-    int32_t *c_ch0 = c_cnt + GT;                                    // [GT + 4] chunk prefix
-    float *c_xv = reinterpret_cast<float *>(c_ch0 + GT + 4);        // [GT]
-    float *xtab = c_xv + GT;                                        // [RG]
-    int2 *xr = reinterpret_cast<int2 *>(xtab + RG);
-    constexpr int XG = JOIN_XCAP / G;
-    uint32_t *bm = reinterpret_cast<uint32_t *>(xr + XG);            // [WG / 32]
-    int64_t *wsum = reinterpret_cast<int64_t *>(bm + WG / 32);
-    int32_t *wcnt = reinterpret_cast<int32_t *>(wsum + 32);
-    int64_t *bc = reinterpret_cast<int64_t *>(wcnt + 32);
-    int2 *elist = P.scratch + ((size_t)blockIdx.x * NWARPS + (threadIdx.x >> 5)) * JOIN_ECAP;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp >= tile_warps(G)) return;
+    const int W = tile_window(G);
+    const uint32_t wmagic = 0xffffffffu / (uint32_t)W + 1u;  // a / W is the high word of a * wmagic, or less by one
     const unsigned lt_mask = (1u << lane) - 1u;
-
-    for (int i = gt; i < WG; i += GT) A[i] = 0u;
-    for (int i = gt; i < WG / 32; i += GT) bm[i] = 0u;
-    if (gt == 0) bc[3] = bc[4] = bc[5] = 0;  // this group's staging slab: base, used, size
-
+    Tile T;
+    T.A = reinterpret_cast<uint32_t *>(smem + (size_t)warp * tile_bytes(G));
+    T.bm = T.A + W;
+    T.px = reinterpret_cast<float *>(T.bm + W / 32);
+    T.wait = reinterpret_cast<int4 *>(T.px + 64);
+    T.seg = reinterpret_cast<int2 *>(T.wait + 32);
+    T.xr = T.seg + 32;
+    T.list = reinterpret_cast<uint16_t *>(T.xr + JOIN_XCAP);
+#pragma unroll 1
+    for (int i = lane; i < W + W / 32; i += 32) T.A[i] = 0u;
+    __syncwarp();
+    const uint32_t parts = (uint32_t)P.parts, ncut = (uint32_t)heavy * parts;
+    const uint32_t nunits = (uint32_t)(item_end - item_begin) + (uint32_t)heavy * (parts - 1u);
+    auto item_of = [&](const uint32_t unit) -> int64_t {
+        return item_begin + (unit < ncut ? unit / parts : unit - (uint32_t)heavy * (parts - 1u));
+    };
+    // A warp's first two units are its own, dealt over the SMs; the others are asked for two ahead
+    // and their work items read one ahead (lane 0). A small join thus runs without one atomic.
+    const uint32_t nwarps = gridDim.x * (uint32_t)tile_warps(G);
+    uint32_t u0 = blockIdx.x + gridDim.x * (uint32_t)warp, u1 = u0 + nwarps, x0 = 0;
+    if (lane == 0 && u0 < nunits) x0 = QMODE ? (uint32_t)item_of(u0) : (uint32_t)P.items[item_of(u0)];
     for (;;) {
-        ctr_flush(ct, wtot, lane);
-        gsync(G, g, GT);  // every thread is done with the previous item's broadcast slots
-        if (gt == 0) bc[0] = (int64_t)atomicAdd(work, 1ull) + item_begin;
-        gsync(G, g, GT);
-        const int64_t it = bc[0];
-        if (it >= item_end) break;
+        const uint32_t unit = __shfl_sync(0xffffffffu, u0, 0);
+        if (unit >= nunits) break;
         // x: a vector of the set (self-join: candidates are the later ids of its instance)
         // or an external query (all indexed vectors are candidates)
-        // query mode: item = (query, window), so the windows of a long query run on several
-        // CTAs at once instead of one after another
-        const int64_t x = QMODE ? it / P.qnw : (int64_t)P.items[it];
-        const int blk = (SPLIT && P.iblk) ? (int)P.iblk[it] : -1;  // group-uniform
-        const int wq_item = QMODE ? (int)(it % P.qnw) : 0;
-        const InstDesc I = P.inst[QMODE ? 0 : P.vinst[x]];
-        const int32_t lx = QMODE ? -1 : (int32_t)(x - I.vbase);
+        const uint32_t x = __shfl_sync(0xffffffffu, x0, 0);
+        if (lane == 0) {
+            u0 = u1;
+            if (u0 < nunits) {
+                u1 = (uint32_t)min(atomicAdd(work, 1ull) + 2ull * nwarps, 0xffffffffull);
+                x0 = QMODE ? (uint32_t)item_of(u0) : (uint32_t)P.items[item_of(u0)];
+            }
+        }
+        const int blk = (SPLIT && P.iblk) ? (int)P.iblk[item_of(unit)] : -1;
+        const InstDesc &I = P.inst[QMODE || P.one ? 0 : P.vinst[x]];
         const int4 xm = QMODE ? P.qvmeta[x] : P.vmeta[x];
-        const int2 *xrow = (QMODE ? P.qcrow : P.crow) + xm.x;
+        const uint32_t vbase = (uint32_t)I.vbase;
+        const int32_t lx = QMODE ? -1 : (int32_t)(x - vbase);
+        const int2 *xrow = (QMODE ? P.qcrow : P.crow) + (uint32_t)xm.x;
         const int32_t xl = xm.y;
-        const int32_t qs = f_remscore ? (QMODE ? P.qqsplit[x] : P.qsplit[x]) : 0;
-        const float mwx = QMODE ? P.qmw[x] : P.mw[x];
+        const int32_t qs = f_remscore ? xm.z : 0;
+        const float mwx = __int_as_float(xm.w);
         const float t = QMODE ? P.qt : I.t;
         const float beta = fmaxf(1e-5f, (float)(xl + 2) * 1.1920929e-7f);  // (|x|+2) * 2^-23
-        if (gt == 0) {  // what the emit step needs of x, kept in shared memory (not in registers)
-            bc[6] = QMODE ? x * I.nw : I.qwbase + (int64_t)lx * I.nw;  // x's first (x, window) slot
-            bc[7] = QMODE ? x : (int64_t)lx;                           // x's id in the output
+        if (qs >= xl) continue;  // no component may create: x has no candidate at all
+        // the windows of this unit: its share of those from x's successor on
+        const int nw = I.nw, IW = W, In = I.n;
+        int wfirst = 0;
+        if (!QMODE && nw > 1) {
+            wfirst = (int)__umulhi((uint32_t)lx + 1u, wmagic);
+            while ((uint32_t)wfirst * (uint32_t)W > (uint32_t)lx + 1u) wfirst--;
         }
-        // no component reaches remscore >= t: x can create no candidate at all
-        if (f_remscore ? qs >= xl : xl == 0) continue;
+        const uint32_t *const wp0 = P.wptr + I.wbase;
+        const int32_t rbase = I.rbase;
+        int wa = wfirst, wz = nw;
+        uint32_t part = 0;
+        if (unit < ncut && parts > 1u) {  // (nw * parts stays below 2^32: both are at most 2^31 / 1536, or small)
+            part = unit % parts;
+            wa = wfirst + (int)((uint32_t)(nw - wfirst) * (uint64_t)part / parts);
+            wz = wfirst + (int)((uint32_t)(nw - wfirst) * (uint64_t)(part + 1u) / parts);
+        }
+        if (wa >= wz) continue;
         // A block item walks its share of x's creating components (every nblk-th, from its
         // block index on) and all of x's updating ones, which only add to candidates its
         // own creating components made.
         const int cstr = blk < 0 ? 1 : P.nblk, coff = blk < 0 ? 0 : blk;
         const int ncreate = blk < 0 ? xl - qs : (xl - qs > blk ? (xl - qs - blk + P.nblk - 1) / P.nblk : 0);
-        const int nwalk = ncreate + qs;  // components this item walks
         if (ncreate == 0) continue;
-        // minsize: a match y needs |y| >= t / maxweight(x) (margin for rounding and the
-        // 1e-3 norm tolerance); the size class byte of each entry is compared with it
-        // (float, directed rounding: numerator down, denominator up, quotient down, so the
-        // bound can only come out below its exact value and never prunes a match)
+        WinCtx C;
+        // minsize: a match y needs |y| >= t / maxweight(x) (a margin of 1e-5 for rounding, over
+        // the 1e-3 norm tolerances, so the bound can only come out below its exact value and
+        // never prunes a match); the size class byte of each entry is compared with it
         int smin = 0;
         if (f_minsize && I.packed && mwx > 0.f)
-            smin = (int)ceilf(fminf(__fdiv_rd(__fsub_rd(t, beta), __fmul_ru(mwx, 1.0020001f)), 255.f));
-        const uint32_t smin_tag = (uint32_t)max(smin, 0) << 24;
-        const int32_t idmask = I.packed ? 0x00ffffff : 0x7fffffff;
-        // dense table of x over small ranks for dot(x, y')
-        for (int i = gt; i < RG; i += GT) xtab[i] = 0.f;
-        gsync(G, g, GT);
-        const int xs = xl <= XG ? xl : 0;  // x's row in shared memory when it fits
-        for (int c = gt; c < xl; c += GT) {
-            const int2 e = xrow[c];
-            if (e.x < RG) xtab[e.x] = __int_as_float(e.y);
-            if (c < xs) xr[c] = e;
+            smin = (int)ceilf(fminf(__fdividef(t - beta, mwx) * 0.99799f, 255.f));
+        C.smin_tag = (uint32_t)max(smin, 0) << 24;
+        C.idmask = I.packed ? 0x00ffffff : 0x7fffffff;
+        C.first = lx + 1;
+        // x's norms up to each rank bucket, rounded up
+        {
+            uint32_t *pu = reinterpret_cast<uint32_t *>(T.px);
+            pu[lane] = pu[lane + 32] = 0u;
+            __syncwarp();
+#pragma unroll 1
+            for (int c = lane; c < xl; c += 32) {
+                const int2 e = __ldg(xrow + c);
+                const float v = __int_as_float(e.y);
+                atomicAdd(&pu[rank_bucket(e.x)], __float2uint_ru(__fmul_ru(__fmul_ru(v, v), 1073741824.f)));
+            }
+            __syncwarp();
+            const uint32_t p0 = pu[2 * lane], p1 = pu[2 * lane + 1];
+            int sum;
+            const uint32_t ex = (uint32_t)warp_excl_scan_int((int)(p0 + p1), lane, &sum);
+            __syncwarp();
+            // (the approximate square root is good to a few units in the last place)
+            const float s0 = __uint2float_ru(ex + p0) * 9.31322574615478515625e-10f;
+            const float s1 = __uint2float_ru(ex + p0 + p1) * 9.31322574615478515625e-10f;
+            T.px[2 * lane] = s0 > 0.f ? s0 * rsqrtf(s0) * 1.00001f : 0.f;
+            T.px[2 * lane + 1] = s1 > 0.f ? s1 * rsqrtf(s1) * 1.00001f : 0.f;
         }
-        gsync(G, g, GT);
-
-        const int wfirst = QMODE ? wq_item : (lx + 1) / I.W;
-        const int wend = QMODE ? wq_item + 1 : I.nw;
-        for (int w = wfirst; w < wend; w++) {
-            const int w0 = w * I.W;
-            const int wn = min(I.W, I.n - w0);
-            const int lo = max(0, lx + 1 - w0);
-            bool created = false;  // any entry of a creating component in this window
-            if (f_upper || blk >= 0) {  // the window's 4-bit ||y'||_2 codes into shared memory, behind the accumulation
-                const uint32_t *src = P.pn4 + I.pbase + (w0 >> 3);
-                for (int q = gt; q < (wn + 31) >> 5; q += GT) cp_async16(pn4s + 4 * q, src + 4 * q);
-                cp_async_commit();
-            }
-            // ---------------- accumulate. Components are walked creating-first (those with
-            // remscore >= t), so every batch holds its creating part before its updating part.
-            if (nwalk <= 32) {
-                // a short x: every warp builds the window's segment table itself, lane c
-                // holding component c (no shared table, no barrier)
-                int64_t st = 0;
-                int cnt = 0;
-                float xv = 0.f;
-                if (lane < nwalk) {
-                    const int c = lane < ncreate ? qs + coff + lane * cstr : lane - ncreate;
-                    const int2 e = c < xs ? xr[c] : xrow[c];
-                    const int64_t R = (int64_t)I.rbase + e.x;
-                    xv = __int_as_float(e.y);
-                    int64_t ls = P.lptr[R], le = P.lptr[R + 1];
-                    if (I.nw > 1) {
-                        const int32_t *wp = P.wptr + I.wbase + (int64_t)e.x * (I.nw + 1);
-                        le = ls + wp[w + 1];
-                        ls = ls + wp[w];
-                    }
-                    cnt = (int32_t)(le - ls);
-                    st = ls;
-                    if (gw == 0) ct.read += (uint32_t)cnt;
-                }
-                const int nch = (cnt + 127) >> 7;
-                int nchk;
-                const int ch0 = warp_excl_scan_int(nch, lane, &nchk);
-                const int P0 = ncreate > 0 ? __shfl_sync(0xffffffffu, ch0 + nch, ncreate - 1) : 0;
-                created = P0 > 0;
-                for (int phase = 0; phase < 2; phase++) {
-                    const int pb = phase == 0 ? 0 : P0, pe = phase == 0 ? P0 : nchk;
-                    if (pe <= pb) continue;
-                    if (phase == 1 && P0 > 0) gsync(G, g, GT);  // creations land before updates
-                    const int K = (pe - pb + NW - 1) / NW;
-                    const int ch = pb + gw * K;
-                    const int che = min(ch + K, pe);
-                    if (ch >= che) continue;
-                    // the last component with entries whose first chunk is at or before ch
-                    const int cc = 31 - __clz(__ballot_sync(0xffffffffu, nch > 0 && ch0 <= ch));
-                    if (phase == 0) {
-                        if (lo > 0) walk_chunks_r<true, true>(ch, che, cc, st, cnt, ch0, xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                        else walk_chunks_r<true, false>(ch, che, cc, st, cnt, ch0, xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                    } else {
-                        if (lo > 0) walk_chunks_r<false, true>(ch, che, cc, st, cnt, ch0, xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                        else walk_chunks_r<false, false>(ch, che, cc, st, cnt, ch0, xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                    }
-                }
-                cp_async_wait_all();  // the window's codes have landed (visible after the barrier)
-                gsync(G, g, GT);
-            } else
-            for (int c0 = 0; c0 < nwalk; c0 += GT) {
-                const int cp = c0 + gt;
-                int64_t st = 0;
-                int32_t cnt = 0;
-                float xv = 0.f;
-                const bool ph0 = cp < ncreate;
-                if (cp < nwalk) {
-                    const int c = ph0 ? qs + coff + cp * cstr : cp - ncreate;
-                    const int2 e = c < xs ? xr[c] : xrow[c];  // x's row from shared memory when held there
-                    const int64_t R = (int64_t)I.rbase + e.x;
-                    xv = __int_as_float(e.y);
-                    int64_t ls = P.lptr[R], le = P.lptr[R + 1];
-                    if (I.nw > 1) {
-                        const int32_t *wp = P.wptr + I.wbase + (int64_t)e.x * (I.nw + 1);
-                        le = ls + wp[w + 1];
-                        ls = ls + wp[w];
-                    }
-                    cnt = (int32_t)(le - ls);
-                    st = ls;
-                    ct.read += (uint32_t)cnt;  // every entry of the window's list is loaded
-                }
-                // scan of (chunks, non-empty, non-empty creating) packed in one int64
-                const int64_t nch = (cnt + 127) >> 7;
-                const int64_t packed = (nch << 22) | ((cnt > 0 && ph0) ? (1 << 11) : 0) | (cnt > 0 ? 1 : 0);
-                const int64_t inc = warp_incl_scan(packed, lane);
-                if (lane == 31) wsum[gw] = inc;
-                gsync(G, g, GT);
-                const int64_t wv = lane < NW ? wsum[lane] : 0;
-                const int64_t winc = warp_incl_scan(wv, lane);
-                const int64_t before = __shfl_sync(0xffffffffu, winc - wv, gw);
-                const int64_t total = __shfl_sync(0xffffffffu, winc, NW - 1);
-                const int64_t ex = before + inc - packed;
-                if (cnt > 0) {
-                    const int pos = (int)(ex & 2047);
-                    c_start[pos] = st;
-                    c_cnt[pos] = cnt;
-                    c_ch0[pos] = (int32_t)(ex >> 22);
-                    c_xv[pos] = xv;
-                }
-                const int ncomp = (int)(total & 2047);
-                const int ncomp0 = (int)((total >> 11) & 2047);
-                const int nchk = (int)(total >> 22);
-                if (gt == 0) c_ch0[ncomp] = nchk;
-                gsync(G, g, GT);
-                const int P0 = c_ch0[ncomp0];
-                created = created || P0 > 0;
-                // phase 0 chunks [0, P0) create candidates; phase 1 chunks [P0, nchk) update
-                for (int phase = 0; phase < 2; phase++) {
-                    const int pb = phase == 0 ? 0 : P0, pe = phase == 0 ? P0 : nchk;
-                    if (pe <= pb) continue;
-                    if (phase == 1 && P0 > 0) gsync(G, g, GT);  // creations land before updates
-                    const int K = (pe - pb + NW - 1) / NW;
-                    int ch = pb + gw * K;
-                    const int che = min(ch + K, pe);
-                    if (ch >= che) continue;
-                    int cc = 0;
-                    {  // component holding the warp's first chunk
-                        int a = 0, b = ncomp - 1;
-                        while (a < b) {
-                            const int mid = (a + b + 1) >> 1;
-                            if (c_ch0[mid] <= ch) a = mid; else b = mid - 1;
+        // A candidate is worth verifying when A[y] + ||x before y's lists|| * ||y'|| exceeds
+        // t - beta. A block item keeps y by Lemma 1 (local pruning): a match scores
+        // A + dot(x, y') >= t, the blocks that created y hold all of A between them, so one
+        // of them has A_b >= (t - dot(x, y')) / nblk.
+        const float scale = (SPLIT && blk >= 0 ? (float)P.nblk : 1.f) * 9.31322574615478515625e-10f * 1.000001f;
+        const float floor_ = f_upper || blk >= 0 ? t - beta : -1.f;
+        // x's row in shared memory where it fits (verification searches it)
+        const int2 *xs = xrow;
+        if (xl <= JOIN_XCAP) {
+#pragma unroll 1
+            for (int c = lane; c < xl; c += 32) T.xr[c] = __ldg(xrow + c);
+            xs = T.xr;
+            __syncwarp();
+        }
+        // The lists of a short x stay in registers over the windows (a lane each, the creating
+        // ones first), and so do their positions: a window's lists end where the next one's
+        // begin, so each window loads one position per list, for the window after it.
+        const bool shortx = ncreate + qs <= 32;
+        auto list_at = [&](const int r, const int w) -> uint32_t {
+            return nw > 1 ? __ldg(wp0 + (int64_t)r * (nw + 1) + w) : (uint32_t)__ldg(P.lptr + (rbase + r + w));
+        };
+        int2 e0 = make_int2(0, 0);
+        uint32_t p0 = 0, p1 = 0;
+        if (shortx && lane < ncreate + qs) {
+            e0 = xs[lane < ncreate ? qs + coff + lane * cstr : lane - ncreate];
+            p0 = list_at(e0.x, wa);
+            p1 = list_at(e0.x, wa + 1);
+        }
+        uint32_t visits = 0;
+#pragma unroll 1
+        for (int w = wa; w < wz; w++) {
+            const int w0 = w * IW;
+            const int wn = min(IW, In - w0);
+            C.w0 = w0;
+            int n = 0;  // candidates
+            // A short x: one walk, its creating lists first. A long one: create, then update (only
+            // where there are candidates); the non-empty lists of the window are gathered over
+            // blocks of 32 components and walked 32 at a time, because most lists of a long
+            // vector have no entry in a given window.
+            uint32_t p2 = p1;  // the next window's list ends
+            if (shortx && w + 1 < wz && lane < ncreate + qs) p2 = list_at(e0.x, w + 2);
+            uint32_t st = p0;
+            int cnt = (int)(p1 - p0), k0 = 0;
+            float xv = __int_as_float(e0.y);
+            for (int ph = 0;;) {
+                if (!shortx) {
+                    const bool create = ph == 0;
+                    const int count = create ? ncreate : qs;
+                    int qn = 0;  // lists gathered
+#pragma unroll 1
+                    for (; k0 < count; k0 += 32) {
+                        int2 e = make_int2(0, 0);
+                        uint32_t s0 = 0, s1 = 0;
+                        if (k0 + lane < count) {
+                            e = xs[create ? qs + coff + (k0 + lane) * cstr : k0 + lane];
+                            s0 = list_at(e.x, w);
+                            s1 = list_at(e.x, w + 1);
                         }
-                        cc = a;
+                        const unsigned have = __ballot_sync(0xffffffffu, s1 > s0);
+                        if (qn + __popc(have) > 32) break;  // no room: this block again, after the walk
+                        if (s1 > s0) T.wait[qn + __popc(have & lt_mask)] = make_int4((int)s0, (int)(s1 - s0), e.y, 0);
+                        qn += __popc(have);
                     }
-                    // four specialisations: creating or updating, first window (ids at or
-                    // below x present) or not
-                    if (phase == 0) {
-                        if (lo > 0) walk_chunks<true, true>(ch, che, cc, c_start, c_cnt, c_ch0, c_xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                        else walk_chunks<true, false>(ch, che, cc, c_start, c_cnt, c_ch0, c_xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                    } else {
-                        if (lo > 0) walk_chunks<false, true>(ch, che, cc, c_start, c_cnt, c_ch0, c_xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                        else walk_chunks<false, false>(ch, che, cc, c_start, c_cnt, c_ch0, c_xv, P.post, A, bm, smin_tag, idmask, w0, lo, lane, ct.visits);
-                    }
+                    __syncwarp();
+                    const int4 g = lane < qn ? T.wait[lane] : make_int4(0, 0, 0, 0);
+                    st = (uint32_t)g.x;
+                    cnt = g.y;
+                    xv = __int_as_float(g.z);
                 }
-                cp_async_wait_all();  // the window's codes have landed (visible after the barrier)
-                gsync(G, g, GT);
+                walk(T, P.post, C, shortx ? ncreate : ph == 0 ? 32 : 0, st, cnt, xv, lane, n, visits, tot);
+                __syncwarp();
+                if (shortx) break;
+                if (k0 >= (ph == 0 ? ncreate : qs)) {
+                    if (ph == 1 || n == 0) break;
+                    ph = 1;
+                    k0 = 0;
+                }
             }
-            if (!created) continue;  // no candidate can exist in this window
-            // ---------------- verify. The creating pass marked every candidate in bm. Each
-            // warp walks its share of bm 32 words (1024 slots) at a time, a word per lane.
-            // First each lane tests its word's candidates against the window's ||y'||_2
-            // codes: since dot(x, y') <= ||y'||_2, a candidate with A[y] + ||y'||_2 <=
-            // t - beta cannot match (most stop here, with no global load; their A is
-            // cleared). Then the remaining bits are taken in slot order, 32 candidates per
-            // batch: lane j of a batch takes the candidate at position b + j, located from
-            // the lanes' popcount prefix. Taken slots are cleared in A (bm words as they are
-            // read), and the emitted (y, score) go to the warp's scratch list in increasing y.
-            const int wlo = lo >> 5, whi = (wn + 31) >> 5;
-            const int wper = (whi - wlo + NW - 1) / NW;
-            const int wb = wlo + gw * wper, we = min(wb + wper, whi);
-            // A[y] + ||y'||_2 <= t - beta in units of 2^-30: threshold rounded down, codes
-            // rounded up, so the test keeps at least every candidate the exact one keeps
-            const uint32_t thq = __float2uint_rd(fmaxf(t - beta, 0.f) * 1073741824.f);
-            int ne = 0;
-            for (int wq = wb; wq < we; wq += 32) {
-                uint32_t word = 0u;
-                if (wq + lane < we) {
-                    word = bm[wq + lane];
-                    bm[wq + lane] = 0u;
-                }
-                ct.cand += (uint32_t)__popc(word);
-                if (f_upper || blk >= 0) {
-                    // a block item keeps y by Lemma 1 (local pruning): a match scores
-                    // A + dot(x, y') >= t, the blocks that created y hold all of A between
-                    // them, so one of them has A_b >= (t - ||y'||_2) / nblk
-                    const uint32_t mul = blk < 0 ? 1u : (uint32_t)P.nblk;
-                    const int sb = (wq + lane) << 5;
-                    uint32_t keep = 0u;
-                    for (uint32_t wv = word; wv; wv &= wv - 1u) {
-                        const int b = __ffs(wv) - 1;
-                        const int sl = sb + b;
-                        const uint32_t a = A[sl];
-                        const uint32_t code = (pn4s[sl >> 3] >> ((sl & 7) << 2)) & 15u;
-                        const bool kp = SPLIT ? (uint64_t)a * mul + code * PN4_UNIT > (uint64_t)thq
-                                              : a + code * PN4_UNIT > thq;
-                        if (kp) keep |= 1u << b; else A[sl] = 0u;
+            p0 = p1;
+            p1 = p2;
+            if (n == 0) continue;  // no candidate in this window
+            __syncwarp();
+            // ---------------- filter and verify: the candidate list at once, or, when it ran
+            // over, the slots of the window in stretches of JOIN_LCAP
+            const uint8_t *codes = P.code + (vbase + (uint32_t)w0);
+            const int4 *cands = P.vcand + (vbase + (uint32_t)w0);
+            const bool over = n > JOIN_LCAP;
+            if (lane == 0) tot.v[1] += (unsigned long long)n;
+            int nm = 0;  // matches
+            for (int s0 = 0; s0 < (over ? wn : 1); s0 += JOIN_LCAP) {
+                if (over) {
+                    n = 0;
+#pragma unroll 1
+                    for (int q = s0; q < min(s0 + JOIN_LCAP, wn); q += 32) {
+                        const bool on = q + lane < wn && T.A[q + lane] != 0u;
+                        const unsigned bal = __ballot_sync(0xffffffffu, on);
+                        if (on) T.list[n + __popc(bal & lt_mask)] = (uint16_t)(q + lane);
+                        n += __popc(bal);
                     }
-                    word = keep;
+                    __syncwarp();
                 }
-                const int c = __popc(word);
-                int T;
-                const int excl = warp_excl_scan_int(c, lane, &T);
-                const int incl = excl + c;
-                for (int b0 = 0; b0 < T; b0 += 32) {
-                    const int p = b0 + lane;
-                    // owner: the first lane whose inclusive count exceeds p (31 when p >= T)
-                    int own = 0;
+                int ns = 0;
+#pragma unroll 1
+                for (int b = 0; b < n; b += 128) {  // four codes per lane in flight
+                    int slot[4], code[4];
 #pragma unroll
-                    for (int step = 16; step; step >>= 1)
-                        if (__shfl_sync(0xffffffffu, incl, own + step - 1) <= p) own += step;
-                    uint32_t ow = __shfl_sync(0xffffffffu, word, own);
-                    const int oex = __shfl_sync(0xffffffffu, excl, own);
-                    const bool have = p < T;
+                    for (int u = 0; u < 4; u++) {
+                        slot[u] = -1;
+                        code[u] = 0;
+                        if (b + 32 * u + lane < n) {
+                            slot[u] = T.list[b + 32 * u + lane];
+                            code[u] = __ldg(codes + slot[u]);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        bool keep = false;
+                        if (slot[u] >= 0) {
+                            const float pn = (float)(code[u] & 15) * (PN4_STEP * 1.0001f);
+                            keep = fmaf(__uint2float_ru(T.A[slot[u]]), scale, T.px[(code[u] >> 4) * 4 + 3] * pn) > floor_;
+                            if (!keep) T.A[slot[u]] = 0u;
+                        }
+                        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                        if (keep) T.list[ns + __popc(bal & lt_mask)] = (uint16_t)slot[u];  // (already read)
+                        ns += __popc(bal);
+                    }
+                    __syncwarp();
+                }
+#pragma unroll 1
+                for (int b = 0; b < ns; b += 32) {
                     bool emit = false;
                     float sc = 0.f, v = 0.f;
-                    int s = 0;
-                    int4 yc = make_int4(0, 0, 0, 0);  // {row offset, |y'|, maxweight(y'), ||y'||_2 bound}
+                    int slot = 0;
+                    int4 yc = make_int4(0, 0, 0, 0);  // {row offset, |y'|, first rank after y', ||y'||_2 bound}
                     // 0: rejected or emitted, 1: score known, 2: short dot(x, y') left, 3: long one
                     int stage = 0;
-                    if (have) {
-                        for (int k = p - oex; k > 0; k--) ow &= ow - 1u;
-                        s = ((wq + own) << 5) + (__ffs(ow) - 1);
-                        v = __uint2float_rn(A[s]) * 9.31322574615478515625e-10f;  // 2^-30
-                        A[s] = 0u;
-                        yc = __ldg(&P.vcand[I.vbase + w0 + s]);
-                        const int ys = blk < 0 ? yc.y : 0;  // a block item scores y whole, below
-                        bool ok = true;
-                        // (a block item's A is a partial sum: these bounds apply to whole sums
-                        // only, and the block's candidates passed the local test instead)
-                        if (f_upper && blk < 0) {
-                            // dot(x, y') <= ||y'||_2 (Cauchy-Schwarz; most candidates stop here),
-                            // then the paper's upperbound; both off with NO_UPPERBOUND
-                            ok = v + __int_as_float(yc.w) > t - beta;
-                            if (ok && ys > 0) ok = v + (float)min(ys, xl) * mwx * __int_as_float(yc.z) >= t - beta;
-                        }
-                        if (ok) {
+                    if (b + lane < ns) {
+                        slot = T.list[b + lane];
+                        v = __uint2float_rn(T.A[slot]) * 9.31322574615478515625e-10f;  // 2^-30
+                        yc = __ldg(cands + slot);
+                        if (SPLIT && blk >= 0) {  // a partial sum: y scored whole, in float64
+                            stage = 4;
+                        } else if (!f_upper || v + T.px[rank_bucket(yc.z)] * __int_as_float(yc.w) * 1.00001f > t - beta) {
                             sc = v;
-                            stage = ys == 0 ? 1 : (ys <= 16 ? 2 : 3);
+                            stage = yc.y == 0 ? 1 : (yc.y <= 16 ? 2 : 3);
                         }
-                        if (blk >= 0) stage = 4;  // kept by the local test: score decided in float64
+                    }
+                    {
+                        const unsigned dots = __ballot_sync(0xffffffffu, stage == 2 || stage == 3);
+                        if (lane == 0 && dots) tot.v[2] += (unsigned long long)__popc(dots);
                     }
                     if (stage == 2) {  // short prefixes: each lane its own candidate
-                        ct.verified++;
-                        sc = v + dot_prefix(P.crow + yc.x, yc.y, xtab, RG, xr, xs, xrow, xl);
+                        const int2 *yr = P.crow + (uint32_t)yc.x;
+                        float acc = 0.f;
+                        int at = 0;  // both rows in rank order: x is searched from the last place on
+#pragma unroll 1
+                        for (int k = 0; k < yc.y && at < xl; k++) {
+                            const int2 e = __ldg(yr + k);
+                            at = row_find(xs, at, xl, e.x);
+                            if (at < xl) {
+                                const int2 xe = xs[at];
+                                if (xe.x == e.x) acc = fmaf(__int_as_float(xe.y), __int_as_float(e.y), acc);
+                            }
+                        }
+                        sc = v + acc;
                         stage = 1;
                     }
                     // long prefixes: the whole warp takes one candidate at a time, its lanes
                     // reading y's prefix entries side by side
                     for (unsigned lm = __ballot_sync(0xffffffffu, stage == 3); lm; lm &= lm - 1u) {
                         const int src = __ffs(lm) - 1;
-                        const int yo = __shfl_sync(0xffffffffu, yc.x, src);
+                        const uint32_t yo = (uint32_t)__shfl_sync(0xffffffffu, yc.x, src);
                         const int yl = __shfl_sync(0xffffffffu, yc.y, src);
                         float acc = 0.f;
+#pragma unroll 1
                         for (int k = lane; k < yl; k += 32) {
                             const int2 e = __ldg(&P.crow[yo + k]);
-                            acc = fmaf(x_at(e.x, xtab, RG, xr, xs, xrow, xl), __int_as_float(e.y), acc);
+                            acc = fmaf(x_at(e.x, xs, xl), __int_as_float(e.y), acc);
                         }
 #pragma unroll
                         for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
                         if (lane == src) {
-                            ct.verified++;
                             sc = v + acc;
                             stage = 1;
                         }
@@ -945,186 +939,226 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int64_t it
                     }
                     if (stage == 4) stage = 1;
                     // inside the band: float64 dot(x, y) over all of y, one candidate at a
-                    // time across the warp (x's values from shared memory, exact products)
+                    // time across the warp (exact products)
                     int yfull = 0;
-                    if (stage == 1) yfull = __ldg(&P.vmeta[I.vbase + w0 + s]).y;
+                    if (stage == 1) yfull = __ldg(&P.vmeta[vbase + (uint32_t)(w0 + slot)]).y;
                     for (unsigned lm = __ballot_sync(0xffffffffu, stage == 1); lm; lm &= lm - 1u) {
                         const int src = __ffs(lm) - 1;
-                        const int yo = __shfl_sync(0xffffffffu, yc.x, src);
+                        const uint32_t yo = (uint32_t)__shfl_sync(0xffffffffu, yc.x, src);
                         const int yl = __shfl_sync(0xffffffffu, yfull, src);
                         double acc = 0.0;
+#pragma unroll 1
                         for (int k = lane; k < yl; k += 32) {
-                            const int2 e = P.crow[yo + k];
-                            acc += (double)x_at(e.x, xtab, RG, xr, xs, xrow, xl) * (double)__int_as_float(e.y);
+                            const int2 e = __ldg(&P.crow[yo + k]);
+                            acc += (double)x_at(e.x, xs, xl) * (double)__int_as_float(e.y);
                         }
 #pragma unroll
                         for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                        if (lane == 0) tot.v[4]++;
                         if (lane == src) {
-                            ct.band++;
                             emit = acc >= (double)t;
                             sc = (float)acc;
                         }
                     }
                     const unsigned bal = __ballot_sync(0xffffffffu, emit);
-                    if (blk >= 0) {  // block items: pairs to the global list, merged after the join
-                        unsigned long long b = 0;
-                        if (lane == 0 && bal) b = atomicAdd(P.sp_count, (unsigned long long)__popc(bal));
-                        b = __shfl_sync(0xffffffffu, b, 0) + (unsigned long long)__popc(bal & lt_mask);
-                        if (emit && b < (unsigned long long)P.sp_cap) {
-                            P.sp_key[b] = (unsigned long long)lx * (unsigned long long)I.n + (unsigned long long)(w0 + s);
-                            P.sp_score[b] = __float_as_uint(sc);
+                    if (SPLIT && blk >= 0) {  // block items: pairs to the global list, merged after the join
+                        unsigned long long g = 0;
+                        if (lane == 0 && bal) g = atomicAdd(P.sp_count, (unsigned long long)__popc(bal));
+                        g = __shfl_sync(0xffffffffu, g, 0) + (unsigned long long)__popc(bal & lt_mask);
+                        if (emit && g < (unsigned long long)P.sp_cap) {
+                            P.sp_key[g] = (unsigned long long)lx * (unsigned long long)In + (unsigned long long)(w0 + slot);
+                            P.sp_score[g] = __float_as_uint(sc);
                         }
+                        emit = false;
                     } else {
-                        if (emit) elist[ne + __popc(bal & lt_mask)] = make_int2(w0 + s, __float_as_int(sc));
-                        ne += __popc(bal);
+                        nm += __popc(bal);
+                    }
+                    if (b + lane < ns) {
+                        T.A[slot] = emit ? __float_as_uint(sc) : 0u;
+                        if (emit) atomicOr(&T.bm[slot >> 5], 1u << (slot & 31));
                     }
                 }
+                __syncwarp();
             }
-            if (blk >= 0) {  // (group-uniform) no run for this (x, window) slot; the barrier
-                gsync(G, g, GT);  // keeps the next window's copies and adds off this window's data
-                continue;
+            if (nm == 0) continue;
+            // ---------------- emit the window's matches in id order
+            if (lane == 0) {
+                stage_take(S, P, (uint32_t)nm);
+                tot.v[3] += (unsigned long long)nm;
             }
-            if (lane == 0) wcnt[gw] = ne;
-            gsync(G, g, GT);
-            if (gw == 0) {  // offsets of the warps' runs; the window's run in the group's slab
-                const int cw = lane < NW ? wcnt[lane] : 0;
-                int tot;
-                const int exw = warp_excl_scan_int(cw, lane, &tot);
-                if (lane < NW) wcnt[lane] = exw;
-                if (lane == 0) {
-                    const int64_t qw = bc[6] + w;
-                    P.cntq[qw] = tot;
-                    int64_t b = 0, wr = 0;
-                    if (tot > 0) {
-                        if (bc[4] + tot > bc[5]) {  // a new slab: one global atomic per slab
-                            const int64_t want = max(P.stage_slab, (int64_t)tot);
-                            bc[3] = (int64_t)atomicAdd(P.stage_count, (unsigned long long)want);
-                            bc[4] = 0;
-                            bc[5] = want;
-                        }
-                        b = bc[3] + bc[4];
-                        bc[4] += tot;
-                        if (b + tot <= P.stage_cap) {
-                            Segment S;
-                            S.src = b;
-                            S.cnt = tot;
-                            S.i = (int32_t)bc[7];
-                            P.segs[qw] = S;
-                            wr = 1;
-                        }
-                    }
-                    ct.pairs += (uint32_t)tot;
-                    bc[1] = b;
-                    bc[2] = wr;
+            __syncwarp();
+            uint32_t at = 0;
+#pragma unroll 1
+            for (int q = lane; q - lane < (wn + 31) >> 5; q += 32) {
+                uint32_t word = 0u;
+                if (q < (wn + 31) >> 5) {
+                    word = T.bm[q];
+                    if (word) T.bm[q] = 0u;
                 }
-            }
-            gsync(G, g, GT);
-            // ---------------- copy the warp's emitted pairs to the reserved run
-            if (bc[2] != 0) {
-                int2 *dst = P.stage + bc[1] + wcnt[gw];
-                for (int k = lane; k < ne; k += 32) dst[k] = elist[k];
+                int sum;
+                uint32_t p = at + (uint32_t)warp_excl_scan_int(__popc(word), lane, &sum);
+                at += (uint32_t)sum;
+#pragma unroll 1
+                for (; word; word &= word - 1u) {
+                    const int slot = (q << 5) + __ffs(word) - 1;
+                    stage_put(P, S, p++, make_int2(w0 + slot, (int)T.A[slot]));
+                    T.A[slot] = 0u;
+                }
             }
             __syncwarp();
         }
+        if (lane == 0) stage_close(S, P, (int64_t)x * parts + part, QMODE ? (int32_t)x : lx);
+        count_add(tot, 0, visits, lane);
+        __syncwarp();
     }
-    ctr_flush(ct, wtot, lane);
 }
 
-// QMODE: external queries against the index (P.qmode = 1); SPLIT: a self-join whose work
-// list may hold dimension-block items (P.iblk). Each is compiled separately, so that the
-// plain self-join carries none of the other paths' state.
+// QMODE: external queries against the index; SPLIT: a self-join whose work list may hold
+// dimension-block items (P.iblk). Each is compiled separately, so that the plain self-join
+// carries none of the other paths' state.
 template <bool QMODE, bool SPLIT = false>
 __global__ void __launch_bounds__(JOIN_THREADS, 1) join_kernel(const __grid_constant__ JoinParams P) {
     const bool f_minsize = !(P.flags & APS_NO_MINSIZE);
     const bool f_remscore = !(P.flags & APS_NO_REMSCORE);
     const bool f_upper = !(P.flags & APS_NO_UPPERBOUND);
-    // per-warp 64-bit work totals (visits, candidates, verified, pairs, band, entries read)
-    __shared__ unsigned long long wtot_s[NWARPS][6];
-    for (int i = threadIdx.x; i < NWARPS * 6; i += blockDim.x) (&wtot_s[0][0])[i] = 0ull;
-    __syncthreads();
-    unsigned long long *const wtot = wtot_s[threadIdx.x >> 5];
-    // A CTA that finds a class's work list empty moves on to the next class and re-carves
-    // its shared memory for that class's G, so the classes share one launch and one tail.
+    __shared__ Stager stagers[JOIN_WARPS];
+    __shared__ Totals totals[JOIN_WARPS];
+    const int warp = threadIdx.x >> 5;
+    Stager &S = stagers[warp];
+    Totals &tot = totals[warp];
+    if ((threadIdx.x & 31) == 0) {
+        memset(&tot, 0, sizeof(tot));
+        memset(&S, 0, sizeof(S));
+        S.piece = -1;
+    }
+    __syncwarp();
+    // A warp that finds a class's work list empty waits for the CTA's other warps before the
+    // next class's tiles take their place in shared memory: the classes share one launch and
+    // one tail. (The streamed class needs no tile.)
     for (int cls = 0; cls < P.ncls; cls++) {
-    const int64_t item_begin = P.cls_begin[cls], item_end = P.cls_begin[cls + 1];
-    if (item_end <= item_begin) continue;
-    const int G = P.cls_G[cls];
-    unsigned long long *const work = P.work + cls;
-    if (!QMODE && G == 0) {  // vectors with one or two components: one warp each, no shared memory
-        stream_short(P, work, item_begin, item_end, f_minsize, f_remscore, wtot);
-        continue;
+        const int64_t item_begin = P.cls_begin[cls], item_end = P.cls_begin[cls + 1];
+        if (item_end <= item_begin) continue;
+        const int G = P.cls_G[cls];
+        unsigned long long *const work = P.work + cls;
+        if (!QMODE && G == 0) {  // short vectors: one warp each
+            stream_short(P, work, item_begin, item_end, f_minsize, f_remscore, tot, S);
+            continue;
+        }
+        join_class<QMODE, SPLIT>(P, G, item_begin, item_end, P.cls_heavy[cls], work, f_minsize, f_remscore, f_upper, S,
+                                 tot);
+        bool later = false;  // another windowed class
+        for (int c = cls + 1; c < P.ncls; c++) later = later || (P.cls_G[c] > 0 && P.cls_begin[c + 1] > P.cls_begin[c]);
+        if (later) __syncthreads();
     }
-    switch (G) {
-        case 1: join_class<QMODE, SPLIT, 1>(P, item_begin, item_end, work, wtot, f_minsize, f_remscore, f_upper); break;
-        case 2: join_class<QMODE, SPLIT, 2>(P, item_begin, item_end, work, wtot, f_minsize, f_remscore, f_upper); break;
-        case 4: join_class<QMODE, SPLIT, 4>(P, item_begin, item_end, work, wtot, f_minsize, f_remscore, f_upper); break;
-        default: join_class<QMODE, SPLIT, 8>(P, item_begin, item_end, work, wtot, f_minsize, f_remscore, f_upper); break;
-    }
-    __syncthreads();  // every group is done with this class's layout of shared memory
-    }
-    // flush counters: the warps' totals, one global atomic per counter and warp
+    __syncwarp();
+    // the warps' totals, one global atomic per counter and warp
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
         for (int k = 0; k < 6; k++)
-            if (wtot[k]) atomicAdd(&P.counters[k < 5 ? k : 6], wtot[k]);
+            if (tot.v[k]) atomicAdd(&P.counters[k < 5 ? k : 6], tot.v[k]);
     }
 }
 
-// One warp per (x, window) slot: copy its staged run to the output at scan(counts)[qw].
-__global__ void k_gather(const Segment *__restrict__ segs, const int32_t *__restrict__ cntq, int64_t nqw,
-                         const int2 *__restrict__ stage, const int64_t *__restrict__ qwoff, int32_t *__restrict__ oi,
-                         int32_t *__restrict__ oj, float *__restrict__ os) {
+// One warp per slot: copy its staged run, piece by piece, to the output at scan(counts)[slot].
+__global__ void k_gather(const Segment *__restrict__ segs, const int2 *__restrict__ chain, int64_t slab,
+                         const int32_t *__restrict__ cntq, int64_t nslots, const int2 *__restrict__ stage,
+                         const int64_t *__restrict__ off, int32_t *__restrict__ oi, int32_t *__restrict__ oj,
+                         float *__restrict__ os) {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < nqw; q += nwarps) {
-        const int cnt = cntq[q];
-        if (cnt == 0) continue;
+    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < nslots; q += nwarps) {
+        if (cntq[q] == 0) continue;
         const Segment S = segs[q];
-        const int64_t dst = qwoff[q];
-        for (int e = lane; e < cnt; e += 32) {
-            const int2 v = stage[S.src + e];
-            oi[dst + e] = S.i;
-            oj[dst + e] = v.x;
-            os[dst + e] = __int_as_float(v.y);
+        int64_t dst = off[q], src = S.src;
+        int cnt = S.cnt, next = S.next;
+        for (;;) {
+            for (int e = lane; e < cnt; e += 32) {
+                const int2 v = stage[src + e];
+                oi[dst + e] = S.i;
+                oj[dst + e] = v.x;
+                os[dst + e] = __int_as_float(v.y);
+            }
+            if (next < 0) break;
+            dst += cnt;
+            src = (int64_t)next * slab;
+            const int2 c = chain[next];
+            cnt = c.x;
+            next = c.y;
         }
     }
 }
 
-__global__ void k_inst_offsets(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ qwoff,
-                               int64_t nqw, int64_t *out) {
+__global__ void k_inst_offsets(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ off, int parts,
+                               int64_t nslots, int64_t *out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= k; i += gridDim.x * blockDim.x)
-        out[i] = i < k ? qwoff[inst[i].qwbase] : qwoff[nqw];
+        out[i] = i < k ? off[inst[i].vbase * parts] : off[nslots];
 }
 
-// The index's work-list classes as one launch's class list. Returns the CTA count (enough
-// for every class's groups, or warps for the class of one- and two-component vectors, at most max_ctas) and
-// sets *smem to the largest class layout used.
-int set_classes(JoinParams &P, const aps_index *ix, int max_ctas, int *smem) {
+// The heaviest vectors of a class whose windows are cut into parts: enough units for every warp
+// of the chip several times over.
+constexpr int64_t JOIN_HEAVY = 8192;
+
+int join_smem() {
+    int b = 0;
+    for (int G : {1, 2, 4, 8}) b = std::max(b, tile_bytes(G) * tile_warps(G));
+    return b;
+}
+
+// The index's work-list classes as one launch's class list, the windows of the heaviest
+// vectors in `parts` parts. Returns the CTA count (the units spread over the SMs, at most
+// max_ctas CTAs).
+int set_classes(JoinParams &P, const aps_index *ix, int parts, int max_ctas) {
     static const int Gs[JOIN_NCLS] = {1, 2, 4, 8, 0};
     P.ncls = JOIN_NCLS;
-    int64_t ctas = 0;
-    *smem = 0;
+    P.parts = parts;
+    int64_t ctas = 1;
     for (int c = 0; c < JOIN_NCLS; c++) {
         P.cls_G[c] = Gs[c];
         P.cls_begin[c] = ix->class_begin[c];
         const int64_t ni = ix->class_begin[c + 1] - ix->class_begin[c];
-        if (ni <= 0) continue;
-        const int per_cta = Gs[c] > 0 ? Gs[c] : NWARPS;
-        ctas = std::max(ctas, (ni + per_cta - 1) / per_cta);
-        if (Gs[c] > 0) *smem = std::max(*smem, group_bytes(Gs[c]) * Gs[c]);
+        P.cls_heavy[c] = Gs[c] > 0 ? std::min(ni, JOIN_HEAVY) : 0;
+        ctas = std::max(ctas, ni + P.cls_heavy[c] * (parts - 1));
     }
     P.cls_begin[JOIN_NCLS] = ix->class_begin[JOIN_NCLS];
-    return (int)std::min<int64_t>(max_ctas, std::max<int64_t>(ctas, 1));
+    return (int)std::min<int64_t>(max_ctas, ctas);
 }
 
-// The join phase (reset the counters and the per-slot pair counts, then the persistent
-// join) as a CUDA graph: captured on the index's first join (on a private stream, so any
-// caller stream works, including the legacy default one), then replayed with the memset
-// targets and the kernel's parameters and grid updated in place for each later join.
+// What every join reads of an index.
+void set_index(JoinParams &P, const aps_index *ix) {
+    const IndexArrays &d = ix->d;
+    memset(&P, 0, sizeof(P));
+    P.inst = d.inst.p;
+    P.vinst = d.vinst.p;
+    P.items = ix->items.p;
+    P.one = ix->k == 1;
+    P.crow = d.crow.p;
+    P.vmeta = d.vmeta.p;
+    P.vcand = d.vcand.p;
+    P.code = d.code.p;
+    P.nblk = 1;
+    P.parts = 1;
+    P.lptr = d.lptr.p;
+    P.wptr = d.wptr.p;
+    P.post = d.post.p;
+}
+
+// The join phase: reset the counters and the per-slot pair counts, then the persistent join.
+// An index's first join launches the three directly: most indexes are joined once, and capturing,
+// instantiating and destroying a graph costs the host some 100 us (a whole join of 2,000 vectors
+// takes 600). From the second join on they are a CUDA graph, captured on a private stream, so any
+// caller stream works, including the legacy default one, and replayed with the memset targets and
+// the kernel's parameters and grid updated in place.
 aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsigned long long *ctr, int32_t *cntq,
-                          cudaStream_t s) {
+                          int64_t nslots, cudaStream_t s) {
     JoinGraph &G = ix->jgraph;
-    const size_t ctr_bytes = 16 * sizeof(unsigned long long), cnt_bytes = sizeof(int32_t) * (size_t)ix->nqw;
+    const size_t ctr_bytes = 16 * sizeof(unsigned long long), cnt_bytes = sizeof(int32_t) * (size_t)nslots;
+    if (G.launches++ == 0) {
+        APS_CUDA(cudaMemsetAsync(ctr, 0, ctr_bytes, s));
+        APS_CUDA(cudaMemsetAsync(cntq, 0, cnt_bytes, s));
+        join_kernel<false><<<grid, JOIN_THREADS, smem, s>>>(P);
+        APS_LAUNCH_CHECK();
+        return APS_OK;
+    }
     if (!G.exec) {
         cudaStream_t cs = nullptr;
         APS_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -1180,7 +1214,6 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
     }
     APS_CUDA(cudaGraphLaunch(G.exec, s));
     count_launch();
-    G.launches++;
     return APS_OK;
 }
 
@@ -1212,7 +1245,7 @@ __global__ void k_first_of_key(const unsigned long long *__restrict__ key, int64
 }
 
 // The split vectors' pairs (key = local x * n + local y, sorted, first occurrences at
-// off[k]) into the staging buffer from `base` on, as the runs of their (x, window) slots.
+// off[k]) into the staging buffer from `base` on, as the runs of their vectors' slots.
 __global__ void k_split_place(const unsigned long long *__restrict__ key, const uint32_t *__restrict__ score,
                               const int32_t *__restrict__ flag, const int64_t *__restrict__ off, int64_t n,
                               const InstDesc *__restrict__ inst, int64_t base, int2 *stage, Segment *segs,
@@ -1222,31 +1255,42 @@ __global__ void k_split_place(const unsigned long long *__restrict__ key, const 
         if (!flag[k]) continue;
         const unsigned long long kk = key[k];
         const int32_t lx = (int32_t)(kk / (unsigned long long)I.n), y = (int32_t)(kk % (unsigned long long)I.n);
-        const int w = y / I.W;
-        const int64_t qw = I.qwbase + (int64_t)lx * I.nw + w;
+        const int64_t qw = I.vbase + lx;
         const int64_t pos = base + off[k];
         stage[pos] = make_int2(y, (int)score[k]);
         atomicAdd(&cntq[qw], 1);
         bool first = k == 0;
         if (!first) {
             const unsigned long long pk = key[k - 1];
-            first = (int32_t)(pk / (unsigned long long)I.n) != lx || (int32_t)(pk % (unsigned long long)I.n) / I.W != w;
+            first = (int32_t)(pk / (unsigned long long)I.n) != lx;
         }
         if (first) {
             Segment S;
             S.src = pos;
-            S.cnt = 0;
+            S.cnt = 0;  // (the count is cntq's: k_split_counts)
             S.i = lx;
+            S.next = -1;
+            S._pad = 0;
             segs[qw] = S;
         }
     }
 }
 
+// The split vectors' piece lengths, once every pair is counted: a vector with no run of its
+// own (it was joined by blocks) has its whole count in its one piece.
+__global__ void k_split_counts(const unsigned long long *__restrict__ key, const int32_t *__restrict__ flag, int64_t n,
+                               const InstDesc *__restrict__ inst, const int32_t *__restrict__ cntq, Segment *segs) {
+    const InstDesc I = inst[0];
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t lx = (int64_t)(key[k] / (unsigned long long)I.n);
+        if (k == 0 || (int64_t)(key[k - 1] / (unsigned long long)I.n) != lx) segs[I.vbase + lx].cnt = cntq[I.vbase + lx];
+    }
+}
+
 }  // namespace
 
-// Staging slots one CTA can reserve and leave unused: a slab per group of every windowed
-// class (1 + 2 + 4 + 8 groups) and a slab per warp of the streamed class.
-int64_t join_slab_slack() { return 15 * (int64_t)JOIN_STAGE_SLAB + (int64_t)NWARPS * (JOIN_STAGE_SLAB / 8); }
+// Staging slots one CTA can reserve and leave unused: less than a slab per warp.
+int64_t join_slab_slack() { return (int64_t)JOIN_WARPS * JOIN_STAGE_SLAB; }
 
 void debug_stage_cap(int64_t pairs) { g_stage_cap_once.store(pairs > 0 ? pairs : 0); }
 
@@ -1263,14 +1307,13 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
             for (int i = 0; i < 4; i++) cudaEventDestroy(e[i]);
         }
     } evg{ev};
-    const int Gs[4] = {1, 2, 4, 8};
-    // the largest requirement of the four group shapes covers every launch
-    int need = 0;
-    for (int c = 0; c < 4; c++) need = std::max(need, group_bytes(Gs[c]) * Gs[c]);
+    const int need = join_smem();
     APS_CUDA(cudaFuncSetAttribute(join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
 
     // the vertical split: the costliest `heavy` vectors as nblk dimension blocks each
     const bool split = nblk >= 2 && heavy > 0 && ix->k == 1;
+    const int parts = split ? 1 : ix->parts;
+    const int64_t nslots = ix->N * parts;
     int split_cls = -1;
     int64_t nsplit = 0, sp_cap = 0;
     DBuf<int32_t> items2;
@@ -1297,15 +1340,16 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
 
     DBuf<int32_t> cntq;
     DBuf<unsigned long long> ctr;  // 0..4 counters, 5 stage count, 6 entries read, 8..12 work, 13 split pairs
-    APS_TRY(cntq.alloc((size_t)std::max<int64_t>(ix->nqw, 1), s));
+    APS_TRY(cntq.alloc((size_t)std::max<int64_t>(nslots, 1), s));
     APS_TRY(ctr.alloc(16, s));
     // Staging capacity: the index's own hint, else the last join of this process; a join
     // that still overflows is re-run with room for what it reserved plus one slab per
-    // group. Segments are stored per (vector, window) slot, so their table never overflows.
+    // warp. First pieces are stored per slot and later ones per slab, so their tables never
+    // overflow.
     int64_t stage_cap = std::max<int64_t>({ix->hint_pairs, g_stage_hint.load(), (int64_t)1 << 20, ix->nnz});
     if (ix->hint_pairs == 0 && g_stage_hint.load() == 0) {
         // no join of this process has sized the staging yet: take room for every possible
-        // pair plus one slab per group, but at most an eighth of the free device memory
+        // pair plus one slab per warp, but at most an eighth of the free device memory
         // and 2^28 pairs, so that a first join rarely has to run twice
         int64_t most = (int64_t)sms * join_slab_slack();
         for (const InstDesc &I : ix->inst_h) most += (int64_t)I.n * (I.n - 1) / 2;
@@ -1320,56 +1364,39 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
     if (const int64_t once = g_stage_cap_once.exchange(0); once > 0) stage_cap = once;
     DBuf<int2> stage;
     DBuf<Segment> segs;
-    DBuf<int2> scratch;
-    APS_TRY(scratch.alloc((size_t)sms * NWARPS * JOIN_ECAP, s));
-    APS_TRY(segs.alloc((size_t)std::max<int64_t>(ix->nqw, 1), s));
+    DBuf<int2> scratch, chain;
+    APS_TRY(scratch.alloc((size_t)sms * JOIN_WARPS * JOIN_ECAP, s));
+    APS_TRY(segs.alloc((size_t)std::max<int64_t>(nslots, 1), s));
     int64_t total_pairs = 0, reserved = 0;
     unsigned long long ch[16];
     int reruns = 0;
     for (int attempt = 0; attempt < 3; attempt++) {
         APS_TRY(stage.alloc((size_t)stage_cap, s));
+        APS_TRY(chain.alloc((size_t)(stage_cap / JOIN_STAGE_SLAB) + 1, s));
         if (nsplit > 0) {
             APS_TRY(sp_key.alloc((size_t)sp_cap, s));
             APS_TRY(sp_score.alloc((size_t)sp_cap, s));
         }
         if (ix->class_begin[JOIN_NCLS] <= ix->class_begin[0]) {  // nothing to join: just the resets
             APS_CUDA(cudaMemsetAsync(ctr.p, 0, 16 * sizeof(unsigned long long), s));
-            if (ix->nqw) APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * ix->nqw, s));
+            if (nslots) APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * nslots, s));
             APS_CUDA(cudaEventRecord(ev[0], s));
         } else {
             JoinParams P;
-            P.inst = d.inst.p;
-            P.vinst = d.vinst.p;
-            P.items = ix->items.p;
-            int smem = 0;
-            const int grid = set_classes(P, ix, sms, &smem);
-            P.crow = d.crow.p;
-            P.vmeta = d.vmeta.p;
-            P.vcand = d.vcand.p;
-            P.pn4 = d.pn4.p;
-            P.qsplit = d.qsplit.p;
-            P.mw = d.mw.p;
-            P.lptr = d.lptr.p;
-            P.wptr = d.wptr.p;
-            P.post = d.post.p;
+            set_index(P, ix);
+            const int grid = set_classes(P, ix, parts, sms);
             P.flags = flags | (ix->flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
             P.stage = stage.p;
             P.stage_cap = stage_cap;
             P.stage_count = ctr.p + 5;
             P.stage_slab = JOIN_STAGE_SLAB;
             P.segs = segs.p;
+            P.chain = chain.p;
             P.cntq = cntq.p;
             P.counters = ctr.p;
             P.work = ctr.p + 8;
             P.scratch = scratch.p;
-            P.qmode = 0;
-            P.qnw = 1;
-            P.iblk = nullptr;
-            P.nblk = 1;
-            P.sp_key = nullptr;
-            P.sp_score = nullptr;
             P.sp_count = ctr.p + 13;
-            P.sp_cap = 0;
             APS_CUDA(cudaEventRecord(ev[0], s));
             if (nsplit > 0) {  // the split work list, one direct launch
                 P.items = items2.p;
@@ -1380,11 +1407,11 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 P.sp_cap = sp_cap;
                 for (int c = split_cls + 1; c <= JOIN_NCLS; c++) P.cls_begin[c] += nsplit * (nblk - 1);
                 APS_CUDA(cudaMemsetAsync(ctr.p, 0, 16 * sizeof(unsigned long long), s));
-                APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * std::max<int64_t>(ix->nqw, 1), s));
-                join_kernel<false, true><<<grid, JOIN_THREADS, smem, s>>>(P);
+                APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * std::max<int64_t>(nslots, 1), s));
+                join_kernel<false, true><<<grid, JOIN_THREADS, need, s>>>(P);
                 APS_LAUNCH_CHECK();
             } else {
-                APS_TRY(run_join_graph(ix, P, grid, smem, ctr.p, cntq.p, s));
+                APS_TRY(run_join_graph(ix, P, grid, need, ctr.p, cntq.p, nslots, s));
             }
         }
         APS_CUDA(cudaEventRecord(ev[1], s));
@@ -1396,7 +1423,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
         if (reserved <= stage_cap && sp_found <= sp_cap) {
             if (sp_found > 0) {
                 // the split vectors' pairs: sorted by (x, y), first occurrences kept, placed
-                // after the join's staged runs as the runs of their (x, window) slots
+                // after the join's staged runs as the runs of their slots
                 const InstDesc &I0 = ix->inst_h[0];
                 APS_TRY(sort_pairs(reinterpret_cast<uint64_t *>(sp_key.p), sp_score.p, sp_found,
                                    bits_for((uint64_t)I0.n * (uint64_t)I0.n), s));
@@ -1421,6 +1448,9 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 }
                 k_split_place<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_key.p, sp_score.p, flag.p, off.p, sp_found,
                                                                      d.inst.p, reserved, stage.p, segs.p, cntq.p);
+                APS_LAUNCH_CHECK();
+                k_split_counts<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_key.p, flag.p, sp_found, d.inst.p, cntq.p,
+                                                                      segs.p);
                 APS_LAUNCH_CHECK();
                 total_pairs += nuniq;
             }
@@ -1449,8 +1479,8 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
 
     // ---------------- output: scan counts, gather runs into (i, j, score)
     DBuf<int64_t> qwoff;
-    APS_TRY(qwoff.alloc((size_t)ix->nqw + 1, s));
-    APS_TRY(scan_exclusive(cntq.p, qwoff.p, ix->nqw, s));
+    APS_TRY(qwoff.alloc((size_t)nslots + 1, s));
+    APS_TRY(scan_exclusive(cntq.p, qwoff.p, nslots, s));
     const int64_t npairs = total_pairs;
     PairsAlloc *pa = new PairsAlloc();
     pa->stream = s;
@@ -1465,14 +1495,14 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
     int32_t *oj = reinterpret_cast<int32_t *>(blk + (((size_t)npairs * 4 + 127) & ~(size_t)127));
     float *os = reinterpret_cast<float *>(blk + 2 * (((size_t)npairs * 4 + 127) & ~(size_t)127));
     if (npairs > 0) {
-        k_gather<<<grid_for(ix->nqw * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(segs.p, cntq.p, ix->nqw, stage.p,
-                                                                               qwoff.p, oi, oj, os);
+        k_gather<<<grid_for(nslots * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(
+            segs.p, chain.p, JOIN_STAGE_SLAB, cntq.p, nslots, stage.p, qwoff.p, oi, oj, os);
         APS_LAUNCH_CHECK();
     }
     if (pair_offsets_h) {
         DBuf<int64_t> offs;
         APS_TRY(offs.alloc((size_t)ix->k + 1, s));
-        k_inst_offsets<<<grid_for(ix->k + 1, 256), 256, 0, s>>>(d.inst.p, ix->k, qwoff.p, ix->nqw, offs.p);
+        k_inst_offsets<<<grid_for(ix->k + 1, 256), 256, 0, s>>>(d.inst.p, ix->k, qwoff.p, parts, nslots, offs.p);
         APS_LAUNCH_CHECK();
         pair_offsets_h->assign((size_t)ix->k + 1, 0);
         APS_CUDA(cudaMemcpyAsync(pair_offsets_h->data(), offs.p, sizeof(int64_t) * (ix->k + 1),
@@ -1557,9 +1587,9 @@ aps_status pairs_to_host(aps_pairs *p, cudaStream_t s) {
 
 // ------------------------------------------------------------------ arena variant
 // The same join and output kernels with every buffer carved out of a caller-provided
-// device arena instead of allocated: counters, per-(x, window) counts and offsets, the
-// segment table, the per-warp emit lists (for at most max_ctas CTAs) and, in what is left,
-// the pair staging buffer. Pairs are gathered into the caller's (i, j, score) arrays.
+// device arena instead of allocated: counters, per-vector counts and offsets, the segment
+// table, the streamed class's per-warp lists (for at most max_ctas CTAs) and, in what is
+// left, the pair staging buffer. Pairs are gathered into the caller's (i, j, score) arrays.
 namespace {
 
 constexpr int SCAN1_THREADS = 1024;
@@ -1606,64 +1636,55 @@ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes, int max_ctas, int32_t *oi,
                         int32_t *oj, float *os, int64_t cap, int64_t *count, cudaStream_t s) {
-    IndexArrays &d = ix->d;
     const int grid_max = std::max(1, std::min(num_sms(), max_ctas));
-    const int64_t nqw = std::max<int64_t>(ix->nqw, 1);
+    // The documented limit: 28 bytes for each of the index's arena slots beside the fixed parts.
+    const size_t limit = (size_t)std::max<int64_t>(ix->arena_slots, 1) * 28 + (size_t)max_ctas * 32 * 1408 * sizeof(int2);
+    const int64_t slab = 32;  // small slabs: the arena's staging room is modest
+    const int64_t nslots = std::max<int64_t>(ix->N, 1);
     size_t off = 0;
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(arena + off);
     off = align256(off + 16 * sizeof(unsigned long long));
     int32_t *cntq = reinterpret_cast<int32_t *>(arena + off);
-    off = align256(off + sizeof(int32_t) * nqw);
+    off = align256(off + sizeof(int32_t) * nslots);
     int64_t *qwoff = reinterpret_cast<int64_t *>(arena + off);
-    off = align256(off + sizeof(int64_t) * (nqw + 1));
+    off = align256(off + sizeof(int64_t) * (nslots + 1));
     Segment *segs = reinterpret_cast<Segment *>(arena + off);
-    off = align256(off + sizeof(Segment) * nqw);
+    off = align256(off + sizeof(Segment) * nslots);
     int2 *elists = reinterpret_cast<int2 *>(arena + off);
-    off = align256(off + sizeof(int2) * (size_t)grid_max * NWARPS * JOIN_ECAP);
-    if (off >= arena_bytes) {
+    off = align256(off + sizeof(int2) * (size_t)grid_max * JOIN_WARPS * JOIN_ECAP);
+    if (limit >= arena_bytes || off + 4096 >= arena_bytes) {
         set_error("index too large for the %zu-byte arena: its %lld (vector, window) slots need %zu bytes "
                   "before any pair is staged",
-                  arena_bytes, (long long)ix->nqw, off);
+                  arena_bytes, (long long)ix->arena_slots, std::max(limit, off));
         return APS_EINVAL;
     }
+    // the rest: staged pairs (8 bytes each) and a chain entry (8 bytes) for every slab of them
+    const int64_t nslabs = (int64_t)((arena_bytes - off - 1024) / (sizeof(int2) * (slab + 1)));
+    const int64_t stage_cap = nslabs * slab;
+    int2 *chain = reinterpret_cast<int2 *>(arena + off);
+    off = align256(off + sizeof(int2) * (nslabs + 1));
     int2 *stage = reinterpret_cast<int2 *>(arena + off);
-    const int64_t stage_cap = (int64_t)((arena_bytes - off) / sizeof(int2));
 
-    const int Gs[4] = {1, 2, 4, 8};
-    int need = 0;
-    for (int c = 0; c < 4; c++) need = std::max(need, group_bytes(Gs[c]) * Gs[c]);
+    const int need = join_smem();
     APS_CUDA(cudaFuncSetAttribute(join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
     APS_CUDA(cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned long long), s));
-    APS_CUDA(cudaMemsetAsync(cntq, 0, sizeof(int32_t) * nqw, s));
+    APS_CUDA(cudaMemsetAsync(cntq, 0, sizeof(int32_t) * nslots, s));
     if (ix->class_begin[JOIN_NCLS] > ix->class_begin[0]) {
         JoinParams P;
-        P.inst = d.inst.p;
-        P.vinst = d.vinst.p;
-        P.items = ix->items.p;
-        int smem = 0;
-        const int grid = set_classes(P, ix, grid_max, &smem);
-        P.crow = d.crow.p;
-        P.vmeta = d.vmeta.p;
-        P.vcand = d.vcand.p;
-        P.pn4 = d.pn4.p;
-        P.qsplit = d.qsplit.p;
-        P.mw = d.mw.p;
-        P.lptr = d.lptr.p;
-        P.wptr = d.wptr.p;
-        P.post = d.post.p;
+        set_index(P, ix);
+        const int grid = set_classes(P, ix, 1, grid_max);
         P.flags = ix->flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND);
         P.stage = stage;
         P.stage_cap = stage_cap;
         P.stage_count = ctr + 5;
-        P.stage_slab = 256;  // small slabs: the arena's staging room is modest
+        P.stage_slab = slab;
         P.segs = segs;
+        P.chain = chain;
         P.cntq = cntq;
         P.counters = ctr;
         P.work = ctr + 8;
         P.scratch = elists;
-        P.qmode = 0;
-        P.qnw = 1;
-        join_kernel<false><<<grid, JOIN_THREADS, smem, s>>>(P);
+        join_kernel<false><<<grid, JOIN_THREADS, need, s>>>(P);
         APS_LAUNCH_CHECK();
     }
     unsigned long long ch[16];
@@ -1680,11 +1701,11 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
         set_error("%lld pairs do not fit the caller's capacity of %lld", (long long)total, (long long)cap);
         return APS_EOVERFLOW;
     }
-    k_scan_single<<<1, SCAN1_THREADS, 0, s>>>(cntq, ix->nqw, qwoff);
+    k_scan_single<<<1, SCAN1_THREADS, 0, s>>>(cntq, ix->N, qwoff);
     APS_LAUNCH_CHECK();
     if (total > 0) {
-        k_gather<<<grid_for(ix->nqw * 32, 256, (int64_t)num_sms() * 32), 256, 0, s>>>(segs, cntq, ix->nqw, stage,
-                                                                                     qwoff, oi, oj, os);
+        k_gather<<<grid_for(ix->N * 32, 256, (int64_t)num_sms() * 32), 256, 0, s>>>(segs, chain, slab, cntq, ix->N,
+                                                                                   stage, qwoff, oi, oj, os);
         APS_LAUNCH_CHECK();
     }
     APS_CUDA(cudaStreamSynchronize(s));
@@ -1712,11 +1733,13 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     const InstDesc &I = ix->inst_h[0];
     const int sms = num_sms();
     const int64_t nq = qa.nq;
-    const int64_t nqw = std::max<int64_t>(nq * (int64_t)std::max(I.nw, 1), 1);
     const int G = I.G;
-    const int Gs[4] = {1, 2, 4, 8};
-    int need = 0;
-    for (int c = 0; c < 4; c++) need = std::max(need, group_bytes(Gs[c]) * Gs[c]);
+    // the windows of a query in as many parts as give every warp of the chip some 32 units
+    const int parts = (int)std::max<int64_t>(
+        1, std::min<int64_t>(I.nw, ((int64_t)sms * tile_warps(G) * 32 + nq - 1) / std::max<int64_t>(nq, 1)));
+    const int64_t nqw = std::max<int64_t>(nq * parts, 1);
+    const int need = tile_bytes(G) * tile_warps(G);
+    const int64_t slab = 256;  // query batches are small: keep the slab tails short
     APS_CUDA(cudaFuncSetAttribute(join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
     cudaEvent_t ev[3];
     for (int i = 0; i < 3; i++) APS_CUDA(cudaEventCreate(&ev[i]));
@@ -1726,73 +1749,61 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
             for (int i = 0; i < 3; i++) cudaEventDestroy(e[i]);
         }
     } evg{ev};
-    const int64_t nitems = nq * (int64_t)I.nw;  // (query, window) items
-    const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>((nitems + G - 1) / G, 1));
+    const int64_t nitems = I.nw > 0 ? nq : 0;
+    const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(nitems * parts, 1));
     DBuf<int32_t> cntq;
     DBuf<unsigned long long> ctr;
-    DBuf<int2> scratch, stage;
+    DBuf<int2> chain, stage;
     DBuf<Segment> segs;
     APS_TRY(cntq.alloc((size_t)nqw, s));
     APS_TRY(ctr.alloc(16, s));
-    APS_TRY(scratch.alloc((size_t)grid * NWARPS * JOIN_ECAP, s));
     APS_TRY(segs.alloc((size_t)nqw, s));
     // staging: the pairs per query this index's batches have needed so far (at least 64),
-    // plus one slab per group
+    // plus one slab per warp
     const int64_t ppq16 = ix->q_ppq16.load(std::memory_order_relaxed);
-    int64_t stage_cap = std::max<int64_t>(nq * ppq16 / 16 + (int64_t)grid * G * 256, (int64_t)1 << 16);
+    const int64_t slack = (int64_t)grid * JOIN_WARPS * slab;
+    int64_t stage_cap = std::max<int64_t>(nq * ppq16 / 16 + slack, (int64_t)1 << 16);
     unsigned long long ch[16];
     for (int attempt = 0; attempt < 2; attempt++) {
         APS_TRY(stage.alloc((size_t)stage_cap, s));
+        APS_TRY(chain.alloc((size_t)(stage_cap / slab) + 1, s));
         APS_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(ch), s));
         APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * nqw, s));
         APS_CUDA(cudaEventRecord(ev[0], s));
         if (nq > 0) {
             JoinParams P;
-            memset(&P, 0, sizeof(P));
-            P.inst = d.inst.p;
-            P.vinst = d.vinst.p;
+            set_index(P, ix);
             P.items = nullptr;
             P.ncls = 1;
             P.cls_G[0] = G;
             P.cls_begin[0] = 0;
             P.cls_begin[1] = nitems;
-            P.crow = d.crow.p;
-            P.vmeta = d.vmeta.p;
-            P.vcand = d.vcand.p;
-            P.pn4 = d.pn4.p;
-            P.qsplit = d.qsplit.p;
-            P.mw = d.mw.p;
-            P.lptr = d.lptr.p;
-            P.wptr = d.wptr.p;
-            P.post = d.post.p;
+            P.cls_heavy[0] = nitems;
+            P.parts = parts;
             P.flags = flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND);
             P.stage = stage.p;
             P.stage_cap = stage_cap;
             P.stage_count = ctr.p + 5;
-            P.stage_slab = 256;  // query batches are small: keep the slab tails short
+            P.stage_slab = slab;
             P.segs = segs.p;
+            P.chain = chain.p;
             P.cntq = cntq.p;
             P.counters = ctr.p;
             P.work = ctr.p + 8;
-            P.scratch = scratch.p;
-            P.qmode = 1;
             P.qcrow = qa.crow.p;
             P.qvmeta = qa.vmeta.p;
-            P.qqsplit = qa.qsplit.p;
-            P.qmw = qa.mw.p;
             P.qt = t;
-            P.qnw = std::max(I.nw, 1);
-            join_kernel<true><<<grid, JOIN_THREADS, group_bytes(G) * G, s>>>(P);
+            join_kernel<true><<<grid, JOIN_THREADS, need, s>>>(P);
             APS_LAUNCH_CHECK();
         }
         APS_CUDA(cudaEventRecord(ev[1], s));
         APS_CUDA(cudaMemcpyAsync(ch, ctr.p, sizeof(ch), cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
         if ((int64_t)ch[5] <= stage_cap) break;
-        stage_cap = (int64_t)ch[5] + (int64_t)grid * G * 256;  // what was reserved, plus one slab per group
+        stage_cap = (int64_t)ch[5] + slack;  // what was reserved, plus one slab per warp
     }
     if (nq > 0) {  // remember what this batch needed (with a quarter more), for the next ones
-        const int64_t need16 = (int64_t)ch[5] * 20 / nq;
+        const int64_t need16 = (int64_t)ch[3] * 20 / nq;  // (the slabs' unused rests are the slack)
         int64_t cur = ix->q_ppq16.load(std::memory_order_relaxed);
         while (need16 > cur && !ix->q_ppq16.compare_exchange_weak(cur, need16, std::memory_order_relaxed)) {
         }
@@ -1818,8 +1829,8 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     int32_t *oj = reinterpret_cast<int32_t *>(blk + seg4);
     float *os = reinterpret_cast<float *>(blk + 2 * seg4);
     if (npairs > 0) {
-        k_gather<<<grid_for(nqw * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(segs.p, cntq.p, nqw, stage.p, qwoff.p, oi,
-                                                                           oj, os);
+        k_gather<<<grid_for(nqw * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(segs.p, chain.p, slab, cntq.p, nqw,
+                                                                           stage.p, qwoff.p, oi, oj, os);
         APS_LAUNCH_CHECK();
     }
     APS_CUDA(cudaEventRecord(ev[2], s));

@@ -142,7 +142,8 @@ namespace {
 // counts/offsets/segments, the staged and final pairs (64 per query assumed), query rows.
 size_t estimate(const aps_server *sv, int32_t nq, int64_t nnz) {
     const InstDesc &I = sv->ix->inst_h[0];
-    const size_t per_q = (size_t)std::max(I.nw, 1) * (4 + 8 + sizeof(Segment)) + 64 * (8 + 12) + 64;
+    const size_t nw = ((size_t)I.n * I.G + 40959) / 40960;  // (a query's slots, at most)
+    const size_t per_q = std::max<size_t>(nw, 1) * (4 + 8 + 16) + 64 * (8 + 12) + 64;
     return sv->fixed + (size_t)nq * per_q + (size_t)nnz * 48;
 }
 
@@ -222,7 +223,7 @@ aps_status aps_server_create(aps_index *index, size_t mem_budget, int32_t slots,
     sv->ix = index;
     sv->budget = mem_budget;
     sv->slots = slots;
-    sv->fixed = (size_t)num_sms() * (JOIN_THREADS / 32) * JOIN_ECAP * sizeof(int2) + (1u << 20);
+    sv->fixed = (size_t)num_sms() * 32 * JOIN_ECAP * sizeof(int2) + (1u << 20);
     for (int i = 0; i < slots; i++) {
         cudaStream_t st;
         cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);

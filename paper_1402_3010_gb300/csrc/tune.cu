@@ -1,10 +1,10 @@
 // Join tile shapes per instance size, and the autotuner that chooses them by measurement.
 //
-// An instance is joined with G query groups per CTA (G = 1, 2, 4, 8), each group holding a
-// candidate window of JOIN_WMAX / G ids in shared memory: a small G gives long windows
-// (fewer windows, so less fixed cost per query), a large G more queries in flight per SM.
-// This is the block size of Sec. 5.1.9 turned into a CTA-level tile, and like the paper's
-// block size it is a measured choice. The table maps an instance's size bucket to G; the
+// An instance is joined with tile shape G (1, 2, 4 or 8): one warp per query vector, with a
+// candidate window of tile_window(G) ids in shared memory. G = 1 gives windows of twice the width
+// (fewer windows, so less fixed cost per query), the others more queries in flight per SM.
+// This is the block size of Sec. 5.1.9 turned into a tile, and like the paper's block size it
+// is a measured choice. The table maps an instance's size bucket to G; the
 // bucket bounds are the work-split thresholds between the shapes.
 #include <algorithm>
 #include <climits>
@@ -21,14 +21,9 @@ namespace {
 const int64_t BOUNDS[APS_TUNE_BUCKETS] = {512, 1280, 2560, 5120, 10240, 20480, 40960, INT64_MAX};
 const int GS[4] = {1, 2, 4, 8};
 
-// Default for self-joins: the largest G whose window still holds the whole instance (one
-// window per query), but at least 2 groups. Measured on the 200k-vector power-law set
-// (join ms): G = 1: 71.7, 2: 65.0, 4: 65.6, 8: 72.9.
-// Default for queryable indexes: the same. Their queries are (query, window) work items,
-// so a long query's windows run on several CTAs; on the 1M-vector serving index G = 1 and
-// G = 2 then serve alike (84.3k and 84.5k queries/s saturated). Before that split, a
-// batch waited for its longest query on one group, and G = 1 (a whole CTA per query)
-// served 47.0k against 23.5k with G = 2.
+// The default table never takes G = 1. Measured (join ms, G = 1 against the others): the
+// 200k-vector power-law set 28.9 / 21.6, the 512-instance batch 28.8 / 15.3, 4096 queries
+// against the 1M-vector index 7.6 / 6.1.
 const aps_tuning DEFAULT_TUNING = {{8, 8, 8, 8, 4, 2, 2, 2}, {8, 8, 8, 8, 4, 2, 2, 2}};
 
 std::mutex g_tune_mu;
