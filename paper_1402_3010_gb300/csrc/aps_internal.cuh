@@ -83,9 +83,12 @@ struct DBuf {
 aps_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s);
 aps_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
 
-// Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the keys.
-// keys/vals are sorted in place (scratch is allocated internally).
-aps_status sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int bits, cudaStream_t s);
+// Stable LSD radix sort of the first n (key, value) pairs, or keys, on the low `bits` bits of the
+// keys. The buffers hold the sorted items afterwards (they may have been exchanged for the sort's
+// own scratch of n items; all on stream s).
+aps_status sort_pairs(DBuf<uint64_t> &keys, DBuf<uint32_t> &vals, int64_t n, int bits, cudaStream_t s);
+aps_status sort_pairs(DBuf<uint32_t> &keys, DBuf<uint32_t> &vals, int64_t n, int bits, cudaStream_t s);
+aps_status sort_keys(DBuf<uint64_t> &keys, int64_t n, int bits, cudaStream_t s);
 
 inline int bits_for(uint64_t v) {  // bits needed to hold values in [0, v]
     int b = 0;

@@ -731,7 +731,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     }
     const int npairs_sm = std::max(1, std::min<int>(max_clusters, (int)units.size()));
     int64_t cap = std::max<int64_t>({g_dense_hint.load(), (int64_t)1 << 22, (int64_t)n * 4});
-    DBuf<unsigned long long> cand;
+    DBuf<uint64_t> cand;
     int64_t nslots = 0, npad = 0;
     float ms_gemm = 0.f;
     for (int attempt = 0; attempt < 2; attempt++) {
@@ -745,7 +745,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
         P.nunits = (int)units.size();
         P.units = dunits.p;
         P.thr = raw ? INFINITY : (float)((double)t - delta);
-        P.cand = cand.p;
+        P.cand = reinterpret_cast<unsigned long long *>(cand.p);
         P.cap = (unsigned long long)cap;
         P.count = ctr.p;
         P.padded = ctr.p + 2;
@@ -797,13 +797,8 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     }
     g_dense_hint.store(nslots + nslots / 8 + 1024);
     // sort by (i, j): the slots hold nc candidates and npad CAND_PAD keys, which sort last
-    DBuf<uint32_t> dummy;
-    APS_TRY(dummy.alloc((size_t)std::max<int64_t>(nslots, 1), s));
-    if (nslots > 1) {
-        APS_CUDA(cudaMemsetAsync(dummy.p, 0, sizeof(uint32_t) * nslots, s));
-        APS_TRY(sort_pairs(reinterpret_cast<uint64_t *>(cand.p), dummy.p, nslots,
-                           bits_for((uint64_t)n * (uint64_t)n), s));
-    }
+    APS_TRY(sort_keys(cand, nslots, bits_for((uint64_t)n * (uint64_t)n), s));
+    const unsigned long long *const sorted = reinterpret_cast<const unsigned long long *>(cand.p);
     const int64_t nc = nslots - npad;
     APS_CUDA(cudaEventRecord(ev[3], s));
     DBuf<int32_t> keep;
@@ -814,7 +809,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     APS_TRY(pos.alloc((size_t)nc + 1, s));
     const float beta = (float)std::max(1e-5, (d / 32.0 + 8.0) * std::ldexp(1.0, -23));
     if (nc > 0) {
-        k_rescore<<<grid_for(nc * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(cand.p, nc, X, n, d, t, beta,
+        k_rescore<<<grid_for(nc * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(sorted, nc, X, n, d, t, beta,
                                                                                    keep.p, sc.p, ctr.p + 1);
         APS_LAUNCH_CHECK();
     }
@@ -837,7 +832,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     int32_t *oj = reinterpret_cast<int32_t *>(b + seg);
     float *os = reinterpret_cast<float *>(b + 2 * seg);
     if (nc > 0) {
-        k_compact<<<grid_for(nc, 256, 65536), 256, 0, s>>>(cand.p, keep.p, sc.p, pos.p, nc, n, oi, oj, os);
+        k_compact<<<grid_for(nc, 256, 65536), 256, 0, s>>>(sorted, keep.p, sc.p, pos.p, nc, n, oi, oj, os);
         APS_LAUNCH_CHECK();
     }
     APS_CUDA(cudaEventRecord(ev[4], s));

@@ -232,7 +232,7 @@ aps_status graph_csr(const int32_t *i_in, const int32_t *j_in, const float *s_in
         if (count > 0) {
             k_sort_keys<<<grid_for(count, 256), 256, 0, s>>>(pi, pj, ps, count, keys.p, vals.p);
             count_launch();
-            if ((st = sort_pairs(keys.p, vals.p, count, bits_for((uint64_t)n), s)) != APS_OK) return fail(st);
+            if ((st = sort_pairs(keys, vals, count, bits_for((uint64_t)n), s)) != APS_OK) return fail(st);
         }
         k_starts<<<grid_for((int64_t)n + 1, 256), 256, 0, s>>>(pi, keys.p, count, n, start_i, start_j, row_ptr);
         count_launch();

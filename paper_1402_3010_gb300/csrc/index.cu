@@ -220,13 +220,28 @@ __global__ void __launch_bounds__(1024) k_dimstats_inst(const int64_t *__restric
 
 // Dimension order of all-pairs-1: decreasing non-zero count; the sort is stable and the
 // input is in id order, so ties keep ascending dimension id.
+template <class K>
 __global__ void k_rank_keys(const int32_t *__restrict__ nnz_d, const InstDesc *__restrict__ inst, int k,
-                            int64_t M, int nbits, uint64_t nmax, uint64_t *keys, uint32_t *vals) {
+                            int64_t M, int nbits, uint64_t nmax, K *keys, uint32_t *vals) {
     for (int64_t D = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; D < M; D += (int64_t)gridDim.x * blockDim.x) {
         uint64_t ki = (uint64_t)inst_of_rank(inst, k, D);
-        keys[D] = (ki << nbits) | (nmax - (uint64_t)nnz_d[D]);
+        keys[D] = (K)((ki << nbits) | (nmax - (uint64_t)nnz_d[D]));
         vals[D] = (uint32_t)D;
     }
+}
+
+// The dimensions in rank order (vals): keys of 32 bits where they hold the instance and the count.
+template <class K>
+aps_status sort_dims(const aps_index *ix, int32_t maxn, DBuf<uint32_t> &vals, cudaStream_t s) {
+    const IndexArrays &d = ix->d;
+    const int nb = bits_for((uint64_t)maxn);
+    DBuf<K> keys;
+    APS_TRY(keys.alloc((size_t)ix->M, s));
+    APS_TRY(vals.alloc((size_t)ix->M, s));
+    k_rank_keys<K><<<grid_for(ix->M, T256), T256, 0, s>>>(d.nnz_d.p, d.inst.p, ix->k, ix->M, nb, (uint64_t)maxn, keys.p,
+                                                          vals.p);
+    APS_LAUNCH_CHECK();
+    return sort_pairs(keys, vals, ix->M, nb + bits_for((uint64_t)(ix->k - 1)), s);
 }
 
 __global__ void k_rank_scatter(const uint32_t *__restrict__ vals, const InstDesc *__restrict__ inst, int k,
@@ -308,7 +323,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
                         const float *__restrict__ cval, const float *__restrict__ mwr,
                         const int32_t *__restrict__ vinst, const InstDesc *__restrict__ inst, int64_t N,
                         uint32_t flags, bool l2, const float *__restrict__ mw, int32_t *split, int32_t *qsplit,
-                        float *mwpre, int4 *vmeta, int4 *vcand, uint8_t *code, int64_t M, uint64_t *pkeys,
+                        float *mwpre, int4 *vmeta, int4 *vcand, uint8_t *code, int64_t M, uint32_t *pkeys,
                         uint32_t *pvals, unsigned long long *nsuf, unsigned long long *njoin) {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -384,7 +399,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
         // past the last rank (it sorts last); the value is the entry's index. The sort is
         // stable and entries arrive in row order, so every list comes out in increasing id.
         for (int64_t p = a + lane; p < b; p += 32) {
-            pkeys[p] = (p - a >= js) ? (uint64_t)I.rbase + (uint64_t)crank[p] : (uint64_t)M;
+            pkeys[p] = (p - a >= js) ? (uint32_t)I.rbase + (uint32_t)crank[p] : (uint32_t)M;
             pvals[p] = (uint32_t)p;
         }
     }
@@ -396,10 +411,10 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
 __global__ void k_post_keys(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
                             const int32_t *__restrict__ erow, const int32_t *__restrict__ vinst,
                             const InstDesc *__restrict__ inst, const int32_t *__restrict__ split, int64_t nnz,
-                            int64_t M, uint64_t *pkeys, uint32_t *pvals) {
+                            int64_t M, uint32_t *pkeys, uint32_t *pvals) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t x = erow[p];
-        pkeys[p] = (p - cptr[x] >= split[x]) ? (uint64_t)inst[vinst[x]].rbase + (uint64_t)crank[p] : (uint64_t)M;
+        pkeys[p] = (p - cptr[x] >= split[x]) ? (uint32_t)inst[vinst[x]].rbase + (uint32_t)crank[p] : (uint32_t)M;
         pvals[p] = (uint32_t)p;
     }
 }
@@ -428,12 +443,12 @@ __global__ void k_post_fill(const uint32_t *__restrict__ vals, const int32_t *__
 
 // List pointers from the sorted posting keys: lptr[R] = first suffix entry with key >= R
 // (binary search; lptr[M] = nsuf).
-__global__ void k_lptr(const uint64_t *__restrict__ keys, int64_t nsuf, int64_t M, int64_t *lptr) {
+__global__ void k_lptr(const uint32_t *__restrict__ keys, int64_t nsuf, int64_t M, int64_t *lptr) {
     for (int64_t R = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; R <= M; R += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = nsuf;
         while (lo < hi) {
             const int64_t mid = (lo + hi) >> 1;
-            if (keys[mid] < (uint64_t)R) lo = mid + 1; else hi = mid;
+            if (keys[mid] < (uint32_t)R) lo = mid + 1; else hi = mid;
         }
         lptr[R] = lo;
     }
@@ -478,9 +493,10 @@ __global__ void k_wptr(const InstDesc *__restrict__ inst, int k, const int64_t *
 // queries first (least-loaded-first idea of the vertical algorithm's binning). Classes 0-3
 // are the instance's tile shape (G = 1, 2, 4, 8); class 4 holds the vectors with one or two
 // components, which the join streams one warp per vector.
+constexpr int ITEM_COST_BITS = 13;
 __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
                             const int64_t *__restrict__ lptr, const int32_t *__restrict__ vinst,
-                            const InstDesc *__restrict__ inst, int64_t N, uint64_t *keys, uint32_t *vals,
+                            const InstDesc *__restrict__ inst, int64_t N, uint32_t *keys, uint32_t *vals,
                             unsigned long long *class_count) {
     // one warp per vector: the lanes read its ranks side by side and look up their lists;
     // the class counts go through shared memory (one global atomic per class and block)
@@ -494,7 +510,7 @@ __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__r
         const int64_t lx = x - I.vbase;
         if (lx >= (int64_t)I.n - 1) {  // no later candidates: after every class
             if (lane == 0) {
-                keys[x] = (uint64_t)JOIN_NCLS << 24;
+                keys[x] = (uint32_t)JOIN_NCLS << ITEM_COST_BITS;
                 vals[x] = (uint32_t)x;
             }
             continue;
@@ -508,13 +524,14 @@ __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__r
 #pragma unroll
         for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
         if (lane == 0) {
-            const double later = (double)(I.n - 1 - lx);
-            const double cost = (double)lsum * later / (double)I.n + later / 8.0 + 32.0;
-            // decreasing cost inside the class, in 24 bits (the costliest saturate together)
-            const uint64_t c = cost >= 16777215.0 ? 0xffffffull : (uint64_t)cost;
+            const float later = (float)(I.n - 1 - lx);
+            const float cost = (float)lsum * (later / (float)I.n) + later * 0.125f + 32.f;
+            // decreasing cost inside the class: the exponent and seven bits of the mantissa (costs
+            // are 32 to 2^63), so that the sort takes two passes instead of four
+            const uint32_t c = min((__float_as_uint(cost) - __float_as_uint(32.f)) >> 16, (1u << ITEM_COST_BITS) - 1u);
             // (a merge of two long lists would be one warp's serial tail: those go by windows)
             const int cls = b - a <= 1 || (b - a == 2 && lsum <= 8192) ? 4 : I.G == 1 ? 0 : I.G == 2 ? 1 : I.G == 4 ? 2 : 3;
-            keys[x] = ((uint64_t)cls << 24) | (0xffffffull - c);
+            keys[x] = ((uint32_t)cls << ITEM_COST_BITS) | ((1u << ITEM_COST_BITS) - 1u - c);
             vals[x] = (uint32_t)x;
             atomicAdd(&ccount[cls], 1ull);
         }
@@ -666,14 +683,11 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     }
     // ---- a2: dimension ranks and rank-ordered rows
     {
-        DBuf<uint64_t> keys;
         DBuf<uint32_t> vals;
-        APS_TRY(keys.alloc((size_t)M, s));
-        APS_TRY(vals.alloc((size_t)M, s));
-        int nb = bits_for((uint64_t)maxn);
-        k_rank_keys<<<gM, T256, 0, s>>>(d.nnz_d.p, d.inst.p, k, M, nb, (uint64_t)maxn, keys.p, vals.p);
-        APS_LAUNCH_CHECK();
-        APS_TRY(sort_pairs(keys.p, vals.p, M, nb + bits_for((uint64_t)(k - 1)), s));
+        if (bits_for((uint64_t)maxn) + bits_for((uint64_t)(k - 1)) <= 32)
+            APS_TRY(sort_dims<uint32_t>(ix, maxn, vals, s));
+        else
+            APS_TRY(sort_dims<uint64_t>(ix, maxn, vals, s));
         k_rank_scatter<<<gM, T256, 0, s>>>(vals.p, d.inst.p, k, M, d.mw_d.p, d.rank_of_dim.p, d.dim_of_rank.p,
                                            d.mwr.p);
         APS_LAUNCH_CHECK();
@@ -691,7 +705,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         if (rb == 0) rb = 1;
         k_canon_keys<<<gE, T256, 0, s>>>(idx, erow.p, d.vinst.p, d.inst.p, d.rank_of_dim.p, nnz, rb, keys.p, vals.p);
         APS_LAUNCH_CHECK();
-        APS_TRY(sort_pairs(keys.p, vals.p, nnz, rb + bits_for((uint64_t)(N - 1)), s));
+        APS_TRY(sort_pairs(keys, vals, nnz, rb + bits_for((uint64_t)(N - 1)), s));
         k_canon_gather<<<gE, T256, 0, s>>>(keys.p, vals.p, vout.p, nnz, (1ull << rb) - 1, d.crank.p, d.cval.p);
         APS_LAUNCH_CHECK();
     }
@@ -700,7 +714,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     APS_TRY(d.vcand.alloc((size_t)std::max<int64_t>(N, 1), s));
     APS_TRY(d.code.alloc((size_t)std::max<int64_t>(N, 1), s));
     // the split also writes each row's posting keys for a4 (and counts the indexed components)
-    DBuf<uint64_t> pkeys;
+    DBuf<uint32_t> pkeys;
     DBuf<uint32_t> pvals;
     APS_TRY(pkeys.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     APS_TRY(pvals.alloc((size_t)std::max<int64_t>(nnz, 1), s));
@@ -712,14 +726,14 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     APS_LAUNCH_CHECK();
     // ---- a4: suffix inverted index
     {
-        DBuf<uint64_t> &keys = pkeys;
+        DBuf<uint32_t> &keys = pkeys;
         DBuf<uint32_t> &vals = pvals;
         unsigned long long cnt3[3] = {0, 0, 0};  // by split, (longest row), in the join's lists
         APS_CUDA(cudaMemcpyAsync(cnt3, nsuf_d, sizeof(cnt3), cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
         ix->nsuf = (int64_t)cnt3[0];
         ix->njoin = (int64_t)cnt3[2];
-        if (nnz > 0) APS_TRY(sort_pairs(keys.p, vals.p, nnz, bits_for((uint64_t)M), s));
+        if (nnz > 0) APS_TRY(sort_pairs(keys, vals, nnz, bits_for((uint64_t)M), s));
         APS_TRY(d.post.alloc((size_t)std::max<int64_t>(ix->njoin, 1), s));
         APS_TRY(d.wptr.alloc((size_t)std::max<int64_t>(nwptr, 1), s));
         if (ix->njoin > 0) {
@@ -743,8 +757,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     }
     // ---- join work list
     {
-        DBuf<uint64_t> keys;
-        DBuf<uint32_t> vals;
+        DBuf<uint32_t> keys, vals;
         APS_TRY(keys.alloc((size_t)std::max<int64_t>(N, 1), s));
         APS_TRY(vals.alloc((size_t)std::max<int64_t>(N, 1), s));
         unsigned long long *cc = err.p;  // reused: one counter per class
@@ -754,7 +767,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
                                                                N, keys.p, vals.p,
                                             cc);
             APS_LAUNCH_CHECK();
-            APS_TRY(sort_pairs(keys.p, vals.p, N, 27, s));  // 3 class bits + 24 cost bits
+            APS_TRY(sort_pairs(keys, vals, N, 3 + ITEM_COST_BITS, s));
         }
         unsigned long long cnt_h[JOIN_NCLS] = {};
         APS_CUDA(cudaMemcpyAsync(cnt_h, cc, sizeof(cnt_h), cudaMemcpyDeviceToHost, s));
@@ -777,8 +790,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
 
 aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> &post, cudaStream_t s) {
     const IndexArrays &d = ix->d;
-    DBuf<uint64_t> keys;
-    DBuf<uint32_t> vals;
+    DBuf<uint32_t> keys, vals;
     DBuf<int32_t> erow;
     APS_TRY(keys.alloc((size_t)std::max<int64_t>(ix->nnz, 1), s));
     APS_TRY(vals.alloc((size_t)std::max<int64_t>(ix->nnz, 1), s));
@@ -791,7 +803,7 @@ aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> 
         k_post_keys<<<grid_for(ix->nnz, T256), T256, 0, s>>>(d.cptr.p, d.crank.p, erow.p, d.vinst.p, d.inst.p,
                                                              d.split.p, ix->nnz, ix->M, keys.p, vals.p);
         APS_LAUNCH_CHECK();
-        APS_TRY(sort_pairs(keys.p, vals.p, ix->nnz, bits_for((uint64_t)ix->M), s));
+        APS_TRY(sort_pairs(keys, vals, ix->nnz, bits_for((uint64_t)ix->M), s));
     }
     if (ix->nsuf > 0) {
         k_post_fill<<<grid_for(ix->nsuf, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p, d.inst.p,
@@ -806,18 +818,36 @@ aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> 
 // ------------------------------------------------------------------ external queries
 namespace {
 
+template <class K>
 __global__ void k_q_keys(const int32_t *__restrict__ qidx, const int32_t *__restrict__ erow,
-                         const int32_t *__restrict__ rank_of_dim, int64_t nnz, int rb, uint64_t *keys, uint32_t *vals) {
+                         const int32_t *__restrict__ rank_of_dim, int64_t nnz, int rb, K *keys, uint32_t *vals) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
-        keys[p] = ((uint64_t)erow[p] << rb) | (uint64_t)rank_of_dim[qidx[p]];
+        keys[p] = (K)(((uint64_t)erow[p] << rb) | (uint64_t)rank_of_dim[qidx[p]]);
         vals[p] = (uint32_t)p;
     }
 }
 
-__global__ void k_q_gather(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
+template <class K>
+__global__ void k_q_gather(const K *__restrict__ keys, const uint32_t *__restrict__ vals,
                            const float *__restrict__ vout, int64_t nnz, uint64_t rmask, int2 *crow) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x)
         crow[q] = make_int2((int32_t)(keys[q] & rmask), __float_as_int(vout[vals[q]]));
+}
+
+// The query rows over the index's ranks, in rank order (keys: row, rank).
+template <class K>
+aps_status sort_queries(const int32_t *qidx, const int32_t *erow, const int32_t *rank_of_dim, const float *vout,
+                        int64_t nnz, int rb, int bits, int2 *crow, cudaStream_t s) {
+    DBuf<K> keys;
+    DBuf<uint32_t> vals;
+    APS_TRY(keys.alloc((size_t)nnz, s));
+    APS_TRY(vals.alloc((size_t)nnz, s));
+    k_q_keys<K><<<grid_for(nnz, T256), T256, 0, s>>>(qidx, erow, rank_of_dim, nnz, rb, keys.p, vals.p);
+    APS_LAUNCH_CHECK();
+    APS_TRY(sort_pairs(keys, vals, nnz, bits, s));
+    k_q_gather<K><<<grid_for(nnz, T256), T256, 0, s>>>(keys.p, vals.p, vout, nnz, (1ull << rb) - 1, crow);
+    APS_LAUNCH_CHECK();
+    return APS_OK;
 }
 
 // Remscore boundary of a query: the first rank-ordered component where
@@ -907,16 +937,12 @@ aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32
     }
     APS_TRY(qa.crow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     if (nnz > 0) {
-        DBuf<uint64_t> keys;
-        DBuf<uint32_t> vals;
-        APS_TRY(keys.alloc((size_t)nnz, s));
-        APS_TRY(vals.alloc((size_t)nnz, s));
         const int rb = std::max(1, bits_for((uint64_t)(ix->maxm - 1)));
-        k_q_keys<<<grid_for(nnz, T256), T256, 0, s>>>(qidx, erow.p, d.rank_of_dim.p, nnz, rb, keys.p, vals.p);
-        APS_LAUNCH_CHECK();
-        APS_TRY(sort_pairs(keys.p, vals.p, nnz, rb + bits_for((uint64_t)std::max(nq - 1, 0)), s));
-        k_q_gather<<<grid_for(nnz, T256), T256, 0, s>>>(keys.p, vals.p, vout.p, nnz, (1ull << rb) - 1, qa.crow.p);
-        APS_LAUNCH_CHECK();
+        const int bits = rb + bits_for((uint64_t)std::max(nq - 1, 0));
+        if (bits <= 32)
+            APS_TRY(sort_queries<uint32_t>(qidx, erow.p, d.rank_of_dim.p, vout.p, nnz, rb, bits, qa.crow.p, s));
+        else
+            APS_TRY(sort_queries<uint64_t>(qidx, erow.p, d.rank_of_dim.p, vout.p, nnz, rb, bits, qa.crow.p, s));
     }
     APS_TRY(qa.vmeta.alloc((size_t)std::max<int64_t>(nq, 1), s));
     if (nq > 0) {

@@ -1318,7 +1318,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
     int64_t nsplit = 0, sp_cap = 0;
     DBuf<int32_t> items2;
     DBuf<int8_t> iblk;
-    DBuf<unsigned long long> sp_key;
+    DBuf<uint64_t> sp_key;
     DBuf<uint32_t> sp_score;
     if (split) {
         // block items come from the windowed classes (G = 1 ... 8), never from the
@@ -1402,7 +1402,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 P.items = items2.p;
                 P.iblk = iblk.p;
                 P.nblk = nblk;
-                P.sp_key = sp_key.p;
+                P.sp_key = reinterpret_cast<unsigned long long *>(sp_key.p);
                 P.sp_score = sp_score.p;
                 P.sp_cap = sp_cap;
                 for (int c = split_cls + 1; c <= JOIN_NCLS; c++) P.cls_begin[c] += nsplit * (nblk - 1);
@@ -1425,13 +1425,13 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 // the split vectors' pairs: sorted by (x, y), first occurrences kept, placed
                 // after the join's staged runs as the runs of their slots
                 const InstDesc &I0 = ix->inst_h[0];
-                APS_TRY(sort_pairs(reinterpret_cast<uint64_t *>(sp_key.p), sp_score.p, sp_found,
-                                   bits_for((uint64_t)I0.n * (uint64_t)I0.n), s));
+                APS_TRY(sort_pairs(sp_key, sp_score, sp_found, bits_for((uint64_t)I0.n * (uint64_t)I0.n), s));
+                const unsigned long long *const sp_sorted = reinterpret_cast<const unsigned long long *>(sp_key.p);
                 DBuf<int32_t> flag;
                 DBuf<int64_t> off;
                 APS_TRY(flag.alloc((size_t)sp_found, s));
                 APS_TRY(off.alloc((size_t)sp_found + 1, s));
-                k_first_of_key<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_key.p, sp_found, flag.p);
+                k_first_of_key<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, sp_found, flag.p);
                 APS_LAUNCH_CHECK();
                 APS_TRY(scan_exclusive(flag.p, off.p, sp_found, s));
                 int64_t nuniq = 0;
@@ -1446,10 +1446,10 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                     std::swap(grown.n, stage.n);
                     stage_cap = reserved + nuniq;
                 }
-                k_split_place<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_key.p, sp_score.p, flag.p, off.p, sp_found,
+                k_split_place<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, sp_score.p, flag.p, off.p, sp_found,
                                                                      d.inst.p, reserved, stage.p, segs.p, cntq.p);
                 APS_LAUNCH_CHECK();
-                k_split_counts<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_key.p, flag.p, sp_found, d.inst.p, cntq.p,
+                k_split_counts<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, flag.p, sp_found, d.inst.p, cntq.p,
                                                                       segs.p);
                 APS_LAUNCH_CHECK();
                 total_pairs += nuniq;

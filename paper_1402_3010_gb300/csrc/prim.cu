@@ -1,6 +1,7 @@
 // Error state, device memory and the generic device primitives (prefix sum, stable
 // radix sort) used by the index build and the output stage.
 #include <atomic>
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -216,150 +217,326 @@ aps_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream
 }
 
 // ------------------------------------------------------------------ radix sort
+// Stable LSD radix sort, 8 bits a pass. One kernel counts the digits of every pass; a pass is
+// then one kernel that reads each item once and writes it once: a tile ranks its items by warp,
+// publishes its digit counts, adds up the earlier tiles' by looking back over what they have
+// published, and writes its items out in digit runs. Against one histogram kernel, a scan (three
+// launches) and a scatter with four block barriers per 256 items for every pass, <SORTFIGURES>.
+// Up to SMALL_MAX items one CTA sorts in shared memory, all passes in one launch.
 namespace {
 
 constexpr int RS_THREADS = 256;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ROUNDS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;
 constexpr int RS_DIGITS = 256;
+constexpr int RS_MAXPASS = 8;
 
-// Digit histogram of each tile, stored digit-major: hist[d * nblocks + block], so that an
-// exclusive scan of the whole array gives each (digit, block) its output offset.
-__global__ void rs_hist_kernel(const uint64_t *__restrict__ keys, int64_t n, int shift,
-                               int32_t *__restrict__ hist) {
-    __shared__ int32_t h[RS_DIGITS];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int r = 0; r < RS_ROUNDS; r++) {
-        int64_t i = base + (int64_t)r * RS_THREADS + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 0xff], 1);
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
+template <class K>
+__device__ __forceinline__ int digit_of(const K k, const int shift) {
+    return (int)((k >> shift) & (K)0xff);
 }
 
-// Stable scatter: a tile is first ranked into shared memory by digit (items visited in
-// input order: round by round, lane order inside a warp, warp order inside a round), then
-// written out in digit runs, each run to consecutive addresses after all earlier items of
-// its digit. rs_smem holds the tile's keys and values (RS_TILE each).
-constexpr int RS_SMEM = RS_TILE * (8 + 4);
-
-__global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const uint64_t *__restrict__ kin,
-                                                                  const uint32_t *__restrict__ vin,
-                                                                  uint64_t *__restrict__ kout,
-                                                                  uint32_t *__restrict__ vout, int64_t n, int shift,
-                                                                  const int64_t *__restrict__ offs) {
-    extern __shared__ __align__(16) unsigned char rs_smem[];
-    uint64_t *sk = reinterpret_cast<uint64_t *>(rs_smem);
-    uint32_t *sv = reinterpret_cast<uint32_t *>(sk + RS_TILE);
-    __shared__ int64_t gbase[RS_DIGITS];  // output offset of (digit, this tile)
-    __shared__ int32_t lbase[RS_DIGITS];  // tile-local start of each digit
-    __shared__ int32_t cur[RS_DIGITS];    // tile-local cursor of each digit
-    __shared__ int32_t wc[RS_WARPS][RS_DIGITS];
-    __shared__ int32_t wsum[RS_WARPS];
+// Digit counts of all passes (gcount[pass][digit]); the last block to finish turns each pass's
+// counts into the digits' first output positions.
+template <class K>
+__global__ void __launch_bounds__(RS_THREADS) rs_count_kernel(const K *__restrict__ keys, int64_t n, int passes,
+                                                              unsigned long long *gcount, uint32_t *done) {
+    __shared__ uint32_t h[RS_MAXPASS][RS_DIGITS];
+    __shared__ unsigned long long wsum[RS_WARPS];
+    __shared__ bool last;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t nb = gridDim.x;
-    const int64_t hi = (int64_t)t * nb + blockIdx.x;
-    gbase[t] = offs[hi];
-    // exclusive scan of the tile's digit counts (offs is the digit-major scan of them)
-    const int c = (int)(offs[hi + 1] - offs[hi]);
-    int inc = c;
+    for (int p = 0; p < passes; p++) h[p][t] = 0u;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * RS_THREADS;
+    for (int64_t i0 = (int64_t)blockIdx.x * RS_THREADS; i0 < n; i0 += stride) {
+        const int64_t i = i0 + t;
+        const bool valid = i < n;
+        const K k = valid ? keys[i] : (K)0;
+        for (int p = 0; p < passes; p++) {
+            const int d = digit_of(k, 8 * p);
+            const int d0 = __shfl_sync(0xffffffffu, d, 0);
+            // (one digit for the whole warp is common in the high passes and among equal keys)
+            const bool same = valid && d == d0;
+            if (__all_sync(0xffffffffu, same)) {
+                if (lane == 0) atomicAdd(&h[p][d], 32u);
+            } else if (valid) {
+                atomicAdd(&h[p][d], 1u);
+            }
+        }
+    }
+    __syncthreads();
+    for (int p = 0; p < passes; p++)
+        if (h[p][t]) atomicAdd(&gcount[p * RS_DIGITS + t], (unsigned long long)h[p][t]);
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int p = 0; p < passes; p++) {
+        const unsigned long long c = *(volatile unsigned long long *)&gcount[p * RS_DIGITS + t];
+        unsigned long long inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        for (int w = 0; w < warp; w++) inc += wsum[w];
+        gcount[p * RS_DIGITS + t] = inc - c;
+        __syncthreads();
+    }
+}
+
+// Ranks of a warp's items among the items of the same digit of this warp so far (whist: the
+// warp's digit counts). Warp-collective; invalid items take no part.
+__device__ __forceinline__ uint32_t warp_rank(uint32_t *whist, const int d, const bool valid, const unsigned lt_mask) {
+    const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : 0x10000);
+    const uint32_t before = (uint32_t)__popc(peers & lt_mask);
+    uint32_t base = 0u;
+    if (valid) base = whist[d];
+    __syncwarp();
+    if (valid && before == 0u) whist[d] = base + (uint32_t)__popc(peers);
+    __syncwarp();
+    return base + before;
+}
+
+constexpr unsigned long long RS_COUNT = 1ull << 62, RS_TOTAL = 2ull << 62, RS_VALUE = (1ull << 62) - 1ull;
+constexpr int RS_SPINS = 1 << 14;  // polls of one earlier tile before its digit is counted here
+
+template <class K, bool VALS, int ITEMS>
+constexpr int rs_smem() { return RS_THREADS * ITEMS * (int)(sizeof(K) + (VALS ? 4 : 0)); }
+
+// One pass. Tiles are taken by ticket, so the earlier tiles that a tile looks back on have all
+// been started. A tile that stays silent for RS_SPINS polls is counted from its keys instead, so
+// the wait always ends.
+template <class K, bool VALS, int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS, 3) rs_pass_kernel(const K *__restrict__ kin,
+                                                             const uint32_t *__restrict__ vin, K *__restrict__ kout,
+                                                             uint32_t *__restrict__ vout, int64_t n, int shift,
+                                                             const unsigned long long *__restrict__ gbase,
+                                                             unsigned long long *status, uint32_t *ticket) {
+    constexpr int TILE = RS_THREADS * ITEMS;
+    extern __shared__ __align__(16) unsigned char rs_mem[];
+    K *sk = reinterpret_cast<K *>(rs_mem);
+    uint32_t *sv = reinterpret_cast<uint32_t *>(sk + TILE);
+    __shared__ uint32_t whist[RS_WARPS][RS_DIGITS];
+    __shared__ int64_t gpos[RS_DIGITS];  // output position of the digit's items minus their place in the tile
+    __shared__ uint32_t wsum[RS_WARPS];
+    __shared__ uint32_t tile_s;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    if (t == 0) tile_s = atomicAdd(ticket, 1u);
+    for (int w = 0; w < RS_WARPS; w++) whist[w][t] = 0u;
+    __syncthreads();
+    const int64_t tile = tile_s;
+    const int tn = (int)min((int64_t)TILE, n - tile * TILE);  // items of the tile
+    const int first = warp * (32 * ITEMS) + lane;             // this lane's first one
+    const K *const kp = kin + tile * TILE + first;
+    K k[ITEMS];
+    uint32_t v[ITEMS], rank[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) k[i] = first + 32 * i < tn ? kp[32 * i] : (K)0;
+    if (VALS) {
+        const uint32_t *const vp = vin + tile * TILE + first;
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++) v[i] = first + 32 * i < tn ? vp[32 * i] : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++)
+        rank[i] = warp_rank(whist[warp], digit_of(k[i], shift), first + 32 * i < tn, lt_mask);
+    __syncthreads();
+    // thread t: digit t. The warps' counts become their offsets, the tile's count is published
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; w++) {
+        const uint32_t x = whist[w][t];
+        whist[w][t] = c;
+        c += x;
+    }
+    volatile unsigned long long *st = status;
+    st[tile * RS_DIGITS + t] = (tile == 0 ? RS_TOTAL : RS_COUNT) | (unsigned long long)c;
+    uint32_t inc = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += y;
     }
     if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    int before = 0;
-    for (int w = 0; w < warp; w++) before += wsum[w];
-    lbase[t] = before + inc - c;
-    cur[t] = before + inc - c;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    const int64_t tile = (int64_t)blockIdx.x * RS_TILE;
-    for (int r = 0; r < RS_ROUNDS; r++) {
-        for (int w = 0; w < RS_WARPS; w++) wc[w][t] = 0;
-        __syncthreads();
-        const int64_t i = tile + (int64_t)r * RS_THREADS + t;
-        const bool valid = i < n;
-        const uint64_t k = valid ? kin[i] : 0;
-        const uint32_t v = valid ? vin[i] : 0;
-        const int d = (int)((k >> shift) & 0xff);
-        const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-        unsigned peers = 0;
-        int rank = 0;
-        if (valid) {
-            peers = __match_any_sync(vmask, d);
-            rank = __popc(peers & lt_mask);
-            if (rank == 0) wc[warp][d] = __popc(peers);
+    for (int w = 0; w < warp; w++) inc += wsum[w];
+    const uint32_t lbase = inc - c;  // place of the digit's first item in the tile
+    unsigned long long before = 0ull;  // the digit's items in earlier tiles
+    for (int64_t q = tile - 1; q >= 0; q--) {
+        unsigned long long x = st[q * RS_DIGITS + t];
+        for (int spin = 0; (x >> 62) == 0ull && spin < RS_SPINS; spin++) {
+            __nanosleep(32);
+            x = st[q * RS_DIGITS + t];
         }
-        __syncthreads();
-        {  // per digit: warp counts -> tile-local warp bases
-            int acc = cur[t];
-            for (int w = 0; w < RS_WARPS; w++) {
-                const int cw = wc[w][t];
-                wc[w][t] = acc;
-                acc += cw;
-            }
-            cur[t] = acc;
+        if ((x >> 62) == 0ull) {
+            for (int64_t e = q * TILE; e < (q + 1) * TILE; e++) x += digit_of(kin[e], shift) == t ? 1ull : 0ull;
         }
-        __syncthreads();
-        if (valid) {
-            const int q = wc[warp][d] + rank;
-            sk[q] = k;
-            sv[q] = v;
-        }
-        __syncthreads();
+        before += x & RS_VALUE;
+        if ((x >> 62) == 2ull) break;
     }
-    // write out in tile order: consecutive items of a digit go to consecutive addresses
-    const int tn = (int)min((int64_t)RS_TILE, n - tile);
+    if (tile > 0) st[tile * RS_DIGITS + t] = RS_TOTAL | (before + (unsigned long long)c);
+    gpos[t] = (int64_t)(gbase[t] + before) - (int64_t)lbase;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; w++) whist[w][t] += lbase;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        if (first + 32 * i < tn) {
+            const uint32_t q = whist[warp][digit_of(k[i], shift)] + rank[i];
+            sk[q] = k[i];
+            if (VALS) sv[q] = v[i];
+        }
+    }
+    __syncthreads();
     for (int q = t; q < tn; q += RS_THREADS) {
-        const uint64_t k = sk[q];
-        const int d = (int)((k >> shift) & 0xff);
-        const int64_t dst = gbase[d] + (q - lbase[d]);
-        kout[dst] = k;
-        vout[dst] = sv[q];
+        const K x = sk[q];
+        const int64_t dst = gpos[digit_of(x, shift)] + q;
+        kout[dst] = x;
+        if (VALS) vout[dst] = sv[q];
     }
+}
+
+// Up to SMALL_MAX items: one CTA, every pass in shared memory.
+constexpr int SMALL_THREADS = 1024;
+constexpr int SMALL_WARPS = SMALL_THREADS / 32;
+constexpr int SMALL_ITEMS = 8;
+constexpr int SMALL_MAX = SMALL_THREADS * SMALL_ITEMS;
+
+template <class K>
+__global__ void __launch_bounds__(SMALL_THREADS) rs_small_kernel(K *keys, uint32_t *vals, int n, int passes) {
+    extern __shared__ __align__(16) unsigned char rs_mem[];
+    K *sk = reinterpret_cast<K *>(rs_mem);
+    uint32_t *sv = reinterpret_cast<uint32_t *>(sk + SMALL_MAX);
+    uint32_t(*whist)[RS_DIGITS] = reinterpret_cast<uint32_t(*)[RS_DIGITS]>(sv + SMALL_MAX);
+    __shared__ uint32_t wsum[8];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int first = warp * (32 * SMALL_ITEMS) + lane;
+    K k[SMALL_ITEMS];
+    uint32_t v[SMALL_ITEMS], rank[SMALL_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SMALL_ITEMS; i++) {
+        const int q = first + 32 * i;
+        k[i] = q < n ? keys[q] : (K)0;
+        v[i] = vals && q < n ? vals[q] : 0u;
+    }
+    for (int p = 0; p < passes; p++) {
+        for (int i = t; i < SMALL_WARPS * RS_DIGITS; i += SMALL_THREADS) (&whist[0][0])[i] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SMALL_ITEMS; i++)
+            rank[i] = warp_rank(whist[warp], digit_of(k[i], 8 * p), first + 32 * i < n, lt_mask);
+        __syncthreads();
+        uint32_t c = 0, inc = 0;
+        if (t < RS_DIGITS) {  // thread t: digit t
+            for (int w = 0; w < SMALL_WARPS; w++) {
+                const uint32_t x = whist[w][t];
+                whist[w][t] = c;
+                c += x;
+            }
+            inc = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) wsum[warp] = inc;
+        }
+        __syncthreads();
+        if (t < RS_DIGITS) {
+            for (int w = 0; w < warp; w++) inc += wsum[w];
+            for (int w = 0; w < SMALL_WARPS; w++) whist[w][t] += inc - c;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SMALL_ITEMS; i++) {
+            if (first + 32 * i < n) {
+                const uint32_t q = whist[warp][digit_of(k[i], 8 * p)] + rank[i];
+                sk[q] = k[i];
+                sv[q] = v[i];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SMALL_ITEMS; i++) {
+            const int q = first + 32 * i;
+            if (q < n) {
+                k[i] = sk[q];
+                v[i] = sv[q];
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < SMALL_ITEMS; i++) {
+        const int q = first + 32 * i;
+        if (q < n) {
+            keys[q] = k[i];
+            if (vals) vals[q] = v[i];
+        }
+    }
+}
+
+template <class K, bool VALS>
+aps_status sort_impl(DBuf<K> &keys, DBuf<uint32_t> *vals, int64_t n, int bits, cudaStream_t s) {
+    if (n <= 1 || bits <= 0) return APS_OK;
+    const int passes = (bits + 7) / 8;
+    if (n <= SMALL_MAX) {
+        constexpr int smem = SMALL_MAX * (int)(sizeof(K) + 4) + SMALL_WARPS * RS_DIGITS * 4;
+        APS_CUDA(cudaFuncSetAttribute(rs_small_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        rs_small_kernel<K><<<1, SMALL_THREADS, smem, s>>>(keys.p, VALS ? vals->p : nullptr, (int)n, passes);
+        APS_LAUNCH_CHECK();
+        return APS_OK;
+    }
+    constexpr int ITEMS = sizeof(K) == 8 ? 16 : 20;
+    constexpr int TILE = RS_THREADS * ITEMS;
+    constexpr int smem = rs_smem<K, VALS, ITEMS>();
+    const int64_t nb = (n + TILE - 1) / TILE;
+    DBuf<K> k2;
+    DBuf<uint32_t> v2;
+    // counts of every pass, then every pass's tile states, then the tickets and the done counter
+    DBuf<unsigned long long> work;
+    const size_t words = (size_t)passes * RS_DIGITS * (size_t)(nb + 1) + RS_MAXPASS;
+    APS_TRY(k2.alloc((size_t)n, s));
+    if (VALS) APS_TRY(v2.alloc((size_t)n, s));
+    APS_TRY(work.alloc(words, s));
+    APS_CUDA(cudaMemsetAsync(work.p, 0, words * sizeof(unsigned long long), s));
+    unsigned long long *gcount = work.p, *status = work.p + (size_t)passes * RS_DIGITS;
+    uint32_t *tickets = reinterpret_cast<uint32_t *>(work.p + words - RS_MAXPASS);
+    APS_CUDA(cudaFuncSetAttribute(rs_pass_kernel<K, VALS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    rs_count_kernel<K><<<grid_for(n, RS_THREADS * 8, (int64_t)num_sms() * 8), RS_THREADS, 0, s>>>(
+        keys.p, n, passes, gcount, tickets + RS_MAXPASS);
+    APS_LAUNCH_CHECK();
+    for (int p = 0; p < passes; p++) {
+        rs_pass_kernel<K, VALS, ITEMS><<<(unsigned)nb, RS_THREADS, smem, s>>>(
+            keys.p, VALS ? vals->p : nullptr, k2.p, VALS ? v2.p : nullptr, n, 8 * p, gcount + p * RS_DIGITS,
+            status + (size_t)p * RS_DIGITS * nb, tickets + p);
+        APS_LAUNCH_CHECK();
+        std::swap(keys.p, k2.p);  // (the sorted items are the caller's, whatever the number of passes)
+        std::swap(keys.n, k2.n);
+        if (VALS) {
+            std::swap(vals->p, v2.p);
+            std::swap(vals->n, v2.n);
+        }
+    }
+    return APS_OK;
 }
 
 }  // namespace
 
-aps_status sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int bits, cudaStream_t s) {
-    if (n <= 1 || bits <= 0) return APS_OK;
-    int passes = (bits + 7) / 8;
-    int64_t nb = (n + RS_TILE - 1) / RS_TILE;
-    DBuf<uint64_t> k2;
-    DBuf<uint32_t> v2;
-    DBuf<int32_t> hist;
-    DBuf<int64_t> offs;
-    APS_TRY(k2.alloc((size_t)n, s));
-    APS_TRY(v2.alloc((size_t)n, s));
-    APS_TRY(hist.alloc((size_t)(nb * RS_DIGITS), s));
-    APS_TRY(offs.alloc((size_t)(nb * RS_DIGITS + 1), s));
-    APS_CUDA(cudaFuncSetAttribute(rs_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM));
-    uint64_t *ka = keys, *kb = k2.p;
-    uint32_t *va = vals, *vb = v2.p;
-    for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
-        rs_hist_kernel<<<(unsigned)nb, RS_THREADS, 0, s>>>(ka, n, shift, hist.p);
-        APS_LAUNCH_CHECK();
-        APS_TRY(scan_exclusive(hist.p, offs.p, nb * RS_DIGITS, s));
-        rs_scatter_kernel<<<(unsigned)nb, RS_THREADS, RS_SMEM, s>>>(ka, va, kb, vb, n, shift, offs.p);
-        APS_LAUNCH_CHECK();
-        uint64_t *tk = ka;
-        ka = kb;
-        kb = tk;
-        uint32_t *tv = va;
-        va = vb;
-        vb = tv;
-    }
-    if (ka != keys) {
-        APS_CUDA(cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s));
-        APS_CUDA(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
-    }
-    return APS_OK;
+aps_status sort_pairs(DBuf<uint64_t> &keys, DBuf<uint32_t> &vals, int64_t n, int bits, cudaStream_t s) {
+    return sort_impl<uint64_t, true>(keys, &vals, n, bits, s);
+}
+aps_status sort_pairs(DBuf<uint32_t> &keys, DBuf<uint32_t> &vals, int64_t n, int bits, cudaStream_t s) {
+    return sort_impl<uint32_t, true>(keys, &vals, n, bits, s);
+}
+aps_status sort_keys(DBuf<uint64_t> &keys, int64_t n, int bits, cudaStream_t s) {
+    return sort_impl<uint64_t, false>(keys, nullptr, n, bits, s);
 }
 
 }  // namespace aps

@@ -32,7 +32,7 @@ __global__ void k_rows_check(const int64_t *__restrict__ indptr, const int32_t *
 }
 
 __global__ void k_list_keys(const int32_t *__restrict__ pi, const int32_t *__restrict__ pj, int64_t count, int32_t n,
-                            uint64_t *keys, uint32_t *vals, unsigned long long *bad) {
+                            uint64_t *keys, unsigned long long *bad) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < count;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t a = pi[p], b = pj[p];
@@ -42,7 +42,6 @@ __global__ void k_list_keys(const int32_t *__restrict__ pi, const int32_t *__res
         } else {
             keys[p] = (uint64_t)a * (uint64_t)n + (uint64_t)b;
         }
-        vals[p] = 0u;
     }
 }
 
@@ -122,9 +121,7 @@ aps_status pairs_verify(const aps_pairs *lists, int32_t k, const int64_t *indptr
     }
     // 1. every list's keys in one buffer (host lists are brought over first)
     DBuf<uint64_t> keys;
-    DBuf<uint32_t> vals;
     APS_TRY(keys.alloc((size_t)std::max<int64_t>(total, 1), s));
-    APS_TRY(vals.alloc((size_t)std::max<int64_t>(total, 1), s));
     int64_t off = 0;
     for (int r = 0; r < k; r++) {
         const int64_t c = lists[r].count;
@@ -139,7 +136,7 @@ aps_status pairs_verify(const aps_pairs *lists, int32_t k, const int64_t *indptr
             pi = hi.p;
             pj = hj.p;
         }
-        k_list_keys<<<grid_for(c, 256), 256, 0, s>>>(pi, pj, c, n, keys.p + off, vals.p + off, bad.p);
+        k_list_keys<<<grid_for(c, 256), 256, 0, s>>>(pi, pj, c, n, keys.p + off, bad.p);
         APS_LAUNCH_CHECK();
         off += c;
         APS_CUDA(cudaStreamSynchronize(s));  // host staging of this list may be released
@@ -151,7 +148,7 @@ aps_status pairs_verify(const aps_pairs *lists, int32_t k, const int64_t *indptr
         return APS_EINVAL;
     }
     // 2. sort and keep the first of each run
-    if (total > 1) APS_TRY(sort_pairs(keys.p, vals.p, total, bits_for((uint64_t)n * (uint64_t)n), s));
+    APS_TRY(sort_keys(keys, total, bits_for((uint64_t)n * (uint64_t)n), s));
     DBuf<int32_t> flag;
     DBuf<int64_t> pos;
     APS_TRY(flag.alloc((size_t)std::max<int64_t>(total, 1), s));
@@ -172,7 +169,6 @@ aps_status pairs_verify(const aps_pairs *lists, int32_t k, const int64_t *indptr
         APS_LAUNCH_CHECK();
     }
     keys.release();
-    vals.release();
     // 3. exact scores, 4. the pairs that reach t
     DBuf<int32_t> keep;
     DBuf<float> sc;
