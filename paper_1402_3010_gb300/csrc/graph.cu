@@ -21,9 +21,12 @@
 namespace aps {
 namespace {
 
-// Smallest index of a pair that is out of range, not i < j, or not after its predecessor.
-__global__ void k_pairs_check(const int32_t *__restrict__ pi, const int32_t *__restrict__ pj, int64_t count,
-                              int32_t n, unsigned long long *bad) {
+// Smallest index of a pair that is out of range, not i < j, or not after its predecessor; and
+// the sort's keys and payload, written whether or not the pairs turn out to be good (one pass
+// over the pairs for both: 40M pairs in 0.27 ms, 0.38 in two).
+__global__ void k_check_keys(const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
+                             const float *__restrict__ ps, int64_t count, int32_t n, unsigned long long *bad,
+                             uint64_t *keys, uint32_t *vals) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < count;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t a = pi[p], b = pj[p];
@@ -33,14 +36,7 @@ __global__ void k_pairs_check(const int32_t *__restrict__ pi, const int32_t *__r
             ok = a0 < a || (a0 == a && b0 < b);
         }
         if (!ok) atomicMin(bad, (unsigned long long)p);
-    }
-}
-
-__global__ void k_sort_keys(const int32_t *__restrict__ pi, const int32_t *__restrict__ pj,
-                            const float *__restrict__ ps, int64_t count, uint64_t *keys, uint32_t *vals) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < count;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        keys[p] = ((uint64_t)(uint32_t)pi[p] << 32) | (uint64_t)(uint32_t)pj[p];
+        keys[p] = ((uint64_t)(uint32_t)a << 32) | (uint64_t)(uint32_t)b;
         vals[p] = __float_as_uint(ps[p]);
     }
 }
@@ -103,41 +99,156 @@ __device__ __forceinline__ unsigned long long knn_key(float w, int32_t id) {
     return ((unsigned long long)b << 32) | (unsigned long long)(0xffffffffu - (uint32_t)id);
 }
 
-// One warp per vertex: k rounds, each taking the largest key below the previous one.
-__global__ void k_knn(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                      const float *__restrict__ w, int32_t n, int32_t k, int32_t *nbr, float *wk) {
+__device__ __forceinline__ void knn_write(unsigned long long key, int32_t *nbr, float *wk) {
+    int32_t id = -1;
+    float wt = 0.f;
+    if (key != 0ull) {
+        id = (int32_t)(0xffffffffu - (uint32_t)(key & 0xffffffffull));
+        uint32_t hb = (uint32_t)(key >> 32);
+        hb = (hb & 0x80000000u) ? (hb & 0x7fffffffu) : ~hb;
+        wt = __uint_as_float(hb);
+    }
+    *nbr = id;
+    *wk = wt;
+}
+
+__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
+    return a > b ? a : b;
+}
+__device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b) {
+    return a < b ? a : b;
+}
+
+// A bitonic sequence across the lanes into descending order.
+__device__ __forceinline__ unsigned long long bitonic_desc(unsigned long long x, int lane) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = (lane & o) ? umin64(x, y) : umax64(x, y);
+    }
+    return x;
+}
+
+// One warp per vertex reads the row once and keeps its 32 * T largest keys so far sorted across
+// the lanes (place t * 32 + lane). Of 32 new keys those above the k-th so far go in one at a time,
+// or, when more than KNN_MERGE do, sorted and merged, so that a row in rising order costs no more
+// than its share. In a row of L neighbours in any order about k * ln(L / k) keys go in at all.
+// 200,000 rows of 400 at k = 16 take 0.37 ms, 1.20 when the row was read k times; the two
+// arrays alone are 0.64 GB, 0.1 ms, and the rest is the 64-bit compares of the insertions.
+constexpr int KNN_MERGE = 8;
+constexpr int KNN_LOADS = 4;
+
+template <int T>
+__global__ void __launch_bounds__(256) k_knn(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                                             const float *__restrict__ w, int32_t n, int32_t k, int32_t *nbr,
+                                             float *wk) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t v = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < n; v += nw) {
         const int64_t b = row_ptr[v], e = row_ptr[v + 1];
-        unsigned long long prev = ~0ull;
-        for (int r = 0; r < k; r++) {
-            unsigned long long best = 0ull;
-            if (prev != 0ull) {
-                for (int64_t q = b + lane; q < e; q += 32) {
-                    const unsigned long long key = knn_key(w[q], col[q]);
-                    if (key < prev && key > best) best = key;
-                }
+        unsigned long long top[T], kth = 0ull;
 #pragma unroll
-                for (int o = 16; o; o >>= 1) {
-                    const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
-                    best = y > best ? y : best;
-                }
+        for (int t = 0; t < T; t++) top[t] = 0ull;
+        for (int64_t q0 = b; q0 < e; q0 += 32 * KNN_LOADS) {
+            unsigned long long key[KNN_LOADS];
+#pragma unroll
+            for (int u = 0; u < KNN_LOADS; u++) {
+                const int64_t q = q0 + 32 * u + lane;
+                key[u] = q < e ? knn_key(w[q], col[q]) : 0ull;
             }
-            if (lane == 0) {
-                int32_t id = -1;
-                float wt = 0.f;
-                if (best != 0ull) {
-                    id = (int32_t)(0xffffffffu - (uint32_t)(best & 0xffffffffull));
-                    uint32_t hb = (uint32_t)(best >> 32);
-                    hb = (hb & 0x80000000u) ? (hb & 0x7fffffffu) : ~hb;
-                    wt = __uint_as_float(hb);
+#pragma unroll
+            for (int u = 0; u < KNN_LOADS; u++) {
+                unsigned m = __ballot_sync(0xffffffffu, key[u] > kth);
+                if (m == 0) continue;
+                if (__popc(m) > KNN_MERGE) {
+                    unsigned long long x = key[u];
+#pragma unroll
+                    for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+                        for (int o = size >> 1; o; o >>= 1) {
+                            const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+                            const bool up = size < 32 && (lane & size) != 0;  // this run rises
+                            x = (((lane & o) != 0) != up) ? umin64(x, y) : umax64(x, y);
+                        }
+                    }
+#pragma unroll
+                    for (int t = 0; t < T; t++) {
+                        const unsigned long long r = __shfl_xor_sync(0xffffffffu, x, 31);
+                        const unsigned long long hi = umax64(top[t], r), lo = umin64(top[t], r);
+                        top[t] = bitonic_desc(hi, lane);
+                        if (t + 1 < T) x = bitonic_desc(lo, lane);
+                    }
+                } else {
+                    while (m) {
+                        const int src = __ffs(m) - 1;
+                        m &= m - 1;
+                        const unsigned long long x = __shfl_sync(0xffffffffu, key[u], src);
+#pragma unroll
+                        for (int t = T - 1; t >= 0; t--) {
+                            unsigned long long before = __shfl_up_sync(0xffffffffu, top[t], 1);
+                            const unsigned long long carry =
+                                t > 0 ? __shfl_sync(0xffffffffu, top[t > 0 ? t - 1 : 0], 31) : ~0ull;
+                            if (lane == 0) before = carry;
+                            top[t] = top[t] > x ? top[t] : umin64(before, x);
+                        }
+                    }
                 }
-                nbr[v * (int64_t)k + r] = id;
-                wk[v * (int64_t)k + r] = wt;
+                // the k-th so far: 0 until k keys were seen
+                unsigned long long last = top[0];
+#pragma unroll
+                for (int t = 1; t < T; t++) last = ((k - 1) >> 5) == t ? top[t] : last;
+                kth = __shfl_sync(0xffffffffu, last, (k - 1) & 31);
             }
-            prev = best;
         }
+#pragma unroll
+        for (int t = 0; t < T; t++)
+            if (t * 32 + lane < k) knn_write(top[t], nbr + v * (int64_t)k + t * 32 + lane, wk + v * (int64_t)k + t * 32 + lane);
+    }
+}
+
+// Up to eight neighbours: every lane keeps its own K largest keys and the warp takes the k largest of
+// all lanes at the end; no order of a row makes this dearer.
+template <int K>
+__global__ void __launch_bounds__(256) k_knn_few(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                                                 const float *__restrict__ w, int32_t n, int32_t k, int32_t *nbr,
+                                                 float *wk) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t v = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < n; v += nw) {
+        const int64_t b = row_ptr[v], e = row_ptr[v + 1];
+        unsigned long long top[K], mine = 0ull;
+#pragma unroll
+        for (int t = 0; t < K; t++) top[t] = 0ull;
+        for (int64_t q0 = b; q0 < e; q0 += 32 * KNN_LOADS) {
+            unsigned long long key[KNN_LOADS];
+#pragma unroll
+            for (int u = 0; u < KNN_LOADS; u++) {
+                const int64_t q = q0 + 32 * u + lane;
+                key[u] = q < e ? knn_key(w[q], col[q]) : 0ull;
+            }
+#pragma unroll
+            for (int u = 0; u < KNN_LOADS; u++) {
+                unsigned long long x = key[u];
+#pragma unroll
+                for (int t = 0; t < K; t++) {
+                    const unsigned long long y = top[t];
+                    top[t] = umax64(x, y);
+                    x = umin64(x, y);
+                }
+            }
+        }
+        for (int r = 0; r < k; r++) {  // keys differ: the lane that holds the largest drops it
+            unsigned long long best = top[0];
+#pragma unroll
+            for (int o = 16; o; o >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, o));
+            if (lane == r) mine = best;
+            if (top[0] == best) {
+#pragma unroll
+                for (int t = 0; t + 1 < K; t++) top[t] = top[t + 1];
+                top[K - 1] = 0ull;
+            }
+        }
+        if (lane < k) knn_write(mine, nbr + v * (int64_t)k + lane, wk + v * (int64_t)k + lane);
     }
 }
 
@@ -178,11 +289,15 @@ aps_status graph_csr(const int32_t *i_in, const int32_t *j_in, const float *s_in
         pj = dj.p;
         ps = ds.p;
     }
+    DBuf<uint64_t> keys;
+    DBuf<uint32_t> vals;
     if (count > 0) {
         DBuf<unsigned long long> bad;
         APS_TRY(bad.alloc(1, s));
+        APS_TRY(keys.alloc((size_t)count, s));
+        APS_TRY(vals.alloc((size_t)count, s));
         APS_CUDA(cudaMemsetAsync(bad.p, 0xff, sizeof(unsigned long long), s));
-        k_pairs_check<<<grid_for(count, 256), 256, 0, s>>>(pi, pj, count, n, bad.p);
+        k_check_keys<<<grid_for(count, 256), 256, 0, s>>>(pi, pj, ps, count, n, bad.p, keys.p, vals.p);
         APS_LAUNCH_CHECK();
         unsigned long long b = 0;
         APS_CUDA(cudaMemcpyAsync(&b, bad.p, sizeof(b), cudaMemcpyDeviceToHost, s));
@@ -223,15 +338,9 @@ aps_status graph_csr(const int32_t *i_in, const int32_t *j_in, const float *s_in
     };
     {
         DBuf<int64_t> start;
-        DBuf<uint64_t> keys;
-        DBuf<uint32_t> vals;
         if ((st = start.alloc(2 * ((size_t)n + 1), s)) != APS_OK) return fail(st);
-        if ((st = keys.alloc((size_t)count, s)) != APS_OK) return fail(st);
-        if ((st = vals.alloc((size_t)count, s)) != APS_OK) return fail(st);
         int64_t *start_i = start.p, *start_j = start.p + n + 1;
         if (count > 0) {
-            k_sort_keys<<<grid_for(count, 256), 256, 0, s>>>(pi, pj, ps, count, keys.p, vals.p);
-            count_launch();
             if ((st = sort_pairs(keys, vals, count, bits_for((uint64_t)n), s)) != APS_OK) return fail(st);
         }
         k_starts<<<grid_for((int64_t)n + 1, 256), 256, 0, s>>>(pi, keys.p, count, n, start_i, start_j, row_ptr);
@@ -289,8 +398,16 @@ aps_status graph_knn(const aps_graph *g, int32_t k, int32_t *nbr, float *wk, uin
         on = dn.p;
         ow = dw.p;
     }
-    k_knn<<<grid_for((int64_t)g->n * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(g->row_ptr, g->col, g->w, g->n,
-                                                                                      k, on, ow);
+    // Up to eight by the lanes' own lists, whose cost grows with k but not with the order of a row
+    // (0.42 ms at k = 6 on the rows above, any order; the warp's list 0.25 in any order, 0.89 where
+    // a row's weights rise, and re-reading the row k times 0.47): from nine on that list is cheaper
+    // in any order, and no dearer than the k passes were from twelve on where they rise.
+    static constexpr decltype(&k_knn<1>) few[8] = {k_knn_few<1>, k_knn_few<2>, k_knn_few<3>, k_knn_few<4>,
+                                                   k_knn_few<5>, k_knn_few<6>, k_knn_few<7>, k_knn_few<8>};
+    const auto knn = k <= 8    ? few[k - 1]
+                     : k <= 32 ? k_knn<1> : k <= 64 ? k_knn<2> : k <= 128 ? k_knn<4> : k_knn<8>;
+    knn<<<grid_for((int64_t)g->n * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(g->row_ptr, g->col, g->w, g->n, k,
+                                                                                    on, ow);
     APS_LAUNCH_CHECK();
     if (!(flags & APS_DEVICE_PTRS)) {
         APS_CUDA(cudaMemcpyAsync(nbr, on, sizeof(int32_t) * (size_t)nk, cudaMemcpyDeviceToHost, s));
