@@ -268,15 +268,7 @@ aps_status aps_pairs_copy_to(const aps_pairs *p, int32_t *i, int32_t *j, float *
         set_error("pairs must not be NULL");
         return APS_EINVAL;
     }
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t n = (size_t)p->count;
-    if (n) {
-        if (i) APS_CUDA(cudaMemcpyAsync(i, p->i, n * 4, cudaMemcpyDefault, s));
-        if (j) APS_CUDA(cudaMemcpyAsync(j, p->j, n * 4, cudaMemcpyDefault, s));
-        if (score) APS_CUDA(cudaMemcpyAsync(score, p->score, n * 4, cudaMemcpyDefault, s));
-    }
-    APS_CUDA(cudaStreamSynchronize(s));
-    return APS_OK;
+    return pairs_copy(p, i, j, score, static_cast<cudaStream_t>(stream));
 }
 
 aps_status aps_batch_all_pairs(int32_t k, const aps_instance *inst, uint32_t flags, void *stream, aps_pairs *outs,

@@ -175,6 +175,8 @@ struct PairsAlloc {          // bookkeeping behind aps_pairs._priv
 };
 
 void pairs_release(aps_pairs *p);
+// Copy a result's arrays to the caller's (host or device, any may be null) and wait.
+aps_status pairs_copy(const aps_pairs *p, int32_t *i, int32_t *j, float *score, cudaStream_t s);
 // Replace device pairs by one pinned host copy.
 aps_status pairs_to_host(aps_pairs *p, cudaStream_t s);
 

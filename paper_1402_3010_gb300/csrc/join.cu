@@ -32,6 +32,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "index.cuh"
@@ -1550,6 +1552,58 @@ void pairs_release(aps_pairs *p) {
     p->i = p->j = nullptr;
     p->score = nullptr;
     p->count = 0;
+}
+
+namespace {
+
+// Whether p is host memory, pinned or not (managed memory is left to the driver).
+bool is_host(const void *p) {
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return pa.type == cudaMemoryTypeUnregistered || pa.type == cudaMemoryTypeHost;
+}
+
+}  // namespace
+
+aps_status pairs_copy(const aps_pairs *p, int32_t *i, int32_t *j, float *score, cudaStream_t s) {
+    const size_t n = (size_t)std::max<int64_t>(p->count, 0);
+    const void *src[3] = {p->i, p->j, p->score};
+    void *dst[3] = {i, j, score};
+    bool all_host = n && !p->on_device;
+    for (int k = 0; k < 3 && all_host; k++) all_host = !dst[k] || is_host(dst[k]);
+    if (all_host) {
+        // A result in pinned host memory to plain host memory: the processor copies it (the driver
+        // moves such copies at 9.5 GB/s), the three arrays side by side where they are large.
+        APS_CUDA(cudaStreamSynchronize(s));
+        std::thread side[2];
+        int running = 0;
+        int own[3], nown = 0;
+        for (int k = 0; k < 3; k++) {
+            if (!dst[k]) continue;
+            if (nown > 0 && n >= ((size_t)1 << 18)) {
+                try {
+                    void *d = dst[k];
+                    const void *a = src[k];
+                    side[running] = std::thread([d, a, n] { memcpy(d, a, n * 4); });
+                    running++;
+                    continue;
+                } catch (const std::system_error &) {  // no thread to be had: copied here
+                }
+            }
+            own[nown++] = k;
+        }
+        for (int q = 0; q < nown; q++) memcpy(dst[own[q]], src[own[q]], n * 4);
+        for (int q = 0; q < running; q++) side[q].join();
+        return APS_OK;
+    } else if (n) {
+        for (int k = 0; k < 3; k++)
+            if (dst[k]) APS_CUDA(cudaMemcpyAsync(dst[k], src[k], n * 4, cudaMemcpyDefault, s));
+    }
+    APS_CUDA(cudaStreamSynchronize(s));
+    return APS_OK;
 }
 
 // Copy device pairs into one pinned host allocation (replacing the device one).
