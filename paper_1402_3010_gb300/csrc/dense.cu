@@ -496,49 +496,106 @@ __global__ void __launch_bounds__(DN_THREADS, 1)
     }
 }
 
-// One warp per row: float64 norm; with normalise, rows are scaled into Y; otherwise a row
-// whose norm is off by more than 1e-3 (or holds a non-finite value) is reported in *bad.
+// One warp per row, the row in registers (at most four float4 a lane): its norm, and the row
+// rounded to BF16. With normalise, rows are scaled into Y by their float64 norm; otherwise a row
+// whose norm is off by more than 1e-3 (or holds a non-finite value) is reported in *bad: float32
+// decides where its sum of squares (off by at most 21 roundings of 2^-24) lies clear of those
+// norms, which no row with a non-finite value does, and float64 the rest. A float64 instruction
+// holds the SM for some 15 cycles a warp: 200,000 rows of 256 took 0.37 ms with float64 for all
+// and 0.12 for the BF16 rows in a pass of their own, 0.075 in one.
 __global__ void k_dense_rows(const float *__restrict__ X, int64_t n, int d, int normalise, float *Y,
-                             unsigned long long *bad) {
+                             __nv_bfloat16 *__restrict__ Xb, unsigned long long *bad) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int d4 = d >> 2;
     for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < n; r += nw) {
-        double ss = 0.0;
-        bool finite = true;
-        for (int e = lane; e < d; e += 32) {
-            const float v = X[r * d + e];
-            finite = finite && isfinite(v);
-            ss += (double)v * (double)v;
+        const float4 *X4 = reinterpret_cast<const float4 *>(X) + r * d4;
+        float4 v[4];
+        float s32 = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            v[u] = lane + 32 * u < d4 ? X4[lane + 32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+            s32 = fmaf(v[u].x, v[u].x, s32);
+            s32 = fmaf(v[u].y, v[u].y, s32);
+            s32 = fmaf(v[u].z, v[u].z, s32);
+            s32 = fmaf(v[u].w, v[u].w, s32);
         }
 #pragma unroll
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        finite = __all_sync(0xffffffffu, finite);
-        const double nrm = sqrt(ss);
-        if (normalise) {
-            const double sc = nrm > 0.0 ? 1.0 / nrm : 0.0;
-            for (int e = lane; e < d; e += 32) Y[r * d + e] = (float)((double)X[r * d + e] * sc);
-            if (lane == 0 && (!finite || nrm == 0.0)) atomicMin(bad, (unsigned long long)r);
-        } else if (lane == 0 && (!finite || fabs(nrm - 1.0) > 1e-3)) {
-            atomicMin(bad, (unsigned long long)r);
+        for (int o = 16; o; o >>= 1) s32 += __shfl_xor_sync(0xffffffffu, s32, o);
+        if (normalise || !(s32 >= 0.9981f && s32 <= 1.0019f)) {
+            double ss = 0.0;
+            bool finite = true;
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const float e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    finite = finite && isfinite(e[q]);
+                    ss += (double)e[q] * (double)e[q];
+                }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            finite = __all_sync(0xffffffffu, finite);
+            const double nrm = sqrt(ss);
+            if (normalise) {
+                const double sc = nrm > 0.0 ? 1.0 / nrm : 0.0;
+                float4 *Y4 = reinterpret_cast<float4 *>(Y) + r * d4;
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    v[u] = make_float4((float)((double)v[u].x * sc), (float)((double)v[u].y * sc),
+                                       (float)((double)v[u].z * sc), (float)((double)v[u].w * sc));
+                    if (lane + 32 * u < d4) Y4[lane + 32 * u] = v[u];
+                }
+                if (lane == 0 && (!finite || nrm == 0.0)) atomicMin(bad, (unsigned long long)r);
+            } else if (lane == 0 && (!finite || fabs(nrm - 1.0) > 1e-3)) {
+                atomicMin(bad, (unsigned long long)r);
+            }
         }
+        __nv_bfloat162 *B2 = reinterpret_cast<__nv_bfloat162 *>(Xb + r * d);
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (lane + 32 * u < d4) {
+                union {
+                    __nv_bfloat162 h[2];
+                    uint2 w;
+                } c;
+                c.h[0] = __floats2bfloat162_rn(v[u].x, v[u].y);
+                c.h[1] = __floats2bfloat162_rn(v[u].z, v[u].w);
+                reinterpret_cast<uint2 *>(B2)[lane + 32 * u] = c.w;
+            }
     }
 }
 
-__global__ void k_to_bf16(const float *__restrict__ X, int64_t n, int d, int64_t n_pad, __nv_bfloat16 *Xb) {
-    const int64_t total = n_pad * d;
+// The BF16 rows alone (rows as they are).
+__global__ void k_to_bf16(const float *__restrict__ X, int64_t n, int d, __nv_bfloat16 *Xb) {
+    const int64_t total = n * d;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
-        Xb[e] = (e < n * d) ? __float2bfloat16_rn(X[e]) : __float2bfloat16_rn(0.f);
+        Xb[e] = __float2bfloat16_rn(X[e]);
 }
 
 // Exact rescoring of the candidates (sorted keys i*n + j). Each warp takes a contiguous run
-// of candidates and scores four at a time, issuing all their row loads (float4) before any
-// arithmetic, so that four pairs' reads are in flight per warp; consecutive candidates share
-// row i, which then comes from L1. float32 dot with a tree reduction; float64 when the
-// float32 score lies within the band of t. X is 16-byte aligned and d % 64 == 0, d <= 512.
-constexpr int RS_BATCH = 4;
+// of candidates, 32 at a time: a lane divides one key into its pair (a 64-bit division costs more
+// than the dot product's own instructions), then RS_BATCH pairs are scored together. Pairs of one
+// i (most batches: candidates come sorted) read row i into registers once; all the row loads
+// (float4) of a batch are issued before any arithmetic. float32 dot with a tree reduction; float64
+// when the float32 score lies within the band of t. X is 16-byte aligned and d % 64 == 0, d <= 512;
+// V = the float4 a lane holds of a row. What bounds it are the j rows, from L2 where X fits there:
+// 200,000 rows of 256 with some 50 candidates each took 2.33 ms, 0.93 now.
+constexpr int RS_MIN = 4;  // candidates a warp at least
 
-__global__ void k_rescore(const unsigned long long *__restrict__ keys, int64_t nc, const float *__restrict__ X, int n,
-                          int d, float t, float beta, int32_t *keep, float *score, unsigned long long *nband) {
+__device__ __forceinline__ float dot4(const float4 &a, const float4 &b, float acc) {
+    acc = fmaf(a.x, b.x, acc);
+    acc = fmaf(a.y, b.y, acc);
+    acc = fmaf(a.z, b.z, acc);
+    return fmaf(a.w, b.w, acc);
+}
+
+template <int V>
+__global__ void __launch_bounds__(256) k_rescore(const unsigned long long *__restrict__ keys, int64_t nc,
+                                                 const float *__restrict__ X, int n, int d, float t, float beta,
+                                                 int32_t *keep, float *score, unsigned long long *nband) {
+    constexpr int RS_BATCH = V <= 2 ? 8 : 4;
     const int lane = threadIdx.x & 31;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -546,56 +603,83 @@ __global__ void k_rescore(const unsigned long long *__restrict__ keys, int64_t n
     const int64_t c0 = wid * per, c1 = min(nc, c0 + per);
     const int d4 = d >> 2;
     const float4 *X4 = reinterpret_cast<const float4 *>(X);
-    for (int64_t c = c0; c < c1; c += RS_BATCH) {
-        int64_t ii[RS_BATCH], jj[RS_BATCH];
-        float acc[RS_BATCH];
+    float4 a[V];
+    int cur = -1;  // the row that a holds
+    for (int64_t cb = c0; cb < c1; cb += 32) {
+        const int cnt = (int)min((int64_t)32, c1 - cb);
+        const unsigned long long k = keys[cb + min(lane, cnt - 1)];
+        const int mi = (int)(k / (unsigned long long)n), mj = (int)(k - (unsigned long long)mi * (unsigned long long)n);
+        float mine = 0.f;  // the score of this lane's candidate
+        for (int g = 0; g < cnt; g += RS_BATCH) {
+            int ii[RS_BATCH], jj[RS_BATCH];
+            float acc[RS_BATCH];
 #pragma unroll
-        for (int u = 0; u < RS_BATCH; u++) {
-            const unsigned long long k = keys[min(c + u, c1 - 1)];
-            ii[u] = (int64_t)(k / (unsigned long long)n);
-            jj[u] = (int64_t)(k % (unsigned long long)n);
-            acc[u] = 0.f;
-        }
+            for (int u = 0; u < RS_BATCH; u++) {  // (lanes from cnt on hold the last candidate)
+                ii[u] = __shfl_sync(0xffffffffu, mi, g + u);
+                jj[u] = __shfl_sync(0xffffffffu, mj, g + u);
+                acc[u] = 0.f;
+            }
+            if (ii[0] == ii[RS_BATCH - 1]) {  // sorted: one i for all
+                float4 b[V][RS_BATCH];
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
-            if (lane + 32 * v < d4) {
-                float4 a[RS_BATCH], b[RS_BATCH];
+                for (int v = 0; v < V; v++)
 #pragma unroll
-                for (int u = 0; u < RS_BATCH; u++) {
-                    a[u] = X4[ii[u] * d4 + lane + 32 * v];
-                    b[u] = X4[jj[u] * d4 + lane + 32 * v];
+                    for (int u = 0; u < RS_BATCH; u++)
+                        b[v][u] = lane + 32 * v < d4 ? X4[(int64_t)jj[u] * d4 + lane + 32 * v]
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (ii[0] != cur) {
+                    cur = ii[0];
+#pragma unroll
+                    for (int v = 0; v < V; v++)
+                        a[v] = lane + 32 * v < d4 ? X4[(int64_t)cur * d4 + lane + 32 * v]
+                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
-                for (int u = 0; u < RS_BATCH; u++) {
-                    acc[u] = fmaf(a[u].x, b[u].x, acc[u]);
-                    acc[u] = fmaf(a[u].y, b[u].y, acc[u]);
-                    acc[u] = fmaf(a[u].z, b[u].z, acc[u]);
-                    acc[u] = fmaf(a[u].w, b[u].w, acc[u]);
+                for (int v = 0; v < V; v++)
+#pragma unroll
+                    for (int u = 0; u < RS_BATCH; u++) acc[u] = dot4(a[v], b[v][u], acc[u]);
+            } else {
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    if (lane + 32 * v < d4) {
+                        float4 x[RS_BATCH], y[RS_BATCH];
+#pragma unroll
+                        for (int u = 0; u < RS_BATCH; u++) {
+                            x[u] = X4[(int64_t)ii[u] * d4 + lane + 32 * v];
+                            y[u] = X4[(int64_t)jj[u] * d4 + lane + 32 * v];
+                        }
+#pragma unroll
+                        for (int u = 0; u < RS_BATCH; u++) acc[u] = dot4(x[u], y[u], acc[u]);
+                    }
                 }
             }
+#pragma unroll
+            for (int u = 0; u < RS_BATCH; u++) {
+#pragma unroll
+                for (int o = 16; o; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+                if (lane == g + u) mine = acc[u];
+            }
         }
+        bool in = lane < cnt && mine >= t;
+        unsigned band = __ballot_sync(0xffffffffu, lane < cnt && fabsf(mine - t) <= beta);
+        if (lane == 0 && band) atomicAdd(nband, (unsigned long long)__popc(band));
+        while (band) {
+            const int q = __ffs(band) - 1;
+            band &= band - 1;
+            const int bi = __shfl_sync(0xffffffffu, mi, q), bj = __shfl_sync(0xffffffffu, mj, q);
+            const float *xi = X + (int64_t)bi * d, *xj = X + (int64_t)bj * d;
+            double a64 = 0.0;
+            for (int e = lane; e < d; e += 32) a64 += (double)xi[e] * (double)xj[e];
 #pragma unroll
-        for (int u = 0; u < RS_BATCH; u++) {
-#pragma unroll
-            for (int o = 16; o; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
-        }
-        for (int u = 0; u < RS_BATCH && c + u < c1; u++) {
-            float s = acc[u];
-            bool in = s >= t;
-            if (fabsf(s - t) <= beta) {
-                const float *xi = X + ii[u] * d, *xj = X + jj[u] * d;
-                double a64 = 0.0;
-                for (int e = lane; e < d; e += 32) a64 += (double)xi[e] * (double)xj[e];
-#pragma unroll
-                for (int o = 16; o; o >>= 1) a64 += __shfl_xor_sync(0xffffffffu, a64, o);
+            for (int o = 16; o; o >>= 1) a64 += __shfl_xor_sync(0xffffffffu, a64, o);
+            if (lane == q) {
                 in = a64 >= (double)t;
-                s = (float)a64;
-                if (lane == 0) atomicAdd(nband, 1ull);
+                mine = (float)a64;
             }
-            if (lane == 0) {
-                keep[c + u] = in ? 1 : 0;
-                score[c + u] = s;
-            }
+        }
+        if (lane < cnt) {
+            keep[cb + lane] = in ? 1 : 0;
+            score[cb + lane] = mine;
         }
     }
 }
@@ -662,8 +746,12 @@ double dense_margin(int d) {
     return (2.0 * u + u * u) * 1.002 + 2.0 * d * std::ldexp(1.0, -23);
 }
 
+static int64_t dense_rows_padded(int64_t n) {
+    return std::max<int64_t>(PAIR_ROWS, (n + PAIR_ROWS - 1) / PAIR_ROWS * PAIR_ROWS);
+}
+
 aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t, cudaStream_t s, aps_pairs *out,
-                                  aps_stats *stats, float *raw) {
+                                  aps_stats *stats, float *raw, const DenseRows *rows) {
     int dev = 0, major = 0, minor = 0;
     APS_CUDA(cudaGetDevice(&dev));
     APS_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
@@ -673,7 +761,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
         return APS_EUNSUPPORTED;
     }
     const int KB = d / KBLK;
-    const int64_t n_pad = std::max<int64_t>(PAIR_ROWS, ((int64_t)n + PAIR_ROWS - 1) / PAIR_ROWS * PAIR_ROWS);
+    const int64_t n_pad = dense_rows_padded(n);
     const int S = std::min(MAX_STAGES, (SMEM_BUDGET - KB * TILE_BYTES) / TILE_BYTES);
     const int smem = (KB + S) * TILE_BYTES + 1024 + 512;  // operands, alignment slack, barriers
     cudaEvent_t ev[5];
@@ -685,12 +773,16 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
         }
     } evg{ev};
     APS_CUDA(cudaEventRecord(ev[0], s));
-    DBuf<__nv_bfloat16> Xb;
-    APS_TRY(Xb.alloc((size_t)(n_pad * d), s));
-    k_to_bf16<<<grid_for(n_pad * d, 256, 65536), 256, 0, s>>>(X, n, d, n_pad, Xb.p);
-    APS_LAUNCH_CHECK();
+    DBuf<__nv_bfloat16> own;
+    if (!rows) {
+        APS_TRY(own.alloc((size_t)(n_pad * d), s));
+        APS_CUDA(cudaMemsetAsync(own.p + (int64_t)n * d, 0, sizeof(__nv_bfloat16) * (size_t)((n_pad - n) * d), s));
+        k_to_bf16<<<grid_for((int64_t)n * d, 256, 65536), 256, 0, s>>>(X, n, d, own.p);
+        APS_LAUNCH_CHECK();
+    }
+    __nv_bfloat16 *const Xb = rows ? static_cast<__nv_bfloat16 *>(rows->xb) : own.p;
     CUtensorMap map;
-    APS_TRY(encode_map(&map, Xb.p, n_pad, d));
+    APS_TRY(encode_map(&map, Xb, n_pad, d));
     // work units: (A block, run of B blocks), B blocks from the diagonal onward
     const int64_t nb = n_pad / PAIR_ROWS;
     std::vector<int4> units;
@@ -809,8 +901,9 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     APS_TRY(pos.alloc((size_t)nc + 1, s));
     const float beta = (float)std::max(1e-5, (d / 32.0 + 8.0) * std::ldexp(1.0, -23));
     if (nc > 0) {
-        k_rescore<<<grid_for(nc * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(sorted, nc, X, n, d, t, beta,
-                                                                                   keep.p, sc.p, ctr.p + 1);
+        const unsigned g = grid_for((nc + RS_MIN - 1) / RS_MIN * 32, 256, (int64_t)num_sms() * 64);
+        const auto rescore = d <= 128 ? k_rescore<1> : d <= 256 ? k_rescore<2> : d <= 384 ? k_rescore<3> : k_rescore<4>;
+        rescore<<<g, 256, 0, s>>>(sorted, nc, X, n, d, t, beta, keep.p, sc.p, ctr.p + 1);
         APS_LAUNCH_CHECK();
     }
     APS_TRY(scan_exclusive(keep.p, pos.p, nc, s));
@@ -838,7 +931,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     APS_CUDA(cudaEventRecord(ev[4], s));
     APS_CUDA(cudaEventSynchronize(ev[4]));
     float ms_total = 0, ms_out = 0;
-    cudaEventElapsedTime(&ms_total, ev[0], ev[4]);
+    cudaEventElapsedTime(&ms_total, rows ? rows->began : ev[0], ev[4]);
     cudaEventElapsedTime(&ms_out, ev[2], ev[4]);
     if (stats) {
         memset(stats, 0, sizeof(*stats));
@@ -877,8 +970,17 @@ aps_status dense_all_pairs(const float *X, int32_t n, int32_t d, float t, uint32
     APS_CUDA(cudaMemsetAsync(bad.p, 0xff, sizeof(unsigned long long), s));
     const bool norm = (flags & APS_NORMALIZE) != 0;
     if (norm) APS_TRY(dy.alloc((size_t)n * d, s));
+    const int64_t n_pad = dense_rows_padded(n);
+    DBuf<__nv_bfloat16> xb;
+    APS_TRY(xb.alloc((size_t)(n_pad * d), s));
+    DenseRows rows;
+    APS_CUDA(cudaEventCreate(&rows.began));
+    APS_CUDA(cudaEventRecord(rows.began, s));
+    rows.xb = xb.p;
+    if (n_pad > n)
+        APS_CUDA(cudaMemsetAsync(xb.p + (int64_t)n * d, 0, sizeof(__nv_bfloat16) * (size_t)((n_pad - n) * d), s));
     if (n > 0) {
-        k_dense_rows<<<grid_for((int64_t)n * 32, 256, 65536), 256, 0, s>>>(Xd, n, d, norm ? 1 : 0, dy.p, bad.p);
+        k_dense_rows<<<grid_for((int64_t)n * 32, 256, 65536), 256, 0, s>>>(Xd, n, d, norm ? 1 : 0, dy.p, xb.p, bad.p);
         APS_LAUNCH_CHECK();
     }
     unsigned long long b = 0;
@@ -891,7 +993,7 @@ aps_status dense_all_pairs(const float *X, int32_t n, int32_t d, float t, uint32
                   b);
         return APS_EINVAL;
     }
-    return dense_all_pairs_device(norm ? dy.p : Xd, n, d, t, s, out, stats, nullptr);
+    return dense_all_pairs_device(norm ? dy.p : Xd, n, d, t, s, out, stats, nullptr, &rows);
 }
 
 // The tensor cores' float32 products S = X_bf16 . X_bf16^T of the dense path (rows as they
@@ -900,7 +1002,7 @@ aps_status dense_all_pairs(const float *X, int32_t n, int32_t d, float t, uint32
 aps_status dense_tensor_products(const float *X, int32_t n, int32_t d, cudaStream_t s, float *raw) {
     aps_pairs none;
     memset(&none, 0, sizeof(none));
-    return dense_all_pairs_device(X, n, d, 0.f, s, &none, nullptr, raw);
+    return dense_all_pairs_device(X, n, d, 0.f, s, &none, nullptr, raw, nullptr);
 }
 
 }  // namespace aps

@@ -238,8 +238,20 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
 // tensor cores with exact rescoring; d % 64 == 0, 64 <= d <= 512.
 aps_status dense_all_pairs(const float *X, int32_t n, int32_t d, float t, uint32_t flags, cudaStream_t s,
                            aps_pairs *out, aps_stats *stats);
+// The BF16 rows (zero rows up to the padded count) that the validation of X has already made, and
+// when it began.
+struct DenseRows {
+    void *xb = nullptr;
+    cudaEvent_t began = nullptr;
+    DenseRows() = default;
+    DenseRows(const DenseRows &) = delete;
+    DenseRows &operator=(const DenseRows &) = delete;
+    ~DenseRows() {
+        if (began) cudaEventDestroy(began);
+    }
+};
 aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t, cudaStream_t s, aps_pairs *out,
-                                  aps_stats *stats, float *raw);
+                                  aps_stats *stats, float *raw, const DenseRows *rows);
 // The tensor cores' float32 products X_bf16 . X_bf16^T of the computed (upper) blocks into
 // raw (row-major n x n, device memory); X on the device.
 aps_status dense_tensor_products(const float *X, int32_t n, int32_t d, cudaStream_t s, float *raw);
