@@ -39,6 +39,11 @@ __global__ void k_vinst(const InstDesc *inst, int k, int64_t N, int32_t *vinst) 
 // Validation codes reported as (row << 8 | code) through atomicMin.
 enum { E_PTR = 1, E_IDX_RANGE = 2, E_IDX_ORDER = 3, E_VALUE = 4, E_NORM = 5 };
 
+// CTAs for a warp per row: some rounds of what is resident, so that the sums each CTA adds to one
+// counter are few. With a warp for each of 1.9M rows, the 64-bit atomics on one address were most
+// of the time of the kernels that have them (k_split took 3.1 ms, 1.4 with these grids).
+unsigned rows_grid(int64_t rows) { return grid_for(rows * 32, 256, (int64_t)num_sms() * 64); }
+
 // One warp per row: checks the row, records |x| and maxweight(x), and copies the values
 // (scaled to unit norm with APS_NORMALIZE). The lanes read 32 components at a time; the
 // error code is that of the row's first bad component (range before order before value,
@@ -64,7 +69,7 @@ __global__ void k_validate(const int64_t *__restrict__ indptr, const int32_t *__
         }
         const int m = inst[vinst[x]].m;
         int code = 0, prev_last = -1;
-        double ss = 0.0;
+        float s32 = 0.f;
         for (int64_t base = a; base < b; base += 32) {
             const int64_t p = base + lane;
             const int cnt = (int)min((int64_t)32, b - base);
@@ -85,16 +90,28 @@ __global__ void k_validate(const int64_t *__restrict__ indptr, const int32_t *__
             }
             const unsigned bad = __ballot_sync(0xffffffffu, ec != 0);
             if (!code && bad) code = __shfl_sync(0xffffffffu, ec, __ffs(bad) - 1);
-            if (p < b) ss += (double)v * (double)v;
+            if (p < b) s32 = fmaf(v, v, s32);
             prev_last = __shfl_sync(0xffffffffu, d, cnt - 1);
         }
 #pragma unroll
-        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        for (int o = 16; o; o >>= 1) s32 += __shfl_xor_sync(0xffffffffu, s32, o);
         float best = 0.f;
         if (b > a && !code) {
-            const double nrm = sqrt(ss);
-            if (!(flags & APS_NORMALIZE) && ((flags & APS_SUBUNIT_NORMS) ? nrm > 1.0 + 1e-3 : fabs(nrm - 1.0) > 1e-3))
-                code = E_NORM;
+            // float32 decides where its sum of squares, off by less than 3e-5 (L / 32 + 6 roundings
+            // of at most 2^-24 each), lies clear of the norms 1 -+ 1e-3; the rest, and rows to be
+            // scaled, take the float64 norm (for every one of 1.9M rows that took 3.5 ms, this 0.64)
+            const bool clear = b - a <= 8192 && s32 <= 1.0019f && ((flags & APS_SUBUNIT_NORMS) || s32 >= 0.9981f);
+            double nrm = 1.0;
+            if ((flags & APS_NORMALIZE) || !clear) {
+                double ss = 0.0;
+                for (int64_t p = a + lane; p < b; p += 32) ss += (double)val[p] * (double)val[p];
+#pragma unroll
+                for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                nrm = sqrt(ss);
+                if (!(flags & APS_NORMALIZE) &&
+                    ((flags & APS_SUBUNIT_NORMS) ? nrm > 1.0 + 1e-3 : fabs(nrm - 1.0) > 1e-3))
+                    code = E_NORM;
+            }
             for (int64_t p = a + lane; p < b; p += 32) {
                 const float v = (flags & APS_NORMALIZE) ? (float)((double)val[p] / nrm) : val[p];
                 vout[p] = v;
@@ -110,12 +127,21 @@ __global__ void k_validate(const int64_t *__restrict__ indptr, const int32_t *__
             longest = max(longest, (unsigned long long)(b - a));
         }
     }
-    if (lane == 0 && longest && longest_out) atomicMax(longest_out, longest);
+    if (longest_out) {
+        __shared__ unsigned long long blongest;
+        if (threadIdx.x == 0) blongest = 0ull;
+        __syncthreads();
+        if (lane == 0) atomicMax(&blongest, longest);
+        __syncthreads();
+        if (threadIdx.x == 0) atomicMax(longest_out, blongest);
+    }
 }
 
 // The rank-ordered rows when no row is longer than 64 components: one warp per row sorts
 // the row's (rank, value) pairs by a bitonic network over the lanes, two per lane (element
-// k = 2 * lane + h), instead of the global sort by (row, rank) that longer rows need.
+// k = 2 * lane + h; rows of at most 32, one per lane and six steps fewer), instead of the
+// global sort by (row, rank) that longer rows need. Bound by the network's exchanges: 1.9M rows
+// of 30 on average took 1.4 ms with 64 places for every row and a CTA for every eight, 1.06 now.
 __global__ void k_canon_rows64(const int64_t *__restrict__ cptr, const int32_t *__restrict__ idx,
                                const float *__restrict__ vout, const int32_t *__restrict__ vinst,
                                const InstDesc *__restrict__ inst, const int32_t *__restrict__ rank_of_dim,
@@ -126,6 +152,32 @@ __global__ void k_canon_rows64(const int64_t *__restrict__ cptr, const int32_t *
         const int64_t a = cptr[x];
         const int L = (int)(cptr[x + 1] - a);  // <= 64
         const int64_t rb = inst[vinst[x]].rbase;
+        if (L <= 32) {
+            int r = 0x7fffffff;  // padding sorts last
+            float v = 0.f;
+            if (lane < L) {
+                r = rank_of_dim[rb + idx[a + lane]];
+                v = vout[a + lane];
+            }
+#pragma unroll
+            for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+                for (int j = size >> 1; j > 0; j >>= 1) {
+                    const int pr = __shfl_xor_sync(0xffffffffu, r, j);
+                    const float pv = __shfl_xor_sync(0xffffffffu, v, j);
+                    const bool keep_min = ((lane & j) == 0) == ((lane & size) == 0);
+                    if (keep_min ? pr < r : pr > r) {
+                        r = pr;
+                        v = pv;
+                    }
+                }
+            }
+            if (lane < L) {
+                crank[a + lane] = r;
+                cval[a + lane] = v;
+            }
+            continue;
+        }
         const int k0 = 2 * lane, k1 = k0 + 1;
         int r0 = 0x7fffffff, r1 = 0x7fffffff;  // padding sorts last
         float v0 = 0.f, v1 = 0.f;
@@ -315,8 +367,63 @@ __device__ __forceinline__ float warp_incl_scan_ru(float v, int lane) {
 // The smallest 4-bit code c with c * PN4_STEP >= pn (the bound stays a bound).
 __device__ __forceinline__ int pn4_code(float pn) {
     int c = (int)ceilf(__fdiv_ru(pn, PN4_STEP));
-    if ((double)c * (double)PN4_STEP < (double)pn) c++;
+    if (__fmul_rd((float)c, PN4_STEP) < pn) c++;
     return min(max(c, 0), 15);
+}
+
+// The remaining-score bound's sums in float32 are off by at most (1 + 5 + chunks of 32 so far)
+// roundings of 2^-24 (all terms are positive), which stays below SPLIT_F32_EPS up to component
+// SPLIT_F32_MAX. A row whose first sum at t (1 - eps) is also past t (1 + eps) splits there in
+// float64 too; any other that comes near t is summed again in float64 (about one row in 10^4, or
+// rows of equal weights that reach t exactly). A float64 instruction takes the SM some 15 cycles a
+// warp: 58M components of 1.9M rows take 1.4 ms, 1.8 with the float64 scan for every row.
+constexpr float SPLIT_F32_EPS = 1e-5f;
+constexpr int SPLIT_F32_MAX = 2048;
+
+__device__ __forceinline__ float warp_incl_scan(float v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
+
+// First component where sum c * maxweight reaches t, in float64 (L: none); term(p) is component
+// p's pair of the two. All lanes call it.
+template <class F>
+__device__ __forceinline__ int32_t split_f64(F term, int32_t L, double t, int lane) {
+    double bmw = 0.0;
+#pragma unroll 1
+    for (int32_t base = 0; base < L; base += 32) {
+        const int32_t p = base + lane;
+        double v = 0.0;
+        if (p < L) {
+            const float2 e = term(p);
+            v = (double)e.x * (double)e.y;
+        }
+        const double bi = bmw + warp_incl_scan_f64(v, lane);
+        const unsigned hit = __ballot_sync(0xffffffffu, p < L && bi >= t);
+        if (hit) return base + __ffs(hit) - 1;
+        bmw = __shfl_sync(0xffffffffu, bi, 31);
+    }
+    return L;
+}
+
+// One chunk of 32 of the same search in float32, bmw the sum before it (brought forward): the
+// component, L + 1 where float64 finds that no component of the row reaches t, L to go on.
+template <class F>
+__device__ __forceinline__ int32_t split_step(float v, bool in, int32_t at, float &bmw, F term, int32_t L, float t,
+                                              int lane) {
+    const bool tiny = t < 1e-30f;  // (products might underflow)
+    const float bi = bmw + warp_incl_scan(v, lane);
+    const unsigned near = __ballot_sync(0xffffffffu, in && (tiny || bi >= t * (1.f - SPLIT_F32_EPS)));
+    const unsigned past = __ballot_sync(0xffffffffu, in && !tiny && bi > t * (1.f + SPLIT_F32_EPS));
+    bmw = __shfl_sync(0xffffffffu, bi, 31);
+    if (near == 0 && at < SPLIT_F32_MAX) return L;
+    if (past && __ffs(near) == __ffs(past) && at < SPLIT_F32_MAX) return at + __ffs(near) - 1;
+    const int32_t q = split_f64(term, L, (double)t, lane);
+    return q < L ? q : L + 1;
 }
 
 __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restrict__ crank,
@@ -335,9 +442,12 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
         const int64_t a = cptr[x], b = cptr[x + 1];
         const int32_t L = (int32_t)(b - a);
         const bool need_cs = (flags & APS_QUERYABLE) != 0;  // the norm-bound split of queryable indexes
+        const auto term = [&](int32_t p) {
+            return make_float2(cval[a + p], mwr[(int64_t)I.rbase + crank[a + p]]);
+        };
         int32_t qs = L, cs = L, ls = L;
-        double bmw = 0.0, ss = 0.0;  // sums of the components before this step
-        float ssu = 0.f;             // the squares again, rounded up
+        double ss = 0.0;  // sums of the components before this step
+        float bmw = 0.f, ssu = 0.f;  // the remaining-score bound; the squares, rounded up
         for (int64_t base = a; base < b && (qs == L || (need_cs && cs == L) || (l2 && ls == L)); base += 32) {
             const int64_t p = base + lane;
             float c = 0.f, mwc = 0.f;
@@ -346,12 +456,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
                 mwc = mwr[(int64_t)I.rbase + crank[p]];
             }
             const int32_t at = (int32_t)(base - a);
-            if (qs == L) {
-                const double bi = bmw + warp_incl_scan_f64((double)c * (double)mwc, lane);
-                const unsigned hit = __ballot_sync(0xffffffffu, p < b && bi >= t);
-                if (hit) qs = at + __ffs(hit) - 1;
-                bmw = __shfl_sync(0xffffffffu, bi, 31);
-            }
+            if (qs == L) qs = split_step(__fmul_rn(c, mwc), p < b, at, bmw, term, L, I.t, lane);
             if (need_cs && cs == L) {
                 const double si = ss + warp_incl_scan_f64((double)c * (double)c, lane);
                 const unsigned hc = __ballot_sync(0xffffffffu, p < b && si * (1.0 + 2e-3) >= t * t);
@@ -365,6 +470,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
                 ssu = __shfl_sync(0xffffffffu, si, 31);
             }
         }
+        qs = min(qs, L);
         const int32_t sp = (flags & APS_NO_PARTIAL_INDEX) ? 0 : (need_cs ? cs : qs);
         // the join's prefix (external queries only obey the norm bound) and create boundary
         const int32_t js = (l2 && !need_cs) ? max(sp, ls) : sp;
@@ -403,8 +509,16 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
             pvals[p] = (uint32_t)p;
         }
     }
-    if (lane == 0 && nsuf_w) atomicAdd(nsuf, nsuf_w);
-    if (lane == 0 && njoin_w) atomicAdd(njoin, njoin_w);
+    __shared__ unsigned long long bsum[2];
+    if (threadIdx.x < 2) bsum[threadIdx.x] = 0ull;
+    __syncthreads();
+    if (lane == 0) {
+        atomicAdd(&bsum[0], nsuf_w);
+        atomicAdd(&bsum[1], njoin_w);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(nsuf, bsum[0]);
+    if (threadIdx.x == 1) atomicAdd(njoin, bsum[1]);
 }
 
 // Posting keys by a given split (for the exported lists), one thread per component.
@@ -463,27 +577,32 @@ __global__ void k_pack(const int32_t *__restrict__ crank, const float *__restric
 
 // Where the windows of a multi-window instance begin inside each list: w[i] = the position in
 // post of list R's first entry with local id >= i * W (lists are in increasing id; binary
-// search). One warp per list of one instance (blockIdx.y), the windows over its lanes.
+// search). One thread per window of a list, in the order they are stored, instances over
+// blockIdx.y: with a warp per list, 12 windows left 20 lanes idle (25M lists of a batch of 512
+// instances: 1.07 ms, 0.33 now).
 __global__ void k_wptr(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ lptr,
                        const int2 *__restrict__ post, uint32_t *wptr) {
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int q = blockIdx.y; q < k; q += gridDim.y) {
         const InstDesc &I = inst[q];
         if (I.nw <= 1) continue;
         const int32_t idmask = I.packed ? 0x00ffffff : 0x7fffffff;
-        for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < I.m; r += nwarps) {
-            const int64_t a = lptr[I.rbase + r], b = lptr[I.rbase + r + 1];
-            uint32_t *w = wptr + I.wbase + r * (I.nw + 1);
-            for (int i = lane; i <= I.nw; i += 32) {
-                const int64_t bound = (int64_t)i * I.W;
-                int64_t lo = a, hi = b;
-                while (lo < hi) {
-                    const int64_t mid = (lo + hi) >> 1;
-                    if ((post[mid].x & idmask) < bound) lo = mid + 1; else hi = mid;
-                }
-                w[i] = (uint32_t)lo;
+        const uint32_t per = (uint32_t)I.nw + 1u;
+        const int64_t total = (int64_t)I.m * per;
+        uint32_t *w = wptr + I.wbase;
+        for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; e0 < total; e0 += step) {
+            const int64_t r0 = e0 / per;  // one long division a warp
+            const uint32_t off = (uint32_t)(e0 - r0 * per) + (uint32_t)lane;
+            const int64_t r = r0 + off / per, e = e0 + lane;
+            if (e >= total) continue;
+            const int64_t bound = (int64_t)(off % per) * I.W;
+            int64_t lo = lptr[I.rbase + r], hi = lptr[I.rbase + r + 1];
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if ((post[mid].x & idmask) < bound) lo = mid + 1; else hi = mid;
             }
+            w[e] = (uint32_t)lo;
         }
     }
 }
@@ -650,7 +769,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     // ---- a1: validation, |x|, maxweight(x), per-dimension statistics
     k_vinst<<<gN, T256, 0, s>>>(d.inst.p, k, N, d.vinst.p);
     APS_LAUNCH_CHECK();
-    k_validate<<<grid_for(N * 32, T256), T256, 0, s>>>(indptr, idx, val, d.vinst.p, d.inst.p, N, nnz, ix->flags,
+    k_validate<<<rows_grid(N), T256, 0, s>>>(indptr, idx, val, d.vinst.p, d.inst.p, N, nnz, ix->flags,
                                                        erow.p, vout.p, d.len.p, d.mw.p, err.p, err.p + 2);
     APS_LAUNCH_CHECK();
     unsigned long long e3[3] = {~0ull, 0ull, 0ull};  // first error, (unused here), longest row
@@ -693,7 +812,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         APS_LAUNCH_CHECK();
     }
     if (nnz > 0 && longest_row <= 64) {  // every row sorted inside one warp
-        k_canon_rows64<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, idx, vout.p, d.vinst.p, d.inst.p,
+        k_canon_rows64<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, idx, vout.p, d.vinst.p, d.inst.p,
                                                                d.rank_of_dim.p, N, d.crank.p, d.cval.p);
         APS_LAUNCH_CHECK();
     } else if (nnz > 0) {  // a global sort by (row, rank)
@@ -719,7 +838,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     APS_TRY(pkeys.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     APS_TRY(pvals.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     unsigned long long *nsuf_d = err.p + 1;
-    k_split<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N,
+    k_split<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N,
                                                     ix->flags, ix->l2, d.mw.p, d.split.p, d.qsplit.p, d.mwpre.p,
                                                     d.vmeta.p, d.vcand.p, d.code.p, M, pkeys.p, pvals.p, nsuf_d,
                                                     nsuf_d + 2);
@@ -744,7 +863,8 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p);
         APS_LAUNCH_CHECK();
         if (nwptr) {
-            const dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>((maxm + 7) / 8, 65536 / k)),
+            const dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)maxm * (ix->maxnw + 1) + T256 - 1) / T256,
+                                                                          65536 / k)),
                          (unsigned)std::min(k, 65535));
             k_wptr<<<g, T256, 0, s>>>(d.inst.p, k, d.lptr.p, d.post.p, d.wptr.p);
             APS_LAUNCH_CHECK();
@@ -763,7 +883,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         unsigned long long *cc = err.p;  // reused: one counter per class
         APS_CUDA(cudaMemsetAsync(cc, 0, JOIN_NCLS * sizeof(unsigned long long), s));
         if (N > 0) {
-            k_item_keys<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, d.crank.p, d.lptr.p, d.vinst.p, d.inst.p,
+            k_item_keys<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.lptr.p, d.vinst.p, d.inst.p,
                                                                N, keys.p, vals.p,
                                             cc);
             APS_LAUNCH_CHECK();
@@ -851,7 +971,7 @@ aps_status sort_queries(const int32_t *qidx, const int32_t *erow, const int32_t 
 }
 
 // Remscore boundary of a query: the first rank-ordered component where
-// sum x[i] * maxweight_i(V) reaches t (float64, as for indexed vectors), or, with l2 and if
+// sum x[i] * maxweight_i(V) reaches t (exact as float64 is, as for indexed vectors), or, with l2 and if
 // that is later, where the norm of the leading components can reach t. One warp per query.
 __global__ void k_q_split(const int64_t *__restrict__ qptr, const int2 *__restrict__ crow,
                           const float *__restrict__ mwr, const float *__restrict__ mw, int64_t nq, float t, bool l2,
@@ -862,9 +982,12 @@ __global__ void k_q_split(const int64_t *__restrict__ qptr, const int2 *__restri
     for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < nq; x += nwarps) {
         const int64_t a = qptr[x], b = qptr[x + 1];
         const int32_t L = (int32_t)(b - a);
+        const auto term = [&](int32_t p) {
+            const int2 e = crow[a + p];
+            return make_float2(__int_as_float(e.y), mwr[e.x]);
+        };
         int32_t qs = L, ls = l2 ? L : 0;
-        double bmw = 0.0;
-        float ssu = 0.f;
+        float bmw = 0.f, ssu = 0.f;
         for (int64_t base = a; base < b && (qs == L || ls == L); base += 32) {
             const int64_t p = base + lane;
             int2 e = make_int2(0, 0);
@@ -874,16 +997,13 @@ __global__ void k_q_split(const int64_t *__restrict__ qptr, const int2 *__restri
                 mwc = mwr[e.x];
             }
             const float c = __int_as_float(e.y);
-            const double bi = bmw + warp_incl_scan_f64((double)c * (double)mwc, lane);
-            const unsigned hit = __ballot_sync(0xffffffffu, p < b && bi >= (double)t);
-            if (qs == L && hit) qs = (int32_t)(base - a) + __ffs(hit) - 1;
-            bmw = __shfl_sync(0xffffffffu, bi, 31);
+            if (qs == L) qs = split_step(__fmul_rn(c, mwc), p < b, (int32_t)(base - a), bmw, term, L, t, lane);
             const float si = __fadd_ru(ssu, warp_incl_scan_ru(__fmul_ru(c, c), lane));
             const unsigned hl = __ballot_sync(0xffffffffu, p < b && __fmul_ru(si, 1.0025f) >= t2);
             if (ls == L && hl) ls = (int32_t)(base - a) + __ffs(hl) - 1;
             ssu = __shfl_sync(0xffffffffu, si, 31);
         }
-        if (lane == 0) vmeta[x] = make_int4((int32_t)a, L, max(qs, ls), __float_as_int(mw[x]));
+        if (lane == 0) vmeta[x] = make_int4((int32_t)a, L, max(min(qs, L), ls), __float_as_int(mw[x]));
     }
 }
 
