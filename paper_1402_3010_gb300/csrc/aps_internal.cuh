@@ -54,6 +54,7 @@ struct DBuf {
     T *p = nullptr;
     size_t n = 0;
     cudaStream_t s = nullptr;
+    bool own = true;  // false: part of another allocation, which outlives this
     DBuf() = default;
     DBuf(const DBuf &) = delete;
     DBuf &operator=(const DBuf &) = delete;
@@ -62,10 +63,18 @@ struct DBuf {
         release();
         s = stream;
         n = count;
+        own = true;
         return dalloc(reinterpret_cast<void **>(&p), (count ? count : 1) * sizeof(T), stream);
     }
+    void view(T *q, size_t count, cudaStream_t stream) {
+        release();
+        p = q;
+        n = count;
+        s = stream;
+        own = false;
+    }
     void release() {
-        if (p) dfree(p, s);
+        if (p && own) dfree(p, s);
         p = nullptr;
         n = 0;
     }
@@ -74,6 +83,19 @@ struct DBuf {
         p = nullptr;
         n = 0;
         return q;
+    }
+};
+
+// Places arrays one after another (256-byte aligned) in one allocation: with base null the sizes
+// are added up, then the same calls on the allocation set the arrays.
+struct Carver {
+    char *base = nullptr;
+    size_t off = 0;
+    cudaStream_t s = nullptr;
+    template <class T>
+    void put(DBuf<T> &b, size_t count) {
+        if (base) b.view(reinterpret_cast<T *>(base + off), count, s);
+        off += ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
     }
 };
 

@@ -796,9 +796,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     APS_TRY(dunits.alloc(units.size(), s));
     APS_CUDA(cudaMemcpyAsync(dunits.p, units.data(), sizeof(int4) * units.size(), cudaMemcpyHostToDevice, s));
     DBuf<unsigned long long> ctr;
-    DBuf<int> err;
-    APS_TRY(ctr.alloc(4, s));
-    APS_TRY(err.alloc(1, s));
+    APS_TRY(ctr.alloc(4, s));  // candidates, (rescored in float64: below), padding, error code
     constexpr int SMEM_MAX = SMEM_BUDGET + 1024 + 512;
     APS_CUDA(cudaFuncSetAttribute(dense_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX));
     const double delta = dense_margin(d);
@@ -829,7 +827,6 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     for (int attempt = 0; attempt < 2; attempt++) {
         APS_TRY(cand.alloc((size_t)cap, s));
         APS_CUDA(cudaMemsetAsync(ctr.p, 0, 4 * sizeof(unsigned long long), s));
-        APS_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
         DenseParams P;
         P.n = n;
         P.KB = KB;
@@ -841,7 +838,7 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
         P.cap = (unsigned long long)cap;
         P.count = ctr.p;
         P.padded = ctr.p + 2;
-        P.err = err.p;
+        P.err = reinterpret_cast<int *>(ctr.p + 3);
         P.wait_ns = WAIT_NS_DEFAULT;
         P.stall = 0;
         P.raw = raw;
@@ -868,11 +865,11 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
         APS_CUDA(cudaLaunchKernelEx(&cfg, dense_gemm_kernel, map, P));
         count_launch();
         APS_CUDA(cudaEventRecord(ev[2], s));
-        unsigned long long cnt[3] = {0, 0, 0};
-        int e_h = 0;
+        unsigned long long cnt[4] = {0, 0, 0, 0};
         APS_CUDA(cudaMemcpyAsync(cnt, ctr.p, sizeof(cnt), cudaMemcpyDeviceToHost, s));
-        APS_CUDA(cudaMemcpyAsync(&e_h, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
+        int e_h = 0;
+        memcpy(&e_h, &cnt[3], sizeof(e_h));
         if (e_h) {
             set_error("dense tensor-core kernel: a pipeline wait timed out (code %d)", e_h);
             return APS_ETIMEOUT;
@@ -898,20 +895,20 @@ aps_status dense_all_pairs_device(const float *X, int32_t n, int32_t d, float t,
     DBuf<int64_t> pos;
     APS_TRY(keep.alloc((size_t)std::max<int64_t>(nc, 1), s));
     APS_TRY(sc.alloc((size_t)std::max<int64_t>(nc, 1), s));
-    APS_TRY(pos.alloc((size_t)nc + 1, s));
+    APS_TRY(pos.alloc((size_t)nc + 2, s));  // and, after the total, the candidates rescored in float64
+    APS_CUDA(cudaMemsetAsync(pos.p + nc + 1, 0, sizeof(int64_t), s));
     const float beta = (float)std::max(1e-5, (d / 32.0 + 8.0) * std::ldexp(1.0, -23));
     if (nc > 0) {
         const unsigned g = grid_for((nc + RS_MIN - 1) / RS_MIN * 32, 256, (int64_t)num_sms() * 64);
         const auto rescore = d <= 128 ? k_rescore<1> : d <= 256 ? k_rescore<2> : d <= 384 ? k_rescore<3> : k_rescore<4>;
-        rescore<<<g, 256, 0, s>>>(sorted, nc, X, n, d, t, beta, keep.p, sc.p, ctr.p + 1);
+        rescore<<<g, 256, 0, s>>>(sorted, nc, X, n, d, t, beta, keep.p, sc.p, reinterpret_cast<unsigned long long *>(pos.p + nc + 1));
         APS_LAUNCH_CHECK();
     }
     APS_TRY(scan_exclusive(keep.p, pos.p, nc, s));
-    int64_t npairs = 0;
-    unsigned long long nband = 0;
-    APS_CUDA(cudaMemcpyAsync(&npairs, pos.p + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    APS_CUDA(cudaMemcpyAsync(&nband, ctr.p + 1, sizeof(nband), cudaMemcpyDeviceToHost, s));
+    int64_t last[2] = {0, 0};
+    APS_CUDA(cudaMemcpyAsync(last, pos.p + nc, sizeof(last), cudaMemcpyDeviceToHost, s));
     APS_CUDA(cudaStreamSynchronize(s));
+    const int64_t npairs = last[0], nband = last[1];
     PairsAlloc *pa = new PairsAlloc();
     pa->stream = s;
     const size_t seg = ((size_t)npairs * 4 + 127) & ~(size_t)127;

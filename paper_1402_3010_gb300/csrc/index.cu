@@ -31,9 +31,23 @@ __device__ __forceinline__ int inst_of_rank(const InstDesc *inst, int k, int64_t
     return lo - 1;
 }
 
-__global__ void k_vinst(const InstDesc *inst, int k, int64_t N, int32_t *vinst) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < N; x += (int64_t)gridDim.x * blockDim.x)
-        vinst[x] = inst_of_vec(inst, k, x);
+// The start of a build in one launch: the row pointers' copy, every vector's instance, empty
+// dimension statistics and counters (err[0] all ones, the others 0) and, for a single instance,
+// its description (by value: no copy from the host). A copy or a reset of its own costs its
+// caller 3 to 15 us, a tenth of the smallest builds in all.
+__global__ void k_setup(const int64_t *__restrict__ indptr, InstDesc one, InstDesc *inst, int k, int64_t N, int64_t M,
+                        int64_t *cptr, int32_t *vinst, int32_t *nnz_d, float *mw_d, unsigned long long *err, int nerr) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (k == 1 && i0 == 0) inst[0] = one;
+    if (i0 < nerr) err[i0] = i0 == 0 ? ~0ull : 0ull;
+    for (int64_t x = i0; x <= N; x += step) {
+        cptr[x] = indptr[x];
+        if (x < N) vinst[x] = k == 1 ? 0 : inst_of_vec(inst, k, x);
+    }
+    for (int64_t d = i0; d < M; d += step) {
+        nnz_d[d] = 0;
+        mw_d[d] = 0.f;
+    }
 }
 
 // Validation codes reported as (row << 8 | code) through atomicMin.
@@ -50,7 +64,7 @@ unsigned rows_grid(int64_t rows) { return grid_for(rows * 32, 256, (int64_t)num_
 // as for a sequential check). The float64 sum of squares is a warp tree sum.
 __global__ void k_validate(const int64_t *__restrict__ indptr, const int32_t *__restrict__ idx,
                            const float *__restrict__ val, const int32_t *__restrict__ vinst,
-                           const InstDesc *__restrict__ inst, int64_t N, int64_t nnz, uint32_t flags,
+                           const InstDesc *__restrict__ inst, int32_t m1, int64_t N, int64_t nnz, uint32_t flags,
                            int32_t *__restrict__ erow, float *__restrict__ vout, int32_t *__restrict__ len,
                            float *__restrict__ mw, unsigned long long *err,
                            unsigned long long *longest_out) {
@@ -67,7 +81,7 @@ __global__ void k_validate(const int64_t *__restrict__ indptr, const int32_t *__
             }
             continue;
         }
-        const int m = inst[vinst[x]].m;
+        const int m = vinst ? inst[vinst[x]].m : m1;
         int code = 0, prev_last = -1;
         float s32 = 0.f;
         for (int64_t base = a; base < b; base += 32) {
@@ -726,51 +740,75 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     ix->inst_h = inst;
     IndexArrays &d = ix->d;
 
-    int64_t nnz = 0;
-    APS_CUDA(cudaMemcpyAsync(&nnz, indptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    int64_t first = 0;
-    APS_CUDA(cudaMemcpyAsync(&first, indptr, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    // the first and the last row pointer, as one strided copy where its pitch may be that wide
+    int64_t ends[2] = {0, 0};
+    if (N >= 1 && N < ((int64_t)1 << 27)) {
+        APS_CUDA(cudaMemcpy2DAsync(ends, sizeof(int64_t), indptr, sizeof(int64_t) * (size_t)N, sizeof(int64_t), 2,
+                                   cudaMemcpyDeviceToHost, s));
+    } else {
+        APS_CUDA(cudaMemcpyAsync(&ends[0], indptr, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        APS_CUDA(cudaMemcpyAsync(&ends[1], indptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    }
     APS_CUDA(cudaStreamSynchronize(s));
+    const int64_t first = ends[0], nnz = ends[1];
     if (first != 0 || nnz < 0 || nnz >= (1ll << 31)) {
         set_error("indptr[0] must be 0 and nnz in [0, 2^31); got indptr[0]=%lld nnz=%lld",
                   (long long)first, (long long)nnz);
         return APS_EINVAL;
     }
     ix->nnz = nnz;
-    APS_TRY(d.inst.alloc((size_t)k, s));
-    APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
-    APS_TRY(d.vinst.alloc((size_t)N, s));
-    APS_TRY(d.cptr.alloc((size_t)N + 1, s));
-    APS_CUDA(cudaMemcpyAsync(d.cptr.p, indptr, sizeof(int64_t) * (N + 1), cudaMemcpyDeviceToDevice, s));
-    APS_TRY(d.len.alloc((size_t)N, s));
-    APS_TRY(d.mw.alloc((size_t)N, s));
-    APS_TRY(d.split.alloc((size_t)N, s));
-    APS_TRY(d.qsplit.alloc((size_t)N, s));
-    APS_TRY(d.mwpre.alloc((size_t)N, s));
-    APS_TRY(d.crank.alloc((size_t)nnz, s));
-    APS_TRY(d.cval.alloc((size_t)nnz, s));
-    APS_TRY(d.nnz_d.alloc((size_t)M, s));
-    APS_TRY(d.mw_d.alloc((size_t)M, s));
-    APS_TRY(d.mwr.alloc((size_t)M, s));
-    APS_TRY(d.rank_of_dim.alloc((size_t)M, s));
-    APS_TRY(d.dim_of_rank.alloc((size_t)M, s));
-    APS_TRY(d.lptr.alloc((size_t)M + 1, s));
-
+    Carver cv;
+    cv.s = s;
+    for (int pass = 0; pass < 2; pass++) {
+        cv.off = 0;
+        cv.put(d.inst, (size_t)k);
+        cv.put(d.vinst, (size_t)N);
+        cv.put(d.cptr, (size_t)N + 1);
+        cv.put(d.len, (size_t)N);
+        cv.put(d.mw, (size_t)N);
+        cv.put(d.split, (size_t)N);
+        cv.put(d.qsplit, (size_t)N);
+        cv.put(d.mwpre, (size_t)N);
+        cv.put(d.crank, (size_t)nnz);
+        cv.put(d.cval, (size_t)nnz);
+        cv.put(d.nnz_d, (size_t)M);
+        cv.put(d.mw_d, (size_t)M);
+        cv.put(d.mwr, (size_t)M);
+        cv.put(d.rank_of_dim, (size_t)M);
+        cv.put(d.dim_of_rank, (size_t)M);
+        cv.put(d.lptr, (size_t)M + 1);
+        cv.put(d.vmeta, (size_t)N);
+        cv.put(d.vcand, (size_t)N);
+        cv.put(d.code, (size_t)N);
+        if (pass == 0) {
+            APS_TRY(d.block.alloc(cv.off, s));
+            cv.base = d.block.p;
+        }
+    }
+    DBuf<char> tblock;
     DBuf<int32_t> erow;
     DBuf<float> vout;
-    DBuf<unsigned long long> err;
-    APS_TRY(erow.alloc((size_t)nnz, s));
-    APS_TRY(vout.alloc((size_t)nnz, s));
-    APS_TRY(err.alloc(JOIN_NCLS, s));
-    APS_CUDA(cudaMemsetAsync(err.p, 0xff, sizeof(unsigned long long), s));
-    APS_CUDA(cudaMemsetAsync(err.p + 1, 0, 3 * sizeof(unsigned long long), s));
+    DBuf<unsigned long long> err;  // {first bad row, components indexed by split, longest row, in the join's lists}, classes
+    cv.base = nullptr;
+    for (int pass = 0; pass < 2; pass++) {
+        cv.off = 0;
+        cv.put(erow, (size_t)nnz);
+        cv.put(vout, (size_t)nnz);
+        cv.put(err, 4 + JOIN_NCLS);
+        if (pass == 0) {
+            APS_TRY(tblock.alloc(cv.off, s));
+            cv.base = tblock.p;
+        }
+    }
+    if (k > 1) APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
 
-    const unsigned gN = grid_for(N, T256), gE = grid_for(nnz, T256), gM = grid_for(M, T256);
+    const unsigned gE = grid_for(nnz, T256), gM = grid_for(M, T256);
     // ---- a1: validation, |x|, maxweight(x), per-dimension statistics
-    k_vinst<<<gN, T256, 0, s>>>(d.inst.p, k, N, d.vinst.p);
+    k_setup<<<grid_for(std::max<int64_t>(N + 1, M), T256), T256, 0, s>>>(
+        indptr, inst[0], d.inst.p, k, N, M, d.cptr.p, d.vinst.p, d.nnz_d.p, d.mw_d.p, err.p, 4 + JOIN_NCLS);
     APS_LAUNCH_CHECK();
-    k_validate<<<rows_grid(N), T256, 0, s>>>(indptr, idx, val, d.vinst.p, d.inst.p, N, nnz, ix->flags,
-                                                       erow.p, vout.p, d.len.p, d.mw.p, err.p, err.p + 2);
+    k_validate<<<rows_grid(N), T256, 0, s>>>(indptr, idx, val, d.vinst.p, d.inst.p, 0, N, nnz, ix->flags, erow.p,
+                                             vout.p, d.len.p, d.mw.p, err.p, err.p + 2);
     APS_LAUNCH_CHECK();
     unsigned long long e3[3] = {~0ull, 0ull, 0ull};  // first error, (unused here), longest row
     APS_CUDA(cudaMemcpyAsync(e3, err.p, sizeof(e3), cudaMemcpyDeviceToHost, s));
@@ -789,8 +827,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
             set_error("invalid input at row %lld: %s", row, code_name(code));
         return APS_EINVAL;
     }
-    APS_CUDA(cudaMemsetAsync(d.nnz_d.p, 0, sizeof(int32_t) * M, s));
-    APS_CUDA(cudaMemsetAsync(d.mw_d.p, 0, sizeof(float) * M, s));
     if (nnz > 0 && k > 1 && maxm <= DIMSTATS_DIMS) {  // a batch of small instances: one CTA each
         const int sm = (int)(sizeof(uint32_t) * (size_t)maxm);
         APS_CUDA(cudaFuncSetAttribute(k_dimstats_inst, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
@@ -829,9 +865,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         APS_LAUNCH_CHECK();
     }
     // ---- a3: partial-indexing split
-    APS_TRY(d.vmeta.alloc((size_t)std::max<int64_t>(N, 1), s));
-    APS_TRY(d.vcand.alloc((size_t)std::max<int64_t>(N, 1), s));
-    APS_TRY(d.code.alloc((size_t)std::max<int64_t>(N, 1), s));
     // the split also writes each row's posting keys for a4 (and counts the indexed components)
     DBuf<uint32_t> pkeys;
     DBuf<uint32_t> pvals;
@@ -880,8 +913,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         DBuf<uint32_t> keys, vals;
         APS_TRY(keys.alloc((size_t)std::max<int64_t>(N, 1), s));
         APS_TRY(vals.alloc((size_t)std::max<int64_t>(N, 1), s));
-        unsigned long long *cc = err.p;  // reused: one counter per class
-        APS_CUDA(cudaMemsetAsync(cc, 0, JOIN_NCLS * sizeof(unsigned long long), s));
+        unsigned long long *cc = err.p + 4;  // one counter per class
         if (N > 0) {
             k_item_keys<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.lptr.p, d.vinst.p, d.inst.p,
                                                                N, keys.p, vals.p,
@@ -1024,18 +1056,9 @@ aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32
     }
     qa.nq = nq;
     qa.nnz = nnz;
-    // the index's single instance describes the dimension space
-    InstDesc qd = ix->inst_h[0];
-    qd.vbase = 0;
-    qd.n = nq;
-    DBuf<InstDesc> dinst;
-    DBuf<int32_t> vinst, erow, len;
+    DBuf<int32_t> erow, len;
     DBuf<float> vout;
     DBuf<unsigned long long> err;
-    APS_TRY(dinst.alloc(1, s));
-    APS_CUDA(cudaMemcpyAsync(dinst.p, &qd, sizeof(InstDesc), cudaMemcpyHostToDevice, s));
-    APS_TRY(vinst.alloc((size_t)std::max<int64_t>(nq, 1), s));
-    APS_CUDA(cudaMemsetAsync(vinst.p, 0, sizeof(int32_t) * std::max<int64_t>(nq, 1), s));
     APS_TRY(erow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     APS_TRY(vout.alloc((size_t)std::max<int64_t>(nnz, 1), s));
     APS_TRY(len.alloc((size_t)std::max<int64_t>(nq, 1), s));
@@ -1043,9 +1066,9 @@ aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32
     APS_TRY(err.alloc(1, s));
     APS_CUDA(cudaMemsetAsync(err.p, 0xff, sizeof(unsigned long long), s));
     if (nq > 0) {
-        k_validate<<<grid_for((int64_t)nq * 32, T256), T256, 0, s>>>(qptr, qidx, qval, vinst.p, dinst.p, nq, nnz,
-                                                                     flags, erow.p, vout.p, len.p, qa.mw.p, err.p,
-                                                                     nullptr);
+        // (the index's single instance gives the dimension space)
+        k_validate<<<rows_grid(nq), T256, 0, s>>>(qptr, qidx, qval, nullptr, nullptr, ix->inst_h[0].m, nq, nnz, flags,
+                                                  erow.p, vout.p, len.p, qa.mw.p, err.p, nullptr);
         APS_LAUNCH_CHECK();
     }
     unsigned long long e_h = ~0ull;
@@ -1067,7 +1090,7 @@ aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32
     APS_TRY(qa.vmeta.alloc((size_t)std::max<int64_t>(nq, 1), s));
     if (nq > 0) {
         const bool l2 = !(flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
-        k_q_split<<<grid_for((int64_t)nq * 32, T256), T256, 0, s>>>(qptr, qa.crow.p, d.mwr.p, qa.mw.p, nq, t, l2,
+        k_q_split<<<rows_grid(nq), T256, 0, s>>>(qptr, qa.crow.p, d.mwr.p, qa.mw.p, nq, t, l2,
                                                                     qa.vmeta.p);
         APS_LAUNCH_CHECK();
     }

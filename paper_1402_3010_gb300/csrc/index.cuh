@@ -95,6 +95,7 @@ struct Segment {
 };
 
 struct IndexArrays {
+    DBuf<char> block;  // the arrays of known size, from inst to code
     DBuf<InstDesc> inst;
     DBuf<int32_t> vinst;  // instance of each vector
     DBuf<int64_t> cptr;

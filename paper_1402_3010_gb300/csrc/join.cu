@@ -1612,8 +1612,9 @@ aps_status pairs_to_host(aps_pairs *p, cudaStream_t s) {
     PairsAlloc *pa = new PairsAlloc();
     pa->on_device = 0;
     pa->stream = s;
-    const size_t n = (size_t)p->count;
-    pa->bytes = std::max<size_t>(n, 1) * 12;
+    // the three arrays as they lie on the device, so that one copy takes a few pairs over
+    const size_t n = (size_t)p->count, seg = (n * 4 + 127) & ~(size_t)127;
+    pa->bytes = std::max<size_t>(2 * seg + n * 4, 12);
     aps_status hst = halloc(&pa->block, pa->bytes);
     if (hst != APS_OK) {
         delete pa;
@@ -1621,9 +1622,12 @@ aps_status pairs_to_host(aps_pairs *p, cudaStream_t s) {
     }
     char *blk = static_cast<char *>(pa->block);
     int32_t *hi = reinterpret_cast<int32_t *>(blk);
-    int32_t *hj = reinterpret_cast<int32_t *>(blk + n * 4);
-    float *hs = reinterpret_cast<float *>(blk + n * 8);
-    if (n) {
+    int32_t *hj = reinterpret_cast<int32_t *>(blk + seg);
+    float *hs = reinterpret_cast<float *>(blk + 2 * seg);
+    const char *di = reinterpret_cast<const char *>(p->i);
+    if (n && reinterpret_cast<const char *>(p->j) == di + seg && reinterpret_cast<const char *>(p->score) == di + 2 * seg) {
+        APS_CUDA(cudaMemcpyAsync(hi, di, 2 * seg + n * 4, cudaMemcpyDeviceToHost, s));
+    } else if (n) {
         APS_CUDA(cudaMemcpyAsync(hi, p->i, n * 4, cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaMemcpyAsync(hj, p->j, n * 4, cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaMemcpyAsync(hs, p->score, n * 4, cudaMemcpyDeviceToHost, s));
@@ -1805,12 +1809,11 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     } evg{ev};
     const int64_t nitems = I.nw > 0 ? nq : 0;
     const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(nitems * parts, 1));
-    DBuf<int32_t> cntq;
-    DBuf<unsigned long long> ctr;
+    DBuf<unsigned long long> ctr;  // 16 counters, then the pair counts of the query parts
     DBuf<int2> chain, stage;
     DBuf<Segment> segs;
-    APS_TRY(cntq.alloc((size_t)nqw, s));
-    APS_TRY(ctr.alloc(16, s));
+    APS_TRY(ctr.alloc(16 + ((size_t)nqw + 1) / 2, s));
+    int32_t *const cntq = reinterpret_cast<int32_t *>(ctr.p + 16);
     APS_TRY(segs.alloc((size_t)nqw, s));
     // staging: the pairs per query this index's batches have needed so far (at least 64),
     // plus one slab per warp
@@ -1821,8 +1824,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     for (int attempt = 0; attempt < 2; attempt++) {
         APS_TRY(stage.alloc((size_t)stage_cap, s));
         APS_TRY(chain.alloc((size_t)(stage_cap / slab) + 1, s));
-        APS_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(ch), s));
-        APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * nqw, s));
+        APS_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(ch) + sizeof(int32_t) * nqw, s));
         APS_CUDA(cudaEventRecord(ev[0], s));
         if (nq > 0) {
             JoinParams P;
@@ -1841,7 +1843,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
             P.stage_slab = slab;
             P.segs = segs.p;
             P.chain = chain.p;
-            P.cntq = cntq.p;
+            P.cntq = cntq;
             P.counters = ctr.p;
             P.work = ctr.p + 8;
             P.qcrow = qa.crow.p;
@@ -1869,7 +1871,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     const int64_t npairs = (int64_t)ch[3];
     DBuf<int64_t> qwoff;
     APS_TRY(qwoff.alloc((size_t)nqw + 1, s));
-    APS_TRY(scan_exclusive(cntq.p, qwoff.p, nqw, s));
+    APS_TRY(scan_exclusive(cntq, qwoff.p, nqw, s));
     PairsAlloc *pa = new PairsAlloc();
     pa->stream = s;
     const size_t seg4 = ((size_t)npairs * 4 + 127) & ~(size_t)127;
@@ -1883,7 +1885,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     int32_t *oj = reinterpret_cast<int32_t *>(blk + seg4);
     float *os = reinterpret_cast<float *>(blk + 2 * seg4);
     if (npairs > 0) {
-        k_gather<<<grid_for(nqw * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(segs.p, chain.p, slab, cntq.p, nqw,
+        k_gather<<<grid_for(nqw * 32, 256, (int64_t)sms * 32), 256, 0, s>>>(segs.p, chain.p, slab, cntq, nqw,
                                                                            stage.p, qwoff.p, oi, oj, os);
         APS_LAUNCH_CHECK();
     }

@@ -173,7 +173,7 @@ __global__ void scan_down_kernel(const T *__restrict__ in, int64_t n, const int6
     __syncthreads();
     int64_t wbase = 0;
     for (int w = 0; w < warp; w++) wbase += warp_tot[w];
-    int64_t run = offs[blockIdx.x] + wbase + inc - local;
+    int64_t run = (offs ? offs[blockIdx.x] : 0) + wbase + inc - local;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         int64_t i = base + k;
@@ -191,10 +191,7 @@ aps_status scan_impl(const T *in, int64_t *out, int64_t n, cudaStream_t s) {
     }
     int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     DBuf<int64_t> offs;
-    if (nb == 1) {
-        APS_TRY(offs.alloc(1, s));
-        APS_CUDA(cudaMemsetAsync(offs.p, 0, sizeof(int64_t), s));
-    } else {
+    if (nb > 1) {
         DBuf<int64_t> sums;
         APS_TRY(sums.alloc((size_t)nb, s));
         scan_reduce_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums.p);
@@ -445,25 +442,30 @@ __global__ void __launch_bounds__(SMALL_THREADS) rs_small_kernel(K *keys, uint32
     __shared__ uint32_t wsum[8];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
-    const int first = warp * (32 * SMALL_ITEMS) + lane;
+    // rounds of 32 items a warp takes, and the warps that have any
+    const int per = (n + SMALL_THREADS - 1) / SMALL_THREADS, used = (n + 32 * per - 1) / (32 * per);
+    const int first = warp * (32 * per) + lane;
     K k[SMALL_ITEMS];
     uint32_t v[SMALL_ITEMS], rank[SMALL_ITEMS];
 #pragma unroll
     for (int i = 0; i < SMALL_ITEMS; i++) {
         const int q = first + 32 * i;
-        k[i] = q < n ? keys[q] : (K)0;
-        v[i] = vals && q < n ? vals[q] : 0u;
+        k[i] = i < per && q < n ? keys[q] : (K)0;
+        v[i] = vals && i < per && q < n ? vals[q] : 0u;
     }
     for (int p = 0; p < passes; p++) {
-        for (int i = t; i < SMALL_WARPS * RS_DIGITS; i += SMALL_THREADS) (&whist[0][0])[i] = 0u;
+        for (int i = t; i < used * RS_DIGITS; i += SMALL_THREADS) (&whist[0][0])[i] = 0u;
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < SMALL_ITEMS; i++)
-            rank[i] = warp_rank(whist[warp], digit_of(k[i], 8 * p), first + 32 * i < n, lt_mask);
+        for (int i = 0; i < SMALL_ITEMS; i++) {
+            rank[i] = 0u;
+            if (i < per && warp < used)  // (the same for the whole warp)
+                rank[i] = warp_rank(whist[warp], digit_of(k[i], 8 * p), first + 32 * i < n, lt_mask);
+        }
         __syncthreads();
         uint32_t c = 0, inc = 0;
         if (t < RS_DIGITS) {  // thread t: digit t
-            for (int w = 0; w < SMALL_WARPS; w++) {
+            for (int w = 0; w < used; w++) {
                 const uint32_t x = whist[w][t];
                 whist[w][t] = c;
                 c += x;
@@ -479,12 +481,12 @@ __global__ void __launch_bounds__(SMALL_THREADS) rs_small_kernel(K *keys, uint32
         __syncthreads();
         if (t < RS_DIGITS) {
             for (int w = 0; w < warp; w++) inc += wsum[w];
-            for (int w = 0; w < SMALL_WARPS; w++) whist[w][t] += inc - c;
+            for (int w = 0; w < used; w++) whist[w][t] += inc - c;
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < SMALL_ITEMS; i++) {
-            if (first + 32 * i < n) {
+            if (i < per && first + 32 * i < n) {
                 const uint32_t q = whist[warp][digit_of(k[i], 8 * p)] + rank[i];
                 sk[q] = k[i];
                 sv[q] = v[i];
@@ -494,7 +496,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) rs_small_kernel(K *keys, uint32
 #pragma unroll
         for (int i = 0; i < SMALL_ITEMS; i++) {
             const int q = first + 32 * i;
-            if (q < n) {
+            if (i < per && q < n) {
                 k[i] = sk[q];
                 v[i] = sv[q];
             }
@@ -504,7 +506,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) rs_small_kernel(K *keys, uint32
 #pragma unroll
     for (int i = 0; i < SMALL_ITEMS; i++) {
         const int q = first + 32 * i;
-        if (q < n) {
+        if (i < per && q < n) {
             keys[q] = k[i];
             if (vals) vals[q] = v[i];
         }
@@ -548,9 +550,11 @@ aps_status sort_impl(DBuf<K> &keys, DBuf<uint32_t> *vals, int64_t n, int bits, c
         APS_LAUNCH_CHECK();
         std::swap(keys.p, k2.p);  // (the sorted items are the caller's, whatever the number of passes)
         std::swap(keys.n, k2.n);
+        std::swap(keys.own, k2.own);
         if (VALS) {
             std::swap(vals->p, v2.p);
             std::swap(vals->n, v2.n);
+            std::swap(vals->own, v2.own);
         }
     }
     return APS_OK;
