@@ -217,10 +217,13 @@ aps_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream
 // Stable LSD radix sort, 8 bits a pass. One kernel counts the digits of every pass; a pass is
 // then one kernel that reads each item once and writes it once: a tile ranks its items by warp,
 // publishes its digit counts, adds up the earlier tiles' by looking back over what they have
-// published, and writes its items out in digit runs. 40M keys with a payload take 0.42 ms a pass
-// and 0.12 for the counts, a third of the copy bandwidth (it was 0.50 with a histogram, a scan of
-// three launches and a scatter for each pass); what bounds it is the instructions of the ranking,
-// then the latency of a tile's chain of steps with 32 warps on an SM.
+// published, and writes its items out in digit runs. 40M keys with a payload take 0.37 ms a pass
+// and 0.12 for the counts, some 40% of the copy bandwidth (it was 0.50 with a histogram, a scan of
+// three launches and a scatter for each pass). What bounds it is a tile's chain of steps: its reads,
+// its ranks, the look-back (hundreds of tiles run side by side) and its writes. So the tiles are
+// large (4096 items at three CTAs an SM beat 3072 at four, 0.42 ms, and 2048 at five, 0.43), and the
+// payload is read after the look-back, which has its registers until then. Nine bits a pass, which
+// saves 18-bit keys a pass, made each pass half again as long.
 // Up to SMALL_MAX items one CTA sorts in shared memory, all passes in one launch.
 namespace {
 
@@ -317,7 +320,7 @@ constexpr int rs_smem() { return RS_THREADS * ITEMS * (int)(sizeof(K) + (VALS ? 
 // been started. A tile that stays silent for RS_SPINS polls is counted from its keys instead, so
 // the wait always ends.
 template <class K, bool VALS, int ITEMS>
-__global__ void __launch_bounds__(RS_THREADS, 4) rs_pass_kernel(const K *__restrict__ kin,
+__global__ void __launch_bounds__(RS_THREADS, 3) rs_pass_kernel(const K *__restrict__ kin,
                                                              const uint32_t *__restrict__ vin, K *__restrict__ kout,
                                                              uint32_t *__restrict__ vout, int64_t n, int shift,
                                                              const unsigned long long *__restrict__ gbase,
@@ -343,11 +346,6 @@ __global__ void __launch_bounds__(RS_THREADS, 4) rs_pass_kernel(const K *__restr
     uint32_t v[ITEMS], rank[ITEMS];
 #pragma unroll
     for (int i = 0; i < ITEMS; i++) k[i] = first + 32 * i < tn ? kp[32 * i] : (K)0;
-    if (VALS) {
-        const uint32_t *const vp = vin + tile * TILE + first;
-#pragma unroll
-        for (int i = 0; i < ITEMS; i++) v[i] = first + 32 * i < tn ? vp[32 * i] : 0u;
-    }
 #pragma unroll
     for (int i = 0; i < ITEMS; i++)
         rank[i] = warp_rank(whist[warp], digit_of(k[i], shift), first + 32 * i < tn, lt_mask);
@@ -409,6 +407,11 @@ __global__ void __launch_bounds__(RS_THREADS, 4) rs_pass_kernel(const K *__restr
     gpos[t] = (int64_t)(gbase[t] + before) - (int64_t)lbase;
 #pragma unroll
     for (int w = 0; w < RS_WARPS; w++) whist[w][t] += lbase;
+    if (VALS) {  // (not earlier: the look-back keeps its registers)
+        const uint32_t *const vp = vin + tile * TILE + first;
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++) v[i] = first + 32 * i < tn ? vp[32 * i] : 0u;
+    }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < ITEMS; i++) {
@@ -565,7 +568,7 @@ aps_status sort_impl(DBuf<K> &keys, DBuf<uint32_t> *vals, int64_t n, int bits, c
     // tile's chain of steps, and a shorter tile's is shorter (31,000 64-bit keys: counts and three
     // passes 24 us, 31 with the larger tiles).
     if (n <= (int64_t)num_sms() * RS_THREADS * 4) return sort_tiles<K, VALS, 4>(keys, vals, n, passes, s);
-    return sort_tiles<K, VALS, sizeof(K) == 8 ? 12 : 16>(keys, vals, n, passes, s);
+    return sort_tiles<K, VALS, sizeof(K) == 8 ? 16 : 20>(keys, vals, n, passes, s);
 }
 
 }  // namespace

@@ -1,7 +1,7 @@
 """The radix sort at the edges of its forms and tiles, through the calls that sort: the graph
 build (64-bit keys with a payload) and the candidate union (64-bit keys alone, with repeats).
 Up to 8192 items take the one-launch form, up to 1024 for each of 152 SMs tiles of 1024, more the
-form of 3072-item tiles. Both results are whole numbers and copied weights, so they are compared exactly."""
+form of 4096-item tiles. Both results are whole numbers and copied weights, so they are compared exactly."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 COUNTS = [1, 31, 257, 3072, 8191, 8192, 8193, 3 * 3072 - 1, 3 * 3072, 3 * 3072 + 1, 70001,
-          152 * 1024, 152 * 1024 + 1, 55 * 3072 - 1, 55 * 3072, 55 * 3072 + 1]
+          152 * 1024, 152 * 1024 + 1, 40 * 4096 - 1, 40 * 4096, 40 * 4096 + 1]
 
 
 @pytest.fixture(scope="module")
