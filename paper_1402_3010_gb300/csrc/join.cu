@@ -26,6 +26,10 @@
 //      the warp reserves in bulk. The run of x (or of its part) is recorded at its slot.
 // A window with more candidates than the list holds is filtered from A itself, in stretches
 // of as many slots as the list has entries.
+// Instruction issue bounds it (2.1 to 2.5 a cycle and SM; no pipe, no memory level near its
+// limit). With groups of warps sharing a window, and barriers between these steps, and lists up
+// to the split alone, the 200,000-row power-law set took 37.2 ms and a batch of 512 instances
+// 58; 21.6 and 14.9 now. 4096 queries against a million rows take 7.2 ms a call (17.2).
 // The output stage scans the per-slot counts and gathers the staged runs into (i, j, score)
 // arrays, which are then in (i, j) order without a sort.
 #include <algorithm>
