@@ -621,6 +621,11 @@ __global__ void k_wptr(const InstDesc *__restrict__ inst, int k, const int64_t *
     }
 }
 
+dim3 wptr_grid(int32_t maxm, int32_t maxnw, int k) {
+    const int64_t blocks = ((int64_t)maxm * (maxnw + 1) + T256 - 1) / T256;
+    return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, 65536 / k)), (unsigned)std::min(k, 65535));
+}
+
 // Join work list: every vector with later candidates in its instance, keyed by
 // (class, decreasing estimated cost) so that the persistent join takes the most expensive
 // queries first (least-loaded-first idea of the vertical algorithm's binning). Classes 0-3
@@ -896,10 +901,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p);
         APS_LAUNCH_CHECK();
         if (nwptr) {
-            const dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)maxm * (ix->maxnw + 1) + T256 - 1) / T256,
-                                                                          65536 / k)),
-                         (unsigned)std::min(k, 65535));
-            k_wptr<<<g, T256, 0, s>>>(d.inst.p, k, d.lptr.p, d.post.p, d.wptr.p);
+            k_wptr<<<wptr_grid(maxm, ix->maxnw, k), T256, 0, s>>>(d.inst.p, k, d.lptr.p, d.post.p, d.wptr.p);
             APS_LAUNCH_CHECK();
         }
         APS_TRY(d.crow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
@@ -964,6 +966,49 @@ aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> 
     }
     k_lptr<<<grid_for(ix->M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, ix->M, lptr.p);
     APS_LAUNCH_CHECK();
+    return APS_OK;
+}
+
+aps_status build_block_index(const aps_index *ix, BlockIndex &b, cudaStream_t s) {
+    const IndexArrays &d = ix->d;
+    const int64_t N = ix->N, M = ix->M, nnz = ix->nnz;
+    DBuf<int32_t> split, qsplit, erow;
+    DBuf<float> mwpre;
+    DBuf<uint32_t> keys, vals;
+    DBuf<unsigned long long> sums;
+    APS_TRY(split.alloc((size_t)N, s));
+    APS_TRY(qsplit.alloc((size_t)N, s));
+    APS_TRY(mwpre.alloc((size_t)N, s));
+    APS_TRY(erow.alloc((size_t)nnz, s));
+    APS_TRY(keys.alloc((size_t)nnz, s));
+    APS_TRY(vals.alloc((size_t)nnz, s));
+    APS_TRY(sums.alloc(2, s));
+    APS_TRY(b.vmeta.alloc((size_t)N, s));
+    APS_TRY(b.vcand.alloc((size_t)N, s));
+    APS_TRY(b.code.alloc((size_t)N, s));
+    APS_TRY(b.lptr.alloc((size_t)M + 1, s));
+    APS_TRY(b.wptr.alloc((size_t)ix->nwptr, s));
+    APS_TRY(b.post.alloc((size_t)ix->nsuf, s));
+    if (N == 0 || nnz == 0) return APS_OK;  // (nothing to join)
+    APS_CUDA(cudaMemsetAsync(sums.p, 0, 2 * sizeof(unsigned long long), s));
+    k_split<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N, ix->flags,
+                                          false, d.mw.p, split.p, qsplit.p, mwpre.p, b.vmeta.p, b.vcand.p, b.code.p, M,
+                                          keys.p, vals.p, sums.p, sums.p + 1);
+    APS_LAUNCH_CHECK();
+    k_rows_of<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, N, erow.p);
+    APS_LAUNCH_CHECK();
+    APS_TRY(sort_pairs(keys, vals, nnz, bits_for((uint64_t)M), s));
+    if (ix->nsuf > 0) {  // (the components from the splits on, as counted by the build)
+        k_post_fill<<<grid_for(ix->nsuf, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p, d.inst.p,
+                                                              ix->nsuf, b.post.p);
+        APS_LAUNCH_CHECK();
+    }
+    k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, M, b.lptr.p);
+    APS_LAUNCH_CHECK();
+    if (ix->nwptr) {
+        k_wptr<<<wptr_grid(ix->maxm, ix->maxnw, ix->k), T256, 0, s>>>(d.inst.p, ix->k, b.lptr.p, b.post.p, b.wptr.p);
+        APS_LAUNCH_CHECK();
+    }
     return APS_OK;
 }
 

@@ -70,6 +70,12 @@ struct JoinParams {
     // makes work item it one of nblk blocks of the vector items[it]; null: none
     const int8_t *iblk;
     int nblk;
+    // a block item's lists, boundaries and prefixes (up to the split alone)
+    const int4 *vmeta_b, *vcand_b;
+    const uint8_t *code_b;
+    const int64_t *lptr_b;
+    const uint32_t *wptr_b;
+    const int2 *post_b;
     unsigned long long *sp_key;    // pairs found by block items: local x * n + local y
     uint32_t *sp_score;            // their float32 scores (bits)
     unsigned long long *sp_count;  // pairs reserved in sp_key / sp_score
@@ -684,7 +690,8 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         }
         const int blk = (SPLIT && P.iblk) ? (int)P.iblk[item_of(unit)] : -1;
         const InstDesc &I = P.inst[QMODE || P.one ? 0 : P.vinst[x]];
-        const int4 xm = QMODE ? P.qvmeta[x] : P.vmeta[x];
+        const bool in_block = SPLIT && blk >= 0;
+        const int4 xm = QMODE ? P.qvmeta[x] : (in_block ? P.vmeta_b : P.vmeta)[x];
         const uint32_t vbase = (uint32_t)I.vbase;
         const int32_t lx = QMODE ? -1 : (int32_t)(x - vbase);
         const int2 *xrow = (QMODE ? P.qcrow : P.crow) + (uint32_t)xm.x;
@@ -701,7 +708,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
             wfirst = (int)__umulhi((uint32_t)lx + 1u, wmagic);
             while ((uint32_t)wfirst * (uint32_t)W > (uint32_t)lx + 1u) wfirst--;
         }
-        const uint32_t *const wp0 = P.wptr + I.wbase;
+        const uint32_t *const wp0 = (in_block ? P.wptr_b : P.wptr) + I.wbase;
+        const int64_t *const lptr = in_block ? P.lptr_b : P.lptr;
+        const int2 *const post = in_block ? P.post_b : P.post;
         const int32_t rbase = I.rbase;
         int wa = wfirst, wz = nw;
         uint32_t part = 0;
@@ -768,7 +777,7 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         // begin, so each window loads one position per list, for the window after it.
         const bool shortx = ncreate + qs <= 32;
         auto list_at = [&](const int r, const int w) -> uint32_t {
-            return nw > 1 ? __ldg(wp0 + (int64_t)r * (nw + 1) + w) : (uint32_t)__ldg(P.lptr + (rbase + r + w));
+            return nw > 1 ? __ldg(wp0 + (int64_t)r * (nw + 1) + w) : (uint32_t)__ldg(lptr + (rbase + r + w));
         };
         int2 e0 = make_int2(0, 0);
         uint32_t p0 = 0, p1 = 0;
@@ -818,7 +827,7 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                     cnt = g.y;
                     xv = __int_as_float(g.z);
                 }
-                walk(T, P.post, C, shortx ? ncreate : ph == 0 ? 32 : 0, st, cnt, xv, lane, n, visits, tot);
+                walk(T, post, C, shortx ? ncreate : ph == 0 ? 32 : 0, st, cnt, xv, lane, n, visits, tot);
                 __syncwarp();
                 if (shortx) break;
                 if (k0 >= (ph == 0 ? ncreate : qs)) {
@@ -833,8 +842,8 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
             __syncwarp();
             // ---------------- filter and verify: the candidate list at once, or, when it ran
             // over, the slots of the window in stretches of JOIN_LCAP
-            const uint8_t *codes = P.code + (vbase + (uint32_t)w0);
-            const int4 *cands = P.vcand + (vbase + (uint32_t)w0);
+            const uint8_t *codes = (in_block ? P.code_b : P.code) + (vbase + (uint32_t)w0);
+            const int4 *cands = (in_block ? P.vcand_b : P.vcand) + (vbase + (uint32_t)w0);
             const bool over = n > JOIN_LCAP;
             if (lane == 0) tot.v[1] += (unsigned long long)n;
             int nm = 0;  // matches
@@ -1254,14 +1263,14 @@ __global__ void k_first_of_key(const unsigned long long *__restrict__ key, int64
 // off[k]) into the staging buffer from `base` on, as the runs of their vectors' slots.
 __global__ void k_split_place(const unsigned long long *__restrict__ key, const uint32_t *__restrict__ score,
                               const int32_t *__restrict__ flag, const int64_t *__restrict__ off, int64_t n,
-                              const InstDesc *__restrict__ inst, int64_t base, int2 *stage, Segment *segs,
-                              int32_t *cntq) {
+                              const InstDesc *__restrict__ inst, int parts, int64_t base, int2 *stage,
+                              Segment *segs, int32_t *cntq) {
     const InstDesc I = inst[0];
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         if (!flag[k]) continue;
         const unsigned long long kk = key[k];
         const int32_t lx = (int32_t)(kk / (unsigned long long)I.n), y = (int32_t)(kk % (unsigned long long)I.n);
-        const int64_t qw = I.vbase + lx;
+        const int64_t qw = (I.vbase + lx) * parts;  // (a split vector has no run of its own in any part)
         const int64_t pos = base + off[k];
         stage[pos] = make_int2(y, (int)score[k]);
         atomicAdd(&cntq[qw], 1);
@@ -1285,11 +1294,12 @@ __global__ void k_split_place(const unsigned long long *__restrict__ key, const 
 // The split vectors' piece lengths, once every pair is counted: a vector with no run of its
 // own (it was joined by blocks) has its whole count in its one piece.
 __global__ void k_split_counts(const unsigned long long *__restrict__ key, const int32_t *__restrict__ flag, int64_t n,
-                               const InstDesc *__restrict__ inst, const int32_t *__restrict__ cntq, Segment *segs) {
+                               const InstDesc *__restrict__ inst, int parts, const int32_t *__restrict__ cntq, Segment *segs) {
     const InstDesc I = inst[0];
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t lx = (int64_t)(key[k] / (unsigned long long)I.n);
-        if (k == 0 || (int64_t)(key[k - 1] / (unsigned long long)I.n) != lx) segs[I.vbase + lx].cnt = cntq[I.vbase + lx];
+        if (k == 0 || (int64_t)(key[k - 1] / (unsigned long long)I.n) != lx)
+            segs[(I.vbase + lx) * parts].cnt = cntq[(I.vbase + lx) * parts];
     }
 }
 
@@ -1318,7 +1328,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
 
     // the vertical split: the costliest `heavy` vectors as nblk dimension blocks each
     const bool split = nblk >= 2 && heavy > 0 && ix->k == 1;
-    const int parts = split ? 1 : ix->parts;
+    const int parts = ix->parts;
     const int64_t nslots = ix->N * parts;
     int split_cls = -1;
     int64_t nsplit = 0, sp_cap = 0;
@@ -1326,6 +1336,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
     DBuf<int8_t> iblk;
     DBuf<uint64_t> sp_key;
     DBuf<uint32_t> sp_score;
+    BlockIndex bx;
     if (split) {
         // block items come from the windowed classes (G = 1 ... 8), never from the
         // streamed class (one- and two-component vectors) that follows them
@@ -1340,6 +1351,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
             APS_TRY(iblk.alloc((size_t)total, s));
             k_split_items<<<grid_for(total, 256), 256, 0, s>>>(ix->items.p, nitems, nsplit, nblk, items2.p, iblk.p);
             APS_LAUNCH_CHECK();
+            if (ix->l2) APS_TRY(build_block_index(ix, bx, s));
             sp_cap = std::max<int64_t>((int64_t)1 << 20, nsplit * 4096);
         }
     }
@@ -1408,10 +1420,21 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 P.items = items2.p;
                 P.iblk = iblk.p;
                 P.nblk = nblk;
+                P.vmeta_b = ix->l2 ? bx.vmeta.p : P.vmeta;
+                P.vcand_b = ix->l2 ? bx.vcand.p : P.vcand;
+                P.code_b = ix->l2 ? bx.code.p : P.code;
+                P.lptr_b = ix->l2 ? bx.lptr.p : P.lptr;
+                P.wptr_b = ix->l2 ? bx.wptr.p : P.wptr;
+                P.post_b = ix->l2 ? bx.post.p : P.post;
                 P.sp_key = reinterpret_cast<unsigned long long *>(sp_key.p);
                 P.sp_score = sp_score.p;
                 P.sp_cap = sp_cap;
                 for (int c = split_cls + 1; c <= JOIN_NCLS; c++) P.cls_begin[c] += nsplit * (nblk - 1);
+                // block items come first and are cut into parts as heavy vectors are: whole, the
+                // longest of them would be one warp's tail (200 vectors in two blocks: 41.2 ms,
+                // 23.8 cut)
+                P.cls_heavy[split_cls] = std::min(P.cls_begin[split_cls + 1] - P.cls_begin[split_cls],
+                                                  std::min(nsplit * nblk, 4 * JOIN_HEAVY) + JOIN_HEAVY);
                 APS_CUDA(cudaMemsetAsync(ctr.p, 0, 16 * sizeof(unsigned long long), s));
                 APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * std::max<int64_t>(nslots, 1), s));
                 join_kernel<false, true><<<grid, JOIN_THREADS, need, s>>>(P);
@@ -1453,10 +1476,10 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                     stage_cap = reserved + nuniq;
                 }
                 k_split_place<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, sp_score.p, flag.p, off.p, sp_found,
-                                                                     d.inst.p, reserved, stage.p, segs.p, cntq.p);
+                                                                     d.inst.p, parts, reserved, stage.p, segs.p, cntq.p);
                 APS_LAUNCH_CHECK();
-                k_split_counts<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, flag.p, sp_found, d.inst.p, cntq.p,
-                                                                      segs.p);
+                k_split_counts<<<grid_for(sp_found, 256), 256, 0, s>>>(sp_sorted, flag.p, sp_found, d.inst.p, parts,
+                                                                      cntq.p, segs.p);
                 APS_LAUNCH_CHECK();
                 total_pairs += nuniq;
             }
