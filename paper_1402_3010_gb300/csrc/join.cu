@@ -1825,7 +1825,9 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     const int64_t nqw = std::max<int64_t>(nq * parts, 1);
     const int need = tile_bytes(G) * tile_warps(G);
     const int64_t slab = 256;  // query batches are small: keep the slab tails short
-    APS_CUDA(cudaFuncSetAttribute(join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
+    // (the limit is the kernel's, not the launch's: the same for every index, or a query of another
+    // shape on another thread could lower it before this launch)
+    APS_CUDA(cudaFuncSetAttribute(join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, join_smem()));
     cudaEvent_t ev[3];
     for (int i = 0; i < 3; i++) APS_CUDA(cudaEventCreate(&ev[i]));
     struct EvGuard {
