@@ -834,7 +834,9 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     }
     if (nnz > 0 && k > 1 && maxm <= DIMSTATS_DIMS) {  // a batch of small instances: one CTA each
         const int sm = (int)(sizeof(uint32_t) * (size_t)maxm);
-        APS_CUDA(cudaFuncSetAttribute(k_dimstats_inst, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+        // (the kernel's limit is shared by every thread: the same for every batch)
+        APS_CUDA(cudaFuncSetAttribute(k_dimstats_inst, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(uint32_t) * DIMSTATS_DIMS));
         k_dimstats_inst<<<k, 1024, sm, s>>>(d.cptr.p, idx, vout.p, d.inst.p, d.nnz_d.p, d.mw_d.p);
         APS_LAUNCH_CHECK();
     } else if (nnz > 0) {

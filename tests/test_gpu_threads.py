@@ -76,3 +76,32 @@ def test_queries_of_two_tile_shapes_from_two_threads(aps):
         aps.aps_set_tuning(aps.aps_get_tuning(), before)
         for h in handles:
             aps.aps_index_free(h)
+
+
+def test_batches_of_different_dimension_counts_from_two_threads(aps):
+    import torch
+
+    rng = np.random.default_rng(102)
+    jobs = []
+    for m in (200, 57344, 20000, 57000):  # all counted in shared memory: 4 bytes a dimension
+        parts = [synth.sparse_vectors(60, m, rng.integers(3, 9, 60), 1.0, "uniform", 102, rng=rng) for _ in range(2)]
+        ptr = np.concatenate([parts[0].indptr, parts[0].nnz + parts[1].indptr[1:]])
+        csr = [torch.from_numpy(a).cuda() for a in (ptr, *(np.concatenate([getattr(p, k) for p in parts])
+                                                           for k in ("idx", "val")))]
+
+        def join(csr=csr, m=m, stream=torch.cuda.Stream()):
+            outs, st = aps.aps_batch_all_pairs_csr([0, 60, 120], *csr, [m, m], [0.3, 0.3], 0, stream)
+            try:
+                return [o.count for o in outs]
+            finally:
+                for o in outs:
+                    aps.aps_pairs_free(o)
+
+        torch.cuda.synchronize()
+        alone = join()
+
+        def same(join=join, alone=alone):
+            assert join() == alone
+
+        jobs.append(same)
+    _at_once(jobs, 1000)
