@@ -46,6 +46,16 @@ aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qi
     DBuf<int64_t> dp;
     DBuf<int32_t> di;
     DBuf<float> dv;
+    std::vector<char> h;  // few host queries, packed
+    // Copies from host memory may still be reading it when the copy call returns: whatever the call
+    // returns, they have ended before h goes and before the caller has its arrays back.
+    struct Copies {
+        cudaStream_t s;
+        bool pending = false;
+        ~Copies() {
+            if (pending) cudaStreamSynchronize(s);
+        }
+    } copies{s};
     const int64_t *p = qptr;
     const int32_t *ii = qidx;
     const float *vv = qval;
@@ -63,14 +73,14 @@ aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qi
         // few queries go as one copy of one buffer (a copy from pageable memory costs its caller 6 us)
         constexpr size_t QUERY_PACK = 32 * 1024;
         if (pb + 2 * eb <= QUERY_PACK) {
-            std::vector<char> h(pb + 2 * eb);
+            h.resize(pb + 2 * eb);
             memcpy(h.data(), qptr, pb);
             if (nnz) {
                 memcpy(h.data() + pb, qidx, eb);
                 memcpy(h.data() + pb + eb, qval, eb);
             }
             APS_TRY(dp.alloc((h.size() + sizeof(int64_t) - 1) / sizeof(int64_t), s));
-            // (pageable memory has been read when the call returns)
+            copies.pending = true;
             APS_CUDA(cudaMemcpyAsync(dp.p, h.data(), h.size(), cudaMemcpyHostToDevice, s));
             ii = reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(dp.p) + pb);
             vv = reinterpret_cast<const float *>(reinterpret_cast<const char *>(dp.p) + pb + eb);
@@ -78,6 +88,7 @@ aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qi
             APS_TRY(dp.alloc((size_t)nq + 1, s));
             APS_TRY(di.alloc((size_t)std::max<int64_t>(nnz, 1), s));
             APS_TRY(dv.alloc((size_t)std::max<int64_t>(nnz, 1), s));
+            copies.pending = true;
             APS_CUDA(cudaMemcpyAsync(dp.p, qptr, pb, cudaMemcpyHostToDevice, s));
             if (nnz) {
                 APS_CUDA(cudaMemcpyAsync(di.p, qidx, eb, cudaMemcpyHostToDevice, s));
@@ -90,6 +101,7 @@ aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qi
     }
     QueryArrays qa;
     APS_TRY(prepare_queries(ix, p, ii, vv, nq, t, flags, s, qa, (flags & APS_DEVICE_PTRS) ? -1 : qptr[nq]));
+    copies.pending = false;  // (the rows' check has been waited for)
     aps_stats local{};
     APS_TRY(join_queries(ix, qa, t, flags, s, out, &local));
     if (stats) *stats = local;
