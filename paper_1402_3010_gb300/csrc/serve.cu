@@ -25,6 +25,9 @@ using namespace aps;
 
 namespace {
 
+// Component counts that a query batch may have, checked before any size is computed from one.
+bool query_nnz_ok(int64_t nnz) { return nnz >= 0 && nnz < (1ll << 31); }
+
 aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qidx, const float *qval, int32_t nq,
                            float t, uint32_t flags, cudaStream_t s, aps_pairs *out, aps_stats *stats) {
     if (!(ix->flags & APS_QUERYABLE)) {
@@ -65,7 +68,7 @@ aps_status query_on_stream(aps_index *ix, const int64_t *qptr, const int32_t *qi
             return APS_EINVAL;
         }
         const int64_t nnz = qptr[nq];
-        if (nnz < 0 || (nnz > 0 && (!qidx || !qval))) {
+        if (!query_nnz_ok(nnz) || (nnz > 0 && (!qidx || !qval))) {
             set_error("bad query CSR");
             return APS_EINVAL;
         }
@@ -333,7 +336,7 @@ aps_status aps_stream_submit(aps_server *sv, const aps_query_req *req, uint64_t 
         return APS_EINVAL;
     }
     const int64_t nnz = req->qptr[req->nq];
-    if (req->qptr[0] != 0 || nnz < 0 || (nnz > 0 && (!req->qidx || !req->qval))) {
+    if (req->qptr[0] != 0 || !query_nnz_ok(nnz) || (nnz > 0 && (!req->qidx || !req->qval))) {
         set_error("bad query CSR");
         return APS_EINVAL;
     }

@@ -168,6 +168,26 @@ int main() {
     }
     return 0;
 }""",
+    # a last row pointer that no array can have is refused before a size is computed from it
+    "huge_counts_are_refused": r"""
+int main() {
+    index_of(10000);
+    aps_server *sv = nullptr;
+    if (aps_server_create(&ix, 1 << 30, 1, &sv) != APS_OK) return 1;
+    const int32_t id = 0;
+    const float val = 1.f;
+    int rc = 0;
+    for (int64_t nnz : {(int64_t)1 << 31, (int64_t)1 << 60, (int64_t)1 << 61, (int64_t)1 << 62, INT64_MAX, (int64_t)-1}) {
+        const int64_t ptr[2] = {0, nnz};
+        aps_pairs out;
+        if (aps_query(&ix, ptr, &id, &val, 1, 0.5f, 0, &out) != APS_EINVAL) rc = 2;
+        const aps_query_req req = {ptr, &id, &val, 1, 0.5f};
+        uint64_t ticket = 0;
+        if (aps_stream_submit(sv, &req, &ticket) != APS_EINVAL) rc = 3;
+    }
+    aps_server_free(sv);
+    return rc;
+}""",
 }
 
 
