@@ -626,6 +626,81 @@ dim3 wptr_grid(int32_t maxm, int32_t maxnw, int k) {
     return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, 65536 / k)), (unsigned)std::min(k, 65535));
 }
 
+// The same per list (wlist): how many starts each list has, where they begin, and the starts, one
+// thread each.
+__global__ void k_wlist_counts(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ lptr, int64_t M,
+                               int per, int32_t *cnt) {
+    for (int64_t R = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; R < M; R += (int64_t)gridDim.x * blockDim.x) {
+        const int nw = inst[inst_of_rank(inst, k, R)].nw;
+        const int groups = window_groups(nw, list_shift(lptr[R + 1] - lptr[R], nw, per));
+        cnt[R] = groups > 1 ? groups + 1 : 0;
+    }
+}
+
+__global__ void k_wlist(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ lptr,
+                        const int64_t *__restrict__ off, int64_t M, int per, uint64_t *wlist) {
+    for (int64_t R = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; R < M; R += (int64_t)gridDim.x * blockDim.x)
+        wlist[R] = (uint64_t)off[R] << 6 |
+                   (uint64_t)list_shift(lptr[R + 1] - lptr[R], inst[inst_of_rank(inst, k, R)].nw, per);
+}
+
+__global__ void k_wlist_starts(const InstDesc *__restrict__ inst, int k, const int64_t *__restrict__ lptr,
+                               const int2 *__restrict__ post, const int64_t *__restrict__ off,
+                               const uint64_t *__restrict__ wlist, int64_t M, int64_t total, uint32_t *wptr) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        int64_t a = 0, b = M;  // the last list that begins at or before e (those without starts begin where the next does)
+        while (a < b) {
+            const int64_t mid = (a + b) >> 1;
+            if (off[mid] <= e) a = mid + 1; else b = mid;
+        }
+        const int64_t R = a - 1;
+        const InstDesc &I = inst[inst_of_rank(inst, k, R)];
+        const int32_t idmask = I.packed ? 0x00ffffff : 0x7fffffff;
+        const int64_t bound = ((e - off[R]) << (wlist[R] & 63)) * I.W;
+        int64_t lo = lptr[R], hi = lptr[R + 1];
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((post[mid].x & idmask) < bound) lo = mid + 1; else hi = mid;
+        }
+        wptr[e] = (uint32_t)lo;
+    }
+}
+
+// The table of window starts of the lists (lptr, post), in the form that the build chose.
+aps_status window_starts(const aps_index *ix, const DBuf<int64_t> &lptr, const DBuf<int2> &post, DBuf<uint32_t> &wptr,
+                         DBuf<uint64_t> &wlist, cudaStream_t s) {
+    const InstDesc *const inst = ix->d.inst.p;
+    const int64_t M = ix->M;
+    if (ix->wper < 0) {
+        APS_TRY(wptr.alloc((size_t)std::max<int64_t>(ix->nwptr, 1), s));
+        if (ix->nwptr) {
+            k_wptr<<<wptr_grid(ix->maxm, ix->maxnw, ix->k), T256, 0, s>>>(inst, ix->k, lptr.p, post.p, wptr.p);
+            APS_LAUNCH_CHECK();
+        }
+        return APS_OK;
+    }
+    DBuf<int32_t> cnt;
+    DBuf<int64_t> off;
+    APS_TRY(cnt.alloc((size_t)M, s));
+    APS_TRY(off.alloc((size_t)M + 1, s));
+    APS_TRY(wlist.alloc((size_t)M, s));
+    k_wlist_counts<<<grid_for(M, T256), T256, 0, s>>>(inst, ix->k, lptr.p, M, ix->wper, cnt.p);
+    APS_LAUNCH_CHECK();
+    APS_TRY(scan_exclusive(cnt.p, off.p, M, s));
+    int64_t total = 0;
+    APS_CUDA(cudaMemcpyAsync(&total, off.p + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    APS_CUDA(cudaStreamSynchronize(s));
+    APS_TRY(wptr.alloc((size_t)std::max<int64_t>(total, 1), s));
+    k_wlist<<<grid_for(M, T256), T256, 0, s>>>(inst, ix->k, lptr.p, off.p, M, ix->wper, wlist.p);
+    APS_LAUNCH_CHECK();
+    if (total) {
+        k_wlist_starts<<<grid_for(total, T256), T256, 0, s>>>(inst, ix->k, lptr.p, post.p, off.p, wlist.p, M, total,
+                                                              wptr.p);
+        APS_LAUNCH_CHECK();
+    }
+    return APS_OK;
+}
+
 // Join work list: every vector with later candidates in its instance, keyed by
 // (class, decreasing estimated cost) so that the persistent join takes the most expensive
 // queries first (least-loaded-first idea of the vertical algorithm's binning). Classes 0-3
@@ -697,6 +772,29 @@ const char *code_name(int c) {
 
 }  // namespace
 
+namespace {
+
+constexpr int64_t WPTR_LARGE = 64 << 20;  // (asking for the free memory takes the host some 10 us)
+
+// Device memory that an allocation can have: free, or kept by the pool without being used.
+size_t memory_at_hand() {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        cudaGetLastError();
+        return SIZE_MAX;
+    }
+    int dev = 0;
+    cudaMemPool_t pool;
+    uint64_t kept = 0, used = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &kept) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && kept > used)
+        fr += kept - used;
+    return fr;
+}
+
+}  // namespace
+
 aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_t *idx, const float *val,
                               const std::vector<InstDesc> &inst_in, cudaStream_t s, const aps_tuning *tune) {
     const int k = (int)inst_in.size();
@@ -762,6 +860,14 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         return APS_EINVAL;
     }
     ix->nnz = nnz;
+    // the table of window starts: every window's where that takes no more than its share and, when it
+    // is large, an eighth of the memory at hand; else by list
+    if (4 * nwptr > window_bytes(nnz, M) || (4 * nwptr > WPTR_LARGE && (uint64_t)nwptr > memory_at_hand() / 32)) {
+        ix->wper = WLIST_ENTRIES;
+        const uint64_t room = memory_at_hand() / 32;
+        while (ix->wper > 0 && (uint64_t)ix->wper * (uint64_t)nnz * 4 > WPTR_LARGE && (uint64_t)ix->wper * (uint64_t)nnz > room)
+            ix->wper /= 2;
+    }
     Carver cv;
     cv.s = s;
     for (int pass = 0; pass < 2; pass++) {
@@ -894,7 +1000,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         ix->njoin = (int64_t)cnt3[2];
         if (nnz > 0) APS_TRY(sort_pairs(keys, vals, nnz, bits_for((uint64_t)M), s));
         APS_TRY(d.post.alloc((size_t)std::max<int64_t>(ix->njoin, 1), s));
-        APS_TRY(d.wptr.alloc((size_t)std::max<int64_t>(nwptr, 1), s));
         if (ix->njoin > 0) {
             k_post_fill<<<grid_for(ix->njoin, T256), T256, 0, s>>>(vals.p, erow.p, d.cval.p, d.len.p, d.vinst.p,
                                                                    d.inst.p, ix->njoin, d.post.p);
@@ -902,10 +1007,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         }
         k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p);
         APS_LAUNCH_CHECK();
-        if (nwptr) {
-            k_wptr<<<wptr_grid(maxm, ix->maxnw, k), T256, 0, s>>>(d.inst.p, k, d.lptr.p, d.post.p, d.wptr.p);
-            APS_LAUNCH_CHECK();
-        }
+        APS_TRY(window_starts(ix, d.lptr, d.post, d.wptr, d.wlist, s));
         APS_TRY(d.crow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
         if (nnz > 0) {
             k_pack<<<gE, T256, 0, s>>>(d.crank.p, d.cval.p, nnz, d.crow.p);
@@ -989,7 +1091,6 @@ aps_status build_block_index(const aps_index *ix, BlockIndex &b, cudaStream_t s)
     APS_TRY(b.vcand.alloc((size_t)N, s));
     APS_TRY(b.code.alloc((size_t)N, s));
     APS_TRY(b.lptr.alloc((size_t)M + 1, s));
-    APS_TRY(b.wptr.alloc((size_t)ix->nwptr, s));
     APS_TRY(b.post.alloc((size_t)ix->nsuf, s));
     if (N == 0 || nnz == 0) return APS_OK;  // (nothing to join)
     APS_CUDA(cudaMemsetAsync(sums.p, 0, 2 * sizeof(unsigned long long), s));
@@ -1007,11 +1108,7 @@ aps_status build_block_index(const aps_index *ix, BlockIndex &b, cudaStream_t s)
     }
     k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, M, b.lptr.p);
     APS_LAUNCH_CHECK();
-    if (ix->nwptr) {
-        k_wptr<<<wptr_grid(ix->maxm, ix->maxnw, ix->k), T256, 0, s>>>(d.inst.p, ix->k, b.lptr.p, b.post.p, b.wptr.p);
-        APS_LAUNCH_CHECK();
-    }
-    return APS_OK;
+    return window_starts(ix, b.lptr, b.post, b.wptr, b.wlist, s);
 }
 
 // ------------------------------------------------------------------ external queries

@@ -83,6 +83,7 @@ struct JoinParams {
     const int64_t *lptr;
     const uint32_t *wptr;
     const int2 *post;
+    const uint64_t *wlist, *wlist_b;  // COARSE: the lists' places in wptr (in wptr_b)
     uint32_t flags;
     int2 *stage;
     int64_t stage_cap;
@@ -250,9 +251,38 @@ __device__ __forceinline__ int64_t first_after(const int2 *__restrict__ post, in
     return m ? a + (__ffs(m) - 1) : b;
 }
 
+// Position in post of the first entry of window w of the list of global rank R, where the table holds
+// groups of windows (instance of nw windows of W ids).
+__device__ __forceinline__ uint32_t list_start(const uint64_t *__restrict__ wlist, const uint32_t *__restrict__ wptr,
+                                               const int64_t *__restrict__ lptr, const int2 *__restrict__ post,
+                                               const int64_t R, const int w, const int nw, const int W,
+                                               const int32_t idmask) {
+    const uint64_t d = __ldg(wlist + R);
+    const int shift = (int)(d & 63u), g = w >> shift;
+    uint32_t lo, hi;
+    if (window_groups(nw, shift) > 1) {
+        const uint32_t *const e = wptr + (d >> 6) + g;
+        lo = __ldg(e);
+        if (g << shift == w) return lo;
+        hi = __ldg(e + 1);
+    } else {
+        lo = (uint32_t)__ldg(lptr + R);
+        if (w == 0) return lo;
+        hi = (uint32_t)__ldg(lptr + R + 1);
+    }
+    if (w >= nw) return hi;
+#pragma unroll 1
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if ((__ldg(&post[mid].x) & idmask) < w * W) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
 // The part of a posting list after x: [first, end) of list rank r of instance I (the
 // search starts in the window of x's successor, whose part of the list holds the answer
 // or ends right before it).
+template <bool COARSE>
 __device__ __forceinline__ void list_after(const JoinParams &P, const InstDesc &I, const int r, const int32_t lx,
                                            const int wf, const int32_t idmask, const int lane, int64_t &first,
                                            int64_t &end) {
@@ -260,7 +290,14 @@ __device__ __forceinline__ void list_after(const JoinParams &P, const InstDesc &
     const int64_t ls = P.lptr[R];
     end = P.lptr[R + 1];
     int64_t a = ls, b = end;
-    if (I.nw > 1) {
+    if (COARSE) {
+        const uint64_t d = P.wlist[R];
+        if (window_groups(I.nw, (int)(d & 63u)) > 1) {
+            const uint32_t *wp = P.wptr + (d >> 6) + (wf >> (int)(d & 63u));
+            a = wp[0];
+            b = wp[1];
+        }
+    } else if (I.nw > 1) {
         const uint32_t *wp = P.wptr + I.wbase + (int64_t)r * (I.nw + 1);
         a = wp[wf];
         b = wp[wf + 1];
@@ -300,6 +337,7 @@ __device__ __forceinline__ int count_below(const int v, const int key) {
 // the warp's scratch list and are then copied as x's run to the staging slab that the warp
 // reserves in bulk; a vector with more matches than the scratch list holds is streamed a
 // second time, writing them there directly.
+template <bool COARSE>
 __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long long *work, const int64_t item_begin,
                                           const int64_t item_end, const bool f_minsize, const bool f_remscore,
                                           Totals &tot, Stager &S) {
@@ -341,8 +379,8 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
         const int32_t idmask = I.packed ? 0x00ffffff : 0x7fffffff;
         const int wf = (lx + 1) / I.W;  // the window of x's successor
         int64_t f0, e0, f1 = 0, e1 = 0;
-        list_after(P, I, xe0.x, lx, wf, idmask, lane, f0, e0);
-        if (xl == 2) list_after(P, I, xe1.x, lx, wf, idmask, lane, f1, e1);
+        list_after<COARSE>(P, I, xe0.x, lx, wf, idmask, lane, f0, e0);
+        if (xl == 2) list_after<COARSE>(P, I, xe1.x, lx, wf, idmask, lane, f1, e1);
         if (lane == 0) tot.v[5] += (unsigned long long)((e0 - f0) + (e1 - f1));
         // pass 0: count the matches, the first JOIN_ECAP into the scratch list; pass 1 (only
         // when there were more): write them all into the reserved run
@@ -643,7 +681,7 @@ __device__ __forceinline__ void walk(const Tile &T, const int2 *__restrict__ pos
 
 // One class of windowed items with tile shape G: every warp takes units (a vector, or one
 // part of a heavy vector's windows) from the class's work list until it is empty.
-template <bool QMODE, bool SPLIT>
+template <bool QMODE, bool SPLIT, bool COARSE>
 __device__ __forceinline__ void join_class(const JoinParams &P, const int G, const int64_t item_begin,
                                            const int64_t item_end, const int64_t heavy, unsigned long long *const work,
                                            const bool f_minsize, const bool f_remscore, const bool f_upper,
@@ -777,6 +815,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         // begin, so each window loads one position per list, for the window after it.
         const bool shortx = ncreate + qs <= 32;
         auto list_at = [&](const int r, const int w) -> uint32_t {
+            if (COARSE)
+                return list_start(in_block ? P.wlist_b : P.wlist, in_block ? P.wptr_b : P.wptr, lptr, post,
+                                  (int64_t)rbase + r, w, nw, IW, C.idmask);
             return nw > 1 ? __ldg(wp0 + (int64_t)r * (nw + 1) + w) : (uint32_t)__ldg(lptr + (rbase + r + w));
         };
         int2 e0 = make_int2(0, 0);
@@ -1029,9 +1070,10 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 }
 
 // QMODE: external queries against the index; SPLIT: a self-join whose work list may hold
-// dimension-block items (P.iblk). Each is compiled separately, so that the plain self-join
+// dimension-block items (P.iblk); COARSE: window starts by list. Each is
+// compiled separately, so that the plain self-join
 // carries none of the other paths' state.
-template <bool QMODE, bool SPLIT = false>
+template <bool QMODE, bool SPLIT, bool COARSE>
 __global__ void __launch_bounds__(JOIN_THREADS, 1) join_kernel(const __grid_constant__ JoinParams P) {
     const bool f_minsize = !(P.flags & APS_NO_MINSIZE);
     const bool f_remscore = !(P.flags & APS_NO_REMSCORE);
@@ -1056,10 +1098,10 @@ __global__ void __launch_bounds__(JOIN_THREADS, 1) join_kernel(const __grid_cons
         const int G = P.cls_G[cls];
         unsigned long long *const work = P.work + cls;
         if (!QMODE && G == 0) {  // short vectors: one warp each
-            stream_short(P, work, item_begin, item_end, f_minsize, f_remscore, tot, S);
+            stream_short<COARSE>(P, work, item_begin, item_end, f_minsize, f_remscore, tot, S);
             continue;
         }
-        join_class<QMODE, SPLIT>(P, G, item_begin, item_end, P.cls_heavy[cls], work, f_minsize, f_remscore, f_upper, S,
+        join_class<QMODE, SPLIT, COARSE>(P, G, item_begin, item_end, P.cls_heavy[cls], work, f_minsize, f_remscore, f_upper, S,
                                  tot);
         bool later = false;  // another windowed class
         for (int c = cls + 1; c < P.ncls; c++) later = later || (P.cls_G[c] > 0 && P.cls_begin[c + 1] > P.cls_begin[c]);
@@ -1138,6 +1180,20 @@ int set_classes(JoinParams &P, const aps_index *ix, int parts, int max_ctas) {
     return (int)std::min<int64_t>(max_ctas, ctas);
 }
 
+// The kernel for an index's self-join (split: with dimension-block items) or for queries of it.
+using JoinKernel = void (*)(const JoinParams);
+JoinKernel self_kernel(const aps_index *ix, bool split = false) {
+    if (split) return ix->wper >= 0 ? join_kernel<false, true, true> : join_kernel<false, true, false>;
+    return ix->wper >= 0 ? join_kernel<false, false, true> : join_kernel<false, false, false>;
+}
+JoinKernel query_kernel(const aps_index *ix) {
+    return ix->wper >= 0 ? join_kernel<true, false, true> : join_kernel<true, false, false>;
+}
+aps_status allow_smem(JoinKernel k) {  // (the same for every index: the limit is shared by all threads)
+    APS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, join_smem()));
+    return APS_OK;
+}
+
 // What every join reads of an index.
 void set_index(JoinParams &P, const aps_index *ix) {
     const IndexArrays &d = ix->d;
@@ -1155,6 +1211,7 @@ void set_index(JoinParams &P, const aps_index *ix) {
     P.lptr = d.lptr.p;
     P.wptr = d.wptr.p;
     P.post = d.post.p;
+    P.wlist = d.wlist.p;
 }
 
 // The join phase: reset the counters and the per-slot pair counts, then the persistent join.
@@ -1170,7 +1227,7 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
     if (G.launches++ == 0) {
         APS_CUDA(cudaMemsetAsync(ctr, 0, ctr_bytes, s));
         APS_CUDA(cudaMemsetAsync(cntq, 0, cnt_bytes, s));
-        join_kernel<false><<<grid, JOIN_THREADS, smem, s>>>(P);
+        self_kernel(ix)<<<grid, JOIN_THREADS, smem, s>>>(P);
         APS_LAUNCH_CHECK();
         return APS_OK;
     }
@@ -1181,7 +1238,7 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
         if (e == cudaSuccess) {
             cudaMemsetAsync(ctr, 0, ctr_bytes, cs);
             cudaMemsetAsync(cntq, 0, cnt_bytes, cs);
-            join_kernel<false><<<grid, JOIN_THREADS, smem, cs>>>(P);
+            self_kernel(ix)<<<grid, JOIN_THREADS, smem, cs>>>(P);
             cudaGraph_t g = nullptr;
             e = cudaStreamEndCapture(cs, &g);
             G.graph = g;
@@ -1220,7 +1277,7 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
         void *args[1] = {&P};
         cudaKernelNodeParams kp;
         memset(&kp, 0, sizeof(kp));
-        kp.func = reinterpret_cast<void *>(join_kernel<false>);
+        kp.func = reinterpret_cast<void *>(self_kernel(ix));
         kp.gridDim = dim3((unsigned)grid);
         kp.blockDim = dim3(JOIN_THREADS);
         kp.sharedMemBytes = (unsigned)smem;
@@ -1324,7 +1381,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
         }
     } evg{ev};
     const int need = join_smem();
-    APS_CUDA(cudaFuncSetAttribute(join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
+    APS_TRY(allow_smem(self_kernel(ix)));
 
     // the vertical split: the costliest `heavy` vectors as nblk dimension blocks each
     const bool split = nblk >= 2 && heavy > 0 && ix->k == 1;
@@ -1345,7 +1402,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
         const int64_t nitems = ix->class_begin[JOIN_NCLS] - ix->class_begin[0];
         nsplit = std::min<int64_t>(heavy, ix->class_begin[4] - ix->class_begin[0]);
         if (nsplit > 0) {
-            APS_CUDA(cudaFuncSetAttribute(join_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
+            APS_TRY(allow_smem(self_kernel(ix, true)));
             const int64_t total = nitems + nsplit * (nblk - 1);
             APS_TRY(items2.alloc((size_t)total, s));
             APS_TRY(iblk.alloc((size_t)total, s));
@@ -1425,6 +1482,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                 P.code_b = ix->l2 ? bx.code.p : P.code;
                 P.lptr_b = ix->l2 ? bx.lptr.p : P.lptr;
                 P.wptr_b = ix->l2 ? bx.wptr.p : P.wptr;
+                P.wlist_b = ix->l2 ? bx.wlist.p : P.wlist;
                 P.post_b = ix->l2 ? bx.post.p : P.post;
                 P.sp_key = reinterpret_cast<unsigned long long *>(sp_key.p);
                 P.sp_score = sp_score.p;
@@ -1437,7 +1495,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                                                   std::min(nsplit * nblk, 4 * JOIN_HEAVY) + JOIN_HEAVY);
                 APS_CUDA(cudaMemsetAsync(ctr.p, 0, 16 * sizeof(unsigned long long), s));
                 APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * std::max<int64_t>(nslots, 1), s));
-                join_kernel<false, true><<<grid, JOIN_THREADS, need, s>>>(P);
+                self_kernel(ix, true)<<<grid, JOIN_THREADS, need, s>>>(P);
                 APS_LAUNCH_CHECK();
             } else {
                 APS_TRY(run_join_graph(ix, P, grid, need, ctr.p, cntq.p, nslots, s));
@@ -1751,7 +1809,7 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
     int2 *stage = reinterpret_cast<int2 *>(arena + off);
 
     const int need = join_smem();
-    APS_CUDA(cudaFuncSetAttribute(join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, need));
+    APS_TRY(allow_smem(self_kernel(ix)));
     APS_CUDA(cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned long long), s));
     APS_CUDA(cudaMemsetAsync(cntq, 0, sizeof(int32_t) * nslots, s));
     if (ix->class_begin[JOIN_NCLS] > ix->class_begin[0]) {
@@ -1769,7 +1827,7 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
         P.counters = ctr;
         P.work = ctr + 8;
         P.scratch = elists;
-        join_kernel<false><<<grid, JOIN_THREADS, need, s>>>(P);
+        self_kernel(ix)<<<grid, JOIN_THREADS, need, s>>>(P);
         APS_LAUNCH_CHECK();
     }
     unsigned long long ch[16];
@@ -1825,9 +1883,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     const int64_t nqw = std::max<int64_t>(nq * parts, 1);
     const int need = tile_bytes(G) * tile_warps(G);
     const int64_t slab = 256;  // query batches are small: keep the slab tails short
-    // (the limit is the kernel's, not the launch's: the same for every index, or a query of another
-    // shape on another thread could lower it before this launch)
-    APS_CUDA(cudaFuncSetAttribute(join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, join_smem()));
+    APS_TRY(allow_smem(query_kernel(ix)));
     cudaEvent_t ev[3];
     for (int i = 0; i < 3; i++) APS_CUDA(cudaEventCreate(&ev[i]));
     struct EvGuard {
@@ -1878,7 +1934,7 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
             P.qcrow = qa.crow.p;
             P.qvmeta = qa.vmeta.p;
             P.qt = t;
-            join_kernel<true><<<grid, JOIN_THREADS, need, s>>>(P);
+            query_kernel(ix)<<<grid, JOIN_THREADS, need, s>>>(P);
             APS_LAUNCH_CHECK();
         }
         APS_CUDA(cudaEventRecord(ev[1], s));
