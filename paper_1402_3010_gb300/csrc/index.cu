@@ -444,7 +444,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
                         const float *__restrict__ cval, const float *__restrict__ mwr,
                         const int32_t *__restrict__ vinst, const InstDesc *__restrict__ inst, int64_t N,
                         uint32_t flags, bool l2, const float *__restrict__ mw, int32_t *split, int32_t *qsplit,
-                        float *mwpre, int4 *vmeta, int4 *vcand, uint8_t *code, int64_t M, uint32_t *pkeys,
+                        float *mwpre, float *mwj, int4 *vmeta, int4 *vcand, uint8_t *code, int64_t M, uint32_t *pkeys,
                         uint32_t *pvals, unsigned long long *nsuf, unsigned long long *njoin) {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -489,18 +489,20 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
         // the join's prefix (external queries only obey the norm bound) and create boundary
         const int32_t js = (l2 && !need_cs) ? max(sp, ls) : sp;
         const int32_t jq = l2 ? max(qs, ls) : qs;
-        // maxweight(x') of the split and an upper bound of the join prefix's norm (float32 with
+        // maxweight(x') of the split and of the join's prefix, and an upper bound of the join prefix's norm (float32 with
         // every operation rounded up, so the bound can only come out above the exact norm;
         // times 1 + 1.1e-3 for the 1e-3 norm tolerance of the vectors it will be dotted with)
-        float best = 0.f, pss = 0.f;
+        float best = 0.f, bestj = 0.f, pss = 0.f;
         for (int64_t p = a + lane; p < a + js; p += 32) {
             const float c = cval[p];
             if (p < a + sp) best = fmaxf(best, c);
+            bestj = fmaxf(bestj, c);
             pss = __fmaf_ru(c, c, pss);
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
             best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+            bestj = fmaxf(bestj, __shfl_xor_sync(0xffffffffu, bestj, o));
             pss = __fadd_ru(pss, __shfl_xor_sync(0xffffffffu, pss, o));
         }
         if (lane == 0) {
@@ -509,6 +511,7 @@ __global__ void k_split(const int64_t *__restrict__ cptr, const int32_t *__restr
             split[x] = sp;
             qsplit[x] = qs;
             mwpre[x] = best;
+            if (mwj) mwj[x] = bestj;
             vmeta[x] = make_int4((int32_t)a, L, jq, __float_as_int(mw[x]));
             vcand[x] = make_int4((int32_t)a, js, rlim, __float_as_int(pn));
             code[x] = (uint8_t)((rank_bucket(rlim) >> 2) << 4 | pn4_code(pn));
@@ -880,6 +883,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         cv.put(d.split, (size_t)N);
         cv.put(d.qsplit, (size_t)N);
         cv.put(d.mwpre, (size_t)N);
+        if (ix->l2) cv.put(d.mwj, (size_t)N);
         cv.put(d.crank, (size_t)nnz);
         cv.put(d.cval, (size_t)nnz);
         cv.put(d.nnz_d, (size_t)M);
@@ -986,7 +990,7 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     unsigned long long *nsuf_d = err.p + 1;
     k_split<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N,
                                                     ix->flags, ix->l2, d.mw.p, d.split.p, d.qsplit.p, d.mwpre.p,
-                                                    d.vmeta.p, d.vcand.p, d.code.p, M, pkeys.p, pvals.p, nsuf_d,
+                                                    d.mwj.p, d.vmeta.p, d.vcand.p, d.code.p, M, pkeys.p, pvals.p, nsuf_d,
                                                     nsuf_d + 2);
     APS_LAUNCH_CHECK();
     // ---- a4: suffix inverted index
@@ -1095,7 +1099,7 @@ aps_status build_block_index(const aps_index *ix, BlockIndex &b, cudaStream_t s)
     if (N == 0 || nnz == 0) return APS_OK;  // (nothing to join)
     APS_CUDA(cudaMemsetAsync(sums.p, 0, 2 * sizeof(unsigned long long), s));
     k_split<<<rows_grid(N), T256, 0, s>>>(d.cptr.p, d.crank.p, d.cval.p, d.mwr.p, d.vinst.p, d.inst.p, N, ix->flags,
-                                          false, d.mw.p, split.p, qsplit.p, mwpre.p, b.vmeta.p, b.vcand.p, b.code.p, M,
+                                          false, d.mw.p, split.p, qsplit.p, mwpre.p, nullptr, b.vmeta.p, b.vcand.p, b.code.p, M,
                                           keys.p, vals.p, sums.p, sums.p + 1);
     APS_LAUNCH_CHECK();
     k_rows_of<<<grid_for(N * 32, T256), T256, 0, s>>>(d.cptr.p, N, erow.p);

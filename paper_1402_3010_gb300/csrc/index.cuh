@@ -5,7 +5,8 @@
 //   crank/cval  each row's components, re-ordered by dimension rank (rank local to the
 //               instance; ranks sort dimensions by decreasing non-zero count)
 //   len, mw, split, qsplit, mwpre [N]   |x|, maxweight(x), |x'| (unindexed prefix),
-//               remscore boundary, maxweight(x')
+//               remscore boundary, maxweight(x') of the split
+//   mwj[N]      maxweight of the join's prefix (below), where that reaches past the split
 //   mwr/nnzr[M] maxweight_i(V) and non-zero count by global rank
 //   lptr[M+1]   posting-list start by global rank
 //   crow[nnz]   the same rows interleaved as {int32 rank, float32 value} (8 bytes)
@@ -131,7 +132,7 @@ struct IndexArrays {
     DBuf<int4> vcand;
     DBuf<uint8_t> code;
     DBuf<int32_t> len, split, qsplit;
-    DBuf<float> mw, mwpre;
+    DBuf<float> mw, mwpre, mwj;
     DBuf<int32_t> rank_of_dim, dim_of_rank, nnz_d;
     DBuf<float> mw_d, mwr;
     DBuf<int64_t> lptr;
