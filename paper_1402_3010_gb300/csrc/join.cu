@@ -681,6 +681,12 @@ __device__ __forceinline__ void walk(const Tile &T, const int2 *__restrict__ pos
     }
 }
 
+// x * y in the units of A, to the nearest. dot(x, y') is summed in them like the entries of the
+// lists, so that a score is rounded to float32 once, wherever y's prefix ends.
+__device__ __forceinline__ uint32_t fixed_product(const float x, const float y) {
+    return __float2uint_rn(x * 1073741824.f * y);
+}
+
 // One class of windowed items with tile shape G: every warp takes units (a vector, or one
 // part of a heavy vector's windows) from the class's work list until it is empty.
 template <bool QMODE, bool SPLIT, bool COARSE>
@@ -932,19 +938,20 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 #pragma unroll 1
                 for (int b = 0; b < ns; b += 32) {
                     bool emit = false;
-                    float sc = 0.f, v = 0.f;
+                    float sc = 0.f;
+                    uint32_t sum = 0u;  // the score so far, in the units of A
                     int slot = 0;
                     int4 yc = make_int4(0, 0, 0, 0);  // {row offset, |y'|, first rank after y', ||y'||_2 bound}
                     // 0: rejected or emitted, 1: score known, 2: short dot(x, y') left, 3: long one
                     int stage = 0;
                     if (b + lane < ns) {
                         slot = T.list[b + lane];
-                        v = __uint2float_rn(T.A[slot]) * 9.31322574615478515625e-10f;  // 2^-30
+                        sum = T.A[slot];
+                        const float v = __uint2float_rn(sum) * 9.31322574615478515625e-10f;  // 2^-30
                         yc = __ldg(cands + slot);
                         if (SPLIT && blk >= 0) {  // a partial sum: y scored whole, in float64
                             stage = 4;
                         } else if (!f_upper || v + T.px[rank_bucket(yc.z)] * __int_as_float(yc.w) * 1.00001f > t - beta) {
-                            sc = v;
                             stage = yc.y == 0 ? 1 : (yc.y <= 16 ? 2 : 3);
                             // The paper's upperbound. On the 200k power-law set it stops 4% of what gets
                             // here, at no cost to be seen; a batch of 4096 queries takes 2% longer with
@@ -964,7 +971,6 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                     }
                     if (stage == 2) {  // short prefixes: each lane its own candidate
                         const int2 *yr = P.crow + (uint32_t)yc.x;
-                        float acc = 0.f;
                         int at = 0;  // both rows in rank order: x is searched from the last place on
 #pragma unroll 1
                         for (int k = 0; k < yc.y && at < xl; k++) {
@@ -972,10 +978,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                             at = row_find(xs, at, xl, e.x);
                             if (at < xl) {
                                 const int2 xe = xs[at];
-                                if (xe.x == e.x) acc = fmaf(__int_as_float(xe.y), __int_as_float(e.y), acc);
+                                if (xe.x == e.x) sum += fixed_product(__int_as_float(xe.y), __int_as_float(e.y));
                             }
                         }
-                        sc = v + acc;
                         stage = 1;
                     }
                     // long prefixes: the whole warp takes one candidate at a time, its lanes
@@ -984,20 +989,20 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                         const int src = __ffs(lm) - 1;
                         const uint32_t yo = (uint32_t)__shfl_sync(0xffffffffu, yc.x, src);
                         const int yl = __shfl_sync(0xffffffffu, yc.y, src);
-                        float acc = 0.f;
+                        uint32_t acc = 0u;
 #pragma unroll 1
                         for (int k = lane; k < yl; k += 32) {
                             const int2 e = __ldg(&P.crow[yo + k]);
-                            acc = fmaf(x_at(e.x, xs, xl), __int_as_float(e.y), acc);
+                            acc += fixed_product(x_at(e.x, xs, xl), __int_as_float(e.y));
                         }
-#pragma unroll
-                        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                        acc = __reduce_add_sync(0xffffffffu, acc);
                         if (lane == src) {
-                            sc = v + acc;
+                            sum += acc;
                             stage = 1;
                         }
                     }
                     if (stage == 1) {
+                        sc = __uint2float_rn(sum) * 9.31322574615478515625e-10f;
                         if (sc >= t + beta) {
                             emit = true;
                             stage = 0;
