@@ -203,9 +203,9 @@ aps_status aps_index_info(const aps_index *index, int32_t *n, int32_t *m, int64_
  * device arrays i, j, score (capacity pairs each); on APS_OK *count pairs sorted by
  * (i, j) are in them. All scratch comes from one fixed 64 MiB device array inside the
  * library (held by every GPU that loads this part of the library until exit) and the
- * join uses at most 32 CTAs. Limits: the index's arena slots (n times the windows of 40960 / G
- * ids that cover it, G from the tile table) must fit the arena with room left to stage pairs
- * (else APS_EINVAL, before any work), and the pairs
+ * join uses at most 32 CTAs. Limits: the index's size, counted in arena slots (n times the
+ * intervals of 40960 / G ids that cover it, G from the tile table) of 28 bytes each, must fit the
+ * arena beside 11.5 MB (else APS_EINVAL, before any work), and the pairs
  * must fit both the staging room and `capacity` (else APS_EOVERFLOW with *count = the
  * number of pairs). The current device must be the index's device, and i, j and score
  * must be device memory of that device (else APS_EINVAL). The first call on a device

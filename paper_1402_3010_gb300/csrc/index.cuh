@@ -31,6 +31,7 @@
 //   wlist[M]    then: where each list's starts begin in wptr << 6 | log2 of the windows of a group
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -223,6 +224,33 @@ struct QueryArrays {
 aps_status prepare_queries(const aps_index *ix, const int64_t *qptr, const int32_t *qidx, const float *qval,
                            int32_t nq, float t, uint32_t flags, cudaStream_t s, QueryArrays &qa,
                            int64_t nnz_known = -1);
+
+// The windows of a query are cut into as many parts (its slots) as give every warp of the chip some
+// 32 units.
+inline int query_parts(const aps_index *ix, int64_t nq) {
+    const InstDesc &I = ix->inst_h[0];
+    const int64_t n = std::max<int64_t>(nq, 1);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(I.nw, ((int64_t)num_sms() * tile_warps(I.G) * 32 + n - 1) / n));
+}
+constexpr int64_t QUERY_SLAB = 256;  // staging slots a warp reserves at a time: query batches are small
+inline int query_ctas(const aps_index *ix, int64_t nq) {
+    return (int)std::min<int64_t>(num_sms(), std::max<int64_t>(ix->inst_h[0].nw > 0 ? nq * query_parts(ix, nq) : 0, 1));
+}
+// Staging of a batch: the pairs per query that this index's batches have needed so far (at least
+// 64), plus one slab per warp.
+inline int64_t query_stage(const aps_index *ix, int64_t nq) {
+    const int64_t slack = (int64_t)query_ctas(ix, nq) * JOIN_WARPS * QUERY_SLAB;
+    return std::max<int64_t>(nq * ix->q_ppq16.load(std::memory_order_relaxed) / 16 + slack, (int64_t)1 << 16);
+}
+// Device bytes that a batch holds while it runs, at most (unless it has more pairs a query than any
+// before): its rows as they came, checked, keyed, sorted (two copies and the sort's tile states) and
+// packed, 60 bytes a component; row pointers, lengths, maxima and descriptions, 48 a query; count,
+// offset and run of every slot; the staged pairs with their slabs' chain, and the final ones.
+inline size_t query_bytes(const aps_index *ix, int64_t nq, int64_t nnz) {
+    const size_t slots = (size_t)nq * (size_t)query_parts(ix, nq), stage = (size_t)query_stage(ix, nq);
+    return ((size_t)1 << 20) + 60 * (size_t)nnz + 48 * (size_t)nq + slots * (4 + 8 + sizeof(Segment)) +
+           stage * sizeof(int2) + stage / QUERY_SLAB * sizeof(int2) + stage * 12;
+}
 
 // Match prepared queries against every indexed vector: pairs (query row, vector id, score)
 // with score >= t, sorted by (query, vector). Safe to call concurrently on different

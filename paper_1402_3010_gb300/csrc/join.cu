@@ -1814,7 +1814,7 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
     int2 *elists = reinterpret_cast<int2 *>(arena + off);
     off = align256(off + sizeof(int2) * (size_t)grid_max * JOIN_WARPS * JOIN_ECAP);
     if (limit >= arena_bytes || off + 4096 >= arena_bytes) {
-        set_error("index too large for the %zu-byte arena: its %lld (vector, window) slots need %zu bytes "
+        set_error("index too large for the %zu-byte arena: its %lld arena slots count as %zu bytes "
                   "before any pair is staged",
                   arena_bytes, (long long)ix->arena_slots, std::max(limit, off));
         return APS_EINVAL;
@@ -1895,12 +1895,10 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
     const int sms = num_sms();
     const int64_t nq = qa.nq;
     const int G = I.G;
-    // the windows of a query in as many parts as give every warp of the chip some 32 units
-    const int parts = (int)std::max<int64_t>(
-        1, std::min<int64_t>(I.nw, ((int64_t)sms * tile_warps(G) * 32 + nq - 1) / std::max<int64_t>(nq, 1)));
+    const int parts = query_parts(ix, nq);
     const int64_t nqw = std::max<int64_t>(nq * parts, 1);
     const int need = tile_bytes(G) * tile_warps(G);
-    const int64_t slab = 256;  // query batches are small: keep the slab tails short
+    const int64_t slab = QUERY_SLAB;
     APS_TRY(allow_smem(query_kernel(ix)));
     cudaEvent_t ev[3];
     for (int i = 0; i < 3; i++) APS_CUDA(cudaEventCreate(&ev[i]));
@@ -1911,18 +1909,15 @@ aps_status join_queries(const aps_index *ix, const QueryArrays &qa, float t, uin
         }
     } evg{ev};
     const int64_t nitems = I.nw > 0 ? nq : 0;
-    const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(nitems * parts, 1));
+    const int grid = query_ctas(ix, nq);
     DBuf<unsigned long long> ctr;  // 16 counters, then the pair counts of the query parts
     DBuf<int2> chain, stage;
     DBuf<Segment> segs;
     APS_TRY(ctr.alloc(16 + ((size_t)nqw + 1) / 2, s));
     int32_t *const cntq = reinterpret_cast<int32_t *>(ctr.p + 16);
     APS_TRY(segs.alloc((size_t)nqw, s));
-    // staging: the pairs per query this index's batches have needed so far (at least 64),
-    // plus one slab per warp
-    const int64_t ppq16 = ix->q_ppq16.load(std::memory_order_relaxed);
     const int64_t slack = (int64_t)grid * JOIN_WARPS * slab;
-    int64_t stage_cap = std::max<int64_t>(nq * ppq16 / 16 + slack, (int64_t)1 << 16);
+    int64_t stage_cap = query_stage(ix, nq);
     unsigned long long ch[16];
     for (int attempt = 0; attempt < 2; attempt++) {
         APS_TRY(stage.alloc((size_t)stage_cap, s));

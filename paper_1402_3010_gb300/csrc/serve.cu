@@ -150,7 +150,6 @@ struct aps_server {
     aps_index *ix = nullptr;
     size_t budget = 0;
     int slots = 0;
-    size_t fixed = 0;  // per-batch scratch independent of the batch size
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::deque<Request *> queue;
@@ -169,15 +168,6 @@ struct aps_server {
 };
 
 namespace {
-
-// Device bytes a batch may hold while it runs: per-warp emit lists, per-(query, window)
-// counts/offsets/segments, the staged and final pairs (64 per query assumed), query rows.
-size_t estimate(const aps_server *sv, int32_t nq, int64_t nnz) {
-    const InstDesc &I = sv->ix->inst_h[0];
-    const size_t nw = ((size_t)I.n * I.G + 40959) / 40960;  // (a query's slots, at most)
-    const size_t per_q = std::max<size_t>(nw, 1) * (4 + 8 + 16) + 64 * (8 + 12) + 64;
-    return sv->fixed + (size_t)nq * per_q + (size_t)nnz * 48;
-}
 
 void worker(aps_server *sv, int slot) {
     cudaSetDevice(sv->ix->device);
@@ -255,7 +245,6 @@ aps_status aps_server_create(aps_index *index, size_t mem_budget, int32_t slots,
     sv->ix = index;
     sv->budget = mem_budget;
     sv->slots = slots;
-    sv->fixed = (size_t)num_sms() * 32 * JOIN_ECAP * sizeof(int2) + (1u << 20);
     for (int i = 0; i < slots; i++) {
         cudaStream_t st;
         cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
@@ -352,7 +341,7 @@ aps_status aps_stream_submit(aps_server *sv, const aps_query_req *req, uint64_t 
     r->t = req->t;
     r->t_submit = now_s();
     std::lock_guard<std::mutex> lk(sv->mu);
-    r->est = estimate(sv, req->nq, nnz);
+    r->est = query_bytes(sv->ix, req->nq, nnz);
     r->ticket = sv->next_ticket++;
     sv->reqs[r->ticket] = r;
     sv->queue.push_back(r);

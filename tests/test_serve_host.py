@@ -188,6 +188,34 @@ int main() {
     aps_server_free(sv);
     return rc;
 }""",
+    # batches whose footprint leaves room for another run side by side: one query against a million rows
+    # holds some 20 MB (its staging most of all)
+    "small_batches_share_a_budget": r"""
+int main() {
+    index_of(1000000);
+    const int32_t id[1] = {3};
+    const float val[1] = {1.f};
+    const int64_t ptr[2] = {0, 1};
+    hold_for = 2;
+    for (size_t budget : {(size_t)48 << 20, (size_t)1}) {  // room for two; for none: one at a time
+        most = 0;
+        if (budget == 1) hold_for = 0;
+        aps_server *sv = nullptr;
+        if (aps_server_create(&ix, budget, 2, &sv) != APS_OK) return 1;
+        uint64_t tk[2];
+        const aps_query_req req = {ptr, id, val, 1, 0.5f};
+        for (uint64_t &t : tk)
+            if (aps_stream_submit(sv, &req, &t) != APS_OK) return 2;
+        for (uint64_t t : tk) {
+            aps_pairs out;
+            if (aps_stream_poll(sv, t, 10000000, &out) != APS_OK) return 3;
+        }
+        aps_server_free(sv);
+        printf("budget %zu: %d at once\n", budget, most);
+        if (most != (budget == 1 ? 1 : 2)) return 4;
+    }
+    return 0;
+}""",
 }
 
 
