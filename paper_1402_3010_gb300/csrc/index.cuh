@@ -104,9 +104,10 @@ struct Segment {
 // bytes a component, 28 a dimension); past that each list has the starts of as many groups of
 // 2^shift windows as there is room for, WLIST_ENTRIES for each of its entries, and the join searches
 // the group. Long lists, which are most of the work, thus keep every window, and a short
-// list's groups hold one entry or none. Where every window fits it is the better one: by list the
-// 200,000-row power-law set takes 34.5 ms a call (25.5), 4096 queries of a million rows 10.2 (7.3), a
-// batch of 512 instances 46.4 (43.2), and lists searched within 16 windows throughout 66 and 17 ms.
+// list's groups hold one entry or none. Two million rows of ten components over a million
+// dimensions: 0.63 GB and 105 ms in the join's kernel, 5.0 GB and 158 ms with every window. Where
+// most lists are long, every window is the better one: by list the 200,000-row power-law set takes
+// 28.1 ms a call (25.3), 4096 queries of a million rows 8.2 (7.0), a batch of 512 instances 45.9 (43.4).
 constexpr int WLIST_ENTRIES = 8;
 inline int64_t window_bytes(int64_t nnz, int64_t M) { return 4 * WLIST_ENTRIES * nnz + 16 * M; }
 

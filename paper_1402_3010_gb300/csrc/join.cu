@@ -253,32 +253,41 @@ __device__ __forceinline__ int64_t first_after(const int2 *__restrict__ post, in
     return m ? a + (__ffs(m) - 1) : b;
 }
 
-// Position in post of the first entry of window w of the list of global rank R, where the table holds
-// groups of windows (instance of nw windows of W ids).
-__device__ __forceinline__ uint32_t list_start(const uint64_t *__restrict__ wlist, const uint32_t *__restrict__ wptr,
-                                               const int64_t *__restrict__ lptr, const int2 *__restrict__ post,
-                                               const int64_t R, const int w, const int nw, const int W,
-                                               const int32_t idmask) {
-    const uint64_t d = __ldg(wlist + R);
-    const int shift = (int)(d & 63u), g = w >> shift;
-    uint32_t lo, hi;
-    if (window_groups(nw, shift) > 1) {
-        const uint32_t *const e = wptr + (d >> 6) + g;
-        lo = __ldg(e);
-        if (g << shift == w) return lo;
-        hi = __ldg(e + 1);
-    } else {
-        lo = (uint32_t)__ldg(lptr + R);
-        if (w == 0) return lo;
-        hi = (uint32_t)__ldg(lptr + R + 1);
-    }
-    if (w >= nw) return hi;
+// First position of post in [lo, hi) (one list, ids increasing) whose id is at or past `bound`, or hi.
+__device__ __forceinline__ uint32_t first_at(const int2 *__restrict__ post, uint32_t lo, uint32_t hi,
+                                             const uint32_t bound, const int32_t idmask) {
 #pragma unroll 1
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
-        if ((__ldg(&post[mid].x) & idmask) < w * W) lo = mid + 1; else hi = mid;
+        if ((uint32_t)(__ldg(&post[mid].x) & idmask) < bound) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// The part of the list of global rank R in window w, [s0, s1), where starts are stored by list
+// (instance of nw windows of W ids). Returns the list's starts where it has every window's, else null.
+__device__ __forceinline__ const uint32_t *list_range(const uint64_t *__restrict__ wlist,
+                                                      const uint32_t *__restrict__ wptr,
+                                                      const int64_t *__restrict__ lptr,
+                                                      const int2 *__restrict__ post, const int64_t R, const int w,
+                                                      const int nw, const int W, const int32_t idmask, uint32_t &s0,
+                                                      uint32_t &s1) {
+    const uint64_t d = __ldg(wlist + R);
+    const int shift = (int)(d & 63u);
+    const uint32_t *const starts = wptr + (d >> 6);
+    const bool grouped = window_groups(nw, shift) > 1;
+    if (grouped) {
+        s0 = __ldg(starts + (w >> shift));
+        s1 = __ldg(starts + (w >> shift) + 1);
+        if (shift == 0) return starts;
+    } else {
+        s0 = (uint32_t)__ldg(lptr + R);
+        s1 = (uint32_t)__ldg(lptr + R + 1);
+    }
+    const int within = (1 << shift) - 1;
+    if (w & within) s0 = first_at(post, s0, s1, (uint32_t)w * (uint32_t)W, idmask);
+    if (((w + 1) & within) && w + 1 < nw) s1 = first_at(post, s0, s1, (uint32_t)(w + 1) * (uint32_t)W, idmask);
+    return nullptr;
 }
 
 // The part of a posting list after x: [first, end) of list rank r of instance I (the
@@ -823,17 +832,31 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         // begin, so each window loads one position per list, for the window after it.
         const bool shortx = ncreate + qs <= 32;
         auto list_at = [&](const int r, const int w) -> uint32_t {
-            if (COARSE)
-                return list_start(in_block ? P.wlist_b : P.wlist, in_block ? P.wptr_b : P.wptr, lptr, post,
-                                  (int64_t)rbase + r, w, nw, IW, C.idmask);
             return nw > 1 ? __ldg(wp0 + (int64_t)r * (nw + 1) + w) : (uint32_t)__ldg(lptr + (rbase + r + w));
+        };
+        auto range_at = [&](const int r, const int w, uint32_t &s0, uint32_t &s1) {  // COARSE
+            return list_range(in_block ? P.wlist_b : P.wlist, in_block ? P.wptr_b : P.wptr, lptr, post, (int64_t)rbase + r,
+                              w, nw, IW, C.idmask, s0, s1);
         };
         int2 e0 = make_int2(0, 0);
         uint32_t p0 = 0, p1 = 0;
+        // COARSE: a list with every window's start is read like the table; of another one, which holds
+        // an entry in few windows, the id at p1 says whether there is anything to look for
+        const uint32_t *starts = nullptr;
+        uint32_t pend = 0, nextid = 0xffffffffu;
+        auto id_at = [&](const uint32_t q) { return q < pend ? (uint32_t)(__ldg(&post[q].x) & C.idmask) : 0xffffffffu; };
         if (shortx && lane < ncreate + qs) {
             e0 = xs[lane < ncreate ? qs + coff + lane * cstr : lane - ncreate];
-            p0 = list_at(e0.x, wa);
-            p1 = list_at(e0.x, wa + 1);
+            if (COARSE) {
+                starts = range_at(e0.x, wa, p0, p1);
+                if (!starts) {
+                    pend = (uint32_t)__ldg(lptr + (rbase + e0.x + 1));
+                    nextid = id_at(p1);
+                }
+            } else {
+                p0 = list_at(e0.x, wa);
+                p1 = list_at(e0.x, wa + 1);
+            }
         }
         uint32_t visits = 0;
 #pragma unroll 1
@@ -847,7 +870,20 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
             // blocks of 32 components and walked 32 at a time, because most lists of a long
             // vector have no entry in a given window.
             uint32_t p2 = p1;  // the next window's list ends
-            if (shortx && w + 1 < wz && lane < ncreate + qs) p2 = list_at(e0.x, w + 2);
+            if (shortx && w + 1 < wz && lane < ncreate + qs) {
+                if (!COARSE) {
+                    p2 = list_at(e0.x, w + 2);
+                } else if (starts) {
+                    p2 = __ldg(starts + w + 2);
+                } else if (const uint32_t bound = (uint32_t)(w + 2) * (uint32_t)IW; nextid < bound) {
+                    p2 = p1 + 1u;
+                    nextid = id_at(p2);
+                    if (nextid < bound) {
+                        p2 = first_at(post, p2 + 1u, pend, bound, C.idmask);
+                        nextid = id_at(p2);
+                    }
+                }
+            }
             uint32_t st = p0;
             int cnt = (int)(p1 - p0), k0 = 0;
             float xv = __int_as_float(e0.y);
@@ -862,8 +898,12 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                         uint32_t s0 = 0, s1 = 0;
                         if (k0 + lane < count) {
                             e = xs[create ? qs + coff + (k0 + lane) * cstr : k0 + lane];
-                            s0 = list_at(e.x, w);
-                            s1 = list_at(e.x, w + 1);
+                            if (COARSE) {
+                                range_at(e.x, w, s0, s1);
+                            } else {
+                                s0 = list_at(e.x, w);
+                                s1 = list_at(e.x, w + 1);
+                            }
                         }
                         const unsigned have = __ballot_sync(0xffffffffu, s1 > s0);
                         if (qn + __popc(have) > 32) break;  // no room: this block again, after the walk
