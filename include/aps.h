@@ -64,8 +64,7 @@ typedef enum aps_status {
  * for aps_build_index. The candidate map is always a dense array here, so each is the
  * paper's "-array" form; all-pairs-2 (every bound on) is the default. NO_UPPERBOUND also
  * turns off the ||y'||_2 pre-filter, the other bound that skips dot(x, y') (and the only one of
- * the two that queries take). Every variant
- * returns the same pairs; they differ in work. */
+ * the two that queries take). Every variant returns the same pairs; they differ in work. */
 #define APS_VARIANT_ALL_PAIRS_0 (APS_NO_PARTIAL_INDEX | APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND)
 #define APS_VARIANT_ALL_PAIRS_0_REMSCORE (APS_NO_PARTIAL_INDEX | APS_NO_MINSIZE | APS_NO_UPPERBOUND)
 #define APS_VARIANT_ALL_PAIRS_0_MINSIZE (APS_NO_PARTIAL_INDEX | APS_NO_REMSCORE | APS_NO_UPPERBOUND)
@@ -184,7 +183,8 @@ aps_status aps_query(aps_index *index, const int64_t *qptr, const int32_t *qidx,
  * NULL. Host arrays, caller-allocated, sizes: len/mw/split/qsplit/mw_pre [n],
  * rank_of_dim/nnz_d/mw_d [m], crank/cval [nnz] (components re-ordered by rank, the
  * CSR row pointers are the input's), list_ptr [m+1] (by rank), post_id/post_w [list_ptr[m]].
- * Errors: APS_EINVAL (NULL index), APS_ECUDA. */
+ * The lists are those of the split, which are made for the call where the join's own lists are
+ * shorter. Errors: APS_EINVAL (NULL index), APS_ENOMEM, APS_ECUDA. */
 aps_status aps_index_export(const aps_index *index, int32_t *len, float *mw, int32_t *nnz_d,
                             float *mw_d, int32_t *rank_of_dim, int32_t *crank, float *cval,
                             int32_t *split, int32_t *qsplit, float *mw_pre, int64_t *list_ptr,
@@ -270,11 +270,11 @@ aps_status aps_batch_all_pairs_csr(int32_t k, const int64_t *row_offsets, const 
 /* ---- join tile shapes and the autotuner ------------------------------------------ */
 /* The join's tile shape for an instance of n vectors: G = 1, 2, 4 or 8 (one warp per query
  * vector with a candidate window in shared memory, the blocks of Sec. 5.1.9 as tiles; G = 1
- * has the widest windows and the fewest warps). G is looked up by the instance's size bucket: bucket b
- * holds 1 + the previous bound <= n <= APS_TUNE_BOUND_b, with bounds 512, 1280, 2560,
- * 5120, 10240, 20480, 40960 and unbounded (aps_tune_bucket). The bucket bounds are the
- * work-split thresholds; the table is process-wide and read by every later index build
- * (aps_build_index and the batched calls). */
+ * has the widest windows and the fewest warps; 2, 4 and 8 are one shape). G is looked up by
+ * the instance's size bucket: bucket b holds 1 + the previous bound <= n <= APS_TUNE_BOUND_b,
+ * with bounds 512, 1280, 2560, 5120, 10240, 20480, 40960 and unbounded (aps_tune_bucket). The
+ * bucket bounds are the work-split thresholds; the table is process-wide and read by every
+ * later index build (aps_build_index and the batched calls). */
 #define APS_TUNE_BUCKETS 8
 
 typedef struct aps_tuning {

@@ -133,7 +133,8 @@ __device__ __forceinline__ unsigned long long bitonic_desc(unsigned long long x,
 // the lanes (place t * 32 + lane). Of 32 new keys those above the k-th so far go in one at a time,
 // or, when more than KNN_MERGE do, sorted and merged, so that a row in rising order costs no more
 // than its share. In a row of L neighbours in any order about k * ln(L / k) keys go in at all.
-// 200,000 rows of 400 at k = 16 take 0.37 ms, 1.20 when the row was read k times; the two
+// 200,000 rows of 400 at k = 16 take 0.38 ms a call, 1.21 when the row was read k times (rows whose
+// lengths differ widely, the ends drawn with probability rank^-1/2: 0.50 and 2.67); the two
 // arrays alone are 0.64 GB, 0.1 ms, and the rest is the 64-bit compares of the insertions.
 constexpr int KNN_MERGE = 8;
 constexpr int KNN_LOADS = 4;
@@ -398,10 +399,11 @@ aps_status graph_knn(const aps_graph *g, int32_t k, int32_t *nbr, float *wk, uin
         on = dn.p;
         ow = dw.p;
     }
-    // Up to eight by the lanes' own lists, whose cost grows with k but not with the order of a row
-    // (0.42 ms at k = 6 on the rows above, any order; the warp's list 0.25 in any order, 0.89 where
-    // a row's weights rise, and re-reading the row k times 0.47): from nine on that list is cheaper
-    // in any order, and no dearer than the k passes were from twelve on where they rise.
+    // Up to eight by the lanes' own lists, whose cost grows with k but not with the order of a row (ms
+    // a call on the rows above: 0.36 at k = 6, 0.45 at 8). From nine on by the warp's list: 0.30 at
+    // k = 9 in no order, and 0.90 at any k where a row's weights rise. Re-reading the row k times took
+    // 0.48 at k = 6, 0.70 at 9, 0.77, 0.84 and 0.92 at 12, in any order, so that of all rows those whose
+    // weights rise are dearer than that at k = 9 to 11.
     static constexpr decltype(&k_knn<1>) few[8] = {k_knn_few<1>, k_knn_few<2>, k_knn_few<3>, k_knn_few<4>,
                                                    k_knn_few<5>, k_knn_few<6>, k_knn_few<7>, k_knn_few<8>};
     const auto knn = k <= 8    ? few[k - 1]

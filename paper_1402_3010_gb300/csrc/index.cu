@@ -359,7 +359,7 @@ __global__ void k_canon_gather(const uint64_t *__restrict__ keys, const uint32_t
 // norm of the leading components, summed in float32 with every operation rounded up, can
 // reach t (times 1.0025 in the square for the norm tolerance of both vectors): no row scores
 // t on such a prefix, so a match has a later component in common. On the 200k power-law set
-// this takes the visits from 1.2e10 to about 3.8e9 and the candidates from 1.6e9 to 6e8.
+// this takes the visits from 1.2e10 to 2.2e9 and the candidates from 1.6e9 to 3.4e8.
 __device__ __forceinline__ double warp_incl_scan_f64(double v, int lane) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -745,7 +745,8 @@ __global__ void k_item_keys(const int64_t *__restrict__ cptr, const int32_t *__r
             // decreasing cost inside the class: the exponent and seven bits of the mantissa (costs
             // are 32 to 2^63), so that the sort takes two passes instead of four
             const uint32_t c = min((__float_as_uint(cost) - __float_as_uint(32.f)) >> 16, (1u << ITEM_COST_BITS) - 1u);
-            // (a merge of two long lists would be one warp's serial tail: those go by windows)
+            // (a merge of two long lists would be one warp's serial tail: those go by windows; 200,000
+            // rows with the line at 1024 / 8192 / 65536 entries / none: 21.9 / 21.6 / 22.0 / 22.0 ms)
             const int cls = b - a <= 1 || (b - a == 2 && lsum <= 8192) ? 4 : I.G == 1 ? 0 : I.G == 2 ? 1 : I.G == 4 ? 2 : 3;
             keys[x] = ((uint32_t)cls << ITEM_COST_BITS) | ((1u << ITEM_COST_BITS) - 1u - c);
             vals[x] = (uint32_t)x;
@@ -841,7 +842,9 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     // every bound on: the join may keep the norm-bounded prefixes to itself
     ix->l2 = !(ix->flags & (APS_NO_PARTIAL_INDEX | APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
     // A heavy vector's windows go to several warps where there are few vectors (2M slots at most)
-    // and enough windows for it: a vector's tables cost a unit about as much as a window does.
+    // and enough windows for it: a vector's tables cost a unit about as much as a window does. (Join
+    // ms with 1 / 4 / 8 / 16 / 32 parts: 30,000 power-law rows 5.6 / 2.2 / 1.68 / 1.75 / 1.78, 200,000
+    // rows 26.1 / 22.1 / 21.7 / 21.6 / 21.6.)
     ix->parts = maxnw < 4 ? 1 : (int32_t)std::max<int64_t>(1, std::min<int64_t>({16, maxnw, ((int64_t)1 << 21) / std::max<int64_t>(N, 1)}));
     ix->inst_h = inst;
     IndexArrays &d = ix->d;

@@ -47,7 +47,11 @@ constexpr int JOIN_THREADS = 32 * JOIN_WARPS;
 // with 12 / 16 / 20 / 24 warps: 200k power-law set 27.1 / 22.0 / 20.6 / 21.0, the 512-instance
 // batch 28.4 / 21.0 / 17.1 / 14.9; 28 and 32 warps spill registers and lose 5 to 30%), and G = 2,
 // 4 and 8 are the same shape; G = 1 has windows of twice the width.
-constexpr int JOIN_LCAP = 256;  // candidate list entries of a warp
+
+// Candidate list entries of a warp (join ms with 128 / 256 / 512: 30,000 power-law rows 2.25 / 1.75 /
+// 1.69, 200,000 rows 23.5 / 21.6 / 22.5, the 512-instance batch 18.0 / 14.9 / 14.0, 4096 queries 6.64 /
+// 6.60 / 6.92: a longer list takes its room from the window).
+constexpr int JOIN_LCAP = 256;
 constexpr int JOIN_SMEM = 232448 - 4096;  // of the 227 KB a CTA can have (the rest: the warps' states)
 __host__ __device__ constexpr int tile_warps(int G) { return G == 1 ? 12 : 24; }
 constexpr int JOIN_XCAP = 64;   // a query row of at most so many components is held in shared memory

@@ -27,10 +27,12 @@
 //      the warp reserves in bulk. The run of x (or of its part) is recorded at its slot.
 // A window with more candidates than the list holds is filtered from A itself, in stretches
 // of as many slots as the list has entries.
-// Instruction issue bounds it (2.1 to 2.5 a cycle and SM; no pipe, no memory level near its
-// limit). With groups of warps sharing a window, and barriers between these steps, and lists up
+// What bounds it is the latency of its loads with the 24 warps that 80 registers a thread allow: at
+// 50,000 rows a scheduler issues in 51% of the cycles (0.8 of its 6 warps ready), the top stall is the
+// long scoreboard (3.6 cycles an issue), and no pipe is above 30% nor L1 above 40 and L2 above 17%.
+// With groups of warps sharing a window, and barriers between these steps, and lists up
 // to the split alone, the 200,000-row power-law set took 37.2 ms and a batch of 512 instances
-// 58; 21.6 and 14.9 now. 4096 queries against a million rows take 7.2 ms a call (17.2).
+// 58; 21.6 and 14.9 now. 4096 queries against a million rows take 7.1 ms a call (17.2).
 // The output stage scans the per-slot counts and gathers the staged runs into (i, j, score)
 // arrays, which are then in (i, j) order without a sort.
 #include <algorithm>
@@ -1209,7 +1211,9 @@ __global__ void k_inst_offsets(const InstDesc *__restrict__ inst, int k, const i
 }
 
 // The heaviest vectors of a class whose windows are cut into parts: enough units for every warp
-// of the chip several times over.
+// of the chip several times over. (Join ms with 1024 / 2048 / 8192 / 32768 of them: 30,000 power-law
+// rows 2.8 / 2.27 / 1.75 / 1.65, 200,000 rows 22.3 / 21.55 / 21.6 / 21.75, 96 instances 1.92 / 1.92 /
+// 1.96 / 2.09.)
 constexpr int64_t JOIN_HEAVY = 8192;
 
 int join_smem() {

@@ -214,7 +214,8 @@ aps_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream
 }
 
 // ------------------------------------------------------------------ radix sort
-// Stable LSD radix sort, 8 bits a pass. One kernel counts the digits of every pass; a pass is
+// Stable LSD radix sort, 8 bits a pass, by the single-pass method with decoupled look-back (Merrill and
+// Garland's scan, 2016; Adinets and Merrill's sort, 2022). One kernel counts the digits of every pass; a pass is
 // then one kernel that reads each item once and writes it once: a tile ranks its items by warp,
 // publishes its digit counts, adds up the earlier tiles' by looking back over what they have
 // published, and writes its items out in digit runs. 40M keys with a payload take 0.37 ms a pass
