@@ -700,7 +700,7 @@ __device__ __forceinline__ uint32_t fixed_product(const float x, const float y) 
 
 // One class of windowed items with tile shape G: every warp takes units (a vector, or one
 // part of a heavy vector's windows) from the class's work list until it is empty.
-template <bool QMODE, bool SPLIT, bool COARSE>
+template <bool QMODE, bool SPLIT, bool COARSE, bool NOUPPER>
 __device__ __forceinline__ void join_class(const JoinParams &P, const int G, const int64_t item_begin,
                                            const int64_t item_end, const int64_t heavy, unsigned long long *const work,
                                            const bool f_minsize, const bool f_remscore, const bool f_upper,
@@ -823,12 +823,30 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         const float floor_ = f_upper || blk >= 0 ? t - beta : -1.f;
         // x's row in shared memory where it fits (verification searches it)
         const int2 *xs = xrow;
-        if (xl <= JOIN_XCAP) {
+        if (xl <= JOIN_XCAP || NOUPPER) {  // (NOUPPER: of a long row, the first components)
 #pragma unroll 1
-            for (int c = lane; c < xl; c += 32) T.xr[c] = __ldg(xrow + c);
-            xs = T.xr;
+            for (int c = lane; c < min(xl, JOIN_XCAP); c += 32) T.xr[c] = __ldg(xrow + c);
+            if (xl <= JOIN_XCAP) xs = T.xr;
             __syncwarp();
         }
+        // x's first component from `at` on whose rank is at least r, and a component. Without the upper
+        // bounds every candidate's prefix is looked up, and prefixes hold low ranks: the first components
+        // of a long row are in shared memory then (the paper's all-pairs-1 on the 200k power-law set: 284
+        // ms, 469 with long rows searched in global memory and empty prefixes verified).
+        auto x_find = [&](int at, const int r) -> int {
+            if (!NOUPPER) return row_find(xs, at, xl, r);
+            if (at < JOIN_XCAP) at = row_find(T.xr, at, min(xl, JOIN_XCAP), r);
+            return at < JOIN_XCAP ? at : row_find(xrow, at, xl, r);
+        };
+        auto x_comp = [&](const int at) -> int2 {
+            return !NOUPPER ? xs[at] : at < JOIN_XCAP ? T.xr[at] : __ldg(xrow + at);
+        };
+        auto x_value = [&](const int r) -> float {
+            if (!NOUPPER) return x_at(r, xs, xl);
+            const int at = x_find(0, r);
+            const int2 e = at < xl ? x_comp(at) : make_int2(-1, 0);
+            return e.x == r ? __int_as_float(e.y) : 0.f;
+        };
         // The lists of a short x stay in registers over the windows (a lane each, the creating
         // ones first), and so do their positions: a window's lists end where the next one's
         // begin, so each window loads one position per list, for the window after it.
@@ -968,7 +986,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
                         bool keep = false;
                         if (slot[u] >= 0) {
                             const float pn = (float)(code[u] & 15) * (PN4_STEP * 1.0001f);
-                            keep = fmaf(__uint2float_ru(T.A[slot[u]]), scale, T.px[(code[u] >> 4) * 4 + 3] * pn) > floor_;
+                            // (no prefix: A is the whole score)
+                            keep = fmaf(__uint2float_ru(T.A[slot[u]]), scale, T.px[(code[u] >> 4) * 4 + 3] * pn) >
+                                   (NOUPPER && (code[u] & 15) == 0 ? t - beta : floor_);
                             if (!keep) T.A[slot[u]] = 0u;
                         }
                         const unsigned bal = __ballot_sync(0xffffffffu, keep);
@@ -1017,9 +1037,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 #pragma unroll 1
                         for (int k = 0; k < yc.y && at < xl; k++) {
                             const int2 e = __ldg(yr + k);
-                            at = row_find(xs, at, xl, e.x);
+                            at = x_find(at, e.x);
                             if (at < xl) {
-                                const int2 xe = xs[at];
+                                const int2 xe = x_comp(at);
                                 if (xe.x == e.x) sum += fixed_product(__int_as_float(xe.y), __int_as_float(e.y));
                             }
                         }
@@ -1035,7 +1055,7 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 #pragma unroll 1
                         for (int k = lane; k < yl; k += 32) {
                             const int2 e = __ldg(&P.crow[yo + k]);
-                            acc += fixed_product(x_at(e.x, xs, xl), __int_as_float(e.y));
+                            acc += fixed_product(x_value(e.x), __int_as_float(e.y));
                         }
                         acc = __reduce_add_sync(0xffffffffu, acc);
                         if (lane == src) {
@@ -1065,7 +1085,7 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 #pragma unroll 1
                         for (int k = lane; k < yl; k += 32) {
                             const int2 e = __ldg(&P.crow[yo + k]);
-                            acc += (double)x_at(e.x, xs, xl) * (double)__int_as_float(e.y);
+                            acc += (double)x_value(e.x) * (double)__int_as_float(e.y);
                         }
 #pragma unroll
                         for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -1129,14 +1149,15 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
 }
 
 // QMODE: external queries against the index; SPLIT: a self-join whose work list may hold
-// dimension-block items (P.iblk); COARSE: window starts by list. Each is
+// dimension-block items (P.iblk); COARSE: window starts by list; NOUPPER: a self-join
+// without the upper bounds (the others read the flag). Each is
 // compiled separately, so that the plain self-join
 // carries none of the other paths' state.
-template <bool QMODE, bool SPLIT, bool COARSE>
+template <bool QMODE, bool SPLIT, bool COARSE, bool NOUPPER>
 __global__ void __launch_bounds__(JOIN_THREADS, 1) join_kernel(const __grid_constant__ JoinParams P) {
     const bool f_minsize = !(P.flags & APS_NO_MINSIZE);
     const bool f_remscore = !(P.flags & APS_NO_REMSCORE);
-    const bool f_upper = !(P.flags & APS_NO_UPPERBOUND);
+    const bool f_upper = !NOUPPER && !(P.flags & APS_NO_UPPERBOUND);
     __shared__ Stager stagers[JOIN_WARPS];
     __shared__ Totals totals[JOIN_WARPS];
     const int warp = threadIdx.x >> 5;
@@ -1160,7 +1181,7 @@ __global__ void __launch_bounds__(JOIN_THREADS, 1) join_kernel(const __grid_cons
             stream_short<COARSE>(P, work, item_begin, item_end, f_minsize, f_remscore, tot, S);
             continue;
         }
-        join_class<QMODE, SPLIT, COARSE>(P, G, item_begin, item_end, P.cls_heavy[cls], work, f_minsize, f_remscore, f_upper, S,
+        join_class<QMODE, SPLIT, COARSE, NOUPPER>(P, G, item_begin, item_end, P.cls_heavy[cls], work, f_minsize, f_remscore, f_upper, S,
                                  tot);
         bool later = false;  // another windowed class
         for (int c = cls + 1; c < P.ncls; c++) later = later || (P.cls_G[c] > 0 && P.cls_begin[c + 1] > P.cls_begin[c]);
@@ -1243,12 +1264,14 @@ int set_classes(JoinParams &P, const aps_index *ix, int parts, int max_ctas) {
 
 // The kernel for an index's self-join (split: with dimension-block items) or for queries of it.
 using JoinKernel = void (*)(const JoinParams);
-JoinKernel self_kernel(const aps_index *ix, bool split = false) {
-    if (split) return ix->wper >= 0 ? join_kernel<false, true, true> : join_kernel<false, true, false>;
-    return ix->wper >= 0 ? join_kernel<false, false, true> : join_kernel<false, false, false>;
+JoinKernel self_kernel(const aps_index *ix, uint32_t flags, bool split = false) {
+    const bool by_list = ix->wper >= 0;
+    if (split) return by_list ? join_kernel<false, true, true, false> : join_kernel<false, true, false, false>;
+    if (by_list) return join_kernel<false, false, true, false>;
+    return flags & APS_NO_UPPERBOUND ? join_kernel<false, false, false, true> : join_kernel<false, false, false, false>;
 }
 JoinKernel query_kernel(const aps_index *ix) {
-    return ix->wper >= 0 ? join_kernel<true, false, true> : join_kernel<true, false, false>;
+    return ix->wper >= 0 ? join_kernel<true, false, true, false> : join_kernel<true, false, false, false>;
 }
 aps_status allow_smem(JoinKernel k) {  // (the same for every index: the limit is shared by all threads)
     APS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, join_smem()));
@@ -1286,10 +1309,12 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
                           int64_t nslots, cudaStream_t s) {
     JoinGraph &G = ix->jgraph;
     const size_t ctr_bytes = 16 * sizeof(unsigned long long), cnt_bytes = sizeof(int32_t) * (size_t)nslots;
+    const JoinKernel kernel = self_kernel(ix, P.flags);
+    APS_TRY(allow_smem(kernel));
     if (G.launches++ == 0) {
         APS_CUDA(cudaMemsetAsync(ctr, 0, ctr_bytes, s));
         APS_CUDA(cudaMemsetAsync(cntq, 0, cnt_bytes, s));
-        self_kernel(ix)<<<grid, JOIN_THREADS, smem, s>>>(P);
+        kernel<<<grid, JOIN_THREADS, smem, s>>>(P);
         APS_LAUNCH_CHECK();
         return APS_OK;
     }
@@ -1300,7 +1325,7 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
         if (e == cudaSuccess) {
             cudaMemsetAsync(ctr, 0, ctr_bytes, cs);
             cudaMemsetAsync(cntq, 0, cnt_bytes, cs);
-            self_kernel(ix)<<<grid, JOIN_THREADS, smem, cs>>>(P);
+            kernel<<<grid, JOIN_THREADS, smem, cs>>>(P);
             cudaGraph_t g = nullptr;
             e = cudaStreamEndCapture(cs, &g);
             G.graph = g;
@@ -1339,7 +1364,7 @@ aps_status run_join_graph(aps_index *ix, JoinParams &P, int grid, int smem, unsi
         void *args[1] = {&P};
         cudaKernelNodeParams kp;
         memset(&kp, 0, sizeof(kp));
-        kp.func = reinterpret_cast<void *>(self_kernel(ix));
+        kp.func = reinterpret_cast<void *>(kernel);
         kp.gridDim = dim3((unsigned)grid);
         kp.blockDim = dim3(JOIN_THREADS);
         kp.sharedMemBytes = (unsigned)smem;
@@ -1443,7 +1468,6 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
         }
     } evg{ev};
     const int need = join_smem();
-    APS_TRY(allow_smem(self_kernel(ix)));
 
     // the vertical split: the costliest `heavy` vectors as nblk dimension blocks each
     const bool split = nblk >= 2 && heavy > 0 && ix->k == 1;
@@ -1464,7 +1488,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
         const int64_t nitems = ix->class_begin[JOIN_NCLS] - ix->class_begin[0];
         nsplit = std::min<int64_t>(heavy, ix->class_begin[4] - ix->class_begin[0]);
         if (nsplit > 0) {
-            APS_TRY(allow_smem(self_kernel(ix, true)));
+            APS_TRY(allow_smem(self_kernel(ix, flags, true)));
             const int64_t total = nitems + nsplit * (nblk - 1);
             APS_TRY(items2.alloc((size_t)total, s));
             APS_TRY(iblk.alloc((size_t)total, s));
@@ -1557,7 +1581,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out, std::ve
                                                   std::min(nsplit * nblk, 4 * JOIN_HEAVY) + JOIN_HEAVY);
                 APS_CUDA(cudaMemsetAsync(ctr.p, 0, 16 * sizeof(unsigned long long), s));
                 APS_CUDA(cudaMemsetAsync(cntq.p, 0, sizeof(int32_t) * std::max<int64_t>(nslots, 1), s));
-                self_kernel(ix, true)<<<grid, JOIN_THREADS, need, s>>>(P);
+                self_kernel(ix, flags, true)<<<grid, JOIN_THREADS, need, s>>>(P);
                 APS_LAUNCH_CHECK();
             } else {
                 APS_TRY(run_join_graph(ix, P, grid, need, ctr.p, cntq.p, nslots, s));
@@ -1871,14 +1895,15 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
     int2 *stage = reinterpret_cast<int2 *>(arena + off);
 
     const int need = join_smem();
-    APS_TRY(allow_smem(self_kernel(ix)));
+    const uint32_t flags = ix->flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND);
+    APS_TRY(allow_smem(self_kernel(ix, flags)));
     APS_CUDA(cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned long long), s));
     APS_CUDA(cudaMemsetAsync(cntq, 0, sizeof(int32_t) * nslots, s));
     if (ix->class_begin[JOIN_NCLS] > ix->class_begin[0]) {
         JoinParams P;
         set_index(P, ix);
         const int grid = set_classes(P, ix, 1, grid_max);
-        P.flags = ix->flags & (APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND);
+        P.flags = flags;
         P.stage = stage;
         P.stage_cap = stage_cap;
         P.stage_count = ctr + 5;
@@ -1889,7 +1914,7 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
         P.counters = ctr;
         P.work = ctr + 8;
         P.scratch = elists;
-        self_kernel(ix)<<<grid, JOIN_THREADS, need, s>>>(P);
+        self_kernel(ix, flags)<<<grid, JOIN_THREADS, need, s>>>(P);
         APS_LAUNCH_CHECK();
     }
     unsigned long long ch[16];
