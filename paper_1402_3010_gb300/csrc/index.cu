@@ -33,7 +33,7 @@ __device__ __forceinline__ int inst_of_rank(const InstDesc *inst, int k, int64_t
 
 // The start of a build in one launch: the row pointers' copy, every vector's instance, empty
 // dimension statistics and counters (err[0] all ones, the others 0) and, for a single instance,
-// its description (by value: no copy from the host). A copy or a reset of its own costs its
+// its description (by value: no copy from the host; its windows follow with the list pointers). A copy or a reset of its own costs its
 // caller 3 to 15 us, a tenth of the smallest builds in all.
 __global__ void k_setup(const int64_t *__restrict__ indptr, InstDesc one, InstDesc *inst, int k, int64_t N, int64_t M,
                         int64_t *cptr, int32_t *vinst, int32_t *nnz_d, float *mw_d, unsigned long long *err, int nerr) {
@@ -574,7 +574,10 @@ __global__ void k_post_fill(const uint32_t *__restrict__ vals, const int32_t *__
 
 // List pointers from the sorted posting keys: lptr[R] = first suffix entry with key >= R
 // (binary search; lptr[M] = nsuf).
-__global__ void k_lptr(const uint32_t *__restrict__ keys, int64_t nsuf, int64_t M, int64_t *lptr) {
+// `inst`, when given, takes a single instance's description with its windows (no copy from the host).
+__global__ void k_lptr(const uint32_t *__restrict__ keys, int64_t nsuf, int64_t M, int64_t *lptr, InstDesc one,
+                       InstDesc *inst) {
+    if (inst && blockIdx.x == 0 && threadIdx.x == 0) *inst = one;
     for (int64_t R = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; R <= M; R += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = nsuf;
         while (lo < hi) {
@@ -806,8 +809,8 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     ix->stream = s;
     // ---- host-side layout of instances: ranks, windows, classes
     std::vector<InstDesc> inst = inst_in;
-    int64_t N = 0, M = 0, arena_slots = 0, nwptr = 0;
-    int32_t maxm = 1, maxn = 1, maxnw = 1;
+    int64_t N = 0, M = 0, arena_slots = 0;
+    int32_t maxm = 1, maxn = 1;
     // tile shape per instance: G query groups per CTA from the size-bucket table (its
     // queryable column for indexes built to answer queries)
     const aps_tuning tu = tune ? *tune : tuning_current();
@@ -817,17 +820,12 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         I.vbase = N;
         I.rbase = (int32_t)M;
         I.G = gtab[tune_bucket(I.n)];
-        I.W = tile_window(I.G);
-        I.nw = I.n > 0 ? (int32_t)(((int64_t)I.n + I.W - 1) / I.W) : 0;
         I.packed = I.n < (1 << 24) ? 1 : 0;
-        I.wbase = nwptr;
         arena_slots += (int64_t)I.n * (((int64_t)I.n * I.G + 40959) / 40960);
-        if (I.nw > 1) nwptr += (int64_t)I.m * (I.nw + 1);
         N += I.n;
         M += I.m;
         maxm = std::max(maxm, I.m);
         maxn = std::max(maxn, I.n);
-        maxnw = std::max(maxnw, I.nw);
     }
     if (M >= (1ll << 31) || N >= (1ll << 31)) {
         set_error("too many vectors or dimensions (limit 2^31 - 1)");
@@ -836,17 +834,9 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
     ix->N = N;
     ix->M = M;
     ix->arena_slots = arena_slots;
-    ix->nwptr = nwptr;
     ix->maxm = maxm;
-    ix->maxnw = maxnw;
     // every bound on: the join may keep the norm-bounded prefixes to itself
     ix->l2 = !(ix->flags & (APS_NO_PARTIAL_INDEX | APS_NO_MINSIZE | APS_NO_REMSCORE | APS_NO_UPPERBOUND));
-    // A heavy vector's windows go to several warps where there are few vectors (2M slots at most)
-    // and enough windows for it: a vector's tables cost a unit about as much as a window does. (Join
-    // ms with 1 / 4 / 8 / 16 / 32 parts: 30,000 power-law rows 5.6 / 2.2 / 1.68 / 1.75 / 1.78, 200,000
-    // rows 26.1 / 22.1 / 21.7 / 21.6 / 21.6.)
-    ix->parts = maxnw < 4 ? 1 : (int32_t)std::max<int64_t>(1, std::min<int64_t>({16, maxnw, ((int64_t)1 << 21) / std::max<int64_t>(N, 1)}));
-    ix->inst_h = inst;
     IndexArrays &d = ix->d;
 
     // the first and the last row pointer, as one strided copy where its pitch may be that wide
@@ -866,14 +856,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         return APS_EINVAL;
     }
     ix->nnz = nnz;
-    // the table of window starts: every window's where that takes no more than its share and, when it
-    // is large, an eighth of the memory at hand; else by list
-    if (4 * nwptr > window_bytes(nnz, M) || (4 * nwptr > WPTR_LARGE && (uint64_t)nwptr > memory_at_hand() / 32)) {
-        ix->wper = WLIST_ENTRIES;
-        const uint64_t room = memory_at_hand() / 32;
-        while (ix->wper > 0 && (uint64_t)ix->wper * (uint64_t)nnz * 4 > WPTR_LARGE && (uint64_t)ix->wper * (uint64_t)nnz > room)
-            ix->wper /= 2;
-    }
     Carver cv;
     cv.s = s;
     for (int pass = 0; pass < 2; pass++) {
@@ -945,6 +927,43 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
             set_error("invalid input at row %lld: %s", row, code_name(code));
         return APS_EINVAL;
     }
+    // windows, and the table of their starts with every window
+    int64_t nwptr = 0;
+    int32_t maxnw = 1;
+    const auto set_windows = [&](int halvings) {
+        nwptr = 0;
+        maxnw = 1;
+        for (InstDesc &I : inst) {
+            I.W = tile_window(I.G) >> halvings;
+            I.nw = I.n > 0 ? (int32_t)(((int64_t)I.n + I.W - 1) / I.W) : 0;
+            I.wbase = nwptr;
+            if (I.nw > 1) nwptr += (int64_t)I.m * (I.nw + 1);
+            maxnw = std::max(maxnw, I.nw);
+        }
+    };
+    int halvings = 0;
+    while (halvings < WINDOW_HALVINGS && N < WINDOWS_LEAST * (tile_window(2) >> halvings)) halvings++;
+    const bool uneven = longest_row > (unsigned long long)(8 * nnz / std::max<int64_t>(N, 1));
+    if (uneven && halvings > 0) halvings = std::min(halvings + 1, WINDOW_HALVINGS);
+    set_windows(halvings);
+    if (maxnw < 4) set_windows(halvings = 0);  // (too few to be cut all the same)
+    while (halvings > 0 && 4 * nwptr > window_bytes(nnz, M)) set_windows(--halvings);  // (wide tables: wide windows)
+    ix->nwptr = nwptr;
+    ix->maxnw = maxnw;
+    // A heavy vector's windows go to several warps where there are few vectors (2M slots at most)
+    // and enough windows for it: a vector's tables cost a unit about as much as a window does. (Join
+    // ms with 1 / 4 / 8 / 16 / 32 parts: 30,000 power-law rows 5.6 / 2.2 / 1.68 / 1.75 / 1.78, 200,000
+    // rows 26.1 / 22.1 / 21.7 / 21.6 / 21.6.)
+    ix->parts = maxnw < 4 ? 1 : (int32_t)std::max<int64_t>(1, std::min<int64_t>({16, maxnw, ((int64_t)1 << 21) / std::max<int64_t>(N, 1)}));
+    ix->inst_h = inst;
+    // the table of window starts: every window's where that takes no more than its share and, when it
+    // is large, an eighth of the memory at hand; else by list
+    if (4 * nwptr > window_bytes(nnz, M) || (4 * nwptr > WPTR_LARGE && (uint64_t)nwptr > memory_at_hand() / 32)) {
+        ix->wper = WLIST_ENTRIES;
+        const uint64_t room = memory_at_hand() / 32;
+        while (ix->wper > 0 && (uint64_t)ix->wper * (uint64_t)nnz * 4 > WPTR_LARGE && (uint64_t)ix->wper * (uint64_t)nnz > room)
+            ix->wper /= 2;
+    }
     if (nnz > 0 && k > 1 && maxm <= DIMSTATS_DIMS) {  // a batch of small instances: one CTA each
         const int sm = (int)(sizeof(uint32_t) * (size_t)maxm);
         // (the kernel's limit is shared by every thread: the same for every batch)
@@ -1012,7 +1031,8 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
                                                                    d.inst.p, ix->njoin, d.post.p);
             APS_LAUNCH_CHECK();
         }
-        k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p);
+        if (k > 1) APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
+        k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p, inst[0], k == 1 ? d.inst.p : nullptr);
         APS_LAUNCH_CHECK();
         APS_TRY(window_starts(ix, d.lptr, d.post, d.wptr, d.wlist, s));
         APS_TRY(d.crow.alloc((size_t)std::max<int64_t>(nnz, 1), s));
@@ -1075,7 +1095,7 @@ aps_status export_postings(const aps_index *ix, DBuf<int64_t> &lptr, DBuf<int2> 
                                                               ix->nsuf, post.p);
         APS_LAUNCH_CHECK();
     }
-    k_lptr<<<grid_for(ix->M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, ix->M, lptr.p);
+    k_lptr<<<grid_for(ix->M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, ix->M, lptr.p, ix->inst_h[0], nullptr);
     APS_LAUNCH_CHECK();
     return APS_OK;
 }
@@ -1113,7 +1133,7 @@ aps_status build_block_index(const aps_index *ix, BlockIndex &b, cudaStream_t s)
                                                               ix->nsuf, b.post.p);
         APS_LAUNCH_CHECK();
     }
-    k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, M, b.lptr.p);
+    k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->nsuf, M, b.lptr.p, ix->inst_h[0], nullptr);
     APS_LAUNCH_CHECK();
     return window_starts(ix, b.lptr, b.post, b.wptr, b.wlist, s);
 }

@@ -84,7 +84,7 @@ struct InstDesc {
     int32_t m;       // dimensions
     int32_t rbase;   // first global rank
     int32_t nw;      // candidate windows
-    int32_t W;       // window width
+    int32_t W;       // window width, at most tile_window(G)
     int32_t G;       // tile shape of this instance's class
     float t;         // threshold
     int32_t packed;  // 1: posting ids carry the size class in their top byte
@@ -101,6 +101,15 @@ struct Segment {
     int32_t next;  // slab of the next piece, or -1
     int32_t _pad;
 };
+
+// Windows of a set of few vectors are halved, at most WINDOW_HALVINGS times, until there are
+// WINDOWS_LEAST of them, which are then cut into parts for a heavy vector (a row of 2,000 components is
+// otherwise one warp's work), and once more where rows are uneven, the longest more than eight times
+// the mean. Kernel ms with windows of 1792 / 896 / 448 / 224 ids: 2,000 power-law rows (t = 0.5) 0.56 /
+// 0.64 / 0.22 / 0.19, 5,000 (t = 0.3) 1.53 / 0.44 / 0.36 / 0.45, 20,000 1.62 / 1.59 / 1.77 / 2.2, 200,000
+// 21.7 / 34.9 / 62.7 / 99; even rows of 100, 8,000 of them, 0.91 / 0.83 / 0.86 / 0.90. (Calls between:
+// 14,000 power-law rows take 1.19 and 1.01 ms at two widths of dimensions, 1.13 and 1.05 with 896.)
+constexpr int WINDOW_HALVINGS = 3, WINDOWS_LEAST = 4;
 
 // The table of window starts. With every window of every list it takes n * m / 448 bytes, whatever
 // the lists hold, so a wide sparse set's would outgrow the rest of its index (ten million rows of

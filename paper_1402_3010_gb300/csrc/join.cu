@@ -553,8 +553,8 @@ __device__ __forceinline__ void stream_short(const JoinParams &P, unsigned long 
 
 // A warp's part of shared memory.
 struct Tile {
-    uint32_t *A;     // [W] accumulated scores, fixed point, units of 2^-30
-    uint32_t *bm;    // [W / 32] the window's matches
+    uint32_t *A;     // [tile_window(G)] accumulated scores, fixed point, units of 2^-30
+    uint32_t *bm;    // [tile_window(G) / 32] the window's matches
     float *px;       // [64] norm of x on the rank buckets 0 .. b
     int4 *wait;      // [32] lists of a long x waiting for a walk: {first position, entries, x's value, -}
     int2 *seg;       // [32] the lists of a run: {first position - place in the run, x's value scaled by 2^30}
@@ -709,7 +709,6 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp >= tile_warps(G)) return;
     const int W = tile_window(G);
-    const uint32_t wmagic = 0xffffffffu / (uint32_t)W + 1u;  // a / W is the high word of a * wmagic, or less by one
     const unsigned lt_mask = (1u << lane) - 1u;
     Tile T;
     T.A = reinterpret_cast<uint32_t *>(smem + (size_t)warp * tile_bytes(G));
@@ -759,12 +758,9 @@ __device__ __forceinline__ void join_class(const JoinParams &P, const int G, con
         const float beta = fmaxf(1e-5f, (float)(xl + 2) * 1.1920929e-7f);  // (|x|+2) * 2^-23
         if (qs >= xl) continue;  // no component may create: x has no candidate at all
         // the windows of this unit: its share of those from x's successor on
-        const int nw = I.nw, IW = W, In = I.n;
+        const int nw = I.nw, IW = I.W, In = I.n;
         int wfirst = 0;
-        if (!QMODE && nw > 1) {
-            wfirst = (int)__umulhi((uint32_t)lx + 1u, wmagic);
-            while ((uint32_t)wfirst * (uint32_t)W > (uint32_t)lx + 1u) wfirst--;
-        }
+        if (!QMODE && nw > 1) wfirst = (lx + 1) / IW;
         const uint32_t *const wp0 = (in_block ? P.wptr_b : P.wptr) + I.wbase;
         const int64_t *const lptr = in_block ? P.lptr_b : P.lptr;
         const int2 *const post = in_block ? P.post_b : P.post;
