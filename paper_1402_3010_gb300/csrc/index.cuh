@@ -317,7 +317,7 @@ aps_status join_all_pairs(aps_index *ix, uint32_t flags, aps_pairs *out,
 // (arena_bytes, 256-byte aligned) and at most max_ctas CTAs; pairs land in the caller's
 // arrays (capacity cap). *count receives the number of pairs, also on APS_EOVERFLOW.
 aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes, int max_ctas, int32_t *oi,
-                        int32_t *oj, float *os, int64_t cap, int64_t *count, cudaStream_t s);
+                        int32_t *oj, float *os, int64_t cap, int64_t *count, cudaStream_t s, int parts = -1);
 
 // Dense all-pairs of X[n, d] (float32 rows; host or device per APS_DEVICE_PTRS) on the
 // tensor cores with exact rescoring; d % 64 == 0, 64 <= d <= 512.

@@ -1860,12 +1860,16 @@ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 }  // namespace
 
 aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes, int max_ctas, int32_t *oi,
-                        int32_t *oj, float *os, int64_t cap, int64_t *count, cudaStream_t s) {
+                        int32_t *oj, float *os, int64_t cap, int64_t *count, cudaStream_t s, int parts) {
     const int grid_max = std::max(1, std::min(num_sms(), max_ctas));
     // The documented limit: 28 bytes for each of the index's arena slots beside the fixed parts.
     const size_t limit = (size_t)std::max<int64_t>(ix->arena_slots, 1) * 28 + (size_t)max_ctas * 32 * 1408 * sizeof(int2);
     const int64_t slab = 32;  // small slabs: the arena's staging room is modest
-    const int64_t nslots = std::max<int64_t>(ix->N, 1);
+    // The heaviest vectors' windows in parts, as in the allocating join, where their slots take no
+    // more than a sixteenth of the arena; if the pairs then do not fit the rest, once more in one.
+    const int64_t part_room = (int64_t)(arena_bytes / 16 / (sizeof(int32_t) + sizeof(int64_t) + sizeof(Segment)));
+    if (parts < 0) parts = (int)std::max<int64_t>(1, std::min<int64_t>(ix->parts, part_room / std::max<int64_t>(ix->N, 1)));
+    const int64_t nslots = std::max<int64_t>(ix->N * parts, 1);
     size_t off = 0;
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(arena + off);
     off = align256(off + 16 * sizeof(unsigned long long));
@@ -1898,7 +1902,7 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
     if (ix->class_begin[JOIN_NCLS] > ix->class_begin[0]) {
         JoinParams P;
         set_index(P, ix);
-        const int grid = set_classes(P, ix, 1, grid_max);
+        const int grid = set_classes(P, ix, parts, grid_max);
         P.flags = flags;
         P.stage = stage;
         P.stage_cap = stage_cap;
@@ -1918,6 +1922,8 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
     APS_CUDA(cudaStreamSynchronize(s));
     const int64_t total = (int64_t)ch[3];
     *count = total;
+    if ((int64_t)ch[5] > stage_cap && parts > 1)
+        return join_noalloc(ix, arena, arena_bytes, max_ctas, oi, oj, os, cap, count, s, 1);
     if ((int64_t)ch[5] > stage_cap) {
         set_error("%lld staged pairs (%lld emitted) exceed the arena's staging room of %lld pairs",
                   (long long)ch[5], (long long)total, (long long)stage_cap);
@@ -1927,11 +1933,11 @@ aps_status join_noalloc(aps_index *ix, unsigned char *arena, size_t arena_bytes,
         set_error("%lld pairs do not fit the caller's capacity of %lld", (long long)total, (long long)cap);
         return APS_EOVERFLOW;
     }
-    k_scan_single<<<1, SCAN1_THREADS, 0, s>>>(cntq, ix->N, qwoff);
+    k_scan_single<<<1, SCAN1_THREADS, 0, s>>>(cntq, ix->N * parts, qwoff);
     APS_LAUNCH_CHECK();
     if (total > 0) {
-        k_gather<<<grid_for(ix->N * 32, 256, (int64_t)num_sms() * 32), 256, 0, s>>>(segs, chain, slab, cntq, ix->N,
-                                                                                   stage, qwoff, oi, oj, os);
+        k_gather<<<grid_for(nslots * 32, 256, (int64_t)num_sms() * 32), 256, 0, s>>>(segs, chain, slab, cntq, nslots,
+                                                                                    stage, qwoff, oi, oj, os);
         APS_LAUNCH_CHECK();
     }
     APS_CUDA(cudaStreamSynchronize(s));

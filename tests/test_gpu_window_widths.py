@@ -84,3 +84,23 @@ def test_batch_of_small_instances(aps):
     outs, _ = aps.aps_batch_all_pairs([(c.indptr, c.idx, c.val, c.n, c.m, t) for c in sets])
     for p, c in zip(outs, sets):
         compare(*_take(aps, p), oracle.bruteforce(c, t), t, c.n, csr=c)
+
+
+def test_noalloc_pairs_that_fit_the_arena_without_parts_alone(aps):
+    """3745 equal rows: 7,010,640 pairs. The arena stages 7,069,248 where each vector has one slot, and
+    6,938,560 with the slots of nine parts a vector: the join runs again in one part."""
+    import torch
+
+    n = 3745
+    ptr = np.arange(n + 1, dtype=np.int64) * 3
+    idx, val = np.tile(np.arange(3, dtype=np.int32), n), np.full(3 * n, 3 ** -0.5, np.float32)
+    h = aps.aps_build_index(ptr, idx, val, n, 3, 0.9)
+    try:
+        want = n * (n - 1) // 2
+        out = [torch.empty(want, dtype=d, device="cuda") for d in (torch.int32, torch.int32, torch.float32)]
+        assert aps.aps_all_pairs_noalloc(h, *out) == want
+    finally:
+        aps.aps_index_free(h)
+    i, j = np.triu_indices(n, 1)
+    assert np.array_equal(out[0].cpu().numpy(), i) and np.array_equal(out[1].cpu().numpy(), j)
+    assert np.abs(out[2].cpu().numpy() - 1).max() < 1e-5
