@@ -1020,6 +1020,8 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
         DBuf<uint32_t> &keys = pkeys;
         DBuf<uint32_t> &vals = pvals;
         unsigned long long cnt3[3] = {0, 0, 0};  // by split, (longest row), in the join's lists
+        // (a batch's descriptions with their windows; waited for here, as `inst` goes with this call)
+        if (k > 1) APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
         APS_CUDA(cudaMemcpyAsync(cnt3, nsuf_d, sizeof(cnt3), cudaMemcpyDeviceToHost, s));
         APS_CUDA(cudaStreamSynchronize(s));
         ix->nsuf = (int64_t)cnt3[0];
@@ -1031,7 +1033,6 @@ aps_status build_index_device(aps_index *ix, const int64_t *indptr, const int32_
                                                                    d.inst.p, ix->njoin, d.post.p);
             APS_LAUNCH_CHECK();
         }
-        if (k > 1) APS_CUDA(cudaMemcpyAsync(d.inst.p, inst.data(), sizeof(InstDesc) * k, cudaMemcpyHostToDevice, s));
         k_lptr<<<grid_for(M + 1, T256), T256, 0, s>>>(keys.p, ix->njoin, M, d.lptr.p, inst[0], k == 1 ? d.inst.p : nullptr);
         APS_LAUNCH_CHECK();
         APS_TRY(window_starts(ix, d.lptr, d.post, d.wptr, d.wlist, s));
