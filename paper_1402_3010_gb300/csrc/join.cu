@@ -26,10 +26,12 @@
 //   5. emit: the bitmap is walked in id order and the (y, score) go to the staging slab that
 //      the warp reserves in bulk. The run of x (or of its part) is recorded at its slot.
 // A window with more candidates than the list holds is filtered from A itself, in stretches
-// of as many slots as the list has entries.
+// of as many slots as the list has entries. (Such windows are dearer than they were with groups of
+// warps, 1.3 to 1.8 times at loose thresholds or over a few dozen dimensions; scanning them in the
+// filter's own loop was no better, 5.9 against 5.2 ms for 50,000 rows at t = 0.4.)
 // What bounds it is the latency of its loads with the 24 warps that 80 registers a thread allow: at
-// 50,000 rows a scheduler issues in 51% of the cycles (0.8 of its 6 warps ready), the top stall is the
-// long scoreboard (3.6 cycles an issue), and no pipe is above 30% nor L1 above 40 and L2 above 17%.
+// 50,000 rows a scheduler issues in half of the cycles (0.8 of its 6 warps ready), the top stall is the
+// long scoreboard (3.7 cycles an issue), no pipe is above 30%, L1 at 40% and L2 at 17%.
 // With groups of warps sharing a window, and barriers between these steps, and lists up
 // to the split alone, the 200,000-row power-law set took 37.2 ms and a batch of 512 instances
 // 58; 21.6 and 14.9 now. 4096 queries against a million rows take 7.1 ms a call (17.2).
